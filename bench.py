@@ -329,12 +329,19 @@ def host_description():
 # Our arm
 # ---------------------------------------------------------------------------
 
-def plan_plain(m, spl, wave=False):
+def plan_plain(m, spl, wave=False, most=0):
     """Launch sizes of m plain steps as the library groups them: launches of
     spl steps (four only on the wavefront schedule, else three), a remainder
     of one avoided where possible (4 = 2 + 2, 5 = 3 + 2), then pairs, then
-    single steps."""
+    single steps.  most > 4: FP32 on the wavefront schedule, whose launches
+    take up to that many steps (lbm_get_launch_steps)."""
     sizes = []
+    if most > 4:
+        while m >= 2:
+            k = most if m >= most and m != most + 1 else ((most + 1) // 2 if m == most + 1 else m)
+            sizes.append(k)
+            m -= k
+        return sizes + [1] * m
     big = 4 if spl >= 4 and wave else (3 if spl >= 3 else 0)
     if big:
         groups, r = divmod(m, big)
@@ -358,19 +365,19 @@ def check_launch_steps(w, spl, wave=False):
     return 4 if (wave and spl >= 4 and w >= 4) else min(spl, 2, w)
 
 
-def launches_per_iterate(iters, check_every, spl, wave=False):
+def launches_per_iterate(iters, check_every, spl, wave=False, most=0):
     """Stream-collide launches of lbm_iterate_checked(iters, check_every) from
     step 0: each window is check_every - 1 plain steps grouped into launches of
     spl steps (the remainder in shorter ones) and ends with the check step,
     the last step of the window's last launch (check_launch_steps)."""
     def window(w):
         last = check_launch_steps(w, spl, wave)
-        return len(plan_plain(w - last, spl, wave)) + 1
+        return len(plan_plain(w - last, spl, wave, most)) + 1
     total, left = 0, iters
     while left >= check_every:
         total += window(check_every)
         left -= check_every
-    return total + len(plan_plain(left, spl, wave))
+    return total + len(plan_plain(left, spl, wave, most))
 
 
 def time_variant(args, dtype, gx_d, gy_d, torch, P, nsteps, nwarm, events=True, spl=None, iters=None,
@@ -394,7 +401,8 @@ def time_variant(args, dtype, gx_d, gy_d, torch, P, nsteps, nwarm, events=True, 
 
     ce = args.check_every
     windows, rest = divmod(iters, ce)
-    block, big = dominant_block(ce, spl, wave_on)
+    most = P.lbm_get_launch_steps(lat.ctx)
+    block, big = dominant_block(ce, spl, wave_on, most)
     nev = nsteps * windows
 
     def one_step(ev_a=None, ev_b=None, dom=None):
@@ -439,7 +447,7 @@ def time_variant(args, dtype, gx_d, gy_d, torch, P, nsteps, nwarm, events=True, 
     dom_launches = nev * (block // big)
     lat.close()
     del out5
-    per_iter = launches_per_iterate(iters, args.check_every, spl, wave_on)
+    per_iter = launches_per_iterate(iters, args.check_every, spl, wave_on, most)
     checks = iters // args.check_every      # each adds one residual-finish launch
     return {"total_ms": total_ms, "iter_ms": iter_ms, "steps": nsteps, "spl": spl, "iters": iters,
             "step_launches": nsteps * per_iter, "launches": nsteps * (per_iter + checks + 1),
@@ -456,12 +464,12 @@ def fp64_peak(P):
         return FP64_PEAK_GINST, "nominal GB300 FP64 rate (1.25 TFLOP/s with FMA = 2 flops); measurement failed: %s" % e
 
 
-def dominant_block(check_every, spl, wave=False):
+def dominant_block(check_every, spl, wave=False, most=0):
     """(steps, k): the first steps of a residual window, which the library
     runs as whole plain launches of k steps each, k the longest launch of the
     window (lbm_iterate_checked plans the window's check_every - 1 plain steps
     so; see plan_plain)."""
-    sizes = plan_plain(check_every - check_launch_steps(check_every, spl, wave), spl, wave)
+    sizes = plan_plain(check_every - check_launch_steps(check_every, spl, wave), spl, wave, most)
     if not sizes:
         return 0, spl
     big = sizes[0]
@@ -565,7 +573,7 @@ def run_ours(args, ws, rank, local):
             "config": workload_config(args),
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": traffic,
-                         "kernel": ("k_wave<%s,%d> (%d fused stream-collide steps per launch, "
+                         "kernel": ("k_strip<%s,%d> (%d fused stream-collide steps per launch, "
                                     "wavefront schedule)" % (args.dtype, spl, spl)) if res["wave"] else
                                    {1: "k_step<%s> (fused stream-collide)",
                                     2: "k_step2<%s> (two fused stream-collide steps per launch)",

@@ -148,7 +148,10 @@ int lbm_get_host_transfer(lbm_ctx *ctx, int *mode);
  * that of the same steps taken one per launch, bit for bit.  With LBM_F16S
  * storage the intermediate states are not rounded to the FP16 storage format,
  * so results differ from one step per launch by less than that format's
- * rounding (and lie closer to the FP64 result).  Available for LBM_F32 and
+ * rounding (and lie closer to the FP64 result).  Since the grouping cannot
+ * change an LBM_F32 state, k = 4 on the wavefront schedule lets LBM_F32
+ * launches take as many steps as suit the lattice, up to seven
+ * (lbm_get_launch_steps); LBM_F16S keeps groups of four.  Available for LBM_F32 and
  * LBM_F16S storage on any lattice; the default is 4 (wavefront schedule) from
  * nx >= 256 and ny >= 8 on, else 3 from nx >= 64 and ny >= 16 on (a smaller
  * lattice fills the on-chip tile more than once and is faster one step per
@@ -159,19 +162,22 @@ int lbm_get_host_transfer(lbm_ctx *ctx, int *mode);
 int lbm_set_steps_per_launch(lbm_ctx *ctx, int k);
 int lbm_get_steps_per_launch(lbm_ctx *ctx, int *k);
 
-/* Wavefront schedule of launches of three or four steps (rows > 0: segments
+/* The most pseudo-time steps a plain (unchecked) launch of this context
+ * advances under its settings.  Errors: LBM_ERR_ARG (null), LBM_ERR_CUDA. */
+int lbm_get_launch_steps(lbm_ctx *ctx, int *k);
+
+/* Wavefront schedule of launches of three or more steps (rows > 0: segments
  * of `rows` rows; rows = -1: segments chosen per launch), or the tile schedule
- * (rows = 0).  On the wavefront schedule a block owns a strip of 256 slot
+ * (rows = 0).  On the wavefront schedule a warp owns a strip of 64 slot
  * columns and a segment of lattice rows and walks down the segment one row per
- * iteration at every step level at once, step j trailing step j - 1 by two
- * rows, each level keeping four rows in shared memory: the halo is 2(k - 1)
- * columns per strip instead of a ring of nodes around every tile.  Same steps
- * and, for LBM_F32, the same bits as one step per launch (see
- * lbm_set_steps_per_launch).  Used where nx >= 256 and ny >= 8; smaller
- * lattices keep the tile schedule.  With rows = -1 a segment is 256 rows,
- * halved (down to 16) while the grid would have fewer than four waves of
- * resident blocks.  Default -1 for LBM_F32 and LBM_F16S storage, 0 for
- * LBM_F64.
+ * iteration at every step level at once, step j trailing step j - 1 by one
+ * row; what a step still needs of the one above it stays in registers: the
+ * halo is k - 1 columns per side of a strip instead of a ring of nodes around
+ * every tile.  Same steps and, for LBM_F32, the same values as one step per
+ * launch (see lbm_set_steps_per_launch).  Used where nx >= 256 and ny >= 8;
+ * smaller lattices keep the tile schedule.  With rows = -1 the segments are
+ * those whose warps just fill a whole number of waves of the device.  Default
+ * -1 for LBM_F32 and LBM_F16S storage, 0 for LBM_F64.
  * Errors: LBM_ERR_ARG (rows outside -1..2^20, or rows != 0 with LBM_F64
  * storage). */
 int lbm_set_wavefront(lbm_ctx *ctx, int rows);

@@ -14,6 +14,7 @@ __device__ __forceinline__ void arena_tile(const BatchArgs& A, const BatchProb& 
     const int64_t n = (int64_t)P.nx * P.ny;
     a.nx = P.nx;
     a.ny = P.ny;
+    a.pitch = P.nx;
     a.plane = n;
     const int src = (P.parity + s) & 1;
     char* ps = src ? A.pop1 : A.pop0;
@@ -106,6 +107,7 @@ __device__ __forceinline__ void arena_tile2(const BatchArgs& A, const BatchProb&
     const int64_t n = (int64_t)P.nx * P.ny;
     a.nx = P.nx;
     a.ny = P.ny;
+    a.pitch = P.nx;
     a.plane = n;
     const int src = (P.parity + s) & 1;
     a.src = (src ? A.pop1 : A.pop0) + P.pop_off;
@@ -169,6 +171,7 @@ __device__ __forceinline__ void arena_wave_item(const BatchArgs& A, const BatchP
     const int64_t n = (int64_t)P.nx * P.ny;
     a.nx = P.nx;
     a.ny = P.ny;
+    a.pitch = P.nx;
     a.plane = n;
     const int src = (P.parity + q) & 1;
     a.src = (src ? A.pop1 : A.pop0) + P.pop_off;

@@ -49,13 +49,14 @@ struct lbm_ctx {
     int device = 0;
     int nx = 0, ny = 0, dtype = 0;
     int64_t n = 0, plane = 0;
+    int pitch = 0;                 // elements between rows (row_pitch)
     lbm_rates rates{};
     bool gen = false;              // non-standard w_12, w_21, w_22
     cudaStream_t stream = nullptr;
     void* pop[2] = {nullptr, nullptr};
     float* car[2] = {nullptr, nullptr};
     void* force = nullptr;         // 2 planes of the storage force type
-    void* snap = nullptr;          // residual snapshot: 2 planes of n entries of 8 bytes (ResSnap)
+    void* snap = nullptr;          // residual snapshot: 2 planes of entries of 8 bytes (ResSnap)
     double* partials = nullptr;    // residual partial sets, kRes doubles each
     int64_t partials_len = 0;      // partial sets the buffer holds
     double* result = nullptr;      // kRes doubles (device)
@@ -84,6 +85,8 @@ struct lbm_ctx {
                                    // with the segment chosen per launch (wave_seg)
     int nsm = 0;                   // multiprocessors of the device
     int64_t nblocks2 = 0;          // grid of the two-step check launch
+    StripShape shape[kStTMax + 1]; // strip launches per step count ([0]: checked), cleared by lbm_set_wavefront
+    int wave_T = 0;                // FP32: steps per plain strip launch (0: not chosen yet)
 };
 
 namespace {
@@ -97,6 +100,7 @@ StepParams params(const lbm_ctx* c, int src) {
     StepParams a{};
     a.nx = c->nx;
     a.ny = c->ny;
+    a.pitch = c->pitch;
     a.plane = c->plane;
     a.src = c->pop[src];
     a.dst = c->pop[src ^ 1];
@@ -138,6 +142,8 @@ cudaError_t finish_residual_launch(lbm_ctx* c, int64_t grid) {
     k_residual_finish<<<1, kFinishThreads, 0, c->stream>>>(c->partials, grid, c->result);
     return cudaGetLastError();
 }
+
+int ensure_partials(lbm_ctx* c, int64_t sets);
 
 cudaError_t launch_step(lbm_ctx* c, bool check) {
     const StepParams a = params(c, c->cur);
@@ -186,28 +192,70 @@ cudaError_t launch_step3(lbm_ctx* c) {
     return e;
 }
 
-// Segment rows of a wavefront launch of T steps: the set value, or (-1)
-// kWvSegDefault halved, down to 16, while the grid would have fewer than four
-// waves of resident blocks (short segments cost 2(T - j) extra rows at level j).
-int wave_seg(const lbm_ctx* c, int T) {
-    if (c->wave > 0) return c->wave;
-    const int minb = c->dtype == LBM_F16S ? (T == 3 ? wv_minb<S_F16S, 3>() : wv_minb<S_F16S, 4>())
-                                          : (T == 3 ? wv_minb<S_F32, 3>() : wv_minb<S_F32, 4>());
-    const int64_t want = 4LL * (c->nsm > 0 ? c->nsm : 1) * minb;
-    int seg = kWvSegDefault;
-    while (seg > 16 && (T == 3 ? wave_blocks<3>(c->nx, c->ny, seg) : wave_blocks<4>(c->nx, c->ny, seg)) < want)
-        seg /= 2;
-    return seg;
+bool wave_on(const lbm_ctx* c) { return c->wave != 0 && wave_fits(c->nx, c->ny); }
+
+// The shape of a strip launch of T steps (kept per context: it depends on the
+// sizes and the lbm_set_wavefront setting only).
+cudaError_t wave_shape(lbm_ctx* c, int T, bool check, StripShape* out) {
+    StripShape& sh = c->shape[check ? 0 : T];
+    if (sh.T == 0) {
+        int warps = 0;
+        const StepParams a = params(c, c->cur);
+        const Coef<float> cf{};
+        const cudaError_t e = c->dtype == LBM_F32 ? strip_f32(a, cf, c->gen, T, check, 1, &warps, c->stream)
+                                                  : strip_f16s(a, cf, c->gen, T, check, 1, &warps, c->stream);
+        if (e != cudaSuccess) return e;
+        sh = strip_shape(c->dtype, T, c->nx, c->ny, c->nsm > 0 ? c->nsm : 1, warps, c->wave);
+    }
+    *out = sh;
+    return cudaSuccess;
 }
 
-// T = 3 or 4 plain steps in one launch: the wavefront kernel where it is on
-// and fits, else (T = 3) the three-step tile kernel.
-cudaError_t launch_multi(lbm_ctx* c, int T) {
-    if (!(c->wave != 0 && wave_fits(c->nx, c->ny))) return T == 3 ? launch_step3(c) : cudaErrorInvalidValue;
+// Steps per plain strip launch of FP32 storage: the count with the fewest
+// modelled cycles per step, memory traffic included (its states are the same
+// bits whatever the grouping).  Every launch moves 72 bytes per node, 3.0
+// cycles per 768 bytes at 6.2 TB/s, unless the lattice stays in the L2 cache.
+cudaError_t wave_steps(lbm_ctx* c, int* T) {
+    if (c->wave_T == 0) {
+        const double bytes = 72.0 * (double)c->n;
+        const double mem = bytes > 1.2e8 ? bytes / 6.2e12 * 2.0e9 : 0.0;
+        double best = 0.0;
+        int bt = 0;
+        for (int t = 4; t <= kStTMax; ++t) {
+            StripShape sh;
+            const cudaError_t e = wave_shape(c, t, false, &sh);
+            if (e != cudaSuccess) return e;
+            const double per = (sh.cost > mem ? sh.cost : mem) / t;
+            if (bt == 0 || per < best) {
+                best = per;
+                bt = t;
+            }
+        }
+        c->wave_T = bt;
+    }
+    *T = c->wave_T;
+    return cudaSuccess;
+}
+
+// Blocks (partial sets) of the checked launch of four steps.
+int64_t strip_check_blocks(const lbm_ctx* c, int seg) {
+    const int64_t items = strip_count(c->dtype, 4, c->nx) * ((c->ny + seg - 1) / seg);
+    return (items + st_nw<4>() - 1) / st_nw<4>();
+}
+
+cudaError_t launch_strip(lbm_ctx* c, int T, bool check) {
+    StripShape sh;
+    cudaError_t e = wave_shape(c, T, check, &sh);
+    if (e != cudaSuccess) return e;
+    int64_t blocks = 0;
+    if (check) {
+        blocks = strip_check_blocks(c, sh.seg);
+        if (ensure_partials(c, blocks) != LBM_OK) return cudaErrorMemoryAllocation;
+    }
     const StepParams a = params(c, c->cur);
-    const int seg = wave_seg(c, T);
-    cudaError_t e = c->dtype == LBM_F32 ? wave_f32(a, coef<float>(c->rates), c->gen, T, false, seg, c->stream)
-                                        : wave_f16s(a, coef<float>(c->rates), c->gen, T, false, seg, c->stream);
+    e = c->dtype == LBM_F32 ? strip_f32(a, coef<float>(c->rates), c->gen, T, check, sh.seg, nullptr, c->stream)
+                            : strip_f16s(a, coef<float>(c->rates), c->gen, T, check, sh.seg, nullptr, c->stream);
+    if (e == cudaSuccess && check) e = finish_residual_launch(c, blocks);
     if (e == cudaSuccess) {
         c->cur ^= 1;
         c->step += T;
@@ -216,33 +264,34 @@ cudaError_t launch_multi(lbm_ctx* c, int T) {
     return e;
 }
 
-int ensure_partials(lbm_ctx* c, int64_t sets);
-
-// Four steps on the wavefront schedule whose last step carries the residual
-// check (one partial set per block, combined by k_residual_finish).
-cudaError_t launch_wave_checked(lbm_ctx* c) {
-    const int seg = wave_seg(c, 4);
-    const int64_t blocks = wave_blocks<4>(c->nx, c->ny, seg);
-    if (ensure_partials(c, blocks) != LBM_OK) return cudaErrorMemoryAllocation;
-    const StepParams a = params(c, c->cur);
-    cudaError_t e = c->dtype == LBM_F32 ? wave_f32(a, coef<float>(c->rates), c->gen, 4, true, seg, c->stream)
-                                        : wave_f16s(a, coef<float>(c->rates), c->gen, 4, true, seg, c->stream);
-    if (e == cudaSuccess) e = finish_residual_launch(c, blocks);
-    if (e == cudaSuccess) {
-        c->cur ^= 1;
-        c->step += 4;
-        c->staged_fields = false;
-    }
-    return e;
+// T = 3 or 4 plain steps in one launch: the strip kernel where it is on and
+// fits, else (T = 3) the three-step tile kernel.
+cudaError_t launch_multi(lbm_ctx* c, int T) {
+    if (!wave_on(c)) return T == 3 ? launch_step3(c) : cudaErrorInvalidValue;
+    return launch_strip(c, T, false);
 }
 
 // n plain steps, grouped into launches of c->spl steps (four only on the
 // wavefront schedule, else three); a remainder of one step is avoided where
 // possible (4 = 2 + 2, 5 = 3 + 2), since a pair of steps costs about as much
-// as one step alone.
+// as one step alone.  FP32 on the wavefront schedule takes up to seven steps
+// per launch (wave_steps); FP16-shifted storage rounds to FP16 where a launch
+// ends, so its groups stay the documented ones.
 cudaError_t run_plain(lbm_ctx* c, int64_t n) {
     cudaError_t e = cudaSuccess;
-    const bool wave = c->wave != 0 && wave_fits(c->nx, c->ny);
+    const bool wave = wave_on(c);
+    if (c->spl >= 4 && wave && c->dtype == LBM_F32) {
+        int T = 0;
+        e = wave_steps(c, &T);
+        while (n >= 2 && e == cudaSuccess) {
+            // whole groups, then the rest in one launch, or two for T + 1
+            const int t = n >= T && n != T + 1 ? T : (n == T + 1 ? (T + 1) / 2 : (int)n);
+            e = launch_strip(c, t, false);
+            n -= t;
+        }
+        if (n > 0 && e == cudaSuccess) e = launch_step(c, false);
+        return e;
+    }
     const int big = c->spl >= 4 && wave ? 4 : (c->spl >= 3 ? 3 : 0);
     if (big) {
         int64_t groups = n / big, r = n % big;
@@ -270,9 +319,9 @@ cudaError_t run_plain(lbm_ctx* c, int64_t n) {
 // costs twice a plain one, a two-step launch with the check 1.3 times).
 cudaError_t run_window(lbm_ctx* c, int64_t to_check) {
     cudaError_t e;
-    if (c->spl >= 4 && to_check >= 4 && c->wave != 0 && wave_fits(c->nx, c->ny)) {
+    if (c->spl >= 4 && to_check >= 4 && wave_on(c)) {
         e = run_plain(c, to_check - 4);
-        return e == cudaSuccess ? launch_wave_checked(c) : e;
+        return e == cudaSuccess ? launch_strip(c, 4, true) : e;
     }
     if (c->spl >= 2 && to_check >= 2) {
         e = run_plain(c, to_check - 2);
@@ -412,10 +461,10 @@ int set_force_dev(lbm_ctx* c, const double* gx, const double* gy) {
     CK(cudaMemsetAsync(c->bad, 0, sizeof(unsigned int), c->stream));
     if (c->dtype == LBM_F64) {
         double* fx = static_cast<double*>(c->force);
-        k_force_ingest<double><<<2048, 256, 0, c->stream>>>(gx, gy, fx, fx + c->plane, c->n, c->absmax, c->bad);
+        k_force_ingest<double><<<2048, 256, 0, c->stream>>>(gx, gy, fx, fx + c->plane, c->n, c->nx, c->pitch, c->absmax, c->bad);
     } else {
         float* fx = static_cast<float*>(c->force);
-        k_force_ingest<float><<<2048, 256, 0, c->stream>>>(gx, gy, fx, fx + c->plane, c->n, c->absmax, c->bad);
+        k_force_ingest<float><<<2048, 256, 0, c->stream>>>(gx, gy, fx, fx + c->plane, c->n, c->nx, c->pitch, c->absmax, c->bad);
     }
     CK(cudaGetLastError());
     c->force_exp = 0;   // converted as given
@@ -519,7 +568,8 @@ int lbm_create_ex(int nx, int ny, double lambda, double mu, int dtype, const lbm
     c->ny = ny;
     c->dtype = dtype;
     c->n = (int64_t)nx * ny;
-    c->plane = round_up(c->n, 128);
+    c->pitch = row_pitch(dtype, nx);
+    c->plane = round_up((int64_t)c->pitch * ny, 128);
     // Table 1 and Eq. relaxation_rate: theta tau_11 = mu, (1-theta)/2 tau_d = mu,
     // (1+theta)/2 tau_s = K = lambda + mu, w = 1/(tau + 1/2).
     const double K = lambda + mu;
@@ -564,11 +614,14 @@ int lbm_create_ex(int nx, int ny, double lambda, double mu, int dtype, const lbm
     }
     if (e == cudaSuccess) e = alloc(&c->force, fb);
     // FP64: two planes of doubles; FP32 / FP16S: two planes of (hi, lo) FP32 pairs
-    const size_t snap_bytes = 16 * (size_t)c->n;
+    const size_t snap_bytes = 16 * (size_t)c->plane;
     if (e == cudaSuccess) e = alloc(&c->snap, snap_bytes);
     c->partials_len = std::max(c->nblocks, c->nblocks2);
-    if (dtype != LBM_F64 && wave_fits(nx, ny))
-        c->partials_len = std::max(c->partials_len, wave_blocks<4>(nx, ny, wave_seg(c, 4)));
+    if (e == cudaSuccess && dtype != LBM_F64 && wave_on(c)) {
+        StripShape sh;
+        e = wave_shape(c, 4, true, &sh);
+        c->partials_len = std::max(c->partials_len, strip_check_blocks(c, sh.seg));
+    }
     if (e == cudaSuccess) e = alloc((void**)&c->partials, sizeof(double) * kRes * c->partials_len);
     if (e == cudaSuccess) e = alloc((void**)&c->result, sizeof(double) * kRes);
     if (e == cudaSuccess) e = alloc((void**)&c->absmax, sizeof(unsigned long long));
@@ -624,6 +677,15 @@ int lbm_get_steps_per_launch(lbm_ctx* c, int* k) {
     return LBM_OK;
 }
 
+int lbm_get_launch_steps(lbm_ctx* c, int* k) {
+    int rc = check_ctx(c);
+    if (rc) return rc;
+    if (!k) return fail(LBM_ERR_ARG, "lbm_get_launch_steps: null pointer");
+    *k = c->spl >= 4 && !wave_on(c) ? 3 : c->spl;
+    if (c->spl >= 4 && wave_on(c) && c->dtype == LBM_F32) CK(wave_steps(c, k));
+    return LBM_OK;
+}
+
 int lbm_set_wavefront(lbm_ctx* c, int rows) {
     int rc = check_ctx(c);
     if (rc) return rc;
@@ -632,6 +694,8 @@ int lbm_set_wavefront(lbm_ctx* c, int rows) {
     if (rows != 0 && c->dtype == LBM_F64)
         return fail(LBM_ERR_ARG, "lbm_set_wavefront: the wavefront kernel needs FP32 or FP16-shifted storage");
     c->wave = rows;
+    for (auto& sh : c->shape) sh = StripShape();
+    c->wave_T = 0;
     return LBM_OK;
 }
 

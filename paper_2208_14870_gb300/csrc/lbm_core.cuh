@@ -245,4 +245,212 @@ __device__ __forceinline__ float4 exact_displacement(const float f[8], float gx,
 __device__ __forceinline__ int wrap_dec(int i, int n) { return i == 0 ? n - 1 : i - 1; }
 __device__ __forceinline__ int wrap_inc(int i, int n) { return i + 1 == n ? 0 : i + 1; }
 
+// ---------------------------------------------------------------------------
+// The per-node arithmetic above for two nodes at a time, in the packed FP32 instructions of sm_103a (add / sub / fma .f32x2:
+// two FP32 operations per issue slot).
+//
+// Every packed operation rounds each half as its scalar counterpart does, and
+// the sums are those above up to powers of two and signs, which
+// rounding commutes with; so a pair holds the values the scalar code computes
+// (the sign of a zero aside).  Two things shape the form:
+//   - the assembler may fuse a packed product into a following packed sum,
+//     so the products of the relaxation (rmul above) are scalar
+//     multiplications with explicit rounding, which it does not fuse; their
+//     factors come from the constant bank;
+//   - a packed constant needs a register pair, or two moves at each use, so
+//     the factors 2, -1/2 and -4 of lbm_core.cuh are folded away: only 1/2 and
+//     -2 remain.
+using pair_t = unsigned long long;   // two FP32 values: low half first
+
+__device__ __forceinline__ pair_t pk(float lo, float hi) {
+    pair_t d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+    return d;
+}
+__device__ __forceinline__ void unpk(pair_t p, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(p));
+}
+__device__ __forceinline__ float pk_lo(pair_t p) {
+    float lo, hi;
+    unpk(p, lo, hi);
+    return lo;
+}
+__device__ __forceinline__ float pk_hi(pair_t p) {
+    float lo, hi;
+    unpk(p, lo, hi);
+    return hi;
+}
+__device__ __forceinline__ pair_t add2(pair_t a, pair_t b) {
+    pair_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ pair_t sub2(pair_t a, pair_t b) {
+    pair_t d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ pair_t fma2(pair_t a, pair_t b, pair_t c) {
+    pair_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ pair_t splat(float v) { return pk(v, v); }
+
+__device__ __forceinline__ pair_t mul1(float c, pair_t p) {   // rounded on its own
+    float lo, hi;
+    unpk(p, lo, hi);
+    return pk(__fmul_rn(c, lo), __fmul_rn(c, hi));
+}
+__device__ __forceinline__ pair_t neg2(pair_t p) { return p ^ 0x8000000080000000ULL; }
+
+// The factors of the pair form: Coef<float> with q_s doubled (moments2 halves
+// m_s), and the two packed constants.  A kernel argument, so that the scalar
+// factors are operands from the constant bank.
+struct PairCoef {
+    pair_t half, nhalf, nfour;
+    float q11, qs2, qd, qw12t, q12, qw21t, q21, q22, qtheta, theta;
+};
+
+__host__ __device__ inline PairCoef pair_coef(const Coef<float>& c) {
+    PairCoef d;
+    d.half = 0x3f0000003f000000ULL;
+    d.nhalf = 0xbf000000bf000000ULL;
+    d.nfour = 0xc0800000c0800000ULL;
+    d.q11 = c.q11;
+    d.qs2 = 2.0f * c.qs;
+    d.qd = c.qd;
+    d.qw12t = c.qw12t;
+    d.q12 = c.q12;
+    d.qw21t = c.qw21t;
+    d.q21 = c.q21;
+    d.q22 = c.q22;
+    d.qtheta = c.qtheta;
+    d.theta = c.theta;
+    return d;
+}
+
+// First stage of the moment butterfly (moments()): the sums and
+// differences of opposite populations.  Populations 6 and 8 enter negated.
+struct Opp2 {
+    pair_t p, nq, r, s;         // f5 + f7, -(f6 + f8), f5 - f7, f6 - f8
+    pair_t a, b, s13, s24;      // f1 - f3, f2 - f4, f1 + f3, f2 + f4
+};
+
+__device__ __forceinline__ Opp2 opposites2(pair_t f1, pair_t f2, pair_t f3, pair_t f4, pair_t f5, pair_t nf6,
+                                           pair_t f7, pair_t nf8) {
+    Opp2 o;
+    o.p = add2(f5, f7);
+    o.nq = add2(nf6, nf8);
+    o.r = sub2(f5, f7);
+    o.s = sub2(nf8, nf6);
+    o.a = sub2(f1, f3);
+    o.b = sub2(f2, f4);
+    o.s13 = add2(f1, f3);
+    o.s24 = add2(f2, f4);
+    return o;
+}
+
+// The same from eight populations as they are.
+__device__ __forceinline__ Opp2 opposites2(const pair_t f[8]) {
+    Opp2 o = opposites2(f[0], f[1], f[2], f[3], f[4], 0, f[6], 0);
+    o.nq = sub2(sub2(0, f[5]), f[7]);
+    o.s = sub2(f[5], f[7]);
+    return o;
+}
+
+struct Mom2 {
+    pair_t m10, m01, m11, msh, md, m12, m21, m22;   // msh = m_s / 2
+};
+
+__device__ __forceinline__ Mom2 moments2(const Opp2& o, const PairCoef& c) {
+    Mom2 m;
+    m.m11 = add2(o.p, o.nq);
+    m.m22 = sub2(o.p, o.nq);
+    m.m12 = sub2(o.r, o.s);
+    m.m21 = add2(o.r, o.s);
+    m.m10 = add2(o.a, m.m12);
+    m.m01 = add2(o.b, m.m21);
+    m.msh = fma2(c.half, add2(o.s13, o.s24), m.m22);
+    m.md = sub2(o.s13, o.s24);
+    return m;
+}
+
+// Post-collision moments in the quarter form (collide()).
+struct Post2 {
+    pair_t m10, m01, m11, ms, md, m12, m21, m22;
+};
+
+template <bool GEN>
+__device__ __forceinline__ Post2 collide2(const Mom2& m, pair_t gx, pair_t gy, const PairCoef& c) {
+    Post2 s;
+    const pair_t u = fma2(c.half, gx, m.m10), v = fma2(c.half, gy, m.m01);
+    s.m10 = add2(m.m10, gx);
+    s.m01 = add2(m.m01, gy);
+    s.m11 = mul1(c.q11, m.m11);
+    s.ms = mul1(c.qs2, m.msh);
+    s.md = mul1(c.qd, m.md);
+    if (GEN) {
+        s.m12 = fma2(splat(c.qw12t), u, mul1(c.q12, m.m12));
+        s.m21 = fma2(splat(c.qw21t), v, mul1(c.q21, m.m21));
+        s.m22 = mul1(c.q22, m.m22);
+    } else {
+        s.m12 = mul1(c.qtheta, u);
+        s.m21 = mul1(c.qtheta, v);
+        s.m22 = 0;
+    }
+    return s;
+}
+
+// Back-transformation (populations()) up to the last sum of
+// each population, which the caller takes one at a time in the order it needs
+// them.
+template <bool ZERO22>
+struct Pop2 {
+    pair_t A, B, P, Q, h1, h2, h3, h4;
+    __device__ __forceinline__ Pop2(const Post2& s, const PairCoef& c) {
+        A = fma2(c.nfour, s.m12, s.m10);
+        B = fma2(c.nfour, s.m21, s.m01);
+        h3 = add2(s.m12, s.m21);
+        h4 = sub2(s.m21, s.m12);
+        const pair_t t = ZERO22 ? s.ms : sub2(s.ms, add2(s.m22, s.m22));
+        P = add2(t, s.md);
+        Q = sub2(t, s.md);
+        h1 = ZERO22 ? s.m11 : add2(s.m22, s.m11);
+        h2 = ZERO22 ? s.m11 : sub2(s.m11, s.m22);
+    }
+    __device__ __forceinline__ pair_t f1(const PairCoef& c) const { return fma2(c.half, A, P); }
+    __device__ __forceinline__ pair_t f2(const PairCoef& c) const { return fma2(c.half, B, Q); }
+    __device__ __forceinline__ pair_t f3(const PairCoef& c) const { return fma2(c.nhalf, A, P); }
+    __device__ __forceinline__ pair_t f4(const PairCoef& c) const { return fma2(c.nhalf, B, Q); }
+    __device__ __forceinline__ pair_t f5() const { return add2(h1, h3); }
+    __device__ __forceinline__ pair_t nf6() const { return sub2(h2, h4); }
+    __device__ __forceinline__ pair_t f7() const { return sub2(h1, h3); }
+    __device__ __forceinline__ pair_t nf8() const { return add2(h2, h4); }
+    __device__ __forceinline__ void all(const PairCoef& c, pair_t f[8]) const {
+        f[0] = f1(c);
+        f[1] = f2(c);
+        f[2] = f3(c);
+        f[3] = f4(c);
+        f[4] = f5();
+        f[5] = neg2(nf6());
+        f[6] = f7();
+        f[7] = neg2(nf8());
+    }
+};
+
+// The pair one column to the right (c_x = +1: the value pulled from x - 1) or
+// to the left (from x + 1) of a warp whose lane l holds columns 2l, 2l + 1.
+// The outermost column receives its own lane's value: a halo column.
+__device__ __forceinline__ pair_t from_left(pair_t p) {
+    float lo, hi;
+    unpk(p, lo, hi);
+    return pk(__shfl_up_sync(0xffffffffu, hi, 1), lo);
+}
+__device__ __forceinline__ pair_t from_right(pair_t p) {
+    float lo, hi;
+    unpk(p, lo, hi);
+    return pk(hi, __shfl_down_sync(0xffffffffu, lo, 1));
+}
+
 }  // namespace lbm

@@ -468,6 +468,7 @@ cudaError_t ArenaEngine::launch_fields(int slot, double* dst) {
     StepParams a{};
     a.nx = p.nx;
     a.ny = p.ny;
+    a.pitch = p.nx;
     a.plane = p.n;
     a.src = pop_[p.parity] + p.pop_off;
     a.dst = pop_[p.parity ^ 1] + p.pop_off;

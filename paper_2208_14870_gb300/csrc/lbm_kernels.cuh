@@ -5,7 +5,8 @@
 // type by lbm_step_f64.cu, lbm_step_f32.cu and lbm_step_f16s.cu.
 //
 // Memory layout (structure of arrays): population p of node (x, y) lives at
-// base + p*plane + y*nx + x; `plane` >= nx*ny is padded to 256 bytes.  The
+// base + p*plane + y*pitch + x (rows padded to whole 16-byte chunks, see
+// row_pitch; `plane` >= pitch*ny is padded to 256 bytes).  The
 // stored state between steps is the post-collision population f*_p(x) of the
 // previous step ("pull" scheme): a step gathers f_p(x) = f*_p(x - c_p) with the
 // periodic wrap done by index arithmetic (Sec. 5.1), collides, and writes
@@ -64,6 +65,7 @@ constexpr int kRes = 5;
 
 struct StepParams {
     int nx, ny;
+    int pitch;              // elements between rows
     int64_t plane;          // elements between planes
     const void* src;        // 8 population planes (storage type)
     void* dst;
@@ -73,7 +75,7 @@ struct StepParams {
     const void* gy;
     float hscale;           // F16S: the state's scale 2^e (see store_f16s)
     float hinv;             // 1 / hscale
-    void* snap;             // residual: u_x, u_y snapshot, 2 planes of nx*ny (ResSnap)
+    void* snap;             // residual: u_x, u_y snapshot, 2 planes (ResSnap)
     double* partials;       // residual: kRes doubles per block
     unsigned int* counter;  // residual: blocks finished, reset by the last block; null:
                             // blocks only write partials (k_residual_finish combines them)
@@ -88,7 +90,7 @@ __device__ __forceinline__ T ldg(const T* p) { return __ldg(p); }
 // of u^t - u^(t-w) over a window of w steps).  Each thread keeps partials over
 // its nodes -- max|du|, max|u| (over nodes and both components), sum du^2,
 // sum u^2 and a non-finite flag -- and the snapshot holds u of the previous
-// check, two planes of nx*ny entries:
+// check, two planes laid out as the populations':
 //   FP64 storage: u from the FP64 collision, FP64 snapshot and partials;
 //   FP32 / FP16S: u as an exact FP32 pair from exact_displacement, the
 //   snapshot as (hi, lo) pairs (16 bytes per node, like two FP64 planes), and
@@ -493,9 +495,9 @@ __device__ __forceinline__ void step_tile(const StepParams& a,
     if (y >= ny) return;
     const G* __restrict__ gxp = static_cast<const G*>(a.gx);
     const G* __restrict__ gyp = static_cast<const G*>(a.gy);
-    const int64_t n = (int64_t)nx * ny;
+    const int64_t n = a.plane;
     const int ym = wrap_dec(y, ny), yp = wrap_inc(y, ny);
-    const int64_t r0 = (int64_t)y * nx, rm = (int64_t)ym * nx, rp = (int64_t)yp * nx;
+    const int64_t r0 = (int64_t)y * a.pitch, rm = (int64_t)ym * a.pitch, rp = (int64_t)yp * a.pitch;
     // Phase 1: issue every load of the thread's V nodes before any store,
     // so that up to V*10 (V*12 with the snapshot) loads are in flight.
     T f[V][8], gx[V], gy[V];
@@ -630,8 +632,8 @@ __device__ __forceinline__ void step2_tile(const StepParams& a, const Coef<float
         for (int b = 0; b < kT2B; ++b) {
             const int k = kb + b;
             const int y = wrap_slot<ANY>(y0 + warp + 8 * k, ny);
-            const int64_t r0 = (int64_t)y * nx;
-            const int64_t rm = (int64_t)wrap_dec(y, ny) * nx, rp = (int64_t)wrap_inc(y, ny) * nx;
+            const int64_t r0 = (int64_t)y * a.pitch;
+            const int64_t rm = (int64_t)wrap_dec(y, ny) * a.pitch, rp = (int64_t)wrap_inc(y, ny) * a.pitch;
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
                 gather<S>(a, r0, rm, rp, X[j], XM[j], XP[j], f[b][j], c.theta);
@@ -652,7 +654,7 @@ __device__ __forceinline__ void step2_tile(const StepParams& a, const Coef<float
             }
         }
     }
-    const int64_t n = (int64_t)nx * ny;
+    const int64_t n = a.plane;
     ResSnap<S> so[kT2Rows][2];
     if (CHECK) {
 #pragma unroll
@@ -662,7 +664,7 @@ __device__ __forceinline__ void step2_tile(const StepParams& a, const Coef<float
             for (int j = 0; j < 2; ++j) {
                 const int col = lane + 32 * j, x = x0 + col;
                 if (r >= 1 && r <= kT2H - 2 && y < ny && col >= 1 && col <= kT2W - 2 && x < nx)
-                    so[k][j] = snap_load<S>(a, n, (int64_t)y * nx + x);
+                    so[k][j] = snap_load<S>(a, n, (int64_t)y * a.pitch + x);
             }
         }
     }
@@ -678,7 +680,7 @@ __device__ __forceinline__ void step2_tile(const StepParams& a, const Coef<float
             const int col = lane + 32 * j;
             const int x = x0 + col;
             if (col < 1 || col > kT2W - 2 || x >= nx) continue;
-            const int64_t idx = (int64_t)y * nx + x;
+            const int64_t idx = (int64_t)y * a.pitch + x;
             const float* s = sm + r * kT2W + col;
             float f[8];
             f[0] = s[0 * PL - 1];               // f_p(x) = f*_p(x - c_p)
@@ -773,8 +775,8 @@ __device__ __forceinline__ void step3_tile(const StepParams& a, const Coef<float
     for (int k = 0; k < kT3Rows; ++k) {
         const int r = warp + 8 * k;
         const int y = wrap_slot<ANY>(y0 + r, ny);
-        const int64_t r0 = (int64_t)y * nx;
-        const int64_t rm = (int64_t)wrap_dec(y, ny) * nx, rp = (int64_t)wrap_inc(y, ny) * nx;
+        const int64_t r0 = (int64_t)y * a.pitch;
+        const int64_t rm = (int64_t)wrap_dec(y, ny) * a.pitch, rp = (int64_t)wrap_inc(y, ny) * a.pitch;
         float f[2][8];
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
@@ -818,7 +820,7 @@ __device__ __forceinline__ void step3_tile(const StepParams& a, const Coef<float
             for (int p = 0; p < 8; ++p) d[p * PL] = fs[p];
         }
     }
-    const int64_t n = (int64_t)nx * ny;
+    const int64_t n = a.plane;
     ResSnap<S> so[kT3Rows][2];
     if (CHECK) {
 #pragma unroll
@@ -828,7 +830,7 @@ __device__ __forceinline__ void step3_tile(const StepParams& a, const Coef<float
             for (int j = 0; j < 2; ++j) {
                 const int col = lane + 32 * j, x = x0 + col;
                 if (r >= 2 && r <= kT3H - 3 && y < ny && col >= 2 && col <= kT3W - 3 && x < nx)
-                    so[k][j] = snap_load<S>(a, n, (int64_t)y * nx + x);
+                    so[k][j] = snap_load<S>(a, n, (int64_t)y * a.pitch + x);
             }
         }
     }
@@ -844,7 +846,7 @@ __device__ __forceinline__ void step3_tile(const StepParams& a, const Coef<float
             const int col = lane + 32 * j;
             const int x = x0 + col;
             if (col < 2 || col > kT3W - 3 || x >= nx) continue;
-            const int64_t idx = (int64_t)y * nx + x;
+            const int64_t idx = (int64_t)y * a.pitch + x;
             const float* s = smB + r * kT3W + col;
             float f[8];
             f[0] = s[0 * PL - 1];
@@ -1012,7 +1014,7 @@ __device__ __forceinline__ void wave_block(const StepParams& a, const Coef<float
     const int ybeg = y0 - (T - 1);                // lattice row of local row 0 (level 1)
     const int iters = rows + 3 * (T - 1);
     const int n1 = rows + 2 * (T - 1);            // rows of level 1
-    const int64_t n = (int64_t)nx * ny;
+    const int64_t n = a.plane;
     // This thread's column of every ring (slot t sits at padded column t + 1,
     // so the pulls of t - 1 and t + 1 stay inside the row for every thread).
     float* const rt = wv_ring + t + 1;
@@ -1041,16 +1043,16 @@ __device__ __forceinline__ void wave_block(const StepParams& a, const Coef<float
     Pulled<S> q[CIRC ? 4 : (PA2 ? 2 : 1)];
     float qg[LA2 ? 2 : 1][2];
     int ly = wrap_slot<false>(ybeg, ny);          // lattice row of the next population load
-    I lr0 = (I)ly * nx, lrm = (I)wrap_dec(ly, ny) * nx, lrp = (I)wrap_inc(ly, ny) * nx;
+    I lr0 = (I)ly * a.pitch, lrm = (I)wrap_dec(ly, ny) * a.pitch, lrp = (I)wrap_inc(ly, ny) * a.pitch;
     int gly = ly;                                 // lattice row of the next force load
     auto advance = [&]() {
         ly = wrap_inc(ly, ny);
         lrm = lr0;
         lr0 = lrp;
-        lrp = (I)wrap_inc(ly, ny) * nx;
+        lrp = (I)wrap_inc(ly, ny) * a.pitch;
     };
     auto load_force = [&](int b) {
-        const I g = (I)gly * nx + x;
+        const I g = (I)gly * a.pitch + x;
         qg[b][0] = ldg(gxp + g);
         qg[b][1] = ldg(gyp + g);
         gly = wrap_inc(gly, ny);
@@ -1062,7 +1064,7 @@ __device__ __forceinline__ void wave_block(const StepParams& a, const Coef<float
     // Residual check on level T: its snapshot entry is loaded one iteration ahead.
     ResSnap<S> so;
     auto snap_next = [&](int i) {
-        so = snap_load<S>(a, n, (int64_t)((I)(ybeg + i - 2 * (T - 1)) * nx + xs));
+        so = snap_load<S>(a, n, (int64_t)((I)(ybeg + i - 2 * (T - 1)) * a.pitch + xs));
     };
 
     // One iteration; FULL: every level active (ring slots fold to constants
@@ -1156,7 +1158,7 @@ __device__ __forceinline__ void wave_block(const StepParams& a, const Coef<float
                 float u, v, fs[8], c10, c01;
                 post_state<S, GEN>(m, gx, gy, c, u, v, fs, c10, c01);
                 if (store_ok) {
-                    const I idx = (I)(ybeg + j) * nx + xs;   // row in [y0, y0 + rows), xs < nx
+                    const I idx = (I)(ybeg + j) * a.pitch + xs;   // row in [y0, y0 + rows), xs < nx
                     if (CHECK) {
                         check_node<S>(a, n, (int64_t)idx, acc, so, f, gx, gy, u, v);
                         if (FULL || i + 1 < iters) snap_next(i + 1);
@@ -1222,15 +1224,403 @@ __device__ __forceinline__ void wave_block(const StepParams& a, const Coef<float
     for (; i < iters; ++i) iter_any(i);
 }
 
-template <int S, bool GEN, int T, bool CHECK, typename I>
-__global__ void __launch_bounds__(kWvW, (wv_minb<S, T>()))
-k_wave(const StepParams a, const Coef<float> c, int seg) {
-    extern __shared__ float wv_ring[];            // (T-1) rings of 6 planes x kWvD rows x kWvRow, staging
-    const int nstrips = (a.nx + wv_ox<T>() - 1) / wv_ox<T>();
-    const int strip = (int)(blockIdx.x % (unsigned)nstrips);
-    const int y0 = (int)(blockIdx.x / (unsigned)nstrips) * seg;
+// ---------------------------------------------------------------------------
+// T pseudo-time steps per launch, one warp per strip of the
+// lattice (FP32 or FP16-shifted storage).
+//
+// A warp owns a strip of 64 slot columns (lane l holds columns 2l and 2l + 1
+// as FP32 pairs, pair_t) and a segment of `rows` output rows, and walks
+// down the segment one row per iteration at all T step levels at once: in
+// iteration i level j updates local row i - (j - 1), one row behind level
+// j - 1.  What a level still needs of the level above it stays in registers:
+//   populations with c_y = +1 (2, 5, 6) of the last two rows it produced,
+//   those with c_y = 0 (1, 3) of the last one, those with c_y = -1 (4, 7, 8)
+//   of the row it produced in this iteration,
+// i.e. eight values per column and level boundary, and the horizontal movers
+// pass between lanes by shuffles.  A warp shares nothing, so there is no
+// barrier: its shared memory holds the rows on their way from global memory
+// (asynchronous copies LA rows ahead, which need no registers; every lane
+// reads back only what it copied itself) and the force of the last rows,
+// which the levels read one after the other.  The halo is T - 1 columns per
+// side and T - 1 rows per end.
+//
+// FP16-shifted storage decodes the stored deviations and carriers of the
+// lane's own columns (one carrier per node instead of the eight a pulled node
+// needs) one row ahead of level 1, which costs one more halo row and column.
+//
+// The per-node operations are lbm_core.cuh's, so FP32 results equal T
+// single-step launches bit for bit.
+constexpr int kStSlots = 64;                     // slot columns of a strip (two per lane)
+constexpr int kStTMax = 7;                       // most steps per launch
+
+template <int S> __host__ __device__ constexpr int st_lag() { return S == S_F16S ? 1 : 0; }
+// halo rows per end, and halo columns: at least as many per side, even on the
+// left so that pairs start on even columns
+template <int S, int T> __host__ __device__ constexpr int st_halo() { return T - 1 + st_lag<S>(); }
+template <int S, int T> __host__ __device__ constexpr int st_left() { return (st_halo<S, T>() + 1) & ~1; }
+template <int S, int T> __host__ __device__ constexpr int st_ox() {
+    return (kStSlots - st_left<S, T>() - st_halo<S, T>()) & ~1;
+}
+// warps per block and resident blocks the kernel is compiled for: what lets
+// the registers of T levels fit twelve warps per SM (measured per T at
+// 16384^2: T = 7 as 64-thread blocks 447 GLUPS, as 128-thread blocks 411)
+template <int T> __host__ __device__ constexpr int st_nw() { return T >= 7 ? 2 : 4; }
+template <int T> __host__ __device__ constexpr int st_minb() { return T >= 7 ? 5 : 2; }
+// rows copied ahead of the rows in use, and population rows held: FP32 has the
+// rows above, at and below level 1 in use, FP16S the decoded row
+template <int S> __host__ __device__ constexpr int st_la() { return S == S_F16S ? 3 : 1; }
+constexpr int kStPR = 4;
+// force rows held: those the levels still read and the rows ahead (a power of two)
+template <int S, int T> __host__ __device__ constexpr int st_ring() {
+    return T + 1 + st_la<S>() <= 4 ? 4 : (T + 1 + st_la<S>() <= 8 ? 8 : 16);
+}
+// One row in shared memory, in 16-byte chunks.  FP32: 72 columns (the strip's
+// and one on either side, from a multiple of four on) of eight planes; FP16S:
+// 72 columns (from a multiple of eight on) of eight planes and the carriers.
+// The force: two planes of 72 columns, in a ring of its own.
+constexpr int kStCols = 72;
+template <int S> __host__ __device__ constexpr int st_row() { return S == S_F16S ? kStCols * (8 * 2 + 8) : kStCols * 8 * 4; }
+constexpr int kStFRow = 2 * kStCols * 4;
+template <int S, int T> __host__ __device__ constexpr int st_warp_smem() {
+    return kStPR * st_row<S>() + st_ring<S, T>() * kStFRow;
+}
+template <int S, int T> __host__ __device__ constexpr int st_smem() { return st_nw<T>() * st_warp_smem<S, T>(); }
+
+template <int B>
+__device__ __forceinline__ void copy_async(uint32_t dst, const void* src) {
+    if constexpr (B == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(dst), "l"(src), "n"(B) : "memory");
+}
+__device__ __forceinline__ pair_t lds_pair(uint32_t a) {
+    pair_t d;
+    asm volatile("ld.shared.b64 %0, [%1];" : "=l"(d) : "r"(a) : "memory");
+    return d;
+}
+__device__ __forceinline__ void lds_pairs(uint32_t a, pair_t& x, pair_t& y) {
+    asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(x), "=l"(y) : "r"(a) : "memory");
+}
+__device__ __forceinline__ uint32_t lds_u32(uint32_t a) {
+    uint32_t d;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(d) : "r"(a) : "memory");
+    return d;
+}
+__device__ __forceinline__ float lds_float(uint32_t a) {
+    float d;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(d) : "r"(a) : "memory");
+    return d;
+}
+// A register pair the assembler cannot rebuild from a constant (it would, at
+// each use, with two moves): a round trip through shared memory.
+__device__ __forceinline__ pair_t opaque(pair_t p, uint32_t a) {
+    asm volatile("st.shared.b64 [%0], %1;" ::"r"(a), "l"(p) : "memory");
+    return lds_pair(a);
+}
+
+// One strip and segment.  sm: the warp's shared memory (shared-space address).
+// The lattice's pitch is a multiple of the columns of a 16-byte chunk
+// (row_pitch).
+template <int S, bool GEN, int T, bool CHECK>
+__device__ __forceinline__ void strip_walk(const StepParams& a, const PairCoef& ca, uint32_t sm, int strip, int y0,
+                                           int rows, ResAcc<S>& acc) {
+    constexpr int LAG = st_lag<S>(), H = st_halo<S, T>(), HL = st_left<S, T>(), OX = st_ox<S, T>(),
+                  LA = st_la<S>(), R = st_ring<S, T>(), ROW = st_row<S>();
+    constexpr int OFF = 1 - LAG;                             // copied row of local row i: i + OFF
+    constexpr int AHEAD = 2 * OFF + LA;                      // rows copied ahead of iteration i
+    constexpr int CA = S == S_F16S ? 8 : 4;                  // columns of a chunk of populations
+    using P = typename StoreT<S>::P;
+    const int nx = a.nx, ny = a.ny, pitch = a.pitch;
+    const int lane = threadIdx.x & 31;
+    PairCoef c = ca;
+    c.half = opaque(ca.half, sm + 8 * lane);
+    c.nhalf = opaque(ca.nhalf, sm + 8 * lane);
+    c.nfour = opaque(ca.nfour, sm + 8 * lane);
+    __syncwarp();
+    const int xs0 = strip * OX - HL;                         // lattice column of slot 0
+    // first column of a row in shared memory (rounded down, also below zero)
+    const int xa0 = ((xs0 - OFF + (1 << 20)) & ~(CA - 1)) - (1 << 20);
+    const int xs = xs0 + 2 * lane;                           // the lane's first column
+    const bool ok = 2 * lane >= HL && 2 * lane < HL + OX && xs < nx;
+    const int64_t n = a.plane;
+    const int nit = rows + 2 * H;
+    const uint32_t frc = sm + kStPR * ROW;                   // force ring
+    const uint32_t own = (uint32_t)(xs - xa0);               // the lane's first column within a row
+    // Copies of a row: 16-byte chunks, chunk q = lane + 32 m (FP32: 18 per
+    // plane, eight populations, then the force; FP16S: 9 per plane, eight
+    // populations, then 36 of the carriers, then the force), or, where a chunk
+    // would straddle the periodic boundary, single columns.
+    constexpr int NP = S == S_F16S ? 108 : 144, NQ = NP + 36, NM = (NQ + 31) / 32;
+    auto wrapx = [&](int x) {
+        x %= nx;
+        return x < 0 ? x + nx : x;
+    };
+    const bool vec = nx >= kStCols && (nx % CA == 0 || (xa0 >= 0 && xa0 + kStCols <= nx));
+    const char* base[NM];
+    unsigned stride[NM];
+    int col[3];
+    const P* src = static_cast<const P*>(a.src);
+    const float* fx = static_cast<const float*>(a.gx);
+    const float* fy = static_cast<const float*>(a.gy);
+    const float2* car = reinterpret_cast<const float2*>(a.csrc);
+    if (vec) {
+#pragma unroll
+        for (int m = 0; m < NM; ++m) {
+            const int q = min(lane + 32 * m, NQ - 1);
+            if (q >= NP) {
+                const int k = q - NP, p = k / 18;
+                base[m] = reinterpret_cast<const char*>((p == 0 ? fx : fy) + wrapx(xa0 + 4 * (k - 18 * p)));
+                stride[m] = 4 * pitch;
+            } else if (S == S_F16S && q >= 72) {
+                base[m] = reinterpret_cast<const char*>(car + wrapx(xa0 + 2 * (q - 72)));
+                stride[m] = 8 * pitch;
+            } else {
+                constexpr int PC = kStCols / CA;             // chunks of a plane
+                const int p = q / PC;
+                base[m] = reinterpret_cast<const char*>(src + p * a.plane + wrapx(xa0 + CA * (q - PC * p)));
+                stride[m] = (unsigned)sizeof(P) * pitch;
+            }
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) col[k] = wrapx(xa0 + lane + 32 * k);
+    }
+    int ly = (y0 - H - OFF) % ny;                            // lattice row of the next copy
+    if (ly < 0) ly += ny;
+    auto copy_row = [&](int i) {
+        const uint32_t pd = sm + (i & (kStPR - 1)) * ROW, fd = frc + (i & (R - 1)) * kStFRow;
+        if (vec) {
+            const uint32_t d = pd + lane * 16, g = fd + lane * 16;
+#pragma unroll
+            for (int m = 0; m < NM; ++m) {
+                const uint32_t dp = d + m * 512, df = g + m * 512 - NP * 16;
+                const uint32_t e = 32 * m + 31 < NP ? dp : (32 * m >= NP ? df : (lane + 32 * m < NP ? dp : df));
+                if (32 * m + 31 < NQ || lane + 32 * m < NQ) copy_async<16>(e, base[m] + (uint64_t)ly * stride[m]);
+            }
+        } else {
+            const int64_t r = (int64_t)ly * pitch;
+            auto columns = [&](auto&& one) {
+                one(0, col[0]);
+                one(1, col[1]);
+                if (lane < kStCols - 64) one(2, col[2]);
+            };
+#pragma unroll 1
+            for (int p = 0; p < 8; ++p) {
+                const P* b = src + p * a.plane + r;
+                const uint32_t d = pd + (p * kStCols + lane) * (uint32_t)sizeof(P);
+                columns([&](int k, int x) {
+                    if constexpr (S == S_F16S)
+                        asm volatile("st.shared.u16 [%0], %1;" ::"r"(d + k * 64), "h"(__half_as_ushort(ldg(b + x)))
+                                     : "memory");
+                    else
+                        copy_async<4>(d + k * 128, b + x);
+                });
+            }
+            columns([&](int k, int x) {
+                copy_async<4>(fd + lane * 4 + k * 128, fx + r + x);
+                copy_async<4>(fd + (kStCols + lane) * 4 + k * 128, fy + r + x);
+                if constexpr (S == S_F16S) copy_async<8>(pd + kStCols * 16 + lane * 8 + k * 256, car + r + x);
+            });
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        ly = wrap_inc(ly, ny);
+    };
+    // level boundaries (FP16S: the first one below the decoded rows)
+    constexpr int NB = T - 1 + LAG;
+    pair_t up[NB > 0 ? NB : 1][2][3], mid[NB > 0 ? NB : 1][2];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) up[b][0][k] = up[b][1][k] = 0;
+        mid[b][0] = mid[b][1] = 0;
+    }
+    int64_t so = (int64_t)y0 * pitch + xs;                   // the lane's first column of the next output row
+
+    // one iteration; K = i mod 2
+    auto iter = [&](int i, auto k_c) {
+        constexpr int K = decltype(k_c)::value;
+        pair_t f[8];
+        ResSnap<S> sn0{}, sn1{};
+        if (CHECK && i >= 2 * H && ok) {
+            sn0 = snap_load<S>(a, n, (int64_t)so);
+            sn1 = snap_load<S>(a, n, (int64_t)so + 1);
+        }
+        __syncwarp();                             // every lane is done with the rows this copy replaces
+        copy_row(i + AHEAD);                      // (rows past the last are copied too: any row is in range)
+        asm volatile("cp.async.wait_group %0;" ::"n"(LA) : "memory");
+        __syncwarp();                             // the rows of this iteration have arrived for every lane
+        // Over boundary b: the pulled populations of the next level meet their
+        // opposites, and only then the boundary's registers take the new row.
+        // Populations 6 and 8 cross negated (Opp2).
+        Opp2 o;
+        auto cross = [&](int b, auto&& g) {
+            const pair_t d4 = g(4), d7 = from_right(g(7)), d8 = from_left(g(8));
+            if (CHECK && b == NB - 1) {
+                f[0] = mid[b][0];
+                f[1] = up[b][K][0];
+                f[2] = mid[b][1];
+                f[3] = d4;
+                f[4] = up[b][K][1];
+                f[5] = neg2(up[b][K][2]);
+                f[6] = d7;
+                f[7] = neg2(d8);
+            }
+            o = opposites2(mid[b][0], up[b][K][0], mid[b][1], d4, up[b][K][1], up[b][K][2], d7, d8);
+            up[b][K][0] = g(2);
+            up[b][K][1] = from_left(g(5));
+            up[b][K][2] = from_right(g(6));
+            mid[b][0] = from_left(g(1));
+            mid[b][1] = from_right(g(3));
+        };
+        if constexpr (S == S_F32) {
+            // f_p(x) = f*_p(x - c_p), from rows i - 1, i and i + 1 (local rows
+            // of the copies start one above the strip's, hence the + 1)
+            constexpr int PL = kStCols * 4;
+            const uint32_t o4 = own * 4, rm = sm + (i & (kStPR - 1)) * ROW + o4,
+                           r0 = sm + ((i + 1) & (kStPR - 1)) * ROW + o4, rp = sm + ((i + 2) & (kStPR - 1)) * ROW + o4;
+            auto left = [&](uint32_t r) { return pk(lds_float(r - 4), lds_float(r)); };
+            auto right = [&](uint32_t r) { return pk(lds_float(r + 4), lds_float(r + 8)); };
+            pair_t w[8];
+            w[0] = left(r0);
+            w[1] = lds_pair(rm + PL);
+            w[2] = right(r0 + 2 * PL);
+            w[3] = lds_pair(rp + 3 * PL);
+            w[4] = left(rm + 4 * PL);
+            w[5] = right(rm + 5 * PL);
+            w[6] = right(rp + 6 * PL);
+            w[7] = left(rp + 7 * PL);
+            o = opposites2(w);
+            if (CHECK && T == 1)
+#pragma unroll
+                for (int p = 0; p < 8; ++p) f[p] = w[p];
+        } else {
+            // the populations of the lane's columns in row i (pull_decode)
+            const uint32_t r = sm + (i & (kStPR - 1)) * ROW;
+            const float k1 = 0.5f * (1.0f - c.theta), k5 = 0.25f * c.theta;
+            pair_t e0, e1;                        // (m*_10, m*_01) of either column
+            lds_pairs(r + kStCols * 16 + own * 8, e0, e1);
+            const pair_t c10 = pk(pk_lo(e0), pk_lo(e1)), c01 = pk(pk_hi(e0), pk_hi(e1));
+            const pair_t sum = add2(c10, c01), dif = sub2(c10, c01);
+            auto stored = [&](int p) {            // (populations 6 and 8 cross negated)
+                uint32_t h = lds_u32(r + (p * kStCols + own) * 2);
+                if (p == 5 || p == 7) h ^= 0x80008000u;
+                const float2 v = __half22float2(*reinterpret_cast<__half2*>(&h));
+                return pk(v.x, v.y);
+            };
+            cross(0, [&](int p) {
+                switch (p) {
+                    case 1: return fma2(splat(k1), c10, stored(0));
+                    case 2: return fma2(splat(k1), c01, stored(1));
+                    case 3: return fma2(splat(-k1), c10, stored(2));
+                    case 4: return fma2(splat(-k1), c01, stored(3));
+                    case 5: return fma2(splat(k5), sum, stored(4));
+                    case 6: return fma2(splat(k5), dif, stored(5));
+                    case 7: return fma2(splat(-k5), sum, stored(6));
+                    default: return fma2(splat(-k5), dif, stored(7));
+                }
+            });
+        }
+#pragma unroll
+        for (int j = 1; j <= T; ++j) {
+            if (i < 2 * (j - 1 + LAG)) break;         // level j starts two rows after level j - 1
+            const uint32_t fr = frc + ((i + OFF - LAG - (j - 1)) & (R - 1)) * kStFRow + own * 4;
+            const pair_t gx = lds_pair(fr), gy = lds_pair(fr + kStCols * 4);
+            const Post2 m = collide2<GEN>(moments2(o, c), gx, gy, c);
+            if (j < T) {
+                const Pop2<!GEN> w(m, c);
+                cross(j - 1 + LAG, [&](int p) {
+                    switch (p) {
+                        case 1: return w.f1(c);
+                        case 2: return w.f2(c);
+                        case 3: return w.f3(c);
+                        case 4: return w.f4(c);
+                        case 5: return w.f5();
+                        case 6: return w.nf6();
+                        case 7: return w.f7();
+                        default: return w.nf8();
+                    }
+                });
+                continue;
+            }
+            // level T: the output row
+            pair_t fs[8];
+            if (CHECK && ok) {
+                float fl[8], fh[8], gxl, gxh, gyl, gyh;
+#pragma unroll
+                for (int p = 0; p < 8; ++p) unpk(f[p], fl[p], fh[p]);
+                unpk(gx, gxl, gxh);
+                unpk(gy, gyl, gyh);
+                check_node<S>(a, n, (int64_t)so, acc, sn0, fl, gxl, gyl, 0.0f, 0.0f);
+                if (xs + 1 < nx) check_node<S>(a, n, (int64_t)so + 1, acc, sn1, fh, gxh, gyh, 0.0f, 0.0f);
+            }
+            if constexpr (S == S_F32) {
+                Pop2<!GEN>(m, c).all(c, fs);
+                if (ok) {
+                    float* d = static_cast<float*>(a.dst);
+#pragma unroll
+                    for (int p = 0; p < 8; ++p) {
+                        *reinterpret_cast<pair_t*>(d + so) = fs[p];   // (an odd lattice's last pair ends in the pad)
+                        d += a.plane;
+                    }
+                }
+            } else {
+                // the deviations, rounded to FP16, and the carriers that absorb
+                // the first moments of the rounding (store_f16s)
+                Post2 w = m;
+                w.m10 = w.m01 = 0;
+                w.m12 = fma2(splat(-c.qtheta), m.m10, m.m12);
+                w.m21 = fma2(splat(-c.qtheta), m.m01, m.m21);
+                Pop2<!GEN>(w, c).all(c, fs);
+                __half* d = static_cast<__half*>(a.dst);
+                pair_t r[8];
+#pragma unroll
+                for (int p = 0; p < 8; ++p) {
+                    float lo, hi;
+                    unpk(fs[p], lo, hi);
+                    const __half2 h = __floats2half2_rn(lo, hi);
+                    if (ok) *reinterpret_cast<__half2*>(d + so) = h;
+                    const float2 b = __half22float2(h);
+                    r[p] = pk(b.x, b.y);
+                    d += a.plane;
+                }
+                const pair_t r46 = sub2(r[4], r[6]), r57 = sub2(r[5], r[7]);
+                const pair_t e10 = add2(sub2(r[0], r[2]), sub2(r46, r57));
+                const pair_t e01 = add2(sub2(r[1], r[3]), add2(r46, r57));
+                float4 v;
+                unpk(sub2(m.m10, e10), v.x, v.z);
+                unpk(sub2(m.m01, e01), v.y, v.w);
+                if (ok) *reinterpret_cast<float4*>(reinterpret_cast<float2*>(a.cdst) + so) = v;
+            }
+            so += pitch;
+        }
+    };
+
+    using K0 = std::integral_constant<int, 0>;
+    using K1 = std::integral_constant<int, 1>;
+#pragma unroll
+    for (int r = 0; r < AHEAD; ++r) copy_row(r);
+    int i = 0;
+    for (;;) {                                    // (one copy of each phase: the code fits the instruction cache)
+        iter(i, K0{});
+        if (++i >= nit) break;
+        iter(i, K1{});
+        if (++i >= nit) break;
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");     // no copy outlives the strip
+}
+
+template <int S, bool GEN, int T, bool CHECK>
+__global__ void __launch_bounds__(32 * st_nw<T>(), st_minb<T>())
+k_strip(const StepParams a, const PairCoef c, int seg, int nstrips, int items) {
+    extern __shared__ float4 st_mem[];
+    const int warp = threadIdx.x >> 5;
+    const int item = (int)blockIdx.x * st_nw<T>() + warp;
     ResAcc<S> acc;
-    wave_block<S, GEN, T, CHECK, I, true>(a, c, wv_ring, strip, y0, min(seg, a.ny - y0), acc);
+    if (item < items) {
+        const int strip = item % nstrips, y0 = (item / nstrips) * seg;
+        const uint32_t sm = (uint32_t)__cvta_generic_to_shared(st_mem) + warp * st_warp_smem<S, T>();
+        strip_walk<S, GEN, T, CHECK>(a, c, sm, strip, y0, min(seg, a.ny - y0), acc);
+    }
     if (CHECK) residual_reduce<S>(a, acc);
 }
 
@@ -1263,7 +1653,7 @@ k_fields(const StepParams a, const Coef<double> c, typename StoreT<S>::T theta, 
     const int x = blockIdx.x * 32 + threadIdx.x;
     if (y >= ny || x >= nx) return;
     const int ym = wrap_dec(y, ny), yp = wrap_inc(y, ny);
-    const int64_t r0 = (int64_t)y * nx, rm = (int64_t)ym * nx, rp = (int64_t)yp * nx;
+    const int64_t r0 = (int64_t)y * a.pitch, rm = (int64_t)ym * a.pitch, rp = (int64_t)yp * a.pitch;
     T f[8];
     gather<S>(a, r0, rm, rp, x, wrap_dec(x, nx), wrap_inc(x, nx), f, theta);
     const int64_t idx = r0 + x;
@@ -1298,7 +1688,7 @@ k_fields(const StepParams a, const Coef<double> c, typename StoreT<S>::T theta, 
     // (FP16S: back from the state's scaled units, a power of two)
     const double un = S == S_F16S ? (double)a.hinv : 1.0;
     const double mb11 = c.b11 * m11, mbs = c.bs * ms, mbd = c.bd * md;
-    const int64_t o = out.tr ? (int64_t)x * ny + y : idx;
+    const int64_t o = out.tr ? (int64_t)x * ny + y : (int64_t)y * nx + x;
     if (out.p[0]) out.p[0][o] = u * un;
     if (out.p[1]) out.p[1][o] = v * un;
     if (out.p[2]) out.p[2][o] = -0.5 * (mbs + mbd) * un;
@@ -1316,10 +1706,10 @@ k_export(const StepParams a, typename StoreT<S>::T theta, double* out) {
     const int x = blockIdx.x * 32 + threadIdx.x;
     if (y >= ny || x >= nx) return;
     const int ym = wrap_dec(y, ny), yp = wrap_inc(y, ny);
-    const int64_t r0 = (int64_t)y * nx, rm = (int64_t)ym * nx, rp = (int64_t)yp * nx;
+    const int64_t r0 = (int64_t)y * a.pitch, rm = (int64_t)ym * a.pitch, rp = (int64_t)yp * a.pitch;
     T f[8];
     gather<S>(a, r0, rm, rp, x, wrap_dec(x, nx), wrap_inc(x, nx), f, theta);
-    const int64_t idx = r0 + x, n = (int64_t)nx * ny;
+    const int64_t idx = (int64_t)y * nx + x, n = (int64_t)nx * ny;
     // (FP16S: back from the state's scaled units; a power of two, exact)
     const double unscale = S == S_F16S ? (double)a.hinv : 1.0;
 #pragma unroll
@@ -1353,7 +1743,7 @@ k_import(const StepParams a, typename StoreT<S>::T theta, const double* in) {
     fs[5] = T(in[5 * n + rp + xm]) * sc;
     fs[6] = T(in[6 * n + rm + xm]) * sc;
     fs[7] = T(in[7 * n + rm + xp]) * sc;
-    const int64_t idx = r0 + x;
+    const int64_t idx = (int64_t)y * a.pitch + x;
     P* d = static_cast<P*>(a.dst);
     if constexpr (S == S_F16S) {
         const Mom<T> s = moments(fs);
@@ -1373,15 +1763,16 @@ k_import(const StepParams a, typename StoreT<S>::T theta, const double* in) {
 // patterns, so an unsigned 64-bit atomicMax suffices) and `bad` set by a
 // non-finite entry.
 template <typename G>
-__global__ void k_force_ingest(const double* gx, const double* gy, G* ox, G* oy, int64_t n,
+__global__ void k_force_ingest(const double* gx, const double* gy, G* ox, G* oy, int64_t n, int nx, int pitch,
                                unsigned long long* absmax, unsigned int* bad) {
     double m = 0.0;
     unsigned int b = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
         const double u = gx[i], v = gy[i];
-        ox[i] = G(u);
-        oy[i] = G(v);
+        const int64_t o = i + (i / nx) * (pitch - nx);   // rows of nx values, pitch apart
+        ox[o] = G(u);
+        oy[o] = G(v);
         if (!(isfinite(u) && isfinite(v))) b = 1;
         m = fmax(m, fmax(fabs(u), fabs(v)));
     }
@@ -1467,6 +1858,14 @@ inline int adapt_period(int period, double r, double r_prev) {
     return (r > 0.95 * r_prev && period < 64) ? (period * 2 > 64 ? 64 : period * 2) : period;
 }
 
+// Elements between rows of a lattice the library lays out itself: rows start
+// on 16-byte boundaries (FP32: four columns, FP16: eight), which the strip
+// kernel's copies need.  Very narrow lattices stay unpadded.
+inline int row_pitch(int dtype, int nx) {
+    const int m = dtype == S_F64 || nx < 32 ? 1 : (dtype == S_F16S ? 8 : 4);
+    return (nx + m - 1) / m * m;
+}
+
 inline int64_t step_tiles(int nx, int ny, int V) {
     return (int64_t)((nx + 32 * V - 1) / (32 * V)) * ((ny + BY - 1) / BY);
 }
@@ -1498,12 +1897,75 @@ inline int64_t wave_blocks(int nx, int ny, int seg) {
     return (int64_t)((nx + wv_ox<T>() - 1) / wv_ox<T>()) * ((ny + seg - 1) / seg);
 }
 
-// T fused steps on the wavefront schedule (T = 3 or 4; check: T = 4 with the
-// residual on the last step); defined with each storage type's kernels.
-cudaError_t wave_f32(const StepParams& a, const Coef<float>& c, bool gen, int T, bool check, int seg,
-                     cudaStream_t st);
-cudaError_t wave_f16s(const StepParams& a, const Coef<float>& c, bool gen, int T, bool check, int seg,
+// Strips of a strip launch of T steps.
+inline int64_t strip_count(int dtype, int T, int nx) {
+    const int halo = T - 1 + (dtype == S_F16S ? 1 : 0), left = (halo + 1) & ~1, ox = (kStSlots - left - halo) & ~1;
+    return (nx + ox - 1) / ox;
+}
+
+struct StripShape {
+    int T = 0, seg = 0;
+    double cost = 0.0;            // modelled cycles of one launch
+};
+
+// Rows per segment of a launch of T steps that takes the fewest cycles on
+// `nsm` multiprocessors of `warps` resident warps each.  A warp's iteration
+// costs about 70 + 115 w cycles per level with w warps on its scheduler, and a
+// segment of seg rows takes seg + 2 (halo rows) iterations, so the best
+// segments are those whose warps just fill a whole number of waves
+// (4096 x 3000, T = 5: 213 to 229 us with 32 to 256 rows chosen by halving,
+// 164 us with the 125 rows that fill one wave).  rows > 0 fixes the segment.
+inline StripShape strip_shape(int dtype, int T, int nx, int ny, int nsm, int warps, int rows) {
+    const int64_t ns = strip_count(dtype, T, nx);
+    const int halo = T - 1 + (dtype == S_F16S ? 1 : 0);
+    StripShape best;
+    auto consider = [&](int64_t seg) {
+        if (seg < 1) seg = 1;
+        if (seg > ny) seg = ny;
+        const int64_t items = ns * ((ny + seg - 1) / seg), slots = (int64_t)nsm * warps;
+        double cost = 0.0;
+        for (int64_t left = items; left > 0; left -= slots) {
+            const int64_t now = left < slots ? left : slots;
+            const double w = (double)((now + 4 * nsm - 1) / (4 * nsm));
+            const double one = (double)(seg + 2 * halo) * (T * (70.0 + 115.0 * w) + 150.0);
+            if (left > 8 * slots) {                // many waves: they run into one another
+                const double waves = (double)(left - 4 * slots) / (double)slots;
+                cost += waves * one;
+                left = 4 * slots + slots;
+                continue;
+            }
+            cost += one;
+        }
+        cost += 4000.0;                            // the launch itself
+        if (best.seg == 0 || cost < best.cost) {
+            best.T = T;
+            best.seg = (int)seg;
+            best.cost = cost;
+        }
+    };
+    if (rows > 0) {
+        consider(rows);
+        return best;
+    }
+    for (int w = 1; w <= 24 * warps / 4; ++w) {     // w warps per scheduler in all
+        const int64_t nseg = (int64_t)4 * nsm * w / ns;
+        if (nseg < 1) continue;
+        const int64_t seg = (ny + nseg - 1) / nseg;
+        if (seg < 4 && best.seg) break;
+        consider(seg < 4 ? 4 : seg);
+    }
+    if (best.seg == 0) consider(256);
+    return best;
+}
+
+// T fused steps on the wavefront schedule (k_strip; FP32: T = 2 .. 7, FP16S:
+// T = 3, 4; check: T = 4 with the residual on the last step), segments of seg
+// rows.  warps non-null: only the resident warps per multiprocessor of that
+// kernel.  Defined with each storage type's kernels.
+cudaError_t strip_f32(const StepParams& a, const Coef<float>& c, bool gen, int T, bool check, int seg, int* warps,
                       cudaStream_t st);
+cudaError_t strip_f16s(const StepParams& a, const Coef<float>& c, bool gen, int T, bool check, int seg, int* warps,
+                       cudaStream_t st);
 
 // Three fused steps (k_step3); defined with each storage type's kernels.
 cudaError_t step3_f32(const StepParams& a, const Coef<float>& c, bool gen, bool check,

@@ -133,6 +133,7 @@ extern "C" int lbm_step_checked_noalloc(int nx, int ny, double lambda, double mu
     StepParams a{};
     a.nx = nx;
     a.ny = ny;
+    a.pitch = nx;
     a.plane = (int64_t)nx * ny;
     a.src = f_src;
     a.dst = f_dst;

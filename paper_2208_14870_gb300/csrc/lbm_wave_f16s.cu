@@ -1,11 +1,15 @@
-// Wavefront kernels (k_wave, three or four steps per launch) for the LBM_F16S
-// population storage; a translation unit of their own so that they compile in
-// parallel with the other kernels.
+// Strip kernels (k_strip, three or four steps per launch) for the LBM_F16S
+// population storage.
 #include "lbm_ops.cuh"
 
 namespace lbm {
-cudaError_t wave_f16s(const StepParams& a, const Coef<float>& c, bool gen, int T, bool check, int seg,
-                      cudaStream_t st) {
-    return launch_wave<S_F16S>(a, c, gen, T, check, seg, st);
+cudaError_t strip_f16s(const StepParams& a, const Coef<float>& c, bool gen, int T, bool check, int seg, int* warps,
+                       cudaStream_t st) {
+    if (check) return T == 4 ? launch_strip_t<S_F16S, 4, true>(a, c, gen, seg, warps, st) : cudaErrorInvalidValue;
+    switch (T) {
+        case 3: return launch_strip_t<S_F16S, 3, false>(a, c, gen, seg, warps, st);
+        case 4: return launch_strip_t<S_F16S, 4, false>(a, c, gen, seg, warps, st);
+        default: return cudaErrorInvalidValue;
+    }
 }
 }  // namespace lbm

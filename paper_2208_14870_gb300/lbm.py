@@ -61,6 +61,7 @@ _SIGS = {
     "lbm_get_host_transfer": (_c.c_int, [_vp, _c.POINTER(_c.c_int)]),
     "lbm_set_steps_per_launch": (_c.c_int, [_vp, _c.c_int]),
     "lbm_get_steps_per_launch": (_c.c_int, [_vp, _c.POINTER(_c.c_int)]),
+    "lbm_get_launch_steps": (_c.c_int, [_vp, _c.POINTER(_c.c_int)]),
     "lbm_set_wavefront": (_c.c_int, [_vp, _c.c_int]),
     "lbm_get_wavefront": (_c.c_int, [_vp, _c.POINTER(_c.c_int)]),
     "lbm_set_force": (_c.c_int, [_vp, _vp, _vp]),
@@ -172,6 +173,12 @@ def lbm_set_steps_per_launch(ctx: int, k: int) -> None:
 def lbm_get_steps_per_launch(ctx: int) -> int:
     k = _c.c_int()
     _check(_lib.lbm_get_steps_per_launch(ctx, _c.byref(k)), "lbm_get_steps_per_launch")
+    return k.value
+
+
+def lbm_get_launch_steps(ctx: int) -> int:
+    k = _c.c_int()
+    _check(_lib.lbm_get_launch_steps(ctx, _c.byref(k)), "lbm_get_launch_steps")
     return k.value
 
 

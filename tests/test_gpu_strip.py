@@ -1,0 +1,65 @@
+"""Strip kernel (two to seven steps per launch, one warp per strip of 64 slot
+columns) against one step per launch, at the sizes where its copies, halos
+and pairs can go wrong: widths that are no multiple of a 16-byte chunk (every
+remainder of eight), odd widths, whole numbers of strips and one column more,
+heights of one segment row, and every step count a launch can take.  FP32
+states must be equal; FP16-shifted states are compared with the three-step
+tile kernel, which rounds to FP16 at the same steps."""
+import numpy as np
+import pytest
+
+import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():  # pragma: no cover
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+from paper_2208_14870_gb300 import Lattice  # noqa: E402
+
+# 280 and 364: whole strips of 56 and 52 output columns (five and seven steps)
+SIZES = [(256, 8), (257, 9), (258, 31), (259, 40), (260, 13), (261, 8), (262, 21), (263, 17),
+         (280, 33), (281, 10), (364, 12), (365, 25), (1000, 61)]
+
+
+def _state(nx, ny, dtype, spl, wave, steps, check_every=None, **kw):
+    lam, mu = W.lame_2d(1.0, 0.3)
+    rng = np.random.RandomState(nx * 1000 + ny)
+    gx, gy = rng.standard_normal((2, ny, nx)) / max(nx, ny) ** 2
+    with Lattice(nx, ny, lam, mu, dtype, **kw) as lat:
+        lat.steps_per_launch = spl
+        lat.wavefront = wave
+        lat.set_force(gx, gy)
+        if check_every:
+            lat.iterate_checked(steps, check_every)
+        else:
+            lat.iterate(steps)
+        return lat.populations()
+
+
+@pytest.mark.parametrize("nx,ny", SIZES)
+@pytest.mark.parametrize("rows", [1, 6, -1])
+def test_f32_equals_single_steps(nx, ny, rows):
+    for steps in (2, 3, 4, 5, 6, 7, 8, 15):
+        ref = _state(nx, ny, "f32", 1, 0, steps)
+        assert np.array_equal(_state(nx, ny, "f32", 4, rows, steps), ref), steps
+
+
+@pytest.mark.parametrize("nx,ny", [(257, 9), (364, 40)])
+def test_f32_general_rates_and_checks(nx, ny):
+    kw = dict(tau12=0.9, tau22=0.3, theta=0.25)
+    for steps in (2, 5, 6, 7, 20):
+        ref = _state(nx, ny, "f32", 1, 0, steps, **kw)
+        assert np.array_equal(_state(nx, ny, "f32", 4, -1, steps, **kw), ref), steps
+    ref = _state(nx, ny, "f32", 1, 0, 37, **kw)
+    assert np.array_equal(_state(nx, ny, "f32", 4, -1, 37, check_every=9, **kw), ref)
+
+
+@pytest.mark.parametrize("nx,ny", SIZES)
+@pytest.mark.parametrize("kw", [dict(), dict(tau12=0.9, tau22=0.3)])
+def test_f16s_equals_tiles(nx, ny, kw):
+    ny = max(ny, 16)
+    for rows in (5, -1):
+        ref = _state(nx, ny, "f16s", 3, 0, 6, **kw)
+        assert np.array_equal(_state(nx, ny, "f16s", 3, rows, 6, **kw), ref)
