@@ -152,7 +152,10 @@ int lbm_get_host_transfer(lbm_ctx *ctx, int *mode);
  * change an LBM_F32 state, k = 4 on the wavefront schedule lets LBM_F32
  * launches take as many steps as suit the lattice, up to seven
  * (lbm_get_launch_steps); LBM_F16S keeps groups of four.  Available for LBM_F32 and
- * LBM_F16S storage on any lattice; the default is 4 (wavefront schedule) from
+ * LBM_F16S storage on any lattice.  Until this function or lbm_set_wavefront is
+ * called, LBM_F32 lattices take whichever schedule their size suits (strips of
+ * the wavefront schedule, or tiles held in registers, of up to twelve steps per
+ * launch), which gives the same states; the default is 4 (wavefront schedule) from
  * nx >= 256 and ny >= 8 on, else 3 from nx >= 64 and ny >= 16 on (a smaller
  * lattice fills the on-chip tile more than once and is faster one step per
  * launch).  LBM_F64 storage always runs one step per

@@ -49,7 +49,8 @@ struct lbm_ctx {
     int device = 0;
     int nx = 0, ny = 0, dtype = 0;
     int64_t n = 0, plane = 0;
-    int pitch = 0;                 // elements between rows (row_pitch)
+    int pitch = 0, ghost = 0;      // elements between rows, ghost columns at either end (row_ghost)
+    bool ghosts_ok = true;         // the current state's ghost columns hold its images
     lbm_rates rates{};
     bool gen = false;              // non-standard w_12, w_21, w_22
     cudaStream_t stream = nullptr;
@@ -87,6 +88,10 @@ struct lbm_ctx {
     int64_t nblocks2 = 0;          // grid of the two-step check launch
     StripShape shape[kStTMax + 1]; // strip launches per step count ([0]: checked), cleared by lbm_set_wavefront
     int wave_T = 0;                // FP32: steps per plain strip launch (0: not chosen yet)
+    bool auto_plan = true;         // FP32: strip or tile launches as they suit the lattice, until the
+                                   // caller sets a schedule (lbm_set_steps_per_launch, lbm_set_wavefront)
+    int plan = 0;                  // 0: not chosen yet, 1: strips, 2: register tiles (tile)
+    TileShape tile;
 };
 
 namespace {
@@ -102,12 +107,16 @@ StepParams params(const lbm_ctx* c, int src) {
     a.ny = c->ny;
     a.pitch = c->pitch;
     a.plane = c->plane;
-    a.src = c->pop[src];
-    a.dst = c->pop[src ^ 1];
-    a.csrc = c->car[src];
-    a.cdst = c->car[src ^ 1];
-    a.gx = c->force;
-    a.gy = static_cast<const char*>(c->force) + c->plane * force_elem_bytes(c->dtype);
+    // (pointers to column 0 of row 0)
+    const size_t po = c->ghost * pop_elem_bytes(c->dtype), fo = c->ghost * force_elem_bytes(c->dtype);
+    a.src = static_cast<const char*>(c->pop[src]) + po;
+    a.dst = static_cast<char*>(c->pop[src ^ 1]) + po;
+    if (c->dtype == LBM_F16S) {
+        a.csrc = c->car[src] + 2 * c->ghost;
+        a.cdst = c->car[src ^ 1] + 2 * c->ghost;
+    }
+    a.gx = static_cast<const char*>(c->force) + fo;
+    a.gy = static_cast<const char*>(c->force) + fo + c->plane * force_elem_bytes(c->dtype);
     a.hscale = c->hscale;
     a.hinv = c->hinv;
     a.snap = c->snap;
@@ -155,6 +164,7 @@ cudaError_t launch_step(lbm_ctx* c, bool check) {
     }
     if (e == cudaSuccess && check) e = finish_residual_launch(c, c->nblocks);
     if (e == cudaSuccess) {
+        c->ghosts_ok = false;
         c->cur ^= 1;
         c->step += 1;
         c->staged_fields = false;
@@ -171,6 +181,7 @@ cudaError_t launch_step2(lbm_ctx* c, bool check) {
                         : step2_f16s(a, coef<float>(c->rates), c->gen, check, (int)c->nblocks2, c->stream);
     if (e == cudaSuccess && check) e = finish_residual_launch(c, c->nblocks2);
     if (e == cudaSuccess) {
+        c->ghosts_ok = false;
         c->cur ^= 1;
         c->step += 2;
         c->staged_fields = false;
@@ -185,6 +196,7 @@ cudaError_t launch_step3(lbm_ctx* c) {
                         ? step3_f32(a, coef<float>(c->rates), c->gen, false, 0, c->stream)
                         : step3_f16s(a, coef<float>(c->rates), c->gen, false, 0, c->stream);
     if (e == cudaSuccess) {
+        c->ghosts_ok = false;
         c->cur ^= 1;
         c->step += 3;
         c->staged_fields = false;
@@ -252,6 +264,14 @@ cudaError_t launch_strip(lbm_ctx* c, int T, bool check) {
         blocks = strip_check_blocks(c, sh.seg);
         if (ensure_partials(c, blocks) != LBM_OK) return cudaErrorMemoryAllocation;
     }
+    if (!c->ghosts_ok) {
+        const StepParams g = params(c, c->cur ^ 1);      // dst = current buffer
+        const dim3 grid((unsigned)std::min<int64_t>(((int64_t)c->ny * 16 * 8 + 255) / 256, 4096));
+        e = c->dtype == LBM_F32 ? launch_after(k_fill_ghosts<S_F32>, grid, dim3(256), 0, c->stream, g)
+                                : launch_after(k_fill_ghosts<S_F16S>, grid, dim3(256), 0, c->stream, g);
+        if (e != cudaSuccess) return e;
+        c->ghosts_ok = true;
+    }
     const StepParams a = params(c, c->cur);
     e = c->dtype == LBM_F32 ? strip_f32(a, coef<float>(c->rates), c->gen, T, check, sh.seg, nullptr, c->stream)
                             : strip_f16s(a, coef<float>(c->rates), c->gen, T, check, sh.seg, nullptr, c->stream);
@@ -261,6 +281,69 @@ cudaError_t launch_strip(lbm_ctx* c, int T, bool check) {
         c->step += T;
         c->staged_fields = false;
     }
+    return e;
+}
+
+// FP32 without a schedule set by the caller: strips or register tiles,
+// whichever the models say takes fewer cycles per step (every plan gives the
+// same states).  Tiles win up to about 10^6 nodes, where a strip launch is bound
+// by the latency of its rows (333 x 517: 1.1 against 2.1 us per step).
+cudaError_t choose_plan(lbm_ctx* c) {
+    if (c->plan) return cudaSuccess;
+    c->tile = tile_shape(c->nx, c->ny, c->nsm > 0 ? c->nsm : 1);
+    c->plan = 2;
+    if (c->ghost) {
+        int T = 0;
+        StripShape sh;
+        cudaError_t e = wave_steps(c, &T);
+        if (e == cudaSuccess) e = wave_shape(c, T, false, &sh);
+        if (e != cudaSuccess) return e;
+        if (sh.cost * c->tile.T < c->tile.cost * T) c->plan = 1;
+    }
+    return cudaSuccess;
+}
+
+bool auto_on(const lbm_ctx* c) { return c->auto_plan && c->dtype == LBM_F32; }
+
+cudaError_t launch_tile(lbm_ctx* c, int T, bool check) {
+    TileShape t = c->tile;
+    t.T = T;
+    const int64_t blocks = tile_count(t, c->nx, c->ny);
+    if (check && ensure_partials(c, blocks) != LBM_OK) return cudaErrorMemoryAllocation;
+    cudaError_t e = tile_f32(params(c, c->cur), coef<float>(c->rates), c->gen, t, check, c->stream);
+    if (e == cudaSuccess && check) e = finish_residual_launch(c, blocks);
+    if (e == cudaSuccess) {
+        c->ghosts_ok = false;
+        c->cur ^= 1;
+        c->step += T;
+        c->staged_fields = false;
+    }
+    return e;
+}
+
+// n steps in as few tile launches as the tile allows, of equal lengths; check:
+// the last step is the residual-check step.
+cudaError_t run_tiles(lbm_ctx* c, int64_t n, bool check) {
+    cudaError_t e = cudaSuccess;
+    for (int64_t left = (n + c->tile.T - 1) / c->tile.T; left > 0 && e == cudaSuccess; --left) {
+        const int t = (int)((n + left - 1) / left);
+        e = launch_tile(c, t, check && left == 1);
+        n -= t;
+    }
+    return e;
+}
+
+// n plain steps in strip launches of up to T steps: whole groups, then the
+// rest in one launch, or two for T + 1.
+cudaError_t run_strips(lbm_ctx* c, int64_t n) {
+    int T = 0;
+    cudaError_t e = wave_steps(c, &T);
+    while (n >= 2 && e == cudaSuccess) {
+        const int t = n >= T && n != T + 1 ? T : (n == T + 1 ? (T + 1) / 2 : (int)n);
+        e = launch_strip(c, t, false);
+        n -= t;
+    }
+    if (n > 0 && e == cudaSuccess) e = launch_step(c, false);
     return e;
 }
 
@@ -280,18 +363,12 @@ cudaError_t launch_multi(lbm_ctx* c, int T) {
 cudaError_t run_plain(lbm_ctx* c, int64_t n) {
     cudaError_t e = cudaSuccess;
     const bool wave = wave_on(c);
-    if (c->spl >= 4 && wave && c->dtype == LBM_F32) {
-        int T = 0;
-        e = wave_steps(c, &T);
-        while (n >= 2 && e == cudaSuccess) {
-            // whole groups, then the rest in one launch, or two for T + 1
-            const int t = n >= T && n != T + 1 ? T : (n == T + 1 ? (T + 1) / 2 : (int)n);
-            e = launch_strip(c, t, false);
-            n -= t;
-        }
-        if (n > 0 && e == cudaSuccess) e = launch_step(c, false);
-        return e;
+    if (auto_on(c)) {
+        e = choose_plan(c);
+        if (e != cudaSuccess) return e;
+        return c->plan == 2 ? run_tiles(c, n, false) : run_strips(c, n);
     }
+    if (c->spl >= 4 && wave && c->dtype == LBM_F32) return run_strips(c, n);
     const int big = c->spl >= 4 && wave ? 4 : (c->spl >= 3 ? 3 : 0);
     if (big) {
         int64_t groups = n / big, r = n % big;
@@ -319,7 +396,16 @@ cudaError_t run_plain(lbm_ctx* c, int64_t n) {
 // costs twice a plain one, a two-step launch with the check 1.3 times).
 cudaError_t run_window(lbm_ctx* c, int64_t to_check) {
     cudaError_t e;
-    if (c->spl >= 4 && to_check >= 4 && wave_on(c)) {
+    if (auto_on(c)) {
+        e = choose_plan(c);
+        if (e != cudaSuccess) return e;
+        if (c->plan == 2) return run_tiles(c, to_check, true);
+        if (to_check < 4) {
+            e = run_strips(c, to_check - 1);
+            return e == cudaSuccess ? launch_step(c, true) : e;
+        }
+    }
+    if (to_check >= 4 && (auto_on(c) || (c->spl >= 4 && wave_on(c)))) {
         e = run_plain(c, to_check - 4);
         return e == cudaSuccess ? launch_strip(c, 4, true) : e;
     }
@@ -460,10 +546,10 @@ int set_force_dev(lbm_ctx* c, const double* gx, const double* gy) {
     CK(cudaMemsetAsync(c->absmax, 0, sizeof(unsigned long long), c->stream));
     CK(cudaMemsetAsync(c->bad, 0, sizeof(unsigned int), c->stream));
     if (c->dtype == LBM_F64) {
-        double* fx = static_cast<double*>(c->force);
+        double* fx = static_cast<double*>(c->force) + c->ghost;
         k_force_ingest<double><<<2048, 256, 0, c->stream>>>(gx, gy, fx, fx + c->plane, c->n, c->nx, c->pitch, c->absmax, c->bad);
     } else {
-        float* fx = static_cast<float*>(c->force);
+        float* fx = static_cast<float*>(c->force) + c->ghost;
         k_force_ingest<float><<<2048, 256, 0, c->stream>>>(gx, gy, fx, fx + c->plane, c->n, c->nx, c->pitch, c->absmax, c->bad);
     }
     CK(cudaGetLastError());
@@ -568,6 +654,7 @@ int lbm_create_ex(int nx, int ny, double lambda, double mu, int dtype, const lbm
     c->ny = ny;
     c->dtype = dtype;
     c->n = (int64_t)nx * ny;
+    c->ghost = row_ghost(dtype, nx);
     c->pitch = row_pitch(dtype, nx);
     c->plane = round_up((int64_t)c->pitch * ny, 128);
     // Table 1 and Eq. relaxation_rate: theta tau_11 = mu, (1-theta)/2 tau_d = mu,
@@ -599,9 +686,10 @@ int lbm_create_ex(int nx, int ny, double lambda, double mu, int dtype, const lbm
         else if (step2_fits(nx, ny)) c->spl = 2;
     }
 
-    const size_t pb = pop_elem_bytes(dtype) * 8 * c->plane;
-    const size_t fb = force_elem_bytes(dtype) * 2 * c->plane;
-    const size_t cb = sizeof(float) * 2 * c->plane;
+    const int slack = c->ghost ? kRowSlack : 0;
+    const size_t pb = pop_elem_bytes(dtype) * (8 * c->plane + slack);
+    const size_t fb = force_elem_bytes(dtype) * (2 * c->plane + slack);
+    const size_t cb = sizeof(float) * 2 * (c->plane + slack);
     auto alloc = [&](void** p, size_t bytes) -> cudaError_t {
         cudaError_t r = cudaMalloc(p, bytes);
         if (r == cudaSuccess) c->bytes += bytes;
@@ -617,10 +705,14 @@ int lbm_create_ex(int nx, int ny, double lambda, double mu, int dtype, const lbm
     const size_t snap_bytes = 16 * (size_t)c->plane;
     if (e == cudaSuccess) e = alloc(&c->snap, snap_bytes);
     c->partials_len = std::max(c->nblocks, c->nblocks2);
-    if (e == cudaSuccess && dtype != LBM_F64 && wave_on(c)) {
+    if (e == cudaSuccess && dtype != LBM_F64 && (wave_on(c) || (dtype == LBM_F32 && c->ghost))) {
         StripShape sh;
         e = wave_shape(c, 4, true, &sh);
         c->partials_len = std::max(c->partials_len, strip_check_blocks(c, sh.seg));
+    }
+    if (e == cudaSuccess && dtype == LBM_F32) {
+        e = choose_plan(c);
+        c->partials_len = std::max(c->partials_len, c->plan == 2 ? tile_count(c->tile, nx, ny) : int64_t(0));
     }
     if (e == cudaSuccess) e = alloc((void**)&c->partials, sizeof(double) * kRes * c->partials_len);
     if (e == cudaSuccess) e = alloc((void**)&c->result, sizeof(double) * kRes);
@@ -666,6 +758,7 @@ int lbm_set_steps_per_launch(lbm_ctx* c, int k) {
         return fail(LBM_ERR_ARG,
                     "lbm_set_steps_per_launch: several steps per launch need FP32 or FP16-shifted storage");
     c->spl = k;
+    c->auto_plan = false;
     return LBM_OK;
 }
 
@@ -682,7 +775,9 @@ int lbm_get_launch_steps(lbm_ctx* c, int* k) {
     if (rc) return rc;
     if (!k) return fail(LBM_ERR_ARG, "lbm_get_launch_steps: null pointer");
     *k = c->spl >= 4 && !wave_on(c) ? 3 : c->spl;
-    if (c->spl >= 4 && wave_on(c) && c->dtype == LBM_F32) CK(wave_steps(c, k));
+    if (auto_on(c)) CK(choose_plan(c));
+    if (auto_on(c) && c->plan == 2) *k = c->tile.T;
+    else if (c->dtype == LBM_F32 && (auto_on(c) || (c->spl >= 4 && wave_on(c)))) CK(wave_steps(c, k));
     return LBM_OK;
 }
 
@@ -694,6 +789,7 @@ int lbm_set_wavefront(lbm_ctx* c, int rows) {
     if (rows != 0 && c->dtype == LBM_F64)
         return fail(LBM_ERR_ARG, "lbm_set_wavefront: the wavefront kernel needs FP32 or FP16-shifted storage");
     c->wave = rows;
+    c->auto_plan = false;
     for (auto& sh : c->shape) sh = StripShape();
     c->wave_T = 0;
     return LBM_OK;
@@ -868,6 +964,7 @@ int lbm_reset(lbm_ctx* c) {
         CK(cudaMemsetAsync(c->car[c->cur], 0, sizeof(float) * 2 * c->plane, c->stream));
     c->step = 0;
     c->snap_valid = false;
+    c->ghosts_ok = true;
     c->state_zero = true;
     c->staged_fields = false;
     if (c->dtype == LBM_F16S && c->gmax > 0.0) {
@@ -1080,6 +1177,7 @@ int lbm_set_populations(lbm_ctx* c, const double* f) {
     }
     CK(e);
     CK(cudaStreamSynchronize(c->stream));
+    c->ghosts_ok = false;
     c->step = 0;
     c->snap_valid = false;
     c->state_zero = false;

@@ -242,6 +242,18 @@ __device__ __forceinline__ float4 exact_displacement(const float f[8], float gx,
     return d;
 }
 
+// Programmatic dependent launch.  A kernel launched with launch_after (below)
+// starts as soon as its predecessor's blocks have exited, without waiting for
+// the stream to see the predecessor completed: it calls after_predecessor()
+// before it touches global memory, which waits until the predecessor's writes
+// are visible.  Launches in a stream otherwise followed one another on a 2.05 us
+// grid (a tile launch of 4.7 us took 6.25).  No kernel lets its successor
+// start earlier than that: blocks of the next strip launch then took the slots
+// the running one left and clumped (1024^2, 400 steps: 2.37 against 1.85 ms).
+__device__ __forceinline__ void after_predecessor() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 __device__ __forceinline__ int wrap_dec(int i, int n) { return i == 0 ? n - 1 : i - 1; }
 __device__ __forceinline__ int wrap_inc(int i, int n) { return i + 1 == n ? 0 : i + 1; }
 
@@ -451,6 +463,22 @@ __device__ __forceinline__ pair_t from_right(pair_t p) {
     float lo, hi;
     unpk(p, lo, hi);
     return pk(hi, __shfl_down_sync(0xffffffffu, lo, 1));
+}
+
+// Launch a kernel that calls after_predecessor().
+template <typename... P, typename... A>
+inline cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
 }  // namespace lbm

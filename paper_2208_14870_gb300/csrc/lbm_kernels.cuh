@@ -5,8 +5,8 @@
 // type by lbm_step_f64.cu, lbm_step_f32.cu and lbm_step_f16s.cu.
 //
 // Memory layout (structure of arrays): population p of node (x, y) lives at
-// base + p*plane + y*pitch + x (rows padded to whole 16-byte chunks, see
-// row_pitch; `plane` >= pitch*ny is padded to 256 bytes).  The
+// base + p*plane + y*pitch + x (`plane` >= pitch*ny is padded to 256 bytes;
+// rows may hold ghost columns, see row_ghost).  The
 // stored state between steps is the post-collision population f*_p(x) of the
 // previous step ("pull" scheme): a step gathers f_p(x) = f*_p(x - c_p) with the
 // periodic wrap done by index arithmetic (Sec. 5.1), collides, and writes
@@ -52,6 +52,7 @@ constexpr int max_vec() {
     return S == S_F64 ? 2 : (S == S_F16S ? LBM_F16S_V : 4);
 }
 constexpr int kThreads = 32 * BY;
+constexpr int kMaxWarps = 16;          // warps of the largest block that reduces residuals
 
 template <int S> struct StoreT;
 // T: collision arithmetic, P: stored population, G: stored force.
@@ -388,7 +389,7 @@ __device__ __forceinline__ void scatter_local(const StepParams& a, int64_t idx,
 // launch.
 template <int S>
 __device__ __forceinline__ void residual_reduce(const StepParams& a, const ResAcc<S>& acc) {
-    __shared__ double sh[kRes][kThreads / 32];
+    __shared__ double sh[kRes][kMaxWarps];
     __shared__ bool is_last;
     const int tid = threadIdx.y * blockDim.x + threadIdx.x;
     const int lane = tid & 31, warp = tid >> 5;
@@ -1250,6 +1251,16 @@ __device__ __forceinline__ void wave_block(const StepParams& a, const Coef<float
 //
 // The per-node operations are lbm_core.cuh's, so FP32 results equal T
 // single-step launches bit for bit.
+//
+// What bounds it: the five-step FP32 launch moves 72 bytes per node at 6.1 TB/s,
+// 0.90 of the measured copy peak (16384^2, 3.16 ms; the block-wide wavefront
+// kernel before it took 3.31 ms for four steps).  An update issues about 50
+// instructions (that kernel: 90), 27 of them arithmetic, two operations each;
+// FP16S four-step launches are issue-bound at 0.74 of the copy peak (0.63).
+// One code copy serves the first iterations too (each level's test is one
+// uniform branch): with a copy of its own for them the code left the
+// instruction cache and the compiler took 202 registers instead of 150.
+constexpr int kGhost = 8;                        // ghost columns per row end (at least kStTMax + 1)
 constexpr int kStSlots = 64;                     // slot columns of a strip (two per lane)
 constexpr int kStTMax = 7;                       // most steps per launch
 
@@ -1261,11 +1272,12 @@ template <int S, int T> __host__ __device__ constexpr int st_left() { return (st
 template <int S, int T> __host__ __device__ constexpr int st_ox() {
     return (kStSlots - st_left<S, T>() - st_halo<S, T>()) & ~1;
 }
-// warps per block and resident blocks the kernel is compiled for: what lets
-// the registers of T levels fit twelve warps per SM (measured per T at
-// 16384^2: T = 7 as 64-thread blocks 447 GLUPS, as 128-thread blocks 411)
+// warps per block and resident blocks the kernel is compiled for: twelve warps
+// per SM (168 registers a thread; at 16384^2 with registers for eight warps
+// 87.6 ms per 100 steps against 79.8; T = 7 as 64-thread blocks 447 GLUPS, as
+// 128-thread blocks 411)
 template <int T> __host__ __device__ constexpr int st_nw() { return T >= 7 ? 2 : 4; }
-template <int T> __host__ __device__ constexpr int st_minb() { return T >= 7 ? 5 : 2; }
+template <int T> __host__ __device__ constexpr int st_minb() { return T >= 7 ? 6 : 3; }
 // rows copied ahead of the rows in use, and population rows held: FP32 has the
 // rows above, at and below level 1 in use, FP16S the decoded row
 template <int S> __host__ __device__ constexpr int st_la() { return S == S_F16S ? 3 : 1; }
@@ -1288,10 +1300,7 @@ template <int S, int T> __host__ __device__ constexpr int st_smem() { return st_
 
 template <int B>
 __device__ __forceinline__ void copy_async(uint32_t dst, const void* src) {
-    if constexpr (B == 16)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-    else
-        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(dst), "l"(src), "n"(B) : "memory");
+    asm volatile("cp.async.cg.shared.global [%0], [%1], %2;" ::"r"(dst), "l"(src), "n"(B) : "memory");
 }
 __device__ __forceinline__ pair_t lds_pair(uint32_t a) {
     pair_t d;
@@ -1306,6 +1315,9 @@ __device__ __forceinline__ uint32_t lds_u32(uint32_t a) {
     asm volatile("ld.shared.u32 %0, [%1];" : "=r"(d) : "r"(a) : "memory");
     return d;
 }
+__device__ __forceinline__ void sts_pair(uint32_t a, pair_t p) {
+    asm volatile("st.shared.b64 [%0], %1;" ::"r"(a), "l"(p) : "memory");
+}
 __device__ __forceinline__ float lds_float(uint32_t a) {
     float d;
     asm volatile("ld.shared.f32 %0, [%1];" : "=f"(d) : "r"(a) : "memory");
@@ -1319,8 +1331,10 @@ __device__ __forceinline__ pair_t opaque(pair_t p, uint32_t a) {
 }
 
 // One strip and segment.  sm: the warp's shared memory (shared-space address).
-// The lattice's pitch is a multiple of the columns of a 16-byte chunk
-// (row_pitch).
+// The lattice's rows carry ghost columns (row_ghost): the kGhost columns
+// beyond either end hold the periodic images, so that a strip's rows are
+// contiguous and its copies aligned wherever it lies; the strips that own the
+// outermost kGhost columns store their images too.
 template <int S, bool GEN, int T, bool CHECK>
 __device__ __forceinline__ void strip_walk(const StepParams& a, const PairCoef& ca, uint32_t sm, int strip, int y0,
                                            int rows, ResAcc<S>& acc) {
@@ -1342,85 +1356,43 @@ __device__ __forceinline__ void strip_walk(const StepParams& a, const PairCoef& 
     const int xa0 = ((xs0 - OFF + (1 << 20)) & ~(CA - 1)) - (1 << 20);
     const int xs = xs0 + 2 * lane;                           // the lane's first column
     const bool ok = 2 * lane >= HL && 2 * lane < HL + OX && xs < nx;
+    const bool two = ok && xs + 1 < nx;                      // (an odd lattice's last column stands alone)
     const int64_t n = a.plane;
     const int nit = rows + 2 * H;
     const uint32_t frc = sm + kStPR * ROW;                   // force ring
     const uint32_t own = (uint32_t)(xs - xa0);               // the lane's first column within a row
     // Copies of a row: 16-byte chunks, chunk q = lane + 32 m (FP32: 18 per
     // plane, eight populations, then the force; FP16S: 9 per plane, eight
-    // populations, then 36 of the carriers, then the force), or, where a chunk
-    // would straddle the periodic boundary, single columns.
+    // populations, then 36 of the carriers, then the force).
     constexpr int NP = S == S_F16S ? 108 : 144, NQ = NP + 36, NM = (NQ + 31) / 32;
-    auto wrapx = [&](int x) {
-        x %= nx;
-        return x < 0 ? x + nx : x;
-    };
-    const bool vec = nx >= kStCols && (nx % CA == 0 || (xa0 >= 0 && xa0 + kStCols <= nx));
     const char* base[NM];
     unsigned stride[NM];
-    int col[3];
-    const P* src = static_cast<const P*>(a.src);
-    const float* fx = static_cast<const float*>(a.gx);
-    const float* fy = static_cast<const float*>(a.gy);
-    const float2* car = reinterpret_cast<const float2*>(a.csrc);
-    if (vec) {
 #pragma unroll
-        for (int m = 0; m < NM; ++m) {
-            const int q = min(lane + 32 * m, NQ - 1);
-            if (q >= NP) {
-                const int k = q - NP, p = k / 18;
-                base[m] = reinterpret_cast<const char*>((p == 0 ? fx : fy) + wrapx(xa0 + 4 * (k - 18 * p)));
-                stride[m] = 4 * pitch;
-            } else if (S == S_F16S && q >= 72) {
-                base[m] = reinterpret_cast<const char*>(car + wrapx(xa0 + 2 * (q - 72)));
-                stride[m] = 8 * pitch;
-            } else {
-                constexpr int PC = kStCols / CA;             // chunks of a plane
-                const int p = q / PC;
-                base[m] = reinterpret_cast<const char*>(src + p * a.plane + wrapx(xa0 + CA * (q - PC * p)));
-                stride[m] = (unsigned)sizeof(P) * pitch;
-            }
+    for (int m = 0; m < NM; ++m) {
+        const int q = min(lane + 32 * m, NQ - 1);
+        if (q >= NP) {
+            const int k = q - NP, p = k / 18;
+            base[m] = reinterpret_cast<const char*>(static_cast<const float*>(p == 0 ? a.gx : a.gy) + xa0 + 4 * (k - 18 * p));
+            stride[m] = 4 * pitch;
+        } else if (S == S_F16S && q >= 72) {
+            base[m] = reinterpret_cast<const char*>(reinterpret_cast<const float2*>(a.csrc) + xa0 + 2 * (q - 72));
+            stride[m] = 8 * pitch;
+        } else {
+            constexpr int PC = kStCols / CA;                 // chunks of a plane
+            const int p = q / PC;
+            base[m] = reinterpret_cast<const char*>(static_cast<const P*>(a.src) + p * a.plane + xa0 + CA * (q - PC * p));
+            stride[m] = (unsigned)sizeof(P) * pitch;
         }
-    } else {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) col[k] = wrapx(xa0 + lane + 32 * k);
     }
     int ly = (y0 - H - OFF) % ny;                            // lattice row of the next copy
     if (ly < 0) ly += ny;
     auto copy_row = [&](int i) {
-        const uint32_t pd = sm + (i & (kStPR - 1)) * ROW, fd = frc + (i & (R - 1)) * kStFRow;
-        if (vec) {
-            const uint32_t d = pd + lane * 16, g = fd + lane * 16;
+        const uint32_t d = sm + (i & (kStPR - 1)) * ROW + lane * 16, g = frc + (i & (R - 1)) * kStFRow + lane * 16;
 #pragma unroll
-            for (int m = 0; m < NM; ++m) {
-                const uint32_t dp = d + m * 512, df = g + m * 512 - NP * 16;
-                const uint32_t e = 32 * m + 31 < NP ? dp : (32 * m >= NP ? df : (lane + 32 * m < NP ? dp : df));
-                if (32 * m + 31 < NQ || lane + 32 * m < NQ) copy_async<16>(e, base[m] + (uint64_t)ly * stride[m]);
-            }
-        } else {
-            const int64_t r = (int64_t)ly * pitch;
-            auto columns = [&](auto&& one) {
-                one(0, col[0]);
-                one(1, col[1]);
-                if (lane < kStCols - 64) one(2, col[2]);
-            };
-#pragma unroll 1
-            for (int p = 0; p < 8; ++p) {
-                const P* b = src + p * a.plane + r;
-                const uint32_t d = pd + (p * kStCols + lane) * (uint32_t)sizeof(P);
-                columns([&](int k, int x) {
-                    if constexpr (S == S_F16S)
-                        asm volatile("st.shared.u16 [%0], %1;" ::"r"(d + k * 64), "h"(__half_as_ushort(ldg(b + x)))
-                                     : "memory");
-                    else
-                        copy_async<4>(d + k * 128, b + x);
-                });
-            }
-            columns([&](int k, int x) {
-                copy_async<4>(fd + lane * 4 + k * 128, fx + r + x);
-                copy_async<4>(fd + (kStCols + lane) * 4 + k * 128, fy + r + x);
-                if constexpr (S == S_F16S) copy_async<8>(pd + kStCols * 16 + lane * 8 + k * 256, car + r + x);
-            });
+        for (int m = 0; m < NM; ++m) {
+            const uint32_t dp = d + m * 512, df = g + m * 512 - NP * 16;
+            const uint32_t e = 32 * m + 31 < NP ? dp : (32 * m >= NP ? df : (lane + 32 * m < NP ? dp : df));
+            if (32 * m + 31 < NQ || lane + 32 * m < NQ) copy_async<16>(e, base[m] + (uint64_t)ly * stride[m]);
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
         ly = wrap_inc(ly, ny);
@@ -1435,6 +1407,19 @@ __device__ __forceinline__ void strip_walk(const StepParams& a, const PairCoef& 
         mid[b][0] = mid[b][1] = 0;
     }
     int64_t so = (int64_t)y0 * pitch + xs;                   // the lane's first column of the next output row
+
+    // The lane's stores besides its pair in place: the odd last column, and the
+    // periodic images of columns near either end (off: from a column to its
+    // image, 0 without one); one(dx, k) stores column k of the pair at the
+    // pair's place + dx.
+    auto image = [&](bool own, int x) { return !own ? 0 : (x < kGhost ? nx : (x >= nx - kGhost ? -nx : 0)); };
+    const int off0 = image(ok, xs), off1 = image(two, xs + 1);
+    const bool edge = __any_sync(0xffffffffu, off0 != 0 || off1 != 0 || ok != two);
+    auto images = [&](auto&& one) {
+        if (ok != two) one(0, 0);
+        if (off0) one(off0, 0);
+        if (off1) one(off1 + 1, 1);
+    };
 
     // one iteration; K = i mod 2
     auto iter = [&](int i, auto k_c) {
@@ -1555,12 +1540,17 @@ __device__ __forceinline__ void strip_walk(const StepParams& a, const PairCoef& 
             }
             if constexpr (S == S_F32) {
                 Pop2<!GEN>(m, c).all(c, fs);
-                if (ok) {
-                    float* d = static_cast<float*>(a.dst);
+                float* d = static_cast<float*>(a.dst) + so;
+                if (two) {
+#pragma unroll
+                    for (int p = 0; p < 8; ++p) *reinterpret_cast<pair_t*>(d + p * a.plane) = fs[p];
+                }
+                if (edge) {
 #pragma unroll
                     for (int p = 0; p < 8; ++p) {
-                        *reinterpret_cast<pair_t*>(d + so) = fs[p];   // (an odd lattice's last pair ends in the pad)
-                        d += a.plane;
+                        float lo, hi;
+                        unpk(fs[p], lo, hi);
+                        images([&](int dx, int k) { d[p * a.plane + dx] = k ? hi : lo; });
                     }
                 }
             } else {
@@ -1571,17 +1561,18 @@ __device__ __forceinline__ void strip_walk(const StepParams& a, const PairCoef& 
                 w.m12 = fma2(splat(-c.qtheta), m.m10, m.m12);
                 w.m21 = fma2(splat(-c.qtheta), m.m01, m.m21);
                 Pop2<!GEN>(w, c).all(c, fs);
-                __half* d = static_cast<__half*>(a.dst);
+                __half* d = static_cast<__half*>(a.dst) + so;
+                __half2 hs[8];
                 pair_t r[8];
 #pragma unroll
                 for (int p = 0; p < 8; ++p) {
                     float lo, hi;
                     unpk(fs[p], lo, hi);
                     const __half2 h = __floats2half2_rn(lo, hi);
-                    if (ok) *reinterpret_cast<__half2*>(d + so) = h;
+                    if (two) *reinterpret_cast<__half2*>(d + p * a.plane) = h;
+                    hs[p] = h;
                     const float2 b = __half22float2(h);
                     r[p] = pk(b.x, b.y);
-                    d += a.plane;
                 }
                 const pair_t r46 = sub2(r[4], r[6]), r57 = sub2(r[5], r[7]);
                 const pair_t e10 = add2(sub2(r[0], r[2]), sub2(r46, r57));
@@ -1589,7 +1580,14 @@ __device__ __forceinline__ void strip_walk(const StepParams& a, const PairCoef& 
                 float4 v;
                 unpk(sub2(m.m10, e10), v.x, v.z);
                 unpk(sub2(m.m01, e01), v.y, v.w);
-                if (ok) *reinterpret_cast<float4*>(reinterpret_cast<float2*>(a.cdst) + so) = v;
+                float2* cd = reinterpret_cast<float2*>(a.cdst) + so;
+                if (two) *reinterpret_cast<float4*>(cd) = v;
+                if (edge) {
+#pragma unroll
+                    for (int p = 0; p < 8; ++p)
+                        images([&](int dx, int k) { d[p * a.plane + dx] = k ? __high2half(hs[p]) : __low2half(hs[p]); });
+                    images([&](int dx, int k) { cd[dx] = k ? make_float2(v.z, v.w) : make_float2(v.x, v.y); });
+                }
             }
             so += pitch;
         }
@@ -1615,6 +1613,7 @@ k_strip(const StepParams a, const PairCoef c, int seg, int nstrips, int items) {
     extern __shared__ float4 st_mem[];
     const int warp = threadIdx.x >> 5;
     const int item = (int)blockIdx.x * st_nw<T>() + warp;
+    after_predecessor();
     ResAcc<S> acc;
     if (item < items) {
         const int strip = item % nstrips, y0 = (item / nstrips) * seg;
@@ -1622,6 +1621,172 @@ k_strip(const StepParams a, const PairCoef c, int seg, int nstrips, int items) {
         strip_walk<S, GEN, T, CHECK>(a, c, sm, strip, y0, min(seg, a.ny - y0), acc);
     }
     if (CHECK) residual_reduce<S>(a, acc);
+}
+
+// ---------------------------------------------------------------------------
+// Several steps per launch of a small lattice (FP32 storage): a block holds
+// one tile in registers.
+//
+// A launch of a small lattice is bound by latency, not by traffic or
+// arithmetic: the strips of k_strip are too few to fill the GPU and each
+// walks its rows one after the other.  Here a block of NW warps owns a tile of
+// 64 slot columns by NW * RR slot rows, warp w rows w * RR .. w * RR + RR - 1
+// with two columns per lane, and keeps every population in registers for all
+// T steps of the launch (T is a run-time count).  A slot's state is held as
+// the pulls of its neighbours will want it: after the collision the horizontal
+// movers are shifted by shuffle, so that a row's next populations are its own
+// (1, 3), those with c_y = +1 (2, 5, 6) of the row below it in memory order and
+// those with c_y = -1 (4, 7, 8) of the row after it -- registers of the same
+// lane, except at the edge of a warp's rows, where six values per column pass
+// through shared memory (double-buffered: one block barrier per step).
+// Tiles overlap by T - 1 slots per side.
+//
+// Any lattice size works: slots wrap periodically, and a lattice smaller than
+// a tile appears in it more than once.
+//
+// Measured (GB300, launches back to back, against what ran before at these
+// sizes): 100 x 75 0.59 us per step (three-step tiles 2.07), 333 x 517 1.13
+// (wavefront 4.0).  A launch of T steps takes 2.8 us (start, loads, stores) and
+// 0.24 us per step (8 warps of two rows) to 0.67 us (12 warps of four): FMA-pipe
+// and latency bound, 2 to 3 warps per scheduler.
+template <int RR, bool GEN, bool CHECK>
+__global__ void __launch_bounds__(512, 1)
+k_tile(const StepParams a, const PairCoef ca, int T, int ntx) {
+    extern __shared__ float4 tile_mem[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int nx = a.nx, ny = a.ny, H = T - 1;
+    const int ox = kStSlots - 2 * H, oy = nw * RR - 2 * H;
+    const int tx = blockIdx.x % ntx, ty = blockIdx.x / ntx;
+    // the lane's pair in the rows the warps exchange: [parity][warp + 1][up, down][3]
+    const uint32_t sm = (uint32_t)__cvta_generic_to_shared(tile_mem) + lane * 8;
+    const uint32_t par_bytes = (uint32_t)(nw + 2) * 6 * 256;
+    PairCoef c = ca;
+    c.half = opaque(ca.half, sm + warp * 256);
+    c.nhalf = opaque(ca.nhalf, sm + warp * 256);
+    c.nfour = opaque(ca.nfour, sm + warp * 256);
+    __syncthreads();
+    after_predecessor();
+    const int xs = tx * ox - H + 2 * lane, ys = ty * oy - H + warp * RR;   // the first slot's node
+    auto wrapped = [](int v, int n) {
+        v %= n;
+        return v < 0 ? v + n : v;
+    };
+    const int xa = wrapped(xs - 1, nx), xb = wrapped(xs, nx), xc = wrapped(xs + 1, nx), xd = wrapped(xs + 2, nx);
+    const float* src = static_cast<const float*>(a.src);
+    const int64_t pl = a.plane;
+    struct Row {
+        pair_t m1, m3, u2, u5, nu6, d4, d7, nd8;
+    } s[RR];
+    pair_t gx[RR], gy[RR];
+    auto ld2 = [&](const float* p, int x0, int x1) { return pk(ldg(p + x0), ldg(p + x1)); };
+#pragma unroll
+    for (int r = 0; r < RR; ++r) {
+        const int64_t row = (int64_t)wrapped(ys + r, ny) * a.pitch;
+        const float* p = src + row;
+        s[r].m1 = ld2(p, xa, xb);
+        s[r].u2 = ld2(p + pl, xb, xc);
+        s[r].m3 = ld2(p + 2 * pl, xc, xd);
+        s[r].d4 = ld2(p + 3 * pl, xb, xc);
+        s[r].u5 = ld2(p + 4 * pl, xa, xb);
+        s[r].nu6 = ld2(p + 5 * pl, xc, xd);
+        s[r].d7 = ld2(p + 6 * pl, xc, xd);
+        s[r].nd8 = ld2(p + 7 * pl, xa, xb);
+        gx[r] = ld2(static_cast<const float*>(a.gx) + row, xb, xc);
+        gy[r] = ld2(static_cast<const float*>(a.gy) + row, xb, xc);
+    }
+#pragma unroll
+    for (int r = 0; r < RR; ++r) {
+        s[r].nu6 = neg2(s[r].nu6);
+        s[r].nd8 = neg2(s[r].nd8);
+    }
+    auto put = [&](uint32_t e, pair_t x, pair_t y, pair_t z) {
+        sts_pair(e, x);
+        sts_pair(e + 256, y);
+        sts_pair(e + 512, z);
+    };
+    auto slot = [&](int w) { return sm + (uint32_t)(w + 1) * (6 * 256); };
+    put(slot(warp), s[RR - 1].u2, s[RR - 1].u5, s[RR - 1].nu6);
+    put(slot(warp) + 768, s[0].d4, s[0].d7, s[0].nd8);
+    if (warp == 0) {               // the row before the tile, whose upward movers step 1 pulls
+        const float* p = src + (int64_t)wrapped(ys - 1, ny) * a.pitch;
+        put(slot(-1), ld2(p + pl, xb, xc), ld2(p + 4 * pl, xa, xb), neg2(ld2(p + 5 * pl, xc, xd)));
+    }
+    if (warp == nw - 1) {          // the row after it
+        const float* p = src + (int64_t)wrapped(ys + RR, ny) * a.pitch;
+        put(slot(nw) + 768, ld2(p + 3 * pl, xb, xc), ld2(p + 6 * pl, xc, xd), neg2(ld2(p + 7 * pl, xa, xb)));
+    }
+    __syncthreads();
+    const int s0 = 2 * lane;
+    const bool ok0 = s0 >= H && s0 < kStSlots - H && xs < nx, ok1 = s0 + 1 >= H && s0 + 1 < kStSlots - H && xs + 1 < nx;
+    ResAcc<S_F32> acc;
+    for (int t = 0; t < T; ++t) {
+        const bool last = t == T - 1;
+        const uint32_t par = (t & 1) ? par_bytes : 0;
+        const uint32_t above = slot(warp - 1) + par, below = slot(warp + 1) + par + 768;
+        pair_t u2 = lds_pair(above), u5 = lds_pair(above + 256), nu6 = lds_pair(above + 512);
+#pragma unroll
+        for (int r = 0; r < RR; ++r) {
+            pair_t d4, d7, nd8;
+            if (r + 1 < RR) {
+                d4 = s[r + 1 < RR ? r + 1 : r].d4;
+                d7 = s[r + 1 < RR ? r + 1 : r].d7;
+                nd8 = s[r + 1 < RR ? r + 1 : r].nd8;
+            } else {
+                d4 = lds_pair(below);
+                d7 = lds_pair(below + 256);
+                nd8 = lds_pair(below + 512);
+            }
+            const Opp2 o = opposites2(s[r].m1, u2, s[r].m3, d4, u5, nu6, d7, nd8);
+            const Post2 m = collide2<GEN>(moments2(o, c), gx[r], gy[r], c);
+            const Pop2<!GEN> w(m, c);
+            if (last) {
+                const int y = ys + r, q = warp * RR + r;
+                if (q >= H && q < nw * RR - H && y < ny) {
+                    pair_t fs[8];
+                    w.all(c, fs);
+                    const int64_t idx = (int64_t)y * a.pitch + xs;
+                    float* d = static_cast<float*>(a.dst) + idx;
+#pragma unroll
+                    for (int p = 0; p < 8; ++p) {
+                        float lo, hi;
+                        unpk(fs[p], lo, hi);
+                        if (ok0) d[p * pl] = lo;
+                        if (ok1) d[p * pl + 1] = hi;
+                    }
+                    if (CHECK) {
+                        const pair_t f[8] = {s[r].m1, u2, s[r].m3, d4, u5, neg2(nu6), d7, neg2(nd8)};
+                        float fl[8], fh[8], gxl, gxh, gyl, gyh;
+#pragma unroll
+                        for (int p = 0; p < 8; ++p) unpk(f[p], fl[p], fh[p]);
+                        unpk(gx[r], gxl, gxh);
+                        unpk(gy[r], gyl, gyh);
+                        if (ok0)
+                            check_node<S_F32>(a, pl, idx, acc, snap_load<S_F32>(a, pl, idx), fl, gxl, gyl, 0.0f, 0.0f);
+                        if (ok1)
+                            check_node<S_F32>(a, pl, idx + 1, acc, snap_load<S_F32>(a, pl, idx + 1), fh, gxh, gyh,
+                                              0.0f, 0.0f);
+                    }
+                }
+            }
+            u2 = s[r].u2;
+            u5 = s[r].u5;
+            nu6 = s[r].nu6;
+            s[r].u2 = w.f2(c);
+            s[r].d4 = w.f4(c);
+            s[r].m1 = from_left(w.f1(c));
+            s[r].m3 = from_right(w.f3(c));
+            s[r].u5 = from_left(w.f5());
+            s[r].nu6 = from_right(w.nf6());
+            s[r].d7 = from_right(w.f7());
+            s[r].nd8 = from_left(w.nf8());
+        }
+        if (last) break;
+        const uint32_t next = slot(warp) + (par_bytes - par);
+        put(next, s[RR - 1].u2, s[RR - 1].u5, s[RR - 1].nu6);
+        put(next + 768, s[0].d4, s[0].d7, s[0].nd8);
+        __syncthreads();
+    }
+    if (CHECK) residual_reduce<S_F32>(a, acc);
 }
 
 // Destinations of the five solution fields u_x, u_y, sigma_xx, sigma_yy,
@@ -1770,9 +1935,20 @@ __global__ void k_force_ingest(const double* gx, const double* gy, G* ox, G* oy,
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
         const double u = gx[i], v = gy[i];
-        const int64_t o = i + (i / nx) * (pitch - nx);   // rows of nx values, pitch apart
+        const int64_t y = i / nx, o = i + y * (pitch - nx);   // rows of nx values, pitch apart
         ox[o] = G(u);
         oy[o] = G(v);
+        if (pitch > nx) {                                      // periodic images (row_ghost)
+            const int x = (int)(i - y * nx);
+            if (x < kGhost) {
+                ox[o + nx] = G(u);
+                oy[o + nx] = G(v);
+            }
+            if (x >= nx - kGhost) {
+                ox[o - nx] = G(u);
+                oy[o - nx] = G(v);
+            }
+        }
         if (!(isfinite(u) && isfinite(v))) b = 1;
         m = fmax(m, fmax(fabs(u), fabs(v)));
     }
@@ -1784,6 +1960,28 @@ __global__ void k_force_ingest(const double* gx, const double* gy, G* ox, G* oy,
     if ((threadIdx.x & 31) == 0) {
         atomicMax(absmax, (unsigned long long)__double_as_longlong(m));
         if (b) atomicOr(bad, 1u);
+    }
+}
+
+// The ghost columns of the state in a.dst (row_ghost), after a kernel that
+// writes only the lattice's own columns: one thread per row, ghost column and
+// plane (and, FP16S, carrier).
+template <int S>
+__global__ void k_fill_ghosts(const StepParams a) {
+    using P = typename StoreT<S>::P;
+    after_predecessor();
+    const int64_t per = (int64_t)a.ny * 2 * kGhost, total = per * (S == S_F16S ? 9 : 8);
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+        const int p = (int)(i / per), g = (int)(i % (2 * kGhost));
+        const int64_t row = (i % per) / (2 * kGhost) * a.pitch;
+        const int64_t to = row + (g < kGhost ? g - kGhost : a.nx + g - kGhost), from = to + (g < kGhost ? a.nx : -a.nx);
+        if (S == S_F16S && p == 8) {
+            float2* c = reinterpret_cast<float2*>(a.cdst);
+            c[to] = c[from];
+        } else {
+            P* d = static_cast<P*>(a.dst) + p * a.plane;
+            d[to] = d[from];
+        }
     }
 }
 
@@ -1858,13 +2056,13 @@ inline int adapt_period(int period, double r, double r_prev) {
     return (r > 0.95 * r_prev && period < 64) ? (period * 2 > 64 ? 64 : period * 2) : period;
 }
 
-// Elements between rows of a lattice the library lays out itself: rows start
-// on 16-byte boundaries (FP32: four columns, FP16: eight), which the strip
-// kernel's copies need.  Very narrow lattices stay unpadded.
-inline int row_pitch(int dtype, int nx) {
-    const int m = dtype == S_F64 || nx < 32 ? 1 : (dtype == S_F16S ? 8 : 4);
-    return (nx + m - 1) / m * m;
-}
+// Rows of a lattice the library lays out itself.  FP32 and FP16S rows from 64
+// columns on (what the strip kernel runs on) hold kGhost ghost columns at
+// either end, the periodic images of the columns at the other one, and start
+// on 16-byte boundaries; column 0 is kGhost elements into the row.
+constexpr int kRowSlack = 128;    // elements a buffer holds beyond its planes: a strip reads past a row's end
+inline int row_ghost(int dtype, int nx) { return dtype != S_F64 && nx >= 64 && nx < (1 << 30) ? kGhost : 0; }
+inline int row_pitch(int dtype, int nx) { return row_ghost(dtype, nx) ? (nx + 2 * kGhost + 7) / 8 * 8 : nx; }
 
 inline int64_t step_tiles(int nx, int ny, int V) {
     return (int64_t)((nx + 32 * V - 1) / (32 * V)) * ((ny + BY - 1) / BY);
@@ -1936,7 +2134,7 @@ inline StripShape strip_shape(int dtype, int T, int nx, int ny, int nsm, int war
             }
             cost += one;
         }
-        cost += 4000.0;                            // the launch itself
+        cost += 3000.0;                            // the launch itself
         if (best.seg == 0 || cost < best.cost) {
             best.T = T;
             best.seg = (int)seg;
@@ -1957,6 +2155,47 @@ inline StripShape strip_shape(int dtype, int T, int nx, int ny, int nsm, int war
     if (best.seg == 0) consider(256);
     return best;
 }
+
+// A tile launch: T steps, blocks of NW warps of RR rows.
+struct TileShape {
+    int T = 0, RR = 0, NW = 0;
+    double cost = 0.0;            // modelled cycles of one launch
+};
+inline int64_t tile_count(const TileShape& t, int nx, int ny) {
+    const int ox = kStSlots - 2 * (t.T - 1), oy = t.NW * t.RR - 2 * (t.T - 1);
+    return (int64_t)((nx + ox - 1) / ox) * ((ny + oy - 1) / oy);
+}
+inline int tile_smem(int NW) { return 2 * (NW + 2) * 6 * 256; }
+
+// The tile launch with the fewest modelled cycles per step.  Fitted to
+// launches back to back on GB300 (2 .. 12 steps, 4 .. 16 warps, one block per
+// multiprocessor): a step costs a warp about 50 + 97 w cycles per row with w
+// warps on its scheduler; start, loads and stores together 3500 cycles and 145
+// per slot row of a multiprocessor.  16 warps are resident.
+inline TileShape tile_shape(int nx, int ny, int nsm) {
+    TileShape best;
+    for (int T = 2; T <= 12; ++T)
+        for (int RR = 2; RR <= 4; RR += 2)
+            for (int NW = 2; NW <= 16; ++NW) {
+                TileShape t;
+                t.T = T;
+                t.RR = RR;
+                t.NW = NW;
+                if (NW * RR - 2 * (T - 1) < 1) continue;
+                const int64_t blocks = tile_count(t, nx, ny), slots = (int64_t)nsm * (16 / NW);
+                const int64_t waves = (blocks + slots - 1) / slots;
+                const int64_t here = ((blocks < slots ? blocks : slots) + nsm - 1) / nsm * NW;   // warps
+                const double w = (double)((here + 3) / 4);
+                t.cost = 3500.0 + (double)waves * (145.0 * RR * here + T * RR * (50.0 + 97.0 * w));
+                if (best.T == 0 || t.cost * best.T < best.cost * t.T) best = t;
+            }
+    return best;
+}
+
+// T fused steps of FP32 storage on register tiles (k_tile); check: the last
+// step is the residual-check step (one partial set per block).
+cudaError_t tile_f32(const StepParams& a, const Coef<float>& c, bool gen, const TileShape& t, bool check,
+                     cudaStream_t st);
 
 // T fused steps on the wavefront schedule (k_strip; FP32: T = 2 .. 7, FP16S:
 // T = 3, 4; check: T = 4 with the residual on the last step), segments of seg

@@ -104,8 +104,8 @@ static cudaError_t launch_strip_k(const StepParams& a, const Coef<float>& c, int
     }
     const int64_t ns = strip_count(S, T, a.nx), items = ns * ((a.ny + seg - 1) / seg);
     if (items > 0x7fffffffLL - 64) return cudaErrorInvalidValue;
-    kernel<<<(unsigned)((items + NW - 1) / NW), 32 * NW, SM, st>>>(a, pair_coef(c), seg, (int)ns, (int)items);
-    return cudaGetLastError();
+    return launch_after(kernel, dim3((unsigned)((items + NW - 1) / NW)), dim3(32 * NW), SM, st, a, pair_coef(c), seg,
+                        (int)ns, (int)items);
 }
 
 template <int S, int T, bool CHECK>

@@ -63,3 +63,27 @@ def test_f16s_equals_tiles(nx, ny, kw):
     for rows in (5, -1):
         ref = _state(nx, ny, "f16s", 3, 0, 6, **kw)
         assert np.array_equal(_state(nx, ny, "f16s", 3, rows, 6, **kw), ref)
+
+
+# Register tiles (k_tile; the default of small FP32 lattices): lattices smaller
+# than a tile, ragged last tiles, odd and unpadded widths, every step count of
+# a window with its checked last launch.
+@pytest.mark.parametrize("nx,ny", [(1, 1), (2, 3), (5, 1), (1, 40), (31, 7), (33, 64), (64, 64), (100, 75), (257, 30),
+                                   (333, 100)])
+@pytest.mark.parametrize("kw", [dict(), dict(tau12=0.9, tau22=0.3)])
+def test_default_plan_equals_single_steps(nx, ny, kw):
+    lam, mu = W.lame_2d(1.0, 0.3)
+    rng = np.random.RandomState(nx * 1000 + ny)
+    gx, gy = rng.standard_normal((2, ny, nx)) / max(nx, ny) ** 2
+    for steps, check in ((1, 0), (2, 0), (3, 0), (13, 0), (29, 1), (40, 7), (41, 20)):
+        res = []
+        for plain in (True, False):
+            with Lattice(nx, ny, lam, mu, "f32", **kw) as lat:
+                if plain:
+                    lat.steps_per_launch, lat.wavefront = 1, 0
+                lat.set_force(gx, gy)
+                r = lat.iterate_checked(steps, check) if check else lat.iterate(steps)
+                res.append((lat.populations(), r))
+        assert np.array_equal(res[0][0], res[1][0]), (steps, check)
+        if check:   # sums of pairs in another order: about 2^-44 relative
+            assert np.allclose(res[0][1], res[1][1], rtol=1e-12, atol=0.0), (steps, check)
