@@ -46,12 +46,13 @@ FALLBACK_HBM_GBS = 6800.0
 WAVE_MIN_NX = 256
 BYTES_PER_LAUNCH_NODE = {"f64": 8 * 8 * 2 + 2 * 8, "f32": 8 * 4 * 2 + 2 * 4, "f16s": (8 * 2 + 2 * 4) * 2 + 2 * 4}
 FORCE_SEED = 0x2208_14870
-# FP64 storage runs its collision on the FP64 pipe: 42 FP64 instructions per
-# lattice update (ncu: 28 DADD, 5 DMUL, 9 DFMA per node), i.e. 51 flops.
+# FP64 storage runs its collision on the FP64 pipe: 34 FP64 instructions per
+# lattice update (collide_f64: 15 additions, 3 products, 16 fused
+# multiply-adds per node), i.e. 50 flops.
 # Every FP64 instruction takes one slot of the pipe, whose nominal rate on
 # GB300 is 1.25 TFLOP/s counting an FMA as 2 flops, i.e. 625 G instructions/s.
-FP64_INSTR_PER_LUP = 42
-FP64_FLOPS_PER_LUP = 51
+FP64_INSTR_PER_LUP = 34
+FP64_FLOPS_PER_LUP = 50
 FP64_PEAK_GINST = 625.0
 # DRAM traffic per stream-collide launch from one ncu capture, keyed by dtype,
 # steps per launch and schedule, with the hash of the kernel code it was taken

@@ -158,8 +158,9 @@ int lbm_get_host_transfer(lbm_ctx *ctx, int *mode);
  * launch), which gives the same states; the default is 4 (wavefront schedule) from
  * nx >= 256 and ny >= 8 on, else 3 from nx >= 64 and ny >= 16 on (a smaller
  * lattice fills the on-chip tile more than once and is faster one step per
- * launch).  LBM_F64 storage always runs one step per
- * launch.  Paper: the scheme advances one step at a time; grouping steps into
+ * launch).  LBM_F64 storage takes k = 1
+ * only (the library itself groups up to three steps of a small LBM_F64 lattice
+ * into a launch, with the same states).  Paper: the scheme advances one step at a time; grouping steps into
  * launches is a schedule of the same steps, not part of the method.
  * Errors: LBM_ERR_ARG (k outside 1..4, or k > 1 with LBM_F64 storage). */
 int lbm_set_steps_per_launch(lbm_ctx *ctx, int k);

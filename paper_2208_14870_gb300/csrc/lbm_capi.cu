@@ -92,6 +92,7 @@ struct lbm_ctx {
                                    // caller sets a schedule (lbm_set_steps_per_launch, lbm_set_wavefront)
     int plan = 0;                  // 0: not chosen yet, 1: strips, 2: register tiles (tile)
     TileShape tile;
+    Tile64Shape tile64;            // FP64
 };
 
 namespace {
@@ -127,8 +128,10 @@ StepParams params(const lbm_ctx* c, int src) {
 }
 
 template <typename T>
-Coef<T> coef(const lbm_rates& r) {
+Coef<T> coef(lbm_rates r) {
     Coef<T> c;
+    // (a multiple of 2^-53, see collide_f64; no change to a theta rounded to FP32)
+    if (sizeof(T) == 8 && r.theta >= kThetaExact) r.theta = theta_f64(r.theta);
     // quarter form (exact scaling by 1/4 before the rounding to T)
     c.q11 = T(0.25 * (1.0 - r.w11));
     c.qs = T(0.25 * (1.0 - r.ws));
@@ -143,6 +146,10 @@ Coef<T> coef(const lbm_rates& r) {
     c.b11 = T(1.0 - 0.5 * r.w11);
     c.bs = T(1.0 - 0.5 * r.ws);
     c.bd = T(1.0 - 0.5 * r.wd);
+    c.qsd = T(0.25 * (1.0 - r.ws) + 0.25 * (1.0 - r.wd));
+    c.qds = T(0.25 * (1.0 - r.ws) - 0.25 * (1.0 - r.wd));
+    c.qs2 = T(0.5 * (1.0 - r.ws));
+    c.twoctheta = T(2.0 * (1.0 - r.theta));
     return c;
 }
 
@@ -154,11 +161,25 @@ cudaError_t finish_residual_launch(lbm_ctx* c, int64_t grid) {
 
 int ensure_partials(lbm_ctx* c, int64_t sets);
 
+// T steps of FP64 storage (check: the last one is the residual-check step).
+cudaError_t launch_tile64(lbm_ctx* c, int T, bool check) {
+    Tile64Shape t = c->tile64;
+    t.T = T;
+    cudaError_t e = tile_f64(params(c, c->cur), coef<double>(c->rates), c->gen, t, check, c->nblocks, c->stream);
+    if (e == cudaSuccess && check) e = finish_residual_launch(c, std::min(tile64_count(t, c->nx, c->ny), c->nblocks));
+    if (e == cudaSuccess) {
+        c->cur ^= 1;
+        c->step += T;
+        c->staged_fields = false;
+    }
+    return e;
+}
+
 cudaError_t launch_step(lbm_ctx* c, bool check) {
     const StepParams a = params(c, c->cur);
     cudaError_t e;
     switch (c->dtype) {
-        case LBM_F64: e = Ops<S_F64>::step(a, coef<double>(c->rates), c->V, c->gen, check, (int)c->nblocks, c->stream); break;
+        case LBM_F64: return launch_tile64(c, 1, check);
         case LBM_F32: e = Ops<S_F32>::step(a, coef<float>(c->rates), c->V, c->gen, check, (int)c->nblocks, c->stream); break;
         default: e = Ops<S_F16S>::step(a, coef<float>(c->rates), c->V, c->gen, check, (int)c->nblocks, c->stream); break;
     }
@@ -321,6 +342,18 @@ cudaError_t launch_tile(lbm_ctx* c, int T, bool check) {
     return e;
 }
 
+// n steps of FP64 storage in tile launches; check: the last step is the
+// residual-check step.
+cudaError_t run_tiles64(lbm_ctx* c, int64_t n, bool check) {
+    cudaError_t e = cudaSuccess;
+    while (n > 0 && e == cudaSuccess) {
+        const int t = (int)std::min<int64_t>(n, c->tile64.T);
+        n -= t;
+        e = launch_tile64(c, t, check && n == 0);
+    }
+    return e;
+}
+
 // n steps in as few tile launches as the tile allows, of equal lengths; check:
 // the last step is the residual-check step.
 cudaError_t run_tiles(lbm_ctx* c, int64_t n, bool check) {
@@ -363,6 +396,7 @@ cudaError_t launch_multi(lbm_ctx* c, int T) {
 cudaError_t run_plain(lbm_ctx* c, int64_t n) {
     cudaError_t e = cudaSuccess;
     const bool wave = wave_on(c);
+    if (c->dtype == LBM_F64) return run_tiles64(c, n, false);
     if (auto_on(c)) {
         e = choose_plan(c);
         if (e != cudaSuccess) return e;
@@ -396,6 +430,7 @@ cudaError_t run_plain(lbm_ctx* c, int64_t n) {
 // costs twice a plain one, a two-step launch with the check 1.3 times).
 cudaError_t run_window(lbm_ctx* c, int64_t to_check) {
     cudaError_t e;
+    if (c->dtype == LBM_F64) return run_tiles64(c, to_check, true);
     if (auto_on(c)) {
         e = choose_plan(c);
         if (e != cudaSuccess) return e;
@@ -669,13 +704,16 @@ int lbm_create_ex(int nx, int ny, double lambda, double mu, int dtype, const lbm
     c->rates.w22 = 1.0 / (tau22 + 0.5);
     c->rates.theta = theta;
     c->gen = !(c->rates.w12 == 1.0 && c->rates.w22 == 1.0);
-    if (dtype == LBM_F64) c->V = nx >= 64 ? 2 : 1;
-    else {
+    if (dtype == LBM_F64 && theta < kThetaExact) c->gen = true;   // collide_f64 needs 1 - theta exact
+    if (dtype == LBM_F64) {
+        c->V = 1;
+        c->tile64 = tile64_shape(nx, ny, c->nsm > 0 ? c->nsm : 1);
+    } else {
         const int vmax = dtype == LBM_F16S ? max_vec<S_F16S>() : max_vec<S_F32>();
         c->V = nx >= 32 * vmax ? vmax : 1;
     }
     // residual-check grids: one block per tile up to kMaxCheckBlocks
-    c->nblocks = std::min(step_tiles(nx, ny, c->V), kMaxCheckBlocks);
+    c->nblocks = std::min(dtype == LBM_F64 ? tile64_count(c->tile64, nx, ny) : step_tiles(nx, ny, c->V), kMaxCheckBlocks);
     if (dtype != LBM_F64) {
         c->nblocks2 = std::min(step2_tiles(nx, ny), kMaxCheckBlocks);
         // four steps per launch on the wavefront schedule where it fits, else
@@ -725,6 +763,7 @@ int lbm_create_ex(int nx, int ny, double lambda, double mu, int dtype, const lbm
     if (e == cudaSuccess && dtype == LBM_F16S) e = cudaMemset(c->car[1], 0, cb);
     if (e == cudaSuccess) e = cudaMemset(c->force, 0, fb);
     if (e == cudaSuccess) e = cudaMemset(c->snap, 0, snap_bytes);
+    if (e == cudaSuccess) e = cudaMemset(c->result, 0, sizeof(double) * kRes);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
         int code = cuda_fail(e, "lbm_create: device allocation");

@@ -519,12 +519,19 @@ __device__ __forceinline__ void step_tile(const StepParams& a,
         const int x = xb + 32 * j;
         if (x < nx) {
             const int64_t idx = r0 + x;
-            const Mom<T> m = moments(f[j]);
-            scatter_local<S, GEN>(a, idx, m, gx[j], gy[j], c);
-            if (CHECK) {
-                T u, v;
-                displacement(m, gx[j], gy[j], u, v);
-                check_node<S>(a, n, idx, acc, so[j], f[j], gx[j], gy[j], u, v);
+            if constexpr (S == S_F64 && !GEN) {
+                T u, v, fs[8];
+                collide_f64(f[j], gx[j], gy[j], c, u, v, fs);
+                store_state<S>(a, idx, fs, 0.0f, 0.0f);
+                if (CHECK) check_node<S>(a, n, idx, acc, so[j], f[j], gx[j], gy[j], u, v);
+            } else {
+                const Mom<T> m = moments(f[j]);
+                scatter_local<S, GEN>(a, idx, m, gx[j], gy[j], c);
+                if (CHECK) {
+                    T u, v;
+                    displacement(m, gx[j], gy[j], u, v);
+                    check_node<S>(a, n, idx, acc, so[j], f[j], gx[j], gy[j], u, v);
+                }
             }
         }
     }
@@ -541,6 +548,95 @@ k_step(const StepParams a, const Coef<typename StoreT<S>::T> c) {
         step_tile<S, V, GEN, CHECK>(a, c, tx, ty, acc);
     }
     if (CHECK) residual_reduce<S>(a, acc);
+}
+
+// Periodic image in [0, n) of a slot coordinate v >= -1.  ANY = false
+// needs n at least the slot span (one conditional subtraction); ANY = true
+// serves any n (a lattice smaller than the slot array appears in it more
+// than once).  The two are separate kernels because the general form costs
+// the large-lattice kernel 4-6 % even where it never takes the long path.
+template <bool ANY>
+__device__ __forceinline__ int wrap_slot(int v, int n) {
+    if (v < 0) v += n;
+    if (ANY && v < 0) v = v % n + n;   // v >= -2 on a lattice of one node
+    if (v >= n) v = (!ANY || v < 2 * n) ? v - n : v % n;
+    return v;
+}
+
+// ---------------------------------------------------------------------------
+// T pseudo-time steps per launch of FP64 storage (T >= 1, a run-time count).
+//
+// FP64 storage is bound by the FP64 pipe (a warp instruction takes 64 cycles of
+// one of an SM's four schedulers, whatever its active lanes), so a small lattice has to be spread
+// over all SMs, in whole warps: a block owns bx x by nodes, holds the states
+// between its steps in shared memory over a halo that shrinks by one node per
+// step, and its threads take the slots of a step in linear order.  Several
+// steps per launch recompute the halos but save launches; tile64_shape weighs
+// the two.  Large lattices take T = 1 (no halo).  Measured: 1500 x 1100 116 us per
+// step (tiles of 64 x 8 with two nodes per thread 121 with the same arithmetic,
+// 137 before it), 0.77 of the FP64 pipe's measured rate in 34 instructions per
+// update; 64 x 64 2.05 us (8.3).
+template <bool GEN, bool CHECK>
+__global__ void __launch_bounds__(128)
+k_tile64(const StepParams a, const Coef<double> c, int T, int bx, int by, int ntx, int64_t ntiles) {
+    extern __shared__ double tile64_mem[];
+    const int nx = a.nx, ny = a.ny, H = T - 1, sw = bx + 2 * H, sh = by + 2 * H, area = sw * sh;
+    const int64_t pl = a.plane;
+    const double* gxp = static_cast<const double*>(a.gx);
+    const double* gyp = static_cast<const double*>(a.gy);
+    double* dst = static_cast<double*>(a.dst);
+    ResAcc<S_F64> acc;
+    after_predecessor();
+    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const int ty = (int)(tile / ntx), tx = (int)(tile - (int64_t)ty * ntx);
+        const int x0 = tx * bx - H, y0 = ty * by - H;         // node of slot (0, 0)
+        for (int t = 0; t < T; ++t) {
+            const bool last = t == T - 1;
+            const int aw = sw - 2 * t, count = aw * (sh - 2 * t);
+            const double* from = tile64_mem + (t & 1) * 8 * area;
+            double* to = tile64_mem + ((t + 1) & 1) * 8 * area;
+            for (int i = threadIdx.x; i < count; i += blockDim.x) {
+                const int q = i / aw, sx = t + i - q * aw, sy = t + q;
+                int x = x0 + sx, y = y0 + sy;
+                if (last && (x >= nx || y >= ny)) continue;
+                if (!last) {
+                    x = wrap_slot<true>(x, nx);
+                    y = wrap_slot<true>(y, ny);
+                }
+                const int64_t row = (int64_t)y * a.pitch, idx = row + x;
+                double f[8];
+                if (t == 0) {
+                    gather<S_F64>(a, row, (int64_t)wrap_dec(y, ny) * a.pitch, (int64_t)wrap_inc(y, ny) * a.pitch, x,
+                                  wrap_dec(x, nx), wrap_inc(x, nx), f, c.theta);
+                } else {
+                    const double* p = from + sy * sw + sx;
+                    f[0] = p[0 * area - 1];                   // f_p(x) = f*_p(x - c_p)
+                    f[1] = p[1 * area - sw];
+                    f[2] = p[2 * area + 1];
+                    f[3] = p[3 * area + sw];
+                    f[4] = p[4 * area - sw - 1];
+                    f[5] = p[5 * area - sw + 1];
+                    f[6] = p[6 * area + sw + 1];
+                    f[7] = p[7 * area + sw - 1];
+                }
+                const double gx = ldg(gxp + idx), gy = ldg(gyp + idx);
+                double u, v, fs[8];
+                if (GEN) collide_populations<true>(moments(f), gx, gy, c, u, v, fs);
+                else collide_f64(f, gx, gy, c, u, v, fs);
+                if (last) {
+                    if (CHECK) check_node<S_F64>(a, pl, idx, acc, snap_load<S_F64>(a, pl, idx), f, gx, gy, u, v);
+#pragma unroll
+                    for (int p = 0; p < 8; ++p) dst[p * pl + idx] = fs[p];
+                } else {
+                    double* o = to + sy * sw + sx;
+#pragma unroll
+                    for (int p = 0; p < 8; ++p) o[p * area] = fs[p];
+                }
+            }
+            if (T > 1) __syncthreads();
+        }
+    }
+    if (CHECK) residual_reduce<S_F64>(a, acc);
 }
 
 // ---------------------------------------------------------------------------
@@ -593,19 +689,6 @@ constexpr int kT2OX = kT2W - 2, kT2OY = kT2H - 2;
 constexpr int kT2Threads = 256;
 constexpr int kT2Smem = 8 * kT2H * kT2W * (int)sizeof(float);
 static_assert(kT2Threads == kThreads, "residual_reduce sizes its scratch by kThreads");
-
-// Periodic image in [0, n) of a slot coordinate v >= -1.  ANY = false
-// needs n at least the slot span (one conditional subtraction); ANY = true
-// serves any n (a lattice smaller than the slot array appears in it more
-// than once).  The two are separate kernels because the general form costs
-// the large-lattice kernel 4-6 % even where it never takes the long path.
-template <bool ANY>
-__device__ __forceinline__ int wrap_slot(int v, int n) {
-    if (v < 0) v += n;
-    if (ANY && v < 0) v = v % n + n;   // v >= -2 on a lattice of one node
-    if (v >= n) v = (!ANY || v < 2 * n) ? v - n : v % n;
-    return v;
-}
 
 template <int S, bool GEN, bool CHECK, bool ANY>
 __device__ __forceinline__ void step2_tile(const StepParams& a, const Coef<float>& c, float* sm,
@@ -2155,6 +2238,48 @@ inline StripShape strip_shape(int dtype, int T, int nx, int ny, int nsm, int war
     if (best.seg == 0) consider(256);
     return best;
 }
+
+// A tile launch of FP64 storage (k_tile64): T steps, blocks of bx x by nodes.
+struct Tile64Shape {
+    int T = 0, bx = 0, by = 0;
+    double cost = 0.0;            // modelled cycles of one launch
+};
+inline int64_t tile64_count(const Tile64Shape& t, int nx, int ny) {
+    return (int64_t)((nx + t.bx - 1) / t.bx) * ((ny + t.by - 1) / t.by);
+}
+inline int tile64_smem(const Tile64Shape& t) {
+    return t.T > 1 ? 2 * 8 * 8 * (t.bx + 2 * (t.T - 1)) * (t.by + 2 * (t.T - 1)) : 0;
+}
+
+// The FP64 tile launch with the fewest modelled cycles per step.  Fitted on
+// GB300 (8 x 8 to 1500 x 1100 lattices, T = 1 .. 5): each of an SM's four
+// schedulers issues one FP64 warp instruction in 64 cycles, so a step takes
+// about 1100 + 2250 ceil(W / 4) cycles with W warps of slots on an SM, and a
+// launch 2800 besides.  64 x 64: T = 3 on 8 x 4 nodes, 2.05 us per step (T = 1
+// 2.94, the 64 x 8 tiles before 8.3); 256 x 256: T = 1 on 32 x 2, 6.8 (9.8).
+inline Tile64Shape tile64_shape(int nx, int ny, int nsm) {
+    const int tiles[4][2] = {{8, 4}, {16, 4}, {32, 2}, {32, 4}};
+    Tile64Shape best;
+    for (int T = 1; T <= 3; ++T)
+        for (const auto& b : tiles) {
+            Tile64Shape t;
+            t.T = T;
+            t.bx = b[0];
+            t.by = b[1];
+            const int64_t here = (tile64_count(t, nx, ny) + nsm - 1) / nsm;   // tiles per SM
+            t.cost = 2800.0;
+            for (int s = 0; s < T; ++s) {
+                const int slots = (t.bx + 2 * (T - 1 - s)) * (t.by + 2 * (T - 1 - s));
+                const int64_t warps = here * ((slots + 31) / 32);
+                t.cost += 1100.0 + 2250.0 * (double)((warps + 3) / 4);
+            }
+            if (best.T == 0 || t.cost * best.T < 0.999 * best.cost * t.T) best = t;
+        }
+    return best;
+}
+
+cudaError_t tile_f64(const StepParams& a, const Coef<double>& c, bool gen, const Tile64Shape& t, bool check,
+                     int64_t max_blocks, cudaStream_t st);
 
 // A tile launch: T steps, blocks of NW warps of RR rows.
 struct TileShape {

@@ -87,3 +87,27 @@ def test_default_plan_equals_single_steps(nx, ny, kw):
         assert np.array_equal(res[0][0], res[1][0]), (steps, check)
         if check:   # sums of pairs in another order: about 2^-44 relative
             assert np.allclose(res[0][1], res[1][1], rtol=1e-12, atol=0.0), (steps, check)
+
+
+# FP64 tiles (k_tile64): several steps per launch against one step per launch
+# (an iterate call of one step is one), on lattices smaller than a tile, ragged
+# ones and large ones.
+@pytest.mark.parametrize("nx,ny", [(1, 1), (3, 2), (7, 5), (33, 1), (64, 64), (100, 75), (130, 257)])
+@pytest.mark.parametrize("kw", [dict(), dict(tau12=0.9, tau22=0.3), dict(theta=0.1)])
+def test_f64_tiles_equal_single_steps(nx, ny, kw):
+    lam, mu = W.lame_2d(1.0, 0.3)
+    rng = np.random.RandomState(nx * 1000 + ny)
+    gx, gy = rng.standard_normal((2, ny, nx)) / max(nx, ny) ** 2
+    with Lattice(nx, ny, lam, mu, "f64", **kw) as a, Lattice(nx, ny, lam, mu, "f64", **kw) as b:
+        a.set_force(gx, gy)
+        b.set_force(gx, gy)
+        for _ in range(11):
+            a.iterate(1)
+        b.iterate(11)
+        assert np.array_equal(a.populations(), b.populations())
+        for _ in range(10):
+            a.iterate_checked(1, 10)
+        ra = a.iterate_checked(9, 10)
+        rb = b.iterate_checked(19, 10)
+        assert np.array_equal(a.populations(), b.populations())
+        assert np.allclose(ra, rb, rtol=1e-13, atol=0.0)
