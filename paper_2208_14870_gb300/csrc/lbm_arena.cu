@@ -1,52 +1,68 @@
-// lbm_arena.cu -- the persistent chunk kernel of the packed lattice arena
-// (see lbm_arena.cuh), one instantiation per storage type (FP32, FP16-shifted)
-// and tile width.
+// lbm_arena.cu -- the kernels of the packed lattice arena (see lbm_arena.cuh):
+// strip items, and the persistent chunk kernels, one instantiation per storage
+// type (FP32, FP16-shifted) and tile width.
 #include "lbm_arena.cuh"
 
 namespace lbm {
 
 namespace cg = cooperative_groups;
 
-template <int S, int V, bool CHECK>
-__device__ __forceinline__ void arena_tile(const BatchArgs& A, const BatchProb& P, int tile,
-                                           int s, ResAcc<S>& acc) {
+constexpr int kArenaNW = 4;   // warps per block of the strip items
+
+// The step parameters and rates of problem P, whose state lies in buffer src.
+template <int S>
+__device__ __forceinline__ StepParams prob_params(const BatchArgs& A, const BatchProb& P, int src) {
     StepParams a{};
-    const int64_t n = (int64_t)P.nx * P.ny;
     a.nx = P.nx;
     a.ny = P.ny;
-    a.pitch = P.nx;
-    a.plane = n;
-    const int src = (P.parity + s) & 1;
-    char* ps = src ? A.pop1 : A.pop0;
-    char* pd = src ? A.pop0 : A.pop1;
-    a.src = ps + P.pop_off;
-    a.dst = pd + P.pop_off;
+    a.pitch = P.pitch;
+    a.plane = P.plane;
+    a.src = (src ? A.pop1 : A.pop0) + P.pop_off;
+    a.dst = (src ? A.pop0 : A.pop1) + P.pop_off;
     if (S == S_F16S) {
-        char* cs = src ? A.car1 : A.car0;
-        char* cd = src ? A.car0 : A.car1;
-        a.csrc = reinterpret_cast<const float*>(cs + P.car_off);
-        a.cdst = reinterpret_cast<float*>(cd + P.car_off);
+        a.csrc = reinterpret_cast<const float*>((src ? A.car1 : A.car0) + P.car_off);
+        a.cdst = reinterpret_cast<float*>((src ? A.car0 : A.car1) + P.car_off);
         a.hscale = P.hscale;
         a.hinv = P.hinv;
     }
-    float* fsb = reinterpret_cast<float*>(A.fs + P.fs_off);
-    a.gx = fsb;
-    a.gy = fsb + n;
-    a.snap = fsb + 2 * n;
+    const float* force = reinterpret_cast<const float*>(A.fs + P.fs_off);
+    a.gx = force;
+    a.gy = force + P.plane;
+    a.snap = A.fs + P.snap_off;
+    return a;
+}
+
+__device__ __forceinline__ Coef<float> prob_coef(const BatchProb& P) {
     Coef<float> c{};
     c.q11 = P.q11;
     c.qs = P.qs;
     c.qd = P.qd;
     c.qtheta = P.qtheta;
     c.theta = P.theta;
+    return c;
+}
+
+template <int S, int V, bool CHECK>
+__device__ __forceinline__ void arena_tile(const BatchArgs& A, const BatchProb& P, int tile,
+                                           int s, ResAcc<S>& acc) {
     const int ntx = (P.nx + 32 * V - 1) / (32 * V);
     const int ty = tile / ntx, tx = tile - ty * ntx;
-    step_tile<S, V, false, CHECK>(a, c, tx, ty, acc);
+    step_tile<S, V, false, CHECK>(prob_params<S>(A, P, (P.parity + s) & 1), prob_coef(P), tx, ty, acc);
+}
+
+// A problem's residual partials (maxima through the bit patterns of
+// non-negative doubles).
+__device__ __forceinline__ void add_to_problem(double* dst, const double w[kRes]) {
+    unsigned long long* d = reinterpret_cast<unsigned long long*>(dst);
+    atomicMax(d + 0, (unsigned long long)__double_as_longlong(w[0]));
+    atomicMax(d + 1, (unsigned long long)__double_as_longlong(w[1]));
+    atomicAdd(dst + 2, w[2]);
+    atomicAdd(dst + 3, w[3]);
+    atomicMax(d + 4, (unsigned long long)__double_as_longlong(w[4]));
 }
 
 // Block reduction of one tile's residual partials (converted to FP64 per
-// thread) into the problem's FP64 accumulator (maxima through the bit
-// patterns of non-negative doubles).
+// thread) into the problem's FP64 accumulator.
 template <int S>
 __device__ __forceinline__ void tile_to_problem(const ResAcc<S>& acc, double* dst,
                                                 double (&red)[kRes][kThreads / 32]) {
@@ -58,20 +74,15 @@ __device__ __forceinline__ void tile_to_problem(const ResAcc<S>& acc, double* ds
         for (int k = 0; k < kRes; ++k) red[k][warp] = v[k];
     __syncthreads();
     if (tid == 0) {
-        double m0 = 0.0, m1 = 0.0, s2 = 0.0, s3 = 0.0, b = 0.0;
+        double m[kRes] = {0.0, 0.0, 0.0, 0.0, 0.0};
         for (int w = 0; w < kThreads / 32; ++w) {
-            m0 = fmax(m0, red[0][w]);
-            m1 = fmax(m1, red[1][w]);
-            s2 += red[2][w];
-            s3 += red[3][w];
-            b = fmax(b, red[4][w]);
+            m[0] = fmax(m[0], red[0][w]);
+            m[1] = fmax(m[1], red[1][w]);
+            m[2] += red[2][w];
+            m[3] += red[3][w];
+            m[4] = fmax(m[4], red[4][w]);
         }
-        unsigned long long* d = reinterpret_cast<unsigned long long*>(dst);
-        atomicMax(d + 0, (unsigned long long)__double_as_longlong(m0));
-        atomicMax(d + 1, (unsigned long long)__double_as_longlong(m1));
-        atomicAdd(dst + 2, s2);
-        atomicAdd(dst + 3, s3);
-        atomicMax(d + 4, (unsigned long long)__double_as_longlong(b));
+        add_to_problem(dst, m);
     }
     __syncthreads();
 }
@@ -103,34 +114,9 @@ __global__ void __launch_bounds__(kThreads, 2) k_arena_chunk(const BatchArgs A) 
 template <int S, bool CHECK>
 __device__ __forceinline__ void arena_tile2(const BatchArgs& A, const BatchProb& P, int tile, int s,
                                             float* sm, ResAcc<S>& acc) {
-    StepParams a{};
-    const int64_t n = (int64_t)P.nx * P.ny;
-    a.nx = P.nx;
-    a.ny = P.ny;
-    a.pitch = P.nx;
-    a.plane = n;
-    const int src = (P.parity + s) & 1;
-    a.src = (src ? A.pop1 : A.pop0) + P.pop_off;
-    a.dst = (src ? A.pop0 : A.pop1) + P.pop_off;
-    if (S == S_F16S) {
-        a.csrc = reinterpret_cast<const float*>((src ? A.car1 : A.car0) + P.car_off);
-        a.cdst = reinterpret_cast<float*>((src ? A.car0 : A.car1) + P.car_off);
-        a.hscale = P.hscale;
-        a.hinv = P.hinv;
-    }
-    float* fsb = reinterpret_cast<float*>(A.fs + P.fs_off);
-    a.gx = fsb;
-    a.gy = fsb + n;
-    a.snap = fsb + 2 * n;
-    Coef<float> c{};
-    c.q11 = P.q11;
-    c.qs = P.qs;
-    c.qd = P.qd;
-    c.qtheta = P.qtheta;
-    c.theta = P.theta;
     const int ntx = (P.nx + kT2OX - 1) / kT2OX;
     const int ty = tile / ntx, tx = tile - ty * ntx;
-    step2_tile<S, false, CHECK, true>(a, c, sm, tx, ty, acc);
+    step2_tile<S, false, CHECK, true>(prob_params<S>(A, P, (P.parity + s) & 1), prob_coef(P), sm, tx, ty, acc);
 }
 
 // The chunk with two steps per tile visit and one grid barrier per pair of
@@ -162,117 +148,112 @@ __global__ void __launch_bounds__(kT2Threads, 2) k_arena_chunk2(const BatchArgs 
     }
 }
 
-// One wavefront item of a wide problem: strip and P.seg-row segment `item`,
-// the four steps of pass q (the buffers swap once per pass).
+// T steps of the listed strip items, one warp each: item (problem, i) is strip
+// i mod strips, segment i / strips of P.seg rows.
+template <int S, int T, bool CHECK>
+__global__ void __launch_bounds__(32 * kArenaNW, 3)
+k_arena_strips(const BatchArgs A, const uint2* items, int count, int group) {
+    extern __shared__ float4 strip_mem[];
+    const int warp = threadIdx.x >> 5, item = (int)blockIdx.x * kArenaNW + warp;
+    if (item >= count) return;
+    after_predecessor();
+    const uint2 tl = items[item];
+    const BatchProb P = A.probs[tl.x];
+    const StepParams a = prob_params<S>(A, P, (P.parity + group) & 1);
+    const PairCoef c = pair_coef(prob_coef(P));
+    const int ns = (P.nx + kArenaOX - 1) / kArenaOX;
+    const int strip = (int)tl.y % ns, y0 = (int)tl.y / ns * P.seg, rows = min(P.seg, P.ny - y0);
+    const uint32_t sm = (uint32_t)__cvta_generic_to_shared(strip_mem) + warp * st_warp_smem<S, T>();
+    ResAcc<S> acc;
+    if (CHECK && P.check) {
+        strip_walk<S, false, T, true, kArenaOX>(a, c, sm, strip, y0, rows, acc);
+        double w[kRes];
+        res_to_double<S>(acc, w);
+        warp_reduce_res(w);
+        if ((threadIdx.x & 31) == 0) add_to_problem(A.acc + (int64_t)tl.x * kRes, w);
+    } else {
+        strip_walk<S, false, T, false, kArenaOX>(a, c, sm, strip, y0, rows, acc);
+    }
+}
+
+// Two steps of the listed two-step tiles, one block each.
 template <int S, bool CHECK>
-__device__ __forceinline__ void arena_wave_item(const BatchArgs& A, const BatchProb& P, int item, int q,
-                                                float* sm, ResAcc<S>& acc) {
-    StepParams a{};
-    const int64_t n = (int64_t)P.nx * P.ny;
-    a.nx = P.nx;
-    a.ny = P.ny;
-    a.pitch = P.nx;
-    a.plane = n;
-    const int src = (P.parity + q) & 1;
-    a.src = (src ? A.pop1 : A.pop0) + P.pop_off;
-    a.dst = (src ? A.pop0 : A.pop1) + P.pop_off;
-    if (S == S_F16S) {
-        a.csrc = reinterpret_cast<const float*>((src ? A.car1 : A.car0) + P.car_off);
-        a.cdst = reinterpret_cast<float*>((src ? A.car0 : A.car1) + P.car_off);
-        a.hscale = P.hscale;
-        a.hinv = P.hinv;
-    }
-    float* fsb = reinterpret_cast<float*>(A.fs + P.fs_off);
-    a.gx = fsb;
-    a.gy = fsb + n;
-    a.snap = fsb + 2 * n;
-    Coef<float> c{};
-    c.q11 = P.q11;
-    c.qs = P.qs;
-    c.qd = P.qd;
-    c.qtheta = P.qtheta;
-    c.theta = P.theta;
-    const int nstrips = (P.nx + wv_ox<4>() - 1) / wv_ox<4>();
-    const int strip = item % nstrips, y0 = (item / nstrips) * P.seg;
-    wave_block<S, false, 4, CHECK, int>(a, c, sm, strip, y0, min(P.seg, P.ny - y0), acc);
-}
-
-// The chunk of the wavefront schedule: nsteps / 4 passes of four steps.  In
-// phase 0 of a pass every listed item is visited once -- a wavefront item
-// advances its part of a wide problem by four steps, a two-step tile its part
-// of a narrow problem by two -- and in phase 1 the two-step tiles (the list's
-// tail, from *nwide) once more.  Blocks take items in list order from an
-// atomic counter per phase (the heavy wavefront items first), and the grid
-// synchronises between phases.  The residual check rides on the last step of
-// the chunk: level 4 of the wavefront items, the second step of the phase-1
-// tiles of the last pass.
-template <int S>
-__global__ void __launch_bounds__(kWvW, 2) k_arena_wave(const BatchArgs A) {
-    cg::grid_group grid = cg::this_grid();
-    extern __shared__ float wsm[];   // wavefront rings, or the two-step slot array
+__global__ void __launch_bounds__(kT2Threads, 2)
+k_arena_pairs(const BatchArgs A, const uint2* items, int group) {
+    extern __shared__ float t2_smem[];
     __shared__ double red[kRes][kThreads / 32];
-    __shared__ int next;
-    const int ntiles = *A.ntiles, nwide = *A.nwide;
-    const int npass = A.nsteps / 4;
-    for (int q = 0; q < npass; ++q) {
-        const bool last = q == npass - 1;
-        for (int phase = 0; phase < 2; ++phase) {
-            const int begin = phase == 0 ? 0 : nwide;
-            int* ctr = A.counters + 2 * q + phase;
-            for (;;) {
-                if (threadIdx.x == 0) next = begin + atomicAdd(ctr, 1);
-                __syncthreads();
-                const int t = next;
-                __syncthreads();   // `next` is rewritten for the following item
-                if (t >= ntiles) break;
-                const uint2 tl = A.tiles[t];
-                const BatchProb P = A.probs[tl.x];
-                ResAcc<S> acc;
-                if (t < nwide) {
-                    const bool check = last && P.check;   // uniform over the block
-                    if (check) {
-                        arena_wave_item<S, true>(A, P, (int)tl.y, q, wsm, acc);
-                        tile_to_problem<S>(acc, A.acc + (int64_t)tl.x * kRes, red);
-                    } else {
-                        arena_wave_item<S, false>(A, P, (int)tl.y, q, wsm, acc);
-                    }
-                } else {
-                    const bool check = last && phase == 1 && P.check;
-                    if (check) {
-                        arena_tile2<S, true>(A, P, (int)tl.y, 2 * q + phase, wsm, acc);
-                        tile_to_problem<S>(acc, A.acc + (int64_t)tl.x * kRes, red);
-                    } else {
-                        arena_tile2<S, false>(A, P, (int)tl.y, 2 * q + phase, wsm, acc);
-                    }
-                }
-                __syncthreads();   // the shared memory is reused by the next item
-            }
-            if (!(last && phase == 1)) grid.sync();
-        }
+    after_predecessor();
+    const uint2 tl = items[blockIdx.x];
+    const BatchProb P = A.probs[tl.x];
+    ResAcc<S> acc;
+    if (CHECK && P.check) {
+        arena_tile2<S, true>(A, P, (int)tl.y, group, t2_smem, acc);
+        tile_to_problem<S>(acc, A.acc + (int64_t)tl.x * kRes, red);
+    } else {
+        arena_tile2<S, false>(A, P, (int)tl.y, group, t2_smem, acc);
     }
 }
 
+// Ghost columns of the listed problems' current states, one block each.
 template <int S>
-static cudaError_t wave_arena_allow_smem() {
-    return cudaFuncSetAttribute(k_arena_wave<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, wv_smem<S, 4>());
+__global__ void __launch_bounds__(256) k_arena_ghosts(const BatchArgs A, const uint2* items) {
+    after_predecessor();
+    const BatchProb P = A.probs[items[blockIdx.x].x];
+    fill_ghosts<S>(prob_params<S>(A, P, P.parity ^ 1), threadIdx.x, blockDim.x);   // (dst: the current state)
 }
 
-template <int S>
-static cudaError_t launch_wave_chunk(const BatchArgs& a, int grid, cudaStream_t st) {
-    if (a.nsteps % 4) return cudaErrorInvalidValue;
-    cudaError_t e = wave_arena_allow_smem<S>();
+template <int S, int T, bool CHECK>
+static cudaError_t launch_strips_k(const BatchArgs& a, const uint2* items, int count, int group, cudaStream_t st) {
+    constexpr int SM = kArenaNW * st_warp_smem<S, T>();
+    const auto kernel = k_arena_strips<S, T, CHECK>;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SM);
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(kWvW);
-    cfg.dynamicSmemBytes = wv_smem<S, 4>();
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_arena_wave<S>, a);
+    return launch_after(kernel, dim3((unsigned)((count + kArenaNW - 1) / kArenaNW)), dim3(32 * kArenaNW), SM, st, a, items,
+                        count, group);
+}
+
+cudaError_t launch_arena_strips(int dtype, int T, bool check, const BatchArgs& a, const uint2* items, int count,
+                                int group, cudaStream_t st) {
+    if (dtype == S_F16S) {
+        if (T == 4)
+            return check ? launch_strips_k<S_F16S, 4, true>(a, items, count, group, st)
+                         : launch_strips_k<S_F16S, 4, false>(a, items, count, group, st);
+        if (T == 2)
+            return check ? launch_strips_k<S_F16S, 2, true>(a, items, count, group, st)
+                         : launch_strips_k<S_F16S, 2, false>(a, items, count, group, st);
+        return cudaErrorInvalidValue;
+    }
+    if (check) {
+        if (T == 5) return launch_strips_k<S_F32, 5, true>(a, items, count, group, st);
+        return T == 4 ? launch_strips_k<S_F32, 4, true>(a, items, count, group, st) : cudaErrorInvalidValue;
+    }
+    switch (T) {
+        case 2: return launch_strips_k<S_F32, 2, false>(a, items, count, group, st);
+        case 3: return launch_strips_k<S_F32, 3, false>(a, items, count, group, st);
+        case 5: return launch_strips_k<S_F32, 5, false>(a, items, count, group, st);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+template <int S, bool CHECK>
+static cudaError_t launch_pairs_k(const BatchArgs& a, const uint2* items, int count, int group, cudaStream_t st) {
+    const cudaError_t e = cudaFuncSetAttribute(k_arena_pairs<S, CHECK>, cudaFuncAttributeMaxDynamicSharedMemorySize, kT2Smem);
+    if (e != cudaSuccess) return e;
+    return launch_after(k_arena_pairs<S, CHECK>, dim3((unsigned)count), dim3(kT2Threads), kT2Smem, st, a, items, group);
+}
+
+cudaError_t launch_arena_pairs(int dtype, bool check, const BatchArgs& a, const uint2* items, int count, int group,
+                               cudaStream_t st) {
+    if (dtype == S_F16S)
+        return check ? launch_pairs_k<S_F16S, true>(a, items, count, group, st)
+                     : launch_pairs_k<S_F16S, false>(a, items, count, group, st);
+    return check ? launch_pairs_k<S_F32, true>(a, items, count, group, st)
+                 : launch_pairs_k<S_F32, false>(a, items, count, group, st);
+}
+
+cudaError_t launch_arena_ghosts(int dtype, const BatchArgs& a, const uint2* items, int count, cudaStream_t st) {
+    return dtype == S_F16S ? launch_after(k_arena_ghosts<S_F16S>, dim3((unsigned)count), dim3(256), 0, st, a, items)
+                           : launch_after(k_arena_ghosts<S_F32>, dim3((unsigned)count), dim3(256), 0, st, a, items);
 }
 
 template <int S>
@@ -314,8 +295,6 @@ static cudaError_t launch_v(const BatchArgs& a, int grid, cudaStream_t st) {
 }
 
 cudaError_t launch_arena_chunk(int dtype, int V, const BatchArgs& a, int grid, cudaStream_t st) {
-    if (V == kTileWave)
-        return dtype == S_F16S ? launch_wave_chunk<S_F16S>(a, grid, st) : launch_wave_chunk<S_F32>(a, grid, st);
     if (V == kTileTwoStep)
         return dtype == S_F16S ? launch_two_step<S_F16S>(a, grid, st) : launch_two_step<S_F32>(a, grid, st);
     if (dtype == S_F16S) {
@@ -349,16 +328,7 @@ static int occ2() {
     return b;
 }
 
-template <int S>
-static int occw() {
-    if (wave_arena_allow_smem<S>() != cudaSuccess) return 0;
-    int b = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_arena_wave<S>, kWvW, wv_smem<S, 4>());
-    return b;
-}
-
 int arena_occupancy(int dtype, int V) {
-    if (V == kTileWave) return dtype == S_F16S ? occw<S_F16S>() : occw<S_F32>();
     if (V == kTileTwoStep) return dtype == S_F16S ? occ2<S_F16S>() : occ2<S_F32>();
     if (dtype == S_F16S) return V == 1 ? occ<S_F16S, 1>() : V == 2 ? occ<S_F16S, 2>() : occ<S_F16S, 4>();
     return V == 1 ? occ<S_F32, 1>() : V == 2 ? occ<S_F32, 2>() : occ<S_F32, 4>();

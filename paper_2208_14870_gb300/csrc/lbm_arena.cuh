@@ -1,22 +1,26 @@
 // lbm_arena.cuh -- packed lattice arena for many independent periodic
-// problems of uneven sizes and material parameters, advanced together by one
-// persistent cooperative kernel per chunk of k steps.
+// problems of uneven sizes and material parameters, advanced together in
+// chunks of k steps.
 //
 // Every problem p owns, in three device buffers,
 //   pop[0], pop[1] : its 8 population planes (ping-pong; FP32 or FP16),
 //   car[0], car[1] : FP16-shifted only: the two FP32 carriers, one float2 per node,
 //   fs             : force (2 FP32 planes) then residual snapshot (2 planes of
 //                    (hi, lo) FP32 pairs),
-// placed by a first-fit allocator (256-byte aligned).  The work of one step
-// is the list of (problem, tile) pairs of the active problems; the kernel
-// walks that list grid-stride, then synchronises the whole grid before the
-// next step (cooperative launch).  The last step of a chunk carries the
-// residual check for the problems flagged in their descriptor (a problem
-// checks every `check_period` chunks of its own steps); its per-problem
-// partial sums go to per-problem FP64 accumulators with atomics.  The host reads them after the chunk, retires
-// converged problems, admits new ones and rebuilds the tile list between
-// chunks; the chunk itself (accumulator reset, kernel, accumulator read-back)
-// is replayed from a CUDA graph.
+// placed by a first-fit allocator (256-byte aligned).  Rows carry ghost columns
+// (row_ghost) where the strips run; a problem that fits the arena only without
+// them is laid out plainly.
+//
+// The strip chunk (kTileWave) launches one kernel per group of steps over the
+// (problem, strip, segment) items of all running problems, one warp per item;
+// the other tile codes run a chunk in one persistent cooperative kernel that
+// walks the (problem, tile) list grid-stride and synchronises the grid between
+// steps.  The last step of a chunk carries the residual check for the problems
+// flagged in their descriptor (a problem checks every `check_period` chunks of
+// its own steps); its per-problem partial sums go to per-problem FP64
+// accumulators with atomics.  The host reads them after the chunk, retires
+// converged problems, admits new ones and rebuilds the item lists between
+// chunks.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -30,11 +34,13 @@
 namespace lbm {
 
 struct BatchProb {
-    int64_t pop_off;   // bytes into each population buffer
+    int64_t pop_off;   // bytes into each population buffer, of column 0
     int64_t car_off;   // bytes into each carrier buffer (F16S)
-    int64_t fs_off;    // bytes into the force/snapshot buffer
-    int nx, ny, check, dtype, parity;   // check: this chunk's last step checks
-    int seg;                            // wavefront chunk: rows per wavefront item
+    int64_t fs_off;    // bytes into the force/snapshot buffer: force planes
+    int64_t snap_off;  // ... and snapshot planes
+    int64_t plane;     // elements between planes
+    int nx, ny, pitch, check, dtype, parity;   // check: this chunk's last step checks
+    int seg;                            // strip chunk: rows per item
     float q11, qs, qd, qtheta, theta, hscale, hinv;   // rates in the quarter form of collide
 };
 
@@ -42,8 +48,6 @@ struct BatchArgs {
     const BatchProb* probs;
     const uint2* tiles;        // (problem, tile)
     const int* ntiles;         // device scalar: number of valid tiles
-    const int* nwide;          // wavefront chunks: the first *nwide tiles are wavefront items
-    int* counters;             // wavefront chunks: one work counter per phase, zero at launch
     char* pop0;
     char* pop1;
     char* car0;
@@ -108,25 +112,27 @@ private:
 // per tile visit and one grid barrier per pair of steps (chunk length even).
 constexpr int kTileTwoStep = 3;
 
-// Tile code of the wavefront chunk: problems from one strip width up advance
-// four steps per visit of a wavefront item (one strip by `seg` rows);
-// narrower ones take two two-step tiles per four steps (chunk length a
-// multiple of 4).  The segment length is chosen when the work list is built:
-// 256 rows, halved (down to 16) while the list would hold fewer than four
-// waves of resident blocks, so that a few large problems still fill the GPU.
+// Tile code of the strip chunk: every launch advances the listed items by a
+// group of steps (FP32 five; FP16S four for lattices from 256 x 8 on and two for
+// smaller ones, as its states round to FP16 where a launch ends).  Strips have
+// kArenaOX output columns whatever the group, so that one item list serves a
+// chunk; problems without ghost columns take pairs of steps on two-step tiles.
+// Chunk lengths: multiples of 4.
 constexpr int kTileWave = 5;
-constexpr int kArenaWaveSegMax = 256;
+constexpr int kArenaOX = 56;
+inline int64_t arena_strips(int nx) { return (nx + kArenaOX - 1) / kArenaOX; }
 
-// (wavefront items address a problem with 32-bit in-plane offsets)
 inline bool arena_wide(int nx, int ny) { return wave_fits(nx, ny) && (int64_t)nx * ny < (int64_t(1) << 31); }
+// Problems the strips run on: ghost columns (images of distinct columns).
+inline bool arena_padded(int nx) { return nx >= 2 * kGhost; }
+inline int arena_pitch(int nx) { return (nx + 2 * kGhost + 7) / 8 * 8; }
 
-// Relative device work per lattice update of an nx x ny problem in the
-// wavefront chunk: a wide problem pays for the slot columns of its 256-column
-// strips; a narrower one runs two-step tiles, at about half the wavefront's
-// rate on a large lattice (GB300: 159 against 308 GLUPS), and pays for the
-// slots of its tiles.
+// Weight of solving an nx x ny problem as given against its transpose: columns
+// of 256-column strips with 250 outputs for lattices from 256 x 8 on, slots of
+// two-step tiles at about half that rate for smaller ones.  A fixed rule: the
+// choice decides the rounding order of the solution and is reported with it.
 inline double arena_cost(int nx, int ny) {
-    if (arena_wide(nx, ny)) return double((nx + wv_ox<4>() - 1) / wv_ox<4>()) * kWvW / nx;
+    if (arena_wide(nx, ny)) return double((nx + 249) / 250) * 256 / nx;
     return 1.94 * (double((nx + kT2OX - 1) / kT2OX) * kT2W / nx) * (double((ny + kT2OY - 1) / kT2OY) * kT2H / ny);
 }
 
@@ -138,22 +144,28 @@ inline double arena_cost(int nx, int ny) {
 // <-> u_y and sigma_xx <-> sigma_yy; only the rounding order differs.
 inline bool arena_transpose(int nx, int ny) { return arena_cost(ny, nx) < 0.95 * arena_cost(nx, ny); }
 
-// Number of tiles of an nx x ny problem for tile code V (seg: rows per
-// wavefront item of the wavefront chunk).
-inline int64_t arena_tiles(int nx, int ny, int V, int seg = kArenaWaveSegMax) {
-    if (V == kTileWave)
-        return arena_wide(nx, ny) ? (int64_t)((nx + wv_ox<4>() - 1) / wv_ox<4>()) * ((ny + seg - 1) / seg)
-                                  : step2_tiles(nx, ny);
+// Number of tiles of an nx x ny problem for the persistent kernels' tile codes.
+inline int64_t arena_tiles(int nx, int ny, int V) {
     return V == kTileTwoStep ? step2_tiles(nx, ny) : step_tiles(nx, ny, V);
 }
 
-// Launch one chunk: nsteps steps of every listed tile (all of storage type
-// dtype: S_F32 or S_F16S), residual check fused into the last step.  Tile
-// code V: width 32*V for V in {1, 2, 4}, kTileTwoStep or kTileWave.
+// Launch one chunk of a persistent kernel: nsteps steps of every listed tile
+// (all of storage type dtype: S_F32 or S_F16S), residual check fused into the
+// last step.  Tile code V: width 32*V for V in {1, 2, 4}, or kTileTwoStep.
 // Cooperative launch: grid must not exceed arena_occupancy(dtype, V) x SM
 // count.
 cudaError_t launch_arena_chunk(int dtype, int V, const BatchArgs& a, int grid, cudaStream_t st);
 // Resident blocks per SM of the chunk kernel.
 int arena_occupancy(int dtype, int V);
+
+// The strip chunk's launches.  T steps of `count` strip items (check: the last
+// step checks the flagged problems); two steps of `count` two-step tiles; the
+// ghost columns of `count` problems (items: problem numbers).  group: how many
+// groups of steps of its problems ran before in this chunk (buffer parity).
+cudaError_t launch_arena_strips(int dtype, int T, bool check, const BatchArgs& a, const uint2* items, int count,
+                                int group, cudaStream_t st);
+cudaError_t launch_arena_pairs(int dtype, bool check, const BatchArgs& a, const uint2* items, int count, int group,
+                               cudaStream_t st);
+cudaError_t launch_arena_ghosts(int dtype, const BatchArgs& a, const uint2* items, int count, cudaStream_t st);
 
 }  // namespace lbm

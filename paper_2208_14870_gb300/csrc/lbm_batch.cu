@@ -5,6 +5,7 @@
 #include <chrono>
 #include <cstdlib>
 #include <cmath>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -37,7 +38,8 @@ std::string signature(int count, const lbm_problem* probs, int dtype, int k) {
     std::nth_element(sides.begin(), sides.begin() + count / 2, sides.end());
     const int med = sides[count / 2];
     auto lg = [](double v) { return (int)std::floor(std::log2(std::max(v, 1.0))); };
-    return device_name() + "|d" + std::to_string(dtype) + "|k" + std::to_string(k) + "|n" +
+    // ("strips": a choice made before the strip chunk does not hold)
+    return device_name() + "|strips|d" + std::to_string(dtype) + "|k" + std::to_string(k) + "|n" +
            std::to_string(lg(count)) + "|s" + std::to_string(lg(med));
 }
 
@@ -54,12 +56,13 @@ extern "C" int lbm_batch_solve(int count, const lbm_problem* probs, int dtype, d
         return bfail(LBM_ERR_ARG, "lbm_batch_solve: dtype must be LBM_F32 or LBM_F16S");
     if (!(tol >= 0.0) || check_every < 2 || max_iters < 1)
         return bfail(LBM_ERR_ARG, "lbm_batch_solve: need tol >= 0, check_every >= 2, max_iters >= 1");
-    int64_t nodes = 0;
+    int64_t nodes = 0, plain = 0;   // with and without ghost columns
     for (int i = 0; i < count; ++i) {
         const lbm_problem& p = probs[i];
         if (p.nx < 1 || p.ny < 1 || !p.gx || !p.gy || !(p.mu > 0.0) || !(p.lambda + p.mu > 0.0))
             return bfail(LBM_ERR_ARG, "lbm_batch_solve: problem " + std::to_string(i) + " is invalid");
-        nodes += (int64_t)p.nx * p.ny;
+        nodes += ArenaEngine::slots_for(p.nx, p.ny);
+        plain += (int64_t)p.nx * p.ny;
     }
     cudaStream_t st = nullptr;
     if (cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess)
@@ -70,9 +73,17 @@ extern "C" int lbm_batch_solve(int count, const lbm_problem* probs, int dtype, d
     int64_t chunks = 0, lups = 0;
     double dev_ms = 0.0;
     {
-        ArenaEngine eng;
-        rc = eng.init(dtype, nodes, count, check_every, st, &err);
+        auto owned = std::make_unique<ArenaEngine>();
+        rc = owned->init(dtype, nodes, count, check_every, st, &err);
+        if (rc == LBM_ERR_OOM && nodes > plain) {   // no room for ghost columns
+            cudaGetLastError();
+            owned = std::make_unique<ArenaEngine>();
+            owned->set_plain();
+            rc = owned->init(dtype, plain, count, check_every, st, &err);
+        }
+        ArenaEngine& eng = *owned;
         if (rc) {
+            owned.reset();
             cudaStreamDestroy(st);
             return bfail(rc, "lbm_batch_solve: " + err);
         }
@@ -84,9 +95,10 @@ extern "C" int lbm_batch_solve(int count, const lbm_problem* probs, int dtype, d
             else if (s < 0) rc = s;
             slot[i] = s;
         }
-        // Autotuner: the first chunks run with tile widths 32, 64 and 128
-        // and, for an even chunk length, with two-step tiles; the fastest per
-        // active node and chunk is kept and cached.
+        // Autotuner: the first chunks run with the strip chunk and two-step
+        // tiles, or, where the chunk length does not allow strips, with two-step
+        // tiles and tile widths 128, 64 and 32; the fastest per active node and
+        // chunk is kept and cached.
         const std::string key = signature(count, probs, dtype, check_every);
         const bool even = check_every % 2 == 0, four = check_every % 4 == 0;
         int V = rc == LBM_OK ? autotune_lookup(key) : 0;
@@ -96,14 +108,15 @@ extern "C" int lbm_batch_solve(int count, const lbm_problem* probs, int dtype, d
             if (fv == 1 || fv == 2 || fv == 4 || (fv == kTileTwoStep && even) || (fv == kTileWave && four))
                 V = fv;
         }
-        // candidates, the likeliest first (the wavefront chunk when the chunk
-        // length allows it)
+        // candidates, the likeliest first
         int cand[5], ncand = 0;
         if (four) cand[ncand++] = kTileWave;
         if (even) cand[ncand++] = kTileTwoStep;
-        cand[ncand++] = 4;
-        cand[ncand++] = 2;
-        cand[ncand++] = 1;
+        if (!four) {
+            cand[ncand++] = 4;
+            cand[ncand++] = 2;
+            cand[ncand++] = 1;
+        }
         double best = 1e300;
         int tuning = V == 0 ? 0 : ncand;
         while (rc == LBM_OK && eng.running() > 0) {

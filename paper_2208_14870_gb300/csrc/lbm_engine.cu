@@ -1,4 +1,5 @@
 // lbm_engine.cu -- host side of the packed lattice arena (lbm_engine.cuh).
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -49,15 +50,23 @@ ArenaEngine::~ArenaEngine() {
     if (d_acc_) cudaFree(d_acc_);
     if (d_tiles_) cudaFree(d_tiles_);
     if (d_ntiles_) cudaFree(d_ntiles_);
-    if (d_nwide_) cudaFree(d_nwide_);
-    if (d_counters_) cudaFree(d_counters_);
     if (d_fields_) cudaFree(d_fields_);
     if (h_acc_) cudaFreeHost(h_acc_);
     if (h_tiles_) cudaFreeHost(h_tiles_);
     if (h_force_) cudaFreeHost(h_force_);
     if (h_fields_) cudaFreeHost(h_fields_);
+    for (int i = 0; i < kClasses - 1; ++i) {
+        if (side_[i]) cudaStreamDestroy(side_[i]);
+        if (join_[i]) cudaEventDestroy(join_[i]);
+    }
+    if (fork_) cudaEventDestroy(fork_);
     if (ev0_) cudaEventDestroy(ev0_);
     if (ev1_) cudaEventDestroy(ev1_);
+}
+
+int64_t ArenaEngine::slots_for(int nx, int ny) {
+    if (arena_transpose(nx, ny)) std::swap(nx, ny);
+    return arena_padded(nx) ? (int64_t)arena_pitch(nx) * ny : (int64_t)nx * ny;
 }
 
 int64_t ArenaEngine::bytes_for(int64_t n) const {
@@ -78,7 +87,8 @@ int ArenaEngine::init(int dtype, int64_t node_capacity, int max_probs, int check
     int dev = 0;
     ECK(cudaGetDevice(&dev));
     ECK(cudaDeviceGetAttribute(&sms_, cudaDevAttrMultiProcessorCount, dev));
-    const int64_t slack = (int64_t)max_probs * kArenaAlign;
+    // (kRowSlack: a strip of the last problem reads past its last row)
+    const int64_t slack = (int64_t)max_probs * kArenaAlign + kRowSlack * 8;
     const int64_t pb = pop_bytes_per_node(dtype) * node_capacity + slack;
     const int64_t cb = car_bytes_per_node(dtype) * node_capacity + slack;
     const int64_t fb = kFsBytesPerNode * node_capacity + slack;
@@ -101,13 +111,51 @@ int ArenaEngine::init(int dtype, int64_t node_capacity, int max_probs, int check
     ECK(cudaMallocHost(&h_acc_, sizeof(double) * kRes * max_probs));
     ECK(cudaMalloc(&d_ntiles_, sizeof(int)));
     ECK(cudaMemsetAsync(d_ntiles_, 0, sizeof(int), st_));
-    ECK(cudaMalloc(&d_nwide_, sizeof(int)));
-    ECK(cudaMemsetAsync(d_nwide_, 0, sizeof(int), st_));
-    ECK(cudaMalloc(&d_counters_, sizeof(int) * 2 * (k_ / 4 + 1)));
+    for (int i = 0; i < kClasses - 1; ++i) {
+        ECK(cudaStreamCreateWithFlags(&side_[i], cudaStreamNonBlocking));
+        ECK(cudaEventCreateWithFlags(&join_[i], cudaEventDisableTiming));
+    }
+    ECK(cudaEventCreateWithFlags(&fork_, cudaEventDisableTiming));
     ECK(cudaEventCreate(&ev0_));
     ECK(cudaEventCreate(&ev1_));
     dev_bytes_ += sizeof(BatchProb) * max_probs + sizeof(double) * kRes * max_probs;
     return LBM_OK;
+}
+
+// Arena memory for p (its lattice set), with ghost columns where the strips run,
+// or without them if the arena could never hold it with them.
+bool ArenaEngine::place(HostProb& p) {
+    for (int plain = arena_padded(p.nx) && !plain_ ? 0 : 1; plain < 2; ++plain) {
+        p.ghost = plain ? 0 : kGhost;
+        p.pitch = plain ? p.nx : arena_pitch(p.nx);
+        p.plane = (int64_t)p.pitch * p.ny;
+        p.pop_bytes = pop_bytes_per_node(dtype_) * p.plane;
+        p.car_bytes = car_bytes_per_node(dtype_) * p.plane;
+        p.fs_bytes = kFsBytesPerNode * p.plane;
+        if (!plain && (p.pop_bytes > apop_.capacity() || p.car_bytes > acar_.capacity() || p.fs_bytes > afs_.capacity()))
+            continue;
+        p.pop_off = apop_.alloc(p.pop_bytes);
+        if (p.pop_off < 0) return false;
+        p.car_off = dtype_ == S_F16S ? acar_.alloc(p.car_bytes) : 0;
+        if (p.car_off < 0) {
+            apop_.release(p.pop_off, p.pop_bytes);
+            return false;
+        }
+        p.fs_off = afs_.alloc(p.fs_bytes);
+        if (p.fs_off < 0) {
+            apop_.release(p.pop_off, p.pop_bytes);
+            if (dtype_ == S_F16S) acar_.release(p.car_off, p.car_bytes);
+            return false;
+        }
+        return true;
+    }
+    return false;
+}
+
+void ArenaEngine::unplace(const HostProb& p) {
+    apop_.release(p.pop_off, p.pop_bytes);
+    if (dtype_ == S_F16S) acar_.release(p.car_off, p.car_bytes);
+    afs_.release(p.fs_off, p.fs_bytes);
 }
 
 int ArenaEngine::admit(int nx, int ny, double lambda, double mu, const double* gx, const double* gy,
@@ -125,78 +173,67 @@ int ArenaEngine::admit(int nx, int ny, double lambda, double mu, const double* g
         }
     if (slot < 0) return -1;
     const int64_t n = (int64_t)nx * ny;
-    HostProb p;
-    p.pop_bytes = pop_bytes_per_node(dtype_) * n;
-    p.car_bytes = car_bytes_per_node(dtype_) * n;
-    p.fs_bytes = kFsBytesPerNode * n;
-    p.pop_off = apop_.alloc(p.pop_bytes);
-    if (p.pop_off < 0) return -1;
-    if (dtype_ == S_F16S) {
-        p.car_off = acar_.alloc(p.car_bytes);
-        if (p.car_off < 0) {
-            apop_.release(p.pop_off, p.pop_bytes);
-            return -1;
-        }
-    } else {
-        p.car_off = 0;
-    }
-    p.fs_off = afs_.alloc(p.fs_bytes);
-    if (p.fs_off < 0) {
-        apop_.release(p.pop_off, p.pop_bytes);
-        if (dtype_ == S_F16S) acar_.release(p.car_off, p.car_bytes);
-        return -1;
-    }
     // a problem that is cheaper on its transpose is solved there: lattice
     // ny x nx, force components exchanged, node (x, y) at x * ny + y
     const bool tr = arena_transpose(nx, ny);
+    HostProb p;
+    p.nx = tr ? ny : nx;
+    p.ny = tr ? nx : ny;
+    p.tr = tr;
+    p.n = n;
+    if (!place(p)) return -1;
     // force -> FP32 staging (pinned), with the FP16 scale from its maximum
-    if (h_force_cap_ < 2 * n) {
+    const int64_t len = 2 * p.plane;
+    if (h_force_cap_ < len) {
         if (h_force_) {
             ECK(cudaStreamSynchronize(st_));
             cudaFreeHost(h_force_);
             h_force_ = nullptr;
         }
-        ECK(cudaMallocHost(&h_force_, sizeof(float) * 2 * n));
-        h_force_cap_ = 2 * n;
+        ECK(cudaMallocHost(&h_force_, sizeof(float) * len));
+        h_force_cap_ = len;
     }
     ECK(cudaStreamSynchronize(st_));  // the staging may still feed a previous copy
     double gmax = 0.0;
-    for (int64_t i = 0; i < n; ++i) {
-        const double a = gx[i], b = gy[i];
-        if (!std::isfinite(a) || !std::isfinite(b)) {
-            apop_.release(p.pop_off, p.pop_bytes);
-            if (dtype_ == S_F16S) acar_.release(p.car_off, p.car_bytes);
-            afs_.release(p.fs_off, p.fs_bytes);
-            if (err) *err = "admit: non-finite force";
-            return LBM_ERR_ARG;
+    // (row y of the arena lattice: its pitch elements are the periodic images of
+    // its columns, ghost columns and padding included)
+    for (int64_t y = 0; y < p.ny; ++y) {
+        float* rx = h_force_ + y * p.pitch;
+        float* ry = rx + p.plane;
+        for (int c = 0; c < p.nx; ++c) {
+            const int64_t i = tr ? (int64_t)c * nx + y : y * nx + c;
+            const double a = gx[i], b = gy[i];
+            if (!std::isfinite(a) || !std::isfinite(b)) {
+                unplace(p);
+                if (err) *err = "admit: non-finite force";
+                return LBM_ERR_ARG;
+            }
+            gmax = std::fmax(gmax, std::fmax(std::fabs(a), std::fabs(b)));
+            rx[p.ghost + c] = (float)(tr ? b : a);
+            ry[p.ghost + c] = (float)(tr ? a : b);
         }
-        gmax = std::fmax(gmax, std::fmax(std::fabs(a), std::fabs(b)));
-        if (tr) {
-            const int64_t t = (i % nx) * ny + i / nx;
-            h_force_[t] = (float)b;
-            h_force_[n + t] = (float)a;
-        } else {
-            h_force_[i] = (float)a;
-            h_force_[n + i] = (float)b;
+        for (int g = 0; g < p.ghost; ++g) {
+            rx[g] = rx[p.nx + g];
+            ry[g] = ry[p.nx + g];
+        }
+        for (int g = p.ghost + p.nx; g < p.pitch; ++g) {
+            rx[g] = rx[g - p.nx];
+            ry[g] = ry[g - p.nx];
         }
     }
-    if (tr) std::swap(nx, ny);
-    p.hexp = dtype_ == S_F16S ? f16s_exponent(gmax, nx, ny) : 0;
+    p.hexp = dtype_ == S_F16S ? f16s_exponent(gmax, p.nx, p.ny) : 0;
     if (p.hexp != 0) {
         // FP16S keeps its state, the force included, in units scaled by 2^hexp
         // (store_f16s); the power of two is exact
         const float sc = std::ldexp(1.0f, p.hexp);
-        for (int64_t i = 0; i < 2 * n; ++i) h_force_[i] *= sc;
+        for (int64_t i = 0; i < len; ++i) h_force_[i] *= sc;
     }
-    ECK(cudaMemcpyAsync(fs_ + p.fs_off, h_force_, sizeof(float) * 2 * n, cudaMemcpyHostToDevice, st_));
-    ECK(cudaMemsetAsync(fs_ + p.fs_off + sizeof(float) * 2 * n, 0, sizeof(float2) * 2 * n, st_));
+    ECK(cudaMemcpyAsync(fs_ + p.fs_off, h_force_, sizeof(float) * len, cudaMemcpyHostToDevice, st_));
+    ECK(cudaMemsetAsync(fs_ + p.fs_off + sizeof(float) * len, 0, sizeof(float2) * 2 * p.plane, st_));
     ECK(cudaMemsetAsync(pop_[0] + p.pop_off, 0, p.pop_bytes, st_));
     if (dtype_ == S_F16S) ECK(cudaMemsetAsync(car_[0] + p.car_off, 0, p.car_bytes, st_));
     p.parity = 0;
-    p.nx = nx;
-    p.ny = ny;
-    p.tr = tr;
-    p.n = n;
+    p.cls = !p.ghost ? C_PAIRS : (dtype_ == S_F16S && !arena_wide(p.nx, p.ny) ? C_SHORT : C_LONG);
     p.lambda = lambda;
     p.mu = mu;
     // Table 1 / Eq. relaxation_rate with theta = 1/3, w_12 = w_21 = w_22 = 1
@@ -219,11 +256,43 @@ int ArenaEngine::admit(int nx, int ny, double lambda, double mu, const double* g
     return slot;
 }
 
-int64_t ArenaEngine::running_tiles(int V, int seg) const {
+int64_t ArenaEngine::running_tiles(int V) const {
     int64_t t = 0;
     for (const auto& p : probs_)
-        if (p.state == P_RUNNING) t += arena_tiles(p.nx, p.ny, V, seg);
+        if (p.state == P_RUNNING) {
+            if (V != kTileWave) t += arena_tiles(p.nx, p.ny, V);
+            else if (p.cls == C_PAIRS) t += step2_tiles(p.nx, p.ny);
+            else t += arena_strips(p.nx) * ((p.ny + wave_seg_ - 1) / wave_seg_);
+        }
     return t;
+}
+
+// Rows per strip item of the running problems, by strip_shape's model: the
+// segments whose warps take the fewest cycles over all problems (a few large
+// problems get short segments, many get long ones).
+int ArenaEngine::choose_seg() const {
+    const int64_t slots = 12LL * sms_;
+    int best = 16;
+    double cost = 0.0;
+    for (int seg = 8; seg <= 512; seg += seg < 32 ? 4 : (seg < 128 ? 16 : 64)) {
+        int64_t items = 0;
+        int rows = 0;
+        for (const auto& p : probs_)
+            if (p.state == P_RUNNING && p.cls != C_PAIRS) {
+                items += arena_strips(p.nx) * ((p.ny + seg - 1) / seg);
+                rows = std::max(rows, std::min(p.ny, seg));
+            }
+        if (items == 0) break;
+        double c = 0.0;
+        const double full = (double)(rows + 8) * (5 * (70.0 + 115.0 * 3) + 150.0);
+        const int64_t waves = (items - 1) / slots, rest = items - waves * slots;
+        c = waves * full + (double)(rows + 8) * (5 * (70.0 + 115.0 * ((rest + 4 * sms_ - 1) / (4 * sms_))) + 150.0);
+        if (cost == 0.0 || c < cost) {
+            cost = c;
+            best = seg;
+        }
+    }
+    return best;
 }
 
 int64_t ArenaEngine::running_nodes() const {
@@ -236,11 +305,13 @@ int64_t ArenaEngine::running_nodes() const {
 int64_t ArenaEngine::resident_bytes() const {
     int64_t b = 0;
     for (const auto& p : probs_)
-        if (p.state != P_FREE) b += bytes_for(p.n);
+        if (p.state != P_FREE) b += bytes_for(p.plane);
     return b;
 }
 
-int ArenaEngine::grid_blocks(int V) const { return arena_occupancy(dtype_, V) * sms_; }
+int ArenaEngine::grid_blocks(int V) const {
+    return V == kTileWave ? strip_blocks_ : arena_occupancy(dtype_, V) * sms_;
+}
 
 int64_t ArenaEngine::free_nodes_hint() const {
     return apop_.largest_free() / pop_bytes_per_node(dtype_);
@@ -248,14 +319,11 @@ int64_t ArenaEngine::free_nodes_hint() const {
 
 int ArenaEngine::upload_tiles(int V, std::string* err) {
     if (V == kTileWave) {
-        // longest segments that still give four waves of resident blocks
-        const int64_t want = 4LL * grid_blocks(V);
-        int seg = kArenaWaveSegMax;
-        while (seg > 16 && running_tiles(V, seg) < want) seg /= 2;
-        if (seg != wave_seg_) desc_dirty_ = true;
-        wave_seg_ = seg;
+        wave_seg_ = choose_seg();
+        desc_dirty_ = true;
     }
-    const int64_t nt = running_tiles(V, wave_seg_);
+    // (strip chunk: one more item per problem, for the ghost columns)
+    const int64_t nt = running_tiles(V) + (V == kTileWave ? nrunning_ : 0);
     if (nt > (int64_t)INT32_MAX) {
         if (err) *err = "arena: too many tiles";
         return LBM_ERR_ARG;
@@ -282,25 +350,36 @@ int ArenaEngine::upload_tiles(int V, std::string* err) {
             }
     }
     ECK(cudaStreamSynchronize(st_));  // the pinned list may feed a previous copy
-    // wavefront chunks list the wide problems' wavefront items first, then the
-    // narrow problems' two-step tiles
-    int64_t t = 0, nwide = 0;
-    for (int pass = (V == kTileWave ? 0 : 1); pass < 2; ++pass) {
+    int64_t t = 0;
+    if (V == kTileWave) {
+        for (int cls = 0; cls < kClasses; ++cls) {
+            class_begin_[cls] = (int)t;
+            for (int s = 0; s < (int)probs_.size(); ++s) {
+                const HostProb& p = probs_[s];
+                if (p.state != P_RUNNING || p.cls != cls) continue;
+                const int64_t m = cls == C_PAIRS ? step2_tiles(p.nx, p.ny)
+                                                 : arena_strips(p.nx) * ((p.ny + wave_seg_ - 1) / wave_seg_);
+                for (int64_t i = 0; i < m; ++i) h_tiles_[t++] = make_uint2((unsigned)s, (unsigned)i);
+            }
+        }
+        class_begin_[kClasses] = (int)t;
+        ghosts_begin_ = (int)t;
+        for (int s = 0; s < (int)probs_.size(); ++s)
+            if (probs_[s].state == P_RUNNING && probs_[s].ghost && !probs_[s].ghosts_ok)
+                h_tiles_[t++] = make_uint2((unsigned)s, 0u);
+        ghosts_end_ = (int)t;
+    } else {
         for (int s = 0; s < (int)probs_.size(); ++s) {
             const HostProb& p = probs_[s];
             if (p.state != P_RUNNING) continue;
-            if (V == kTileWave && arena_wide(p.nx, p.ny) != (pass == 0)) continue;
-            const int64_t m = arena_tiles(p.nx, p.ny, V, wave_seg_);
+            const int64_t m = arena_tiles(p.nx, p.ny, V);
             for (int64_t i = 0; i < m; ++i) h_tiles_[t++] = make_uint2((unsigned)s, (unsigned)i);
         }
-        if (pass == 0) nwide = t;
     }
-    static thread_local int nt_host[2];
-    nt_host[0] = (int)nt;
-    nt_host[1] = (int)nwide;
-    if (nt > 0) ECK(cudaMemcpyAsync(d_tiles_, h_tiles_, sizeof(uint2) * nt, cudaMemcpyHostToDevice, st_));
-    ECK(cudaMemcpyAsync(d_ntiles_, &nt_host[0], sizeof(int), cudaMemcpyHostToDevice, st_));
-    ECK(cudaMemcpyAsync(d_nwide_, &nt_host[1], sizeof(int), cudaMemcpyHostToDevice, st_));
+    static thread_local int nt_host;
+    nt_host = (int)t;
+    if (t > 0) ECK(cudaMemcpyAsync(d_tiles_, h_tiles_, sizeof(uint2) * t, cudaMemcpyHostToDevice, st_));
+    ECK(cudaMemcpyAsync(d_ntiles_, &nt_host, sizeof(int), cudaMemcpyHostToDevice, st_));
     ECK(cudaStreamSynchronize(st_));
     tiles_V_ = V;
     tiles_dirty_ = false;
@@ -312,8 +391,6 @@ BatchArgs ArenaEngine::chunk_args() const {
     a.probs = d_probs_;
     a.tiles = d_tiles_;
     a.ntiles = d_ntiles_;
-    a.nwide = d_nwide_;
-    a.counters = d_counters_;
     a.pop0 = pop_[0];
     a.pop1 = pop_[1];
     a.car0 = car_[0];
@@ -336,7 +413,6 @@ int ArenaEngine::ensure_graph(int V, std::string* err) {
     cudaError_t e = cudaStreamBeginCapture(st_, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
         cudaMemsetAsync(d_acc_, 0, sizeof(double) * kRes * probs_.size(), st_);
-        if (V == kTileWave) cudaMemsetAsync(d_counters_, 0, sizeof(int) * 2 * (k_ / 4), st_);
         launch_arena_chunk(dtype_, V, a, grid, st_);
         cudaMemcpyAsync(h_acc_, d_acc_, sizeof(double) * kRes * probs_.size(), cudaMemcpyDeviceToHost, st_);
         e = cudaStreamEndCapture(st_, &g);
@@ -348,6 +424,50 @@ int ArenaEngine::ensure_graph(int V, std::string* err) {
         graph_[V] = nullptr;
         graph_failed_[V] = true;
     }
+    return LBM_OK;
+}
+
+// Steps of the launches that advance a class of problems by a chunk of k steps
+// (k a multiple of 4); the last one carries the check.
+static std::vector<int> chunk_groups(int dtype, int cls, int k) {
+    if (cls == C_PAIRS || cls == C_SHORT) return std::vector<int>(k / 2, 2);
+    if (dtype == S_F16S || k < 5) return std::vector<int>(k / 4, 4);
+    // fives after the rest (two threes where it would be one step)
+    std::vector<int> g;
+    const int r = k % 5;
+    if (r == 1) g = {3, 3};
+    else if (r == 4) g = {2, 2};
+    else if (r) g = {r};
+    g.resize(g.size() + (k - (r == 1 ? 6 : r)) / 5, 5);
+    return g;
+}
+
+// One chunk on strips: the classes side by side, each a sequence of launches.
+int ArenaEngine::launch_strip_chunk(std::string* err) {
+    const BatchArgs a = chunk_args();
+    ECK(cudaMemsetAsync(d_acc_, 0, sizeof(double) * kRes * probs_.size(), st_));
+    if (ghosts_end_ > ghosts_begin_)
+        ECK(launch_arena_ghosts(dtype_, a, d_tiles_ + ghosts_begin_, ghosts_end_ - ghosts_begin_, st_));
+    int busy[kClasses], nb = 0;
+    for (int c = 0; c < kClasses; ++c)
+        if (class_begin_[c + 1] > class_begin_[c]) busy[nb++] = c;
+    if (nb > 1) ECK(cudaEventRecord(fork_, st_));
+    for (int b = nb - 1; b >= 0; --b) {          // the first class last, on the engine's own stream
+        const int c = busy[b], count = class_begin_[c + 1] - class_begin_[c];
+        const cudaStream_t st = b == 0 ? st_ : side_[b - 1];
+        if (b > 0) ECK(cudaStreamWaitEvent(st, fork_, 0));
+        const uint2* items = d_tiles_ + class_begin_[c];
+        strip_blocks_ = std::max(strip_blocks_, c == C_PAIRS ? count : (count + 3) / 4);
+        const std::vector<int> groups = chunk_groups(dtype_, c, k_);
+        for (int g = 0; g < (int)groups.size(); ++g) {
+            const bool check = g + 1 == (int)groups.size();
+            if (c == C_PAIRS) ECK(launch_arena_pairs(dtype_, check, a, items, count, g, st));
+            else ECK(launch_arena_strips(dtype_, groups[g], check, a, items, count, g, st));
+        }
+        if (b > 0) ECK(cudaEventRecord(join_[b - 1], st));
+    }
+    for (int b = 1; b < nb; ++b) ECK(cudaStreamWaitEvent(st_, join_[b - 1], 0));
+    ECK(cudaMemcpyAsync(h_acc_, d_acc_, sizeof(double) * kRes * probs_.size(), cudaMemcpyDeviceToHost, st_));
     return LBM_OK;
 }
 
@@ -376,11 +496,15 @@ int ArenaEngine::run_chunk(int V, float* device_ms, std::string* err) {
         for (size_t i = 0; i < probs_.size(); ++i) {
             const HostProb& p = probs_[i];
             BatchProb& b = d[i];
-            b.pop_off = p.pop_off;
-            b.car_off = p.car_off;
-            b.fs_off = p.fs_off;
+            // (of column 0)
+            b.pop_off = p.pop_off + p.ghost * pop_bytes_per_node(dtype_) / 8;
+            b.car_off = p.car_off + p.ghost * car_bytes_per_node(dtype_);
+            b.fs_off = p.fs_off + p.ghost * (int64_t)sizeof(float);
+            b.snap_off = p.fs_off + 2 * p.plane * (int64_t)sizeof(float);
+            b.plane = p.plane;
             b.nx = p.nx;
             b.ny = p.ny;
+            b.pitch = p.pitch;
             b.check = p.check_now ? 1 : 0;
             b.dtype = dtype_;
             b.parity = p.parity;
@@ -397,15 +521,17 @@ int ArenaEngine::run_chunk(int V, float* device_ms, std::string* err) {
         ECK(cudaStreamSynchronize(st_));
         desc_dirty_ = false;
     }
-    int rc = ensure_graph(V, err);
+    int rc = V == kTileWave ? LBM_OK : ensure_graph(V, err);
     if (rc) return rc;
     ECK(cudaEventRecord(ev0_, st_));
-    if (graph_[V]) {
+    if (V == kTileWave) {
+        rc = launch_strip_chunk(err);
+        if (rc) return rc;
+    } else if (graph_[V]) {
         ECK(cudaGraphLaunch(graph_[V], st_));
     } else {
         const BatchArgs a = chunk_args();
         ECK(cudaMemsetAsync(d_acc_, 0, sizeof(double) * kRes * probs_.size(), st_));
-        if (V == kTileWave) ECK(cudaMemsetAsync(d_counters_, 0, sizeof(int) * 2 * (k_ / 4), st_));
         ECK(launch_arena_chunk(dtype_, V, a, grid_blocks(V), st_));
         ECK(cudaMemcpyAsync(h_acc_, d_acc_, sizeof(double) * kRes * probs_.size(), cudaMemcpyDeviceToHost, st_));
     }
@@ -417,10 +543,15 @@ int ArenaEngine::run_chunk(int V, float* device_ms, std::string* err) {
         if (p.state != P_RUNNING) continue;
         p.steps += k_;
         p.lups += p.n * k_;
-        // the buffers swap once per launch-level step: k steps, k/2 pairs, or
-        // (wavefront chunk) k/4 passes of a wide problem, k/2 pairs of a narrow one
-        const int64_t swaps = V == kTileWave ? (arena_wide(p.nx, p.ny) ? k_ / 4 : k_ / 2)
+        // the buffers swap once per group of steps: k steps, k/2 pairs, or (strip
+        // chunk) the groups of the problem's class
+        const int64_t swaps = V == kTileWave ? (int64_t)chunk_groups(dtype_, p.cls, k_).size()
                                              : (V == kTileTwoStep ? k_ / 2 : k_);
+        if (V != kTileWave) p.ghosts_ok = false;
+        else if (!p.ghosts_ok) {
+            p.ghosts_ok = true;
+            tiles_dirty_ = true;      // (the list of stale ghost columns)
+        }
         if (swaps & 1) {
             p.parity ^= 1;
             desc_dirty_ = true;
@@ -468,20 +599,20 @@ cudaError_t ArenaEngine::launch_fields(int slot, double* dst) {
     StepParams a{};
     a.nx = p.nx;
     a.ny = p.ny;
-    a.pitch = p.nx;
-    a.plane = p.n;
-    a.src = pop_[p.parity] + p.pop_off;
-    a.dst = pop_[p.parity ^ 1] + p.pop_off;
+    a.pitch = p.pitch;
+    a.plane = p.plane;
+    const int64_t po = p.pop_off + p.ghost * pop_bytes_per_node(dtype_) / 8;
+    a.src = pop_[p.parity] + po;
+    a.dst = pop_[p.parity ^ 1] + po;
     if (dtype_ == S_F16S) {
-        a.csrc = reinterpret_cast<const float*>(car_[p.parity] + p.car_off);
-        a.cdst = reinterpret_cast<float*>(car_[p.parity ^ 1] + p.car_off);
+        const int64_t co = p.car_off + p.ghost * car_bytes_per_node(dtype_);
+        a.csrc = reinterpret_cast<const float*>(car_[p.parity] + co);
+        a.cdst = reinterpret_cast<float*>(car_[p.parity ^ 1] + co);
         a.hscale = std::ldexp(1.0f, p.hexp);
         a.hinv = std::ldexp(1.0f, -p.hexp);
     }
-    float* fsb = reinterpret_cast<float*>(fs_ + p.fs_off);
-    a.gx = fsb;
-    a.gy = fsb + p.n;
-    a.snap = fsb + 2 * p.n;
+    a.gx = fs_ + p.fs_off + p.ghost * sizeof(float);
+    a.gy = fs_ + p.fs_off + (p.ghost + p.plane) * sizeof(float);
     const double theta = 1.0 / 3.0, K = p.lambda + p.mu;
     const double w11 = 1.0 / (p.mu / theta + 0.5), ws = 1.0 / (2.0 * K / (1.0 + theta) + 0.5),
                  wd = 1.0 / (2.0 * p.mu / (1.0 - theta) + 0.5);
@@ -587,9 +718,7 @@ void ArenaEngine::release(int slot) {
         --nrunning_;
         tiles_dirty_ = true;
     }
-    apop_.release(p.pop_off, p.pop_bytes);
-    if (dtype_ == S_F16S) acar_.release(p.car_off, p.car_bytes);
-    afs_.release(p.fs_off, p.fs_bytes);
+    unplace(p);
     p = HostProb();
 }
 

@@ -15,11 +15,20 @@ namespace lbm {
 
 enum ProbState { P_FREE = 0, P_RUNNING = 1, P_DONE = 2 };
 
+// Strip chunk: strips of the storage type's long groups (FP32 five steps, FP16S
+// four), strips of pairs of steps (FP16S below 256 x 8), two-step tiles
+// (problems without ghost columns).
+enum ProbClass { C_LONG = 0, C_SHORT = 1, C_PAIRS = 2, kClasses = 3 };
+
 struct HostProb {
     int state = P_FREE;
     int nx = 0, ny = 0;            // the arena lattice (the caller's, or its transpose)
     bool tr = false;               // solved transposed (arena_transpose)
     int64_t n = 0;
+    int pitch = 0, ghost = 0;      // row layout (ghost columns at either end, or none)
+    int64_t plane = 0;             // elements between planes
+    int cls = 0;                   // strip chunk: which launches advance it (ProbClass)
+    bool ghosts_ok = true;         // the current state's ghost columns hold its images
     double lambda = 0.0, mu = 0.0;
     int64_t pop_off = -1, car_off = -1, fs_off = -1;
     int64_t pop_bytes = 0, car_bytes = 0, fs_bytes = 0;
@@ -43,13 +52,18 @@ class ArenaEngine {
 public:
     ~ArenaEngine();
     // dtype: S_F32 or S_F16S.  Capacities in nodes (population / carrier /
-    // force+snapshot bytes follow from the storage type).
+    // force+snapshot bytes follow from the storage type); a problem with ghost
+    // columns takes slots_for nodes, one laid out plainly its own.
     int init(int dtype, int64_t node_capacity, int max_probs, int check_every, cudaStream_t st,
              std::string* err);
+    // Lay every problem out without ghost columns (before init).
+    void set_plain() { plain_ = true; }
     int dtype() const { return dtype_; }
     int check_every() const { return k_; }
     // Bytes of device memory a problem of n nodes needs in this arena.
     int64_t bytes_for(int64_t n) const;
+    // Nodes a problem takes with ghost columns (in the orientation it is solved in).
+    static int64_t slots_for(int nx, int ny);
     // Admit a problem; returns slot >= 0, -1 if it does not fit now, or a
     // negative lbm status (< -1) on error.  gx, gy: host FP64, nx*ny each.
     int admit(int nx, int ny, double lambda, double mu, const double* gx, const double* gy,
@@ -67,11 +81,12 @@ public:
     void release(int slot);
     const HostProb& prob(int slot) const { return probs_[slot]; }
     int running() const { return nrunning_; }
-    int64_t running_tiles(int V, int seg = kArenaWaveSegMax) const;
+    int64_t running_tiles(int V) const;
     int64_t running_nodes() const;
     // Arena bytes held by admitted problems (running or finished, not released).
     int64_t resident_bytes() const;
     int max_probs() const { return (int)probs_.size(); }
+    // Blocks of a chunk's launches (strip chunk: of the largest launch so far).
     int grid_blocks(int V) const;
     int64_t free_nodes_hint() const;
     int64_t device_bytes() const { return dev_bytes_; }
@@ -79,12 +94,17 @@ public:
 
 private:
     int upload_tiles(int V, std::string* err);
+    int choose_seg() const;
+    int launch_strip_chunk(std::string* err);
+    bool place(HostProb& p);
+    void unplace(const HostProb& p);
     BatchArgs chunk_args() const;
     cudaError_t launch_fields(int slot, double* dst);
     int ensure_fields_buffer(int64_t len, std::string* err);
     int ensure_graph(int V, std::string* err);
 
     int dtype_ = S_F32;
+    bool plain_ = false;
     int k_ = 100;
     cudaStream_t st_ = nullptr;
     int sms_ = 1;
@@ -99,12 +119,15 @@ private:
     uint2* d_tiles_ = nullptr;
     int64_t tiles_cap_ = 0;
     int* d_ntiles_ = nullptr;
-    int* d_nwide_ = nullptr;          // wavefront chunks: wavefront items at the list's head
-    int* d_counters_ = nullptr;       // wavefront chunks: a work counter per phase (2 per pass)
+    int class_begin_[kClasses + 1] = {0, 0, 0, 0};   // strip chunk: item ranges of the classes
+    int strip_blocks_ = 0;                            // largest launch so far
+    int ghosts_begin_ = 0, ghosts_end_ = 0;           // ... and of the problems whose ghost columns are stale
+    cudaStream_t side_[kClasses - 1] = {nullptr, nullptr};   // the classes run side by side
+    cudaEvent_t fork_ = nullptr, join_[kClasses - 1] = {nullptr, nullptr};
     uint2* h_tiles_ = nullptr;        // pinned
     int64_t h_tiles_cap_ = 0;
     int tiles_V_ = 0;                 // V the device tile list was built for
-    int wave_seg_ = kArenaWaveSegMax; // rows per wavefront item of the current list
+    int wave_seg_ = 0;                // rows per strip item of the current list
     bool tiles_dirty_ = true;
     bool desc_dirty_ = true;
     float* h_force_ = nullptr;        // pinned FP32 staging

@@ -1418,10 +1418,12 @@ __device__ __forceinline__ pair_t opaque(pair_t p, uint32_t a) {
 // beyond either end hold the periodic images, so that a strip's rows are
 // contiguous and its copies aligned wherever it lies; the strips that own the
 // outermost kGhost columns store their images too.
-template <int S, bool GEN, int T, bool CHECK>
+// OX: output columns of a strip (at most st_ox).
+template <int S, bool GEN, int T, bool CHECK, int OX = st_ox<S, T>()>
 __device__ __forceinline__ void strip_walk(const StepParams& a, const PairCoef& ca, uint32_t sm, int strip, int y0,
                                            int rows, ResAcc<S>& acc) {
-    constexpr int LAG = st_lag<S>(), H = st_halo<S, T>(), HL = st_left<S, T>(), OX = st_ox<S, T>(),
+    static_assert(OX % 2 == 0 && OX <= st_ox<S, T>(), "pairs, within the slots");
+    constexpr int LAG = st_lag<S>(), H = st_halo<S, T>(), HL = st_left<S, T>(),
                   LA = st_la<S>(), R = st_ring<S, T>(), ROW = st_row<S>();
     constexpr int OFF = 1 - LAG;                             // copied row of local row i: i + OFF
     constexpr int AHEAD = 2 * OFF + LA;                      // rows copied ahead of iteration i
@@ -2047,14 +2049,13 @@ __global__ void k_force_ingest(const double* gx, const double* gy, G* ox, G* oy,
 }
 
 // The ghost columns of the state in a.dst (row_ghost), after a kernel that
-// writes only the lattice's own columns: one thread per row, ghost column and
-// plane (and, FP16S, carrier).
+// writes only the lattice's own columns: thread `i` of `step` takes rows, ghost
+// columns and planes (and, FP16S, carriers) in turn.
 template <int S>
-__global__ void k_fill_ghosts(const StepParams a) {
+__device__ __forceinline__ void fill_ghosts(const StepParams& a, int64_t i, int64_t step) {
     using P = typename StoreT<S>::P;
-    after_predecessor();
     const int64_t per = (int64_t)a.ny * 2 * kGhost, total = per * (S == S_F16S ? 9 : 8);
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+    for (; i < total; i += step) {
         const int p = (int)(i / per), g = (int)(i % (2 * kGhost));
         const int64_t row = (i % per) / (2 * kGhost) * a.pitch;
         const int64_t to = row + (g < kGhost ? g - kGhost : a.nx + g - kGhost), from = to + (g < kGhost ? a.nx : -a.nx);
@@ -2066,6 +2067,12 @@ __global__ void k_fill_ghosts(const StepParams a) {
             d[to] = d[from];
         }
     }
+}
+
+template <int S>
+__global__ void k_fill_ghosts(const StepParams a) {
+    after_predecessor();
+    fill_ghosts<S>(a, blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
 }
 
 // F16S: multiply every stored deviation by `factor` (a power of two).

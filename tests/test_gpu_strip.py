@@ -16,6 +16,7 @@ pytestmark = pytest.mark.gpu
 if not torch.cuda.is_available():  # pragma: no cover
     pytest.skip("no CUDA device", allow_module_level=True)
 
+import paper_2208_14870_gb300 as P  # noqa: E402
 from paper_2208_14870_gb300 import Lattice  # noqa: E402
 
 # 280 and 364: whole strips of 56 and 52 output columns (five and seven steps)
@@ -111,3 +112,61 @@ def test_f64_tiles_equal_single_steps(nx, ny, kw):
         rb = b.iterate_checked(19, 10)
         assert np.array_equal(a.populations(), b.populations())
         assert np.allclose(ra, rb, rtol=1e-13, atol=0.0)
+
+
+def _problems(sizes):
+    out = []
+    for i, (nx, ny) in enumerate(sizes):
+        gx, gy = np.random.RandomState(i).standard_normal((2, ny, nx)) / max(nx, ny) ** 2
+        out.append((nx, ny, *W.lame_2d(1.0, 0.1 + 0.02 * i), gx, gy))
+    return out
+
+
+def _alone(prob, steps, transposed):
+    """Fields of the problem as a single FP32 lattice, in the arena's orientation."""
+    nx, ny, lam, mu, gx, gy = prob
+    if transposed:
+        nx, ny, gx, gy = ny, nx, gy.T, gx.T
+    with Lattice(nx, ny, lam, mu, "f32") as lat:
+        lat.set_force(gx, gy)
+        lat.iterate(steps)
+        f = lat.fields()
+    return f.transpose(0, 2, 1)[[1, 0, 3, 2, 4]] if transposed else f
+
+
+# Strip items of the arena: widths without ghost columns (below 16), narrower
+# than a strip, whole strips of 56 columns and one more, with every chunk length
+# that leaves another rest of five.
+@pytest.mark.parametrize("k", [4, 8, 12, 16, 100])
+def test_arena_strips_equal_single_lattices(k, monkeypatch):
+    monkeypatch.setenv("LBM_BATCH_TILE_V", str(P.LBM_TILE_WAVE))
+    probs = _problems([(1, 1), (5, 9), (15, 40), (16, 16), (17, 30), (56, 20), (57, 20), (112, 33), (113, 70), (64, 300),
+                       (255, 9), (257, 64), (300, 31)])
+    steps = 2 * k
+    res, rep = P.batch_solve(probs, "f32", 0.0, k, steps)
+    assert rep["tile_v"] == P.LBM_TILE_WAVE
+    for p, r in zip(probs, res):
+        assert r["iters"] == steps
+        assert np.array_equal(r["fields"], _alone(p, steps, r["transposed"])), p[:2]
+
+
+def test_arena_f16s_strips_round_where_tiles_do(monkeypatch):
+    # below 256 x 8 both round the state to FP16 every second step
+    probs = _problems([(1, 1), (15, 40), (16, 16), (57, 20), (112, 33), (113, 70), (64, 300), (255, 9)])
+    res = []
+    for v in (P.LBM_TILE_WAVE, P.LBM_TILE_TWO_STEP):
+        monkeypatch.setenv("LBM_BATCH_TILE_V", str(v))
+        res.append(P.batch_solve(probs, "f16s", 0.0, 8, 24)[0])
+    for a, b in zip(*res):
+        if a["fields"].shape[2] < 256 and a["fields"].shape[1] < 256:
+            assert np.array_equal(a["fields"], b["fields"])
+
+
+def test_arena_problem_that_fits_only_without_ghost_columns():
+    # 32 columns and eight ghost columns per side take half as much again: a
+    # budget between the two
+    prob = _problems([(32, 200)])[0]
+    n = 32 * 200
+    with P.Server(max(1 << 20, 2 * int(n * 88 * 1.2)), check_every=100) as srv:
+        r = srv.wait(srv.submit(*prob, dtype="f32", tol=0.0, max_iters=200))
+    assert np.array_equal(r["fields"], _alone(prob, 200, r["transposed"]))
