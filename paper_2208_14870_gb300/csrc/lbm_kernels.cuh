@@ -968,347 +968,6 @@ k_step3(const StepParams a, const Coef<float> c) {
 }
 
 // ---------------------------------------------------------------------------
-// Wavefront schedule of T pseudo-time steps per launch (FP32 or FP16-shifted
-// storage; T = 3 or 4).
-//
-// A block of 32*NW threads owns a strip of W = 32*NW slot columns (thread t
-// = column t for the whole launch) and a segment of `seg` output rows, and
-// walks down the segment one row per iteration at every step level at once:
-// in iteration i, step tau (1..T) updates the row of local index i - 2(tau - 1)
-// (local row j is lattice row ybeg + j, ybeg = y0 - (T - 1)), so step tau
-// trails step tau - 1 by two rows and only reads rows that step tau - 1
-// finished in earlier iterations.  Step 1 pulls f*(t) from global memory,
-// steps 2..T-1 pull from and write to rings of kWvD = 4 rows per level in
-// shared memory (local row j in ring slot j mod 4), and step T stores
-// f*(t+T) of the strip's W - 2(T-1) inner columns to global memory.  One
-// block barrier per iteration separates a ring slot's last read from its next
-// write.  The halo costs 2(T-1) of W columns and 2(T - tau) extra rows of
-// level tau per segment, and a level's ring holds four rows instead of a
-// whole tile, so four steps per launch fit.
-//
-// The vertical movers c_2 = (0, 1) and c_4 = (0, -1) are pulled from the
-// thread's own column, so they skip the rings: each level boundary keeps them
-// in a per-thread delay line (population 2 of the last three rows produced,
-// population 4 of the last one), and the rings hold the six other
-// populations.  Step 1 pulls into registers one row ahead of its use (FP32
-// with LBM_WV_LA2_F32: two rows) and loads the force two rows ahead (FP16S:
-// one row; its pulls carry the FP32 carriers too).
-//
-// Instruction economy (the kernel issues, it does not wait on HBM): the
-// iterations in which every level is active run in groups of four, so every
-// ring slot is a compile-time offset from one per-thread address and no
-// level tests whether it is active; only the first 3(T-1) and the last few
-// iterations of a segment take the general path.  The force of a thread's
-// column for the last 2(T-1)+1 rows stays in registers (step tau uses the row
-// step 1 loaded 2(tau-1) iterations earlier).  With I = int (lattices below
-// 2^31 nodes) global addresses are a 32-bit in-plane offset on a per-plane
-// base.
-//
-// CHECK: step T is the residual-check step (its input state is u^(t+T-1));
-// its snapshot loads run one iteration ahead, and the block's partials go to
-// StepParams::partials (k_residual_finish combines them).
-//
-// The per-node arithmetic is the single step's: FP32 results equal T
-// single-step launches bit for bit (FP16S keeps the intermediate states in
-// FP32).  Lattices from W x 8 nodes up.
-#ifndef LBM_WV_NW
-#define LBM_WV_NW 8
-#endif
-// step 1: populations loaded two rows ahead (1) or one (0), per storage type
-// (FP16S pulls hold three times the registers; two rows ahead measured 1 %
-// slower)
-#ifndef LBM_WV_LA2_F32
-#define LBM_WV_LA2_F32 1
-#endif
-#ifndef LBM_WV_LA2_F16S
-#define LBM_WV_LA2_F16S 0
-#endif
-constexpr int kWvNW = LBM_WV_NW;                 // warps per block
-constexpr int kWvW = 32 * kWvNW;                 // strip width (slot columns)
-constexpr int kWvRow = kWvW + 2;                 // ring row: the strip plus one pad column per side
-constexpr int kWvD = 4;                          // ring rows per level
-constexpr int kWvRP = 6;                         // populations held in a ring (all but 2 and 4)
-constexpr int kWvSegDefault = 256;               // output rows per block segment (default)
-template <int S>
-__host__ __device__ constexpr bool wv_la2() {
-    return S == S_F16S ? LBM_WV_LA2_F16S != 0 : LBM_WV_LA2_F32 != 0;
-}
-// step 1 collides its row at the start of the iteration (1), so its decoded
-// populations die before the other levels run and its load buffers are free
-// for the next row, or after the other levels (0), so its loads are issued
-// earlier.  Defaults: the faster at 16384^2 on GB300 (FP32 after: 3.34 against
-// 3.77 ms per four-step launch; FP16S first: 3.48 against 3.72 ms)
-#ifndef LBM_WV_L1FIRST_F32
-#define LBM_WV_L1FIRST_F32 0
-#endif
-#ifndef LBM_WV_L1FIRST_F16S
-#define LBM_WV_L1FIRST_F16S 1
-#endif
-// FP32: step 1's load buffers and the delay lines of population 2 as
-// circular buffers of four, indexed by the iteration's phase in its group of
-// four (no register copies: 3.31 against 3.35 ms per four-step launch at
-// 16384^2 on GB300), or (0) two buffers whose pulls are copied before the
-// reload, and delay lines shifted every iteration
-#ifndef LBM_WV_CIRC
-#define LBM_WV_CIRC 1
-#endif
-template <int S>
-__host__ __device__ constexpr bool wv_l1first() {
-    return S == S_F16S ? LBM_WV_L1FIRST_F16S != 0 : LBM_WV_L1FIRST_F32 != 0;
-}
-static_assert(kWvW <= kThreads, "residual_reduce sizes its scratch by kThreads");
-template <int T> __host__ __device__ constexpr int wv_ox() { return kWvW - 2 * (T - 1); }
-template <int S, int T> __host__ __device__ constexpr int wv_smem() {
-    return (T - 1) * kWvRP * kWvD * kWvRow * (int)sizeof(float);
-}
-// resident blocks per SM the kernel is compiled for: what 228 KB of shared
-// memory per SM allows (1 KB reserved per block), at most LBM_WV_MINB (the
-// register budget: 128 registers a thread at two blocks of 256 threads)
-#ifndef LBM_WV_MINB
-#define LBM_WV_MINB 2
-#endif
-template <int S, int T> constexpr int wv_minb() {
-    return (233472 / (wv_smem<S, T>() + 1024)) < LBM_WV_MINB ? (233472 / (wv_smem<S, T>() + 1024))
-                                                             : LBM_WV_MINB;
-}
-
-// One block's share of a wavefront launch: strip `strip`, output rows y0 ..
-// y0 + rows - 1, T steps; wv_ring is the block's (T-1) rings.  With CHECK the thread's residual partials of
-// level T are accumulated into acc.  Called by k_wave (one block per strip
-// and segment) and by the batched arena (one call per work item).
-template <int S, bool GEN, int T, bool CHECK, typename I, bool CIRC_OK = false>
-__device__ __forceinline__ void wave_block(const StepParams& a, const Coef<float>& c, float* wv_ring,
-                                           int strip, int y0, int rows, ResAcc<S>& acc) {
-    static_assert(T >= 2 && T <= 4, "two to four steps per launch");
-    constexpr int W = kWvW, R = kWvRow, OX = wv_ox<T>(), PL = kWvD * kWvRow, RP = kWvRP * PL, D = kWvD - 1;
-    constexpr bool PA2 = wv_la2<S>();             // populations two rows ahead
-    constexpr bool L1FIRST = wv_l1first<S>();     // step 1 collides before the other levels
-    // (CIRC_OK: the single-lattice kernel; the batched arena's kernel, which also
-    // holds the two-step tiles, spills more with the larger code and keeps the
-    // copies: 2048 problems of sides 32 to 1024 ran at 141 against 165 GLUPS with them)
-    constexpr bool CIRC = CIRC_OK && LBM_WV_CIRC != 0 && S == S_F32 && PA2 && !L1FIRST;
-    const int nx = a.nx, ny = a.ny;
-    const int t = threadIdx.x;
-    const int xs = strip * OX - (T - 1) + t;      // lattice column of slot t (unwrapped)
-    const int x = wrap_slot<false>(xs, nx);
-    const int xm = wrap_dec(x, nx), xp = wrap_inc(x, nx);
-    const bool store_ok = t >= T - 1 && t <= W - T && xs < nx;
-    const float* __restrict__ gxp = static_cast<const float*>(a.gx);
-    const float* __restrict__ gyp = static_cast<const float*>(a.gy);
-    const int ybeg = y0 - (T - 1);                // lattice row of local row 0 (level 1)
-    const int iters = rows + 3 * (T - 1);
-    const int n1 = rows + 2 * (T - 1);            // rows of level 1
-    const int64_t n = a.plane;
-    // This thread's column of every ring (slot t sits at padded column t + 1,
-    // so the pulls of t - 1 and t + 1 stay inside the row for every thread).
-    float* const rt = wv_ring + t + 1;
-    // Force of the thread's column in local rows i, i - 1, ..., i - 2(T - 1)
-    // (i the iteration): level tau uses entry 2(tau - 1).
-    constexpr int NH = 2 * (T - 1) + 1;
-    float hx[NH], hy[NH];
-#pragma unroll
-    for (int k = 0; k < NH; ++k) hx[k] = hy[k] = 0.0f;
-    // Delay lines of the vertical movers at the T - 1 level boundaries: v2[r][k]
-    // is population 2 (index 1) of the row ring r's producer made k + 1
-    // productions ago, v4[r] population 4 (index 3) of its last row.  The
-    // consumer (level r + 2) of local row j reads population 2 of row j - 1
-    // (made three iterations earlier) and population 4 of row j + 1 (one
-    // iteration earlier) before the producer (level r + 1) of the same
-    // iteration shifts the line; producers run in consecutive iterations, from
-    // three iterations before their consumer's first to one before its last.
-    float v2[T - 1][4], v4[T - 1];
-#pragma unroll
-    for (int r = 0; r < T - 1; ++r) v2[r][0] = v2[r][1] = v2[r][2] = v2[r][3] = v4[r] = 0.0f;
-    // Step 1's pulls (one row ahead, PA2: two) and the force (LA2: two rows
-    // ahead, else one) in registers.  The row offsets of the next row to load
-    // advance one row per load (rows are loaded in order), with the periodic
-    // wrap.
-    constexpr bool LA2 = S == S_F32 || PA2;
-    Pulled<S> q[CIRC ? 4 : (PA2 ? 2 : 1)];
-    float qg[LA2 ? 2 : 1][2];
-    int ly = wrap_slot<false>(ybeg, ny);          // lattice row of the next population load
-    I lr0 = (I)ly * a.pitch, lrm = (I)wrap_dec(ly, ny) * a.pitch, lrp = (I)wrap_inc(ly, ny) * a.pitch;
-    int gly = ly;                                 // lattice row of the next force load
-    auto advance = [&]() {
-        ly = wrap_inc(ly, ny);
-        lrm = lr0;
-        lr0 = lrp;
-        lrp = (I)wrap_inc(ly, ny) * a.pitch;
-    };
-    auto load_force = [&](int b) {
-        const I g = (I)gly * a.pitch + x;
-        qg[b][0] = ldg(gxp + g);
-        qg[b][1] = ldg(gyp + g);
-        gly = wrap_inc(gly, ny);
-    };
-    auto load1 = [&](int b) {
-        pull_load<S, I>(a, lr0, lrm, lrp, x, xm, xp, q[b]);
-        advance();
-    };
-    // Residual check on level T: its snapshot entry is loaded one iteration ahead.
-    ResSnap<S> so;
-    auto snap_next = [&](int i) {
-        so = snap_load<S>(a, n, (int64_t)((I)(ybeg + i - 2 * (T - 1)) * a.pitch + xs));
-    };
-
-    // One iteration; FULL: every level active (ring slots fold to constants
-    // when i is a compile-time offset from a multiple of four).
-    // Halo threads of a level compute values no valid slot reads (their pulls
-    // stay inside the padded ring rows), so no level branches per thread; only
-    // the stores of level T are predicated.
-    auto iter = [&](int i, auto full_c, auto buf_c) {
-        constexpr bool FULL = decltype(full_c)::value;
-        constexpr int K = decltype(buf_c)::value;   // phase: i mod 4 (CIRC), else i mod 2
-        constexpr int b = LA2 ? (K & 1) : 0;        // load buffers of local row i (i mod 2 with
-                                                    // two rows ahead, else 0)
-        const bool l1 = FULL || i < n1;
-#pragma unroll
-        for (int k = NH - 1; k > 0; --k) {
-            hx[k] = hx[k - 1];
-            hy[k] = hy[k - 1];
-        }
-        hx[0] = qg[b][0];
-        hy[0] = qg[b][1];
-        // step 1 on local row i: its populations 2 and 4 (t2, t4) enter the
-        // delay lines after the levels below have read them
-        float f1[8], t2 = 0.0f, t4 = 0.0f;
-        auto level1 = [&]() {
-            float u, v, fs[8];
-            collide_populations<GEN>(moments(f1), hx[0], hy[0], c, u, v, fs);
-            float* d = rt + (i & D) * R;
-            d[0 * PL] = fs[0];
-            d[1 * PL] = fs[2];
-            d[2 * PL] = fs[4];
-            d[3 * PL] = fs[5];
-            d[4 * PL] = fs[6];
-            d[5 * PL] = fs[7];
-            t2 = fs[1];
-            t4 = fs[3];
-        };
-        if (l1) {
-            if constexpr (CIRC) {
-                // row i + 2 into the buffer row i - 2 left; row i stays in
-                // buffer K until step 1 collides it below
-                if (FULL || i + 2 < n1) load1((K + 2) & 3);
-            } else {
-                constexpr int bq = PA2 ? b : 0;
-                pull_decode<S>(a, q[bq], f1, c.theta);
-                // L1FIRST: collide row i before reloading its buffers (ring slot i
-                // mod 4 is not among the slots the levels below read)
-                if constexpr (L1FIRST) level1();
-                if (FULL || i + (PA2 ? 2 : 1) < n1) load1(bq);
-            }
-            if (FULL || i + (LA2 ? 2 : 1) < n1) load_force(b);
-        }
-        // Levels T..2: local row j = i - 2(tau - 1), pulled from ring tau - 1.
-#pragma unroll
-        for (int tau = T; tau >= 2; --tau) {
-            // active rows y0 - (T - tau) .. y0 + rows - 1 + (T - tau)
-            if (!FULL && (i < 3 * (tau - 1) || i > rows + 2 * T + tau - 4)) continue;
-            const int j = i - 2 * (tau - 1);
-            const float* sp = rt + (tau - 2) * RP;
-            const int rm = ((j - 1) & D) * R, r0 = (j & D) * R, rp = ((j + 1) & D) * R;
-            float f[8];
-            f[0] = sp[0 * PL + r0 - 1];          // f_p(x) = f*_p(x - c_p)
-            f[1] = CIRC ? v2[tau - 2][(K + 1) & 3] : v2[tau - 2][2];   // made 3 iterations ago
-            f[2] = sp[1 * PL + r0 + 1];
-            f[3] = v4[tau - 2];
-            f[4] = sp[2 * PL + rm - 1];
-            f[5] = sp[3 * PL + rm + 1];
-            f[6] = sp[4 * PL + rp + 1];
-            f[7] = sp[5 * PL + rp - 1];
-            const float gx = hx[2 * (tau - 1)], gy = hy[2 * (tau - 1)];
-            const Mom<float> m = moments(f);
-            if (tau < T) {
-                float u, v, fs[8];
-                collide_populations<GEN>(m, gx, gy, c, u, v, fs);
-                float* d = rt + (tau - 1) * RP + r0;
-                d[0 * PL] = fs[0];
-                d[1 * PL] = fs[2];
-                d[2 * PL] = fs[4];
-                d[3 * PL] = fs[5];
-                d[4 * PL] = fs[6];
-                d[5 * PL] = fs[7];
-                if constexpr (CIRC) {
-                    v2[tau - 1][K] = fs[1];
-                } else {
-                    v2[tau - 1][2] = v2[tau - 1][1];
-                    v2[tau - 1][1] = v2[tau - 1][0];
-                    v2[tau - 1][0] = fs[1];
-                }
-                v4[tau - 1] = fs[3];
-            } else {
-                // every thread collides; only the stores are predicated
-                float u, v, fs[8], c10, c01;
-                post_state<S, GEN>(m, gx, gy, c, u, v, fs, c10, c01);
-                if (store_ok) {
-                    const I idx = (I)(ybeg + j) * a.pitch + xs;   // row in [y0, y0 + rows), xs < nx
-                    if (CHECK) {
-                        check_node<S>(a, n, (int64_t)idx, acc, so, f, gx, gy, u, v);
-                        if (FULL || i + 1 < iters) snap_next(i + 1);
-                    }
-                    store_state<S>(a, (int64_t)idx, fs, c10, c01);
-                }
-            }
-        }
-        if (l1) {
-            if constexpr (CIRC) {
-                pull_decode<S>(a, q[K], f1, c.theta);
-                level1();
-                v2[0][K] = t2;
-            } else {
-                if constexpr (!L1FIRST) level1();
-                v2[0][2] = v2[0][1];
-                v2[0][1] = v2[0][0];
-                v2[0][0] = t2;
-            }
-            v4[0] = t4;
-        }
-        __syncthreads();
-    };
-
-    load1(0);
-    if (PA2 && n1 > 1) load1(1);
-    load_force(0);
-    if (LA2 && n1 > 1) load_force(1);
-    const int fb = 3 * (T - 1);                   // first iteration with every level active
-    // last one whose level 1 still loads ahead
-    const int fe = n1 - 1 - (LA2 || PA2 ? 2 : 1);
-    if (CHECK && store_ok) snap_next(fb);         // level T's first row is y0
-    const int m0 = (fb + 3) >> 2, m1 = (fe + 1) >> 2;   // groups i = 4m .. 4m + 3 within [fb, fe]
-    using B0 = std::integral_constant<int, 0>;
-    using B1 = std::integral_constant<int, 1>;
-    using B2 = std::integral_constant<int, CIRC ? 2 : 0>;
-    using B3 = std::integral_constant<int, CIRC ? 3 : 1>;
-    auto iter_any = [&](int i) {
-        if constexpr (CIRC) {
-            switch (i & 3) {
-                case 0: iter(i, std::false_type{}, B0{}); break;
-                case 1: iter(i, std::false_type{}, B1{}); break;
-                case 2: iter(i, std::false_type{}, B2{}); break;
-                default: iter(i, std::false_type{}, B3{}); break;
-            }
-        } else {
-            if (LA2 && (i & 1)) iter(i, std::false_type{}, B1{});
-            else iter(i, std::false_type{}, B0{});
-        }
-    };
-    int i = 0;
-    if (m1 > m0) {
-        for (; i < 4 * m0; ++i) iter_any(i);
-        for (int m = m0; m < m1; ++m) {
-            const int ib = m << 2;
-            iter(ib, std::true_type{}, B0{});
-            iter(ib + 1, std::true_type{}, B1{});
-            iter(ib + 2, std::true_type{}, B2{});
-            iter(ib + 3, std::true_type{}, B3{});
-        }
-        i = 4 * m1;
-    }
-    for (; i < iters; ++i) iter_any(i);
-}
-
-// ---------------------------------------------------------------------------
 // T pseudo-time steps per launch, one warp per strip of the
 // lattice (FP32 or FP16-shifted storage).
 //
@@ -2176,14 +1835,9 @@ inline int64_t step3_tiles(int nx, int ny) {
     return (int64_t)((nx + kT3OX - 1) / kT3OX) * ((ny + kT3OY - 1) / kT3OY);
 }
 
-// Wavefront launches (k_wave) of a single lattice: from one strip width by 8
-// rows up (the slot wrap is a single conditional subtraction there).
-inline bool wave_fits(int nx, int ny) { return nx >= kWvW && ny >= 8; }
-
-template <int T>
-inline int64_t wave_blocks(int nx, int ny, int seg) {
-    return (int64_t)((nx + wv_ox<T>() - 1) / wv_ox<T>()) * ((ny + seg - 1) / seg);
-}
+// The wavefront schedule's lattices (the documented limit of
+// lbm_set_wavefront; FP16S: four steps per launch from here on).
+inline bool wave_fits(int nx, int ny) { return nx >= 256 && ny >= 8; }
 
 // Strips of a strip launch of T steps.
 inline int64_t strip_count(int dtype, int T, int nx) {
