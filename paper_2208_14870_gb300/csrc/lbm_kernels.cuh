@@ -1023,7 +1023,7 @@ template <int T> __host__ __device__ constexpr int st_minb() { return T >= 7 ? 6
 // rows copied ahead of the rows in use, and population rows held: FP32 has the
 // rows above, at and below level 1 in use, FP16S the decoded row
 template <int S> __host__ __device__ constexpr int st_la() { return S == S_F16S ? 3 : 1; }
-constexpr int kStPR = 4;
+constexpr int kWvD = 4;
 // force rows held: those the levels still read and the rows ahead (a power of two)
 template <int S, int T> __host__ __device__ constexpr int st_ring() {
     return T + 1 + st_la<S>() <= 4 ? 4 : (T + 1 + st_la<S>() <= 8 ? 8 : 16);
@@ -1036,7 +1036,7 @@ constexpr int kStCols = 72;
 template <int S> __host__ __device__ constexpr int st_row() { return S == S_F16S ? kStCols * (8 * 2 + 8) : kStCols * 8 * 4; }
 constexpr int kStFRow = 2 * kStCols * 4;
 template <int S, int T> __host__ __device__ constexpr int st_warp_smem() {
-    return kStPR * st_row<S>() + st_ring<S, T>() * kStFRow;
+    return kWvD * st_row<S>() + st_ring<S, T>() * kStFRow;
 }
 template <int S, int T> __host__ __device__ constexpr int st_smem() { return st_nw<T>() * st_warp_smem<S, T>(); }
 
@@ -1103,7 +1103,7 @@ __device__ __forceinline__ void strip_walk(const StepParams& a, const PairCoef& 
     const bool two = ok && xs + 1 < nx;                      // (an odd lattice's last column stands alone)
     const int64_t n = a.plane;
     const int nit = rows + 2 * H;
-    const uint32_t frc = sm + kStPR * ROW;                   // force ring
+    const uint32_t frc = sm + kWvD * ROW;                   // force ring
     const uint32_t own = (uint32_t)(xs - xa0);               // the lane's first column within a row
     // Copies of a row: 16-byte chunks, chunk q = lane + 32 m (FP32: 18 per
     // plane, eight populations, then the force; FP16S: 9 per plane, eight
@@ -1131,7 +1131,7 @@ __device__ __forceinline__ void strip_walk(const StepParams& a, const PairCoef& 
     int ly = (y0 - H - OFF) % ny;                            // lattice row of the next copy
     if (ly < 0) ly += ny;
     auto copy_row = [&](int i) {
-        const uint32_t d = sm + (i & (kStPR - 1)) * ROW + lane * 16, g = frc + (i & (R - 1)) * kStFRow + lane * 16;
+        const uint32_t d = sm + (i & (kWvD - 1)) * ROW + lane * 16, g = frc + (i & (R - 1)) * kStFRow + lane * 16;
 #pragma unroll
         for (int m = 0; m < NM; ++m) {
             const uint32_t dp = d + m * 512, df = g + m * 512 - NP * 16;
@@ -1205,8 +1205,8 @@ __device__ __forceinline__ void strip_walk(const StepParams& a, const PairCoef& 
             // f_p(x) = f*_p(x - c_p), from rows i - 1, i and i + 1 (local rows
             // of the copies start one above the strip's, hence the + 1)
             constexpr int PL = kStCols * 4;
-            const uint32_t o4 = own * 4, rm = sm + (i & (kStPR - 1)) * ROW + o4,
-                           r0 = sm + ((i + 1) & (kStPR - 1)) * ROW + o4, rp = sm + ((i + 2) & (kStPR - 1)) * ROW + o4;
+            const uint32_t o4 = own * 4, rm = sm + (i & (kWvD - 1)) * ROW + o4,
+                           r0 = sm + ((i + 1) & (kWvD - 1)) * ROW + o4, rp = sm + ((i + 2) & (kWvD - 1)) * ROW + o4;
             auto left = [&](uint32_t r) { return pk(lds_float(r - 4), lds_float(r)); };
             auto right = [&](uint32_t r) { return pk(lds_float(r + 4), lds_float(r + 8)); };
             pair_t w[8];
@@ -1224,7 +1224,7 @@ __device__ __forceinline__ void strip_walk(const StepParams& a, const PairCoef& 
                 for (int p = 0; p < 8; ++p) f[p] = w[p];
         } else {
             // the populations of the lane's columns in row i (pull_decode)
-            const uint32_t r = sm + (i & (kStPR - 1)) * ROW;
+            const uint32_t r = sm + (i & (kWvD - 1)) * ROW;
             const float k1 = 0.5f * (1.0f - c.theta), k5 = 0.25f * c.theta;
             pair_t e0, e1;                        // (m*_10, m*_01) of either column
             lds_pairs(r + kStCols * 16 + own * 8, e0, e1);
@@ -1837,7 +1837,8 @@ inline int64_t step3_tiles(int nx, int ny) {
 
 // The wavefront schedule's lattices (the documented limit of
 // lbm_set_wavefront; FP16S: four steps per launch from here on).
-inline bool wave_fits(int nx, int ny) { return nx >= 256 && ny >= 8; }
+#define LBM_WV_NW 8   // in warps of 32 columns
+inline bool wave_fits(int nx, int ny) { return nx >= 32 * LBM_WV_NW && ny >= 8; }
 
 // Strips of a strip launch of T steps.
 inline int64_t strip_count(int dtype, int T, int nx) {
