@@ -202,6 +202,47 @@ __global__ void __launch_bounds__(256) k_arena_ghosts(const BatchArgs A, const u
     fill_ghosts<S>(prob_params<S>(A, P, P.parity ^ 1), threadIdx.x, blockDim.x);   // (dst: the current state)
 }
 
+__global__ void __launch_bounds__(256) k_arena_force(const ForceIn f) {
+    double m = 0.0;
+    unsigned int bad = 0;
+    const int64_t n = (int64_t)f.nx * f.ny;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t y = i / f.nx;
+        const int x = (int)(i - y * f.nx);
+        const int64_t h = f.tr ? (int64_t)x * f.hx + y : y * f.hx + x;
+        const double u = f.gx[h], v = f.gy[h];
+        if (!(isfinite(u) && isfinite(v))) bad = 1;
+        m = fmax(m, fmax(fabs(u), fabs(v)));
+        float* o = f.out + y * f.pitch + f.ghost + x;
+        const float gx = (float)(f.tr ? v : u), gy = (float)(f.tr ? u : v);
+        o[0] = gx;
+        o[f.plane] = gy;
+        if (x < f.ghost) {
+            o[f.nx] = gx;
+            o[f.plane + f.nx] = gy;
+        }
+        if (x >= f.nx - f.ghost) {
+            o[-f.nx] = gx;
+            o[f.plane - f.nx] = gy;
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+        bad |= __shfl_xor_sync(0xffffffffu, bad, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(f.stat, (unsigned long long)__double_as_longlong(m));
+        if (bad) atomicOr(f.stat + 1, 1ULL);
+    }
+}
+
+cudaError_t launch_arena_force(const ForceIn& f, cudaStream_t st) {
+    const int64_t n = (int64_t)f.nx * f.ny, blocks = (n + 1023) / 1024;
+    k_arena_force<<<(unsigned)(blocks < 2048 ? blocks : 2048), 256, 0, st>>>(f);
+    return cudaGetLastError();
+}
+
 template <int S, int T, bool CHECK>
 static cudaError_t launch_strips_k(const BatchArgs& a, const uint2* items, int count, int group, cudaStream_t st) {
     constexpr int SM = kArenaNW * st_warp_smem<S, T>();

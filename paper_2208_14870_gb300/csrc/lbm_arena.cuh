@@ -166,6 +166,20 @@ cudaError_t launch_arena_strips(int dtype, int T, bool check, const BatchArgs& a
                                 int group, cudaStream_t st);
 cudaError_t launch_arena_pairs(int dtype, bool check, const BatchArgs& a, const uint2* items, int count, int group,
                                cudaStream_t st);
+// A problem's force from the caller's FP64 arrays (device memory, hx columns per
+// row) into its FP32 planes of `plane` elements: rows of nx columns with their
+// ghost columns, transposed with the components exchanged for a problem solved
+// on its transpose.  stat[0]: max |g| (bit pattern of a non-negative double),
+// stat[1]: non-zero for a non-finite entry; both zero before.
+struct ForceIn {
+    const double *gx, *gy;
+    int hx, tr;
+    float* out;                // row 0, first ghost column
+    int nx, ny, pitch, ghost;
+    int64_t plane;
+    unsigned long long* stat;
+};
+cudaError_t launch_arena_force(const ForceIn& f, cudaStream_t st);
 cudaError_t launch_arena_ghosts(int dtype, const BatchArgs& a, const uint2* items, int count, cudaStream_t st);
 
 }  // namespace lbm

@@ -7,10 +7,13 @@
 #include <cmath>
 #include <memory>
 #include <string>
+#include <thread>
+#include <utility>
 #include <vector>
 
 #include "../../include/lbm.h"
 #include "lbm_engine.cuh"
+#include "lbm_host.cuh"
 
 using namespace lbm;
 
@@ -87,6 +90,30 @@ extern "C" int lbm_batch_solve(int count, const lbm_problem* probs, int dtype, d
             cudaStreamDestroy(st);
             return bfail(rc, "lbm_batch_solve: " + err);
         }
+        // Bring the callers' result arrays into memory while the device works
+        // (fresh pages would slow the field copies down tenfold).
+        std::vector<std::pair<double*, size_t>> fresh;
+        for (int i = 0; i < count; ++i)
+            for (double* o : {results[i].ux, results[i].uy, results[i].sxx, results[i].syy, results[i].sxy}) {
+                const size_t bytes = sizeof(double) * (size_t)probs[i].nx * probs[i].ny;
+                if (!o) continue;
+                if (!fresh.empty() && (char*)fresh.back().first + fresh.back().second == (char*)o) fresh.back().second += bytes;
+                else fresh.emplace_back(o, bytes);
+            }
+        struct Join {
+            std::thread t;
+            ~Join() { if (t.joinable()) t.join(); }
+        } populate;
+        if (!fresh.empty()) {
+            try {
+                populate.t = std::thread([&fresh] {
+                    host_parallel(fresh.size(), 1, [&](size_t b, size_t e) {
+                        for (size_t i = b; i < e; ++i) host_populate(fresh[i].first, fresh[i].second);
+                    });
+                });
+            } catch (...) {   // (no thread to be had: the copies take the faults)
+            }
+        }
         std::vector<int> slot(count);
         for (int i = 0; i < count && rc == LBM_OK; ++i) {
             const lbm_problem& p = probs[i];
@@ -95,6 +122,7 @@ extern "C" int lbm_batch_solve(int count, const lbm_problem* probs, int dtype, d
             else if (s < 0) rc = s;
             slot[i] = s;
         }
+        if (rc == LBM_OK) rc = eng.check_forces(&err);
         // Autotuner: the first chunks run with the strip chunk and two-step
         // tiles, or, where the chunk length does not allow strips, with two-step
         // tiles and tile widths 128, 64 and 32; the fastest per active node and
@@ -155,6 +183,7 @@ extern "C" int lbm_batch_solve(int count, const lbm_problem* probs, int dtype, d
                 want.push_back(slot[i]);
                 outs.insert(outs.end(), o, o + 5);
             }
+            if (populate.t.joinable()) populate.t.join();
             rc = eng.recover_many((int)want.size(), want.data(), outs.data(), &err);
         }
     }

@@ -51,10 +51,10 @@ ArenaEngine::~ArenaEngine() {
     if (d_tiles_) cudaFree(d_tiles_);
     if (d_ntiles_) cudaFree(d_ntiles_);
     if (d_fields_) cudaFree(d_fields_);
+    if (d_force_) cudaFree(d_force_);
+    if (d_stat_) cudaFree(d_stat_);
     if (h_acc_) cudaFreeHost(h_acc_);
     if (h_tiles_) cudaFreeHost(h_tiles_);
-    if (h_force_) cudaFreeHost(h_force_);
-    if (h_fields_) cudaFreeHost(h_fields_);
     for (int i = 0; i < kClasses - 1; ++i) {
         if (side_[i]) cudaStreamDestroy(side_[i]);
         if (join_[i]) cudaEventDestroy(join_[i]);
@@ -109,6 +109,8 @@ int ArenaEngine::init(int dtype, int64_t node_capacity, int max_probs, int check
     ECK(cudaMalloc(&d_probs_, sizeof(BatchProb) * max_probs));
     ECK(cudaMalloc(&d_acc_, sizeof(double) * kRes * max_probs));
     ECK(cudaMallocHost(&h_acc_, sizeof(double) * kRes * max_probs));
+    ECK(cudaMalloc(&d_stat_, 2 * sizeof(unsigned long long) * max_probs));
+    ECK(cudaMemsetAsync(d_stat_, 0, 2 * sizeof(unsigned long long) * max_probs, st_));
     ECK(cudaMalloc(&d_ntiles_, sizeof(int)));
     ECK(cudaMemsetAsync(d_ntiles_, 0, sizeof(int), st_));
     for (int i = 0; i < kClasses - 1; ++i) {
@@ -182,54 +184,57 @@ int ArenaEngine::admit(int nx, int ny, double lambda, double mu, const double* g
     p.tr = tr;
     p.n = n;
     if (!place(p)) return -1;
-    // force -> FP32 staging (pinned), with the FP16 scale from its maximum
+    // the force: copied as given, converted, transposed and checked on the device
     const int64_t len = 2 * p.plane;
-    if (h_force_cap_ < len) {
-        if (h_force_) {
+    if (d_force_cap_ < 2 * n) {
+        if (d_force_) {
             ECK(cudaStreamSynchronize(st_));
-            cudaFreeHost(h_force_);
-            h_force_ = nullptr;
+            cudaFree(d_force_);
+            d_force_ = nullptr;
+            d_force_cap_ = 0;
         }
-        ECK(cudaMallocHost(&h_force_, sizeof(float) * len));
-        h_force_cap_ = len;
+        const int64_t cap = std::max<int64_t>(2 * n, int64_t(1) << 20);
+        ECK(cudaMalloc(&d_force_, sizeof(double) * cap));
+        d_force_cap_ = cap;
     }
-    ECK(cudaStreamSynchronize(st_));  // the staging may still feed a previous copy
-    double gmax = 0.0;
-    // (row y of the arena lattice: its pitch elements are the periodic images of
-    // its columns, ghost columns and padding included)
-    for (int64_t y = 0; y < p.ny; ++y) {
-        float* rx = h_force_ + y * p.pitch;
-        float* ry = rx + p.plane;
-        for (int c = 0; c < p.nx; ++c) {
-            const int64_t i = tr ? (int64_t)c * nx + y : y * nx + c;
-            const double a = gx[i], b = gy[i];
-            if (!std::isfinite(a) || !std::isfinite(b)) {
-                unplace(p);
-                if (err) *err = "admit: non-finite force";
-                return LBM_ERR_ARG;
-            }
-            gmax = std::fmax(gmax, std::fmax(std::fabs(a), std::fabs(b)));
-            rx[p.ghost + c] = (float)(tr ? b : a);
-            ry[p.ghost + c] = (float)(tr ? a : b);
-        }
-        for (int g = 0; g < p.ghost; ++g) {
-            rx[g] = rx[p.nx + g];
-            ry[g] = ry[p.nx + g];
-        }
-        for (int g = p.ghost + p.nx; g < p.pitch; ++g) {
-            rx[g] = rx[g - p.nx];
-            ry[g] = ry[g - p.nx];
-        }
-    }
-    p.hexp = dtype_ == S_F16S ? f16s_exponent(gmax, p.nx, p.ny) : 0;
-    if (p.hexp != 0) {
+    unsigned long long* stat = d_stat_ + 2 * slot;
+    float* force = reinterpret_cast<float*>(fs_ + p.fs_off);
+    ECK(cudaMemcpyAsync(d_force_, gx, sizeof(double) * n, cudaMemcpyHostToDevice, st_));
+    ECK(cudaMemcpyAsync(d_force_ + n, gy, sizeof(double) * n, cudaMemcpyHostToDevice, st_));
+    ECK(cudaMemsetAsync(stat, 0, 2 * sizeof(unsigned long long), st_));
+    ECK(cudaMemsetAsync(force, 0, p.fs_bytes, st_));
+    ForceIn f{};
+    f.gx = d_force_;
+    f.gy = d_force_ + n;
+    f.hx = nx;
+    f.tr = tr ? 1 : 0;
+    f.out = force;
+    f.nx = p.nx;
+    f.ny = p.ny;
+    f.pitch = p.pitch;
+    f.ghost = p.ghost;
+    f.plane = p.plane;
+    f.stat = stat;
+    ECK(launch_arena_force(f, st_));
+    if (dtype_ == S_F16S) {
         // FP16S keeps its state, the force included, in units scaled by 2^hexp
-        // (store_f16s); the power of two is exact
-        const float sc = std::ldexp(1.0f, p.hexp);
-        for (int64_t i = 0; i < len; ++i) h_force_[i] *= sc;
+        // from max |g| (store_f16s); the power of two is exact
+        unsigned long long got[2];
+        ECK(cudaMemcpyAsync(got, stat, sizeof(got), cudaMemcpyDeviceToHost, st_));
+        ECK(cudaStreamSynchronize(st_));
+        double gmax;
+        std::memcpy(&gmax, &got[0], sizeof(double));
+        if (got[1]) {
+            unplace(p);
+            if (err) *err = "admit: non-finite force";
+            return LBM_ERR_ARG;
+        }
+        p.hexp = f16s_exponent(gmax, p.nx, p.ny);
+        if (p.hexp != 0) {
+            k_scale_float<<<256, 256, 0, st_>>>(force, len, std::ldexp(1.0f, p.hexp));
+            ECK(cudaGetLastError());
+        }
     }
-    ECK(cudaMemcpyAsync(fs_ + p.fs_off, h_force_, sizeof(float) * len, cudaMemcpyHostToDevice, st_));
-    ECK(cudaMemsetAsync(fs_ + p.fs_off + sizeof(float) * len, 0, sizeof(float2) * 2 * p.plane, st_));
     ECK(cudaMemsetAsync(pop_[0] + p.pop_off, 0, p.pop_bytes, st_));
     if (dtype_ == S_F16S) ECK(cudaMemsetAsync(car_[0] + p.car_off, 0, p.car_bytes, st_));
     p.parity = 0;
@@ -265,6 +270,18 @@ int64_t ArenaEngine::running_tiles(int V) const {
             else t += arena_strips(p.nx) * ((p.ny + wave_seg_ - 1) / wave_seg_);
         }
     return t;
+}
+
+int ArenaEngine::check_forces(std::string* err) {
+    std::vector<unsigned long long> got(2 * probs_.size());
+    ECK(cudaMemcpyAsync(got.data(), d_stat_, sizeof(unsigned long long) * got.size(), cudaMemcpyDeviceToHost, st_));
+    ECK(cudaStreamSynchronize(st_));
+    for (size_t i = 0; i < probs_.size(); ++i)
+        if (got[2 * i + 1]) {
+            if (err) *err = "admit: non-finite force";
+            return LBM_ERR_ARG;
+        }
+    return LBM_OK;
 }
 
 // Rows per strip item of the running problems, by strip_shape's model: the
@@ -646,66 +663,47 @@ int ArenaEngine::ensure_fields_buffer(int64_t len, std::string* err) {
     return LBM_OK;
 }
 
-int ArenaEngine::recover(int slot, double* ux, double* uy, double* sxx, double* syy, double* sxy,
-                         std::string* err) {
-    const HostProb& p = probs_[slot];
-    if (p.state == P_FREE) {
-        if (err) *err = "recover: empty slot";
-        return LBM_ERR_STATE;
-    }
-    int rc = ensure_fields_buffer(5 * p.n, err);
-    if (rc) return rc;
-    ECK(launch_fields(slot, d_fields_));
-    double* outs[5] = {ux, uy, sxx, syy, sxy};
-    for (int i = 0; i < 5; ++i)
-        if (outs[i])
-            ECK(cudaMemcpyAsync(outs[i], d_fields_ + i * p.n, sizeof(double) * p.n,
-                                cudaMemcpyDeviceToHost, st_));
-    ECK(cudaStreamSynchronize(st_));
-    return LBM_OK;
-}
-
 int ArenaEngine::recover_many(int count, const int* slots, double* const* outs, std::string* err) {
-    // Problems are packed into blocks of kRecoverBlock doubles: one field
-    // launch per problem into a device block, one copy of the block into a
-    // pinned host block, one synchronisation, then host copies into the
-    // callers' arrays.  A problem larger than a block goes alone.
+    // Problems are packed into blocks of kRecoverBlock doubles (a larger problem
+    // is a block of its own): one field launch per problem into a device block,
+    // then copies straight into the callers' arrays, one per problem where its
+    // five arrays lie one after the other.
     constexpr int64_t kRecoverBlock = int64_t(4) << 20;   // 32 MB of FP64
-    for (int i = 0; i < count; ++i)
-        if (probs_[slots[i]].state == P_FREE) {
+    int64_t need = 0, all = 0;
+    for (int i = 0; i < count; ++i) {
+        const HostProb& p = probs_[slots[i]];
+        if (p.state == P_FREE) {
             if (err) *err = "recover: empty slot";
             return LBM_ERR_STATE;
         }
-    int rc = ensure_fields_buffer(kRecoverBlock, err);
-    if (rc) return rc;
-    if (!h_fields_) {
-        ECK(cudaMallocHost(&h_fields_, sizeof(double) * kRecoverBlock));
+        need = std::max(need, 5 * p.n);
+        all += 5 * p.n;
     }
+    if (count == 0) return LBM_OK;
+    int rc = ensure_fields_buffer(std::max(need, std::min(all, kRecoverBlock)), err);
+    if (rc) return rc;
     for (int i = 0; i < count;) {
-        if (5 * probs_[slots[i]].n > kRecoverBlock) {
-            double* const* o = outs + 5 * (int64_t)i;
-            rc = recover(slots[i], o[0], o[1], o[2], o[3], o[4], err);
-            if (rc) return rc;
-            ++i;
-            continue;
-        }
         int j = i;
         int64_t used = 0;
-        for (; j < count && 5 * probs_[slots[j]].n <= kRecoverBlock - used; ++j) {
+        for (; j < count && (j == i || used + 5 * probs_[slots[j]].n <= d_fields_cap_); ++j) {
             ECK(launch_fields(slots[j], d_fields_ + used));
             used += 5 * probs_[slots[j]].n;
         }
-        ECK(cudaMemcpyAsync(h_fields_, d_fields_, sizeof(double) * used, cudaMemcpyDeviceToHost, st_));
-        ECK(cudaStreamSynchronize(st_));
         int64_t off = 0;
         for (int q = i; q < j; ++q) {
             const int64_t n = probs_[slots[q]].n;
-            for (int f = 0; f < 5; ++f) {
-                double* dst = outs[5 * (int64_t)q + f];
-                if (dst) std::memcpy(dst, h_fields_ + off + f * n, sizeof(double) * n);
+            double* const* o = outs + 5 * (int64_t)q;
+            for (int f = 0; f < 5;) {
+                int g = f + 1;
+                while (o[f] && g < 5 && o[g] == o[f] + (g - f) * n) ++g;
+                if (o[f])
+                    ECK(cudaMemcpyAsync(o[f], d_fields_ + off + f * n, sizeof(double) * n * (g - f),
+                                        cudaMemcpyDeviceToHost, st_));
+                f = g;
             }
             off += 5 * n;
         }
+        ECK(cudaStreamSynchronize(st_));
         i = j;
     }
     return LBM_OK;

@@ -66,17 +66,18 @@ public:
     static int64_t slots_for(int nx, int ny);
     // Admit a problem; returns slot >= 0, -1 if it does not fit now, or a
     // negative lbm status (< -1) on error.  gx, gy: host FP64, nx*ny each.
+    // FP32: the force is checked later, by check_forces.
     int admit(int nx, int ny, double lambda, double mu, const double* gx, const double* gy,
               double tol, int64_t max_iters, std::string* err);
+    // LBM_ERR_ARG if a problem admitted since init has a non-finite force entry
+    // (FP16S problems are refused by admit already).
+    int check_forces(std::string* err);
     // One chunk of check_every steps for every running problem; afterwards
     // finished problems are in state P_DONE (not yet released).
     int run_chunk(int V, float* device_ms, std::string* err);
-    // Solution fields of a finished (or running) problem into host arrays
-    // (nullable), FP64, lattice units.
-    int recover(int slot, double* ux, double* uy, double* sxx, double* syy, double* sxy,
-                std::string* err);
-    // The same for count problems at once; outs holds 5 nullable host arrays
-    // (ux, uy, sxx, syy, sxy) per problem.  Few copies and synchronisations.
+    // Solution fields of count finished (or running) problems into host arrays,
+    // FP64, lattice units; outs holds 5 nullable host arrays (ux, uy, sxx, syy,
+    // sxy) per problem.
     int recover_many(int count, const int* slots, double* const* outs, std::string* err);
     void release(int slot);
     const HostProb& prob(int slot) const { return probs_[slot]; }
@@ -130,11 +131,11 @@ private:
     int wave_seg_ = 0;                // rows per strip item of the current list
     bool tiles_dirty_ = true;
     bool desc_dirty_ = true;
-    float* h_force_ = nullptr;        // pinned FP32 staging
-    int64_t h_force_cap_ = 0;
+    double* d_force_ = nullptr;       // FP64 staging of the caller's force
+    int64_t d_force_cap_ = 0;
+    unsigned long long* d_stat_ = nullptr;   // per problem: max |g|, non-finite flag (ForceIn)
     double* d_fields_ = nullptr;      // FP64 staging for recovery
     int64_t d_fields_cap_ = 0;
-    double* h_fields_ = nullptr;      // pinned block for recover_many
     cudaGraphExec_t graph_[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
     bool graph_failed_[6] = {false, false, false, false, false, false};
     cudaEvent_t ev0_ = nullptr, ev1_ = nullptr;

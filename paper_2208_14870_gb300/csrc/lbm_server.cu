@@ -11,6 +11,7 @@
 // host memory owned by the request, their arena memory is freed for the next
 // admissions, and their latency (submission to completion) is recorded.
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <condition_variable>
@@ -25,6 +26,7 @@
 
 #include "../../include/lbm.h"
 #include "lbm_engine.cuh"
+#include "lbm_host.cuh"
 
 using namespace lbm;
 
@@ -39,8 +41,8 @@ struct Request {
     int nx = 0, ny = 0, dtype = LBM_F32;
     double lambda = 0.0, mu = 0.0, tol = 0.0;
     int64_t max_iters = 0;
-    std::vector<double> gx, gy;
-    std::vector<double> fields;   // 5 * nx * ny once done
+    std::unique_ptr<double[]> gx, gy;       // until admitted
+    std::unique_ptr<double[]> fields;       // 5 * nx * ny once done
     int state = R_QUEUED;
     int status = LBM_OK;
     int64_t iters = 0;
@@ -171,7 +173,7 @@ int lbm_server::admit_locked() {
             continue;
         }
         std::string err;
-        const int s = arena[a]->admit(r.nx, r.ny, r.lambda, r.mu, r.gx.data(), r.gy.data(), r.tol,
+        const int s = arena[a]->admit(r.nx, r.ny, r.lambda, r.mu, r.gx.get(), r.gy.get(), r.tol,
                                       r.max_iters, &err);
         if (s >= 0) {
             r.state = R_RUNNING;
@@ -179,8 +181,8 @@ int lbm_server::admit_locked() {
             r.slot = s;
             r.t_admit = clk::now();
             slot_owner[a][s] = r.ticket;
-            std::vector<double>().swap(r.gx);  // the arena holds the force now
-            std::vector<double>().swap(r.gy);
+            r.gx.reset();  // the arena holds the force now
+            r.gy.reset();
             it = queue.erase(it);
             continue;
         }
@@ -200,12 +202,16 @@ void lbm_server::retire(int a, const std::vector<int>& slots, std::unique_lock<s
     for (int slot : slots) {
         Request& r = *reqs[slot_owner[a][slot]];
         const int64_t n = (int64_t)r.nx * r.ny;
-        r.fields.assign((size_t)5 * n, 0.0);
-        double* f = r.fields.data();
+        r.fields.reset(new double[(size_t)5 * n]);
+        double* f = r.fields.get();
         for (int k = 0; k < 5; ++k) outs.push_back(f + k * n);
     }
     std::string err;
     lk.unlock();
+    for (size_t i = 0; i < slots.size(); ++i) {
+        const size_t bytes = 5 * sizeof(double) * (size_t)arena[a]->prob(slots[i]).n;
+        host_parallel(bytes, size_t(4) << 20, [&](size_t b, size_t e) { host_populate((char*)outs[5 * i] + b, e - b); });
+    }
     const int rc = arena[a]->recover_many((int)slots.size(), slots.data(), outs.data(), &err);
     lk.lock();
     if (rc != LBM_OK) {
@@ -316,11 +322,19 @@ int lbm_server_submit(lbm_server* s, const lbm_problem* p, int dtype, double tol
     r->mu = p->mu;
     r->tol = tol;
     r->max_iters = max_iters;
-    r->gx.assign(p->gx, p->gx + n);
-    r->gy.assign(p->gy, p->gy + n);
-    for (int64_t i = 0; i < n; ++i)
-        if (!std::isfinite(r->gx[i]) || !std::isfinite(r->gy[i]))
-            return set_last_error(LBM_ERR_ARG, "lbm_server_submit: non-finite force");
+    r->gx.reset(new double[n]);
+    r->gy.reset(new double[n]);
+    std::atomic<bool> bad{false};
+    host_parallel((size_t)n, size_t(1) << 17, [&](size_t b, size_t e) {
+        bool any = false;
+        for (size_t i = b; i < e; ++i) {
+            r->gx[i] = p->gx[i];
+            r->gy[i] = p->gy[i];
+            any |= !std::isfinite(r->gx[i]) || !std::isfinite(r->gy[i]);
+        }
+        if (any) bad = true;
+    });
+    if (bad) return set_last_error(LBM_ERR_ARG, "lbm_server_submit: non-finite force");
     {
         std::lock_guard<std::mutex> lk(s->mu);
         if (s->failed != LBM_OK)
@@ -348,9 +362,13 @@ static int take_result(lbm_server* s, Request& r, lbm_result* out) {
         out->transposed = r.transposed;
         const int64_t n = (int64_t)r.nx * r.ny;
         double* dst[5] = {out->ux, out->uy, out->sxx, out->syy, out->sxy};
-        if (!r.fields.empty())
-            for (int i = 0; i < 5; ++i)
-                if (dst[i]) std::memcpy(dst[i], r.fields.data() + i * n, sizeof(double) * n);
+        if (r.fields)
+            for (int i = 0; i < 5;) {
+                int j = i + 1;                 // (one copy where the arrays lie one after the other)
+                while (dst[i] && j < 5 && dst[j] == dst[i] + (j - i) * n) ++j;
+                if (dst[i]) host_copy(dst[i], r.fields.get() + i * n, sizeof(double) * n * (j - i));
+                i = j;
+            }
     }
     s->reqs.erase(r.ticket);
     return LBM_OK;
