@@ -330,19 +330,12 @@ def host_description():
 # Our arm
 # ---------------------------------------------------------------------------
 
-def plan_plain(m, spl, wave=False, most=0):
+def plan_plain(m, spl, wave=False):
     """Launch sizes of m plain steps as the library groups them: launches of
     spl steps (four only on the wavefront schedule, else three), a remainder
     of one avoided where possible (4 = 2 + 2, 5 = 3 + 2), then pairs, then
-    single steps.  most > 4: FP32 on the wavefront schedule, whose launches
-    take up to that many steps (lbm_get_launch_steps)."""
+    single steps."""
     sizes = []
-    if most > 4:
-        while m >= 2:
-            k = most if m >= most and m != most + 1 else ((most + 1) // 2 if m == most + 1 else m)
-            sizes.append(k)
-            m -= k
-        return sizes + [1] * m
     big = 4 if spl >= 4 and wave else (3 if spl >= 3 else 0)
     if big:
         groups, r = divmod(m, big)
@@ -366,19 +359,19 @@ def check_launch_steps(w, spl, wave=False):
     return 4 if (wave and spl >= 4 and w >= 4) else min(spl, 2, w)
 
 
-def launches_per_iterate(iters, check_every, spl, wave=False, most=0):
+def launches_per_iterate(iters, check_every, spl, wave=False):
     """Stream-collide launches of lbm_iterate_checked(iters, check_every) from
     step 0: each window is check_every - 1 plain steps grouped into launches of
     spl steps (the remainder in shorter ones) and ends with the check step,
     the last step of the window's last launch (check_launch_steps)."""
     def window(w):
         last = check_launch_steps(w, spl, wave)
-        return len(plan_plain(w - last, spl, wave, most)) + 1
+        return len(plan_plain(w - last, spl, wave)) + 1
     total, left = 0, iters
     while left >= check_every:
         total += window(check_every)
         left -= check_every
-    return total + len(plan_plain(left, spl, wave, most))
+    return total + len(plan_plain(left, spl, wave))
 
 
 def time_variant(args, dtype, gx_d, gy_d, torch, P, nsteps, nwarm, events=True, spl=None, iters=None,
@@ -402,8 +395,12 @@ def time_variant(args, dtype, gx_d, gy_d, torch, P, nsteps, nwarm, events=True, 
 
     ce = args.check_every
     windows, rest = divmod(iters, ce)
+    block, big = dominant_block(ce, spl, wave_on)
     most = P.lbm_get_launch_steps(lat.ctx)
-    block, big = dominant_block(ce, spl, wave_on, most)
+    if most > big:
+        # FP32 without a set schedule: launches of `most` steps, and a window
+        # ends with a checked launch of at most `most`
+        block, big = max(0, ce - 5) // most * most, most
     nev = nsteps * windows
 
     def one_step(ev_a=None, ev_b=None, dom=None):
@@ -437,6 +434,7 @@ def time_variant(args, dtype, gx_d, gy_d, torch, P, nsteps, nwarm, events=True, 
     devs = [torch.cuda.Event(enable_timing=True) for _ in range(2 * nev)]
     t_start = torch.cuda.Event(enable_timing=True)
     t_end = torch.cuda.Event(enable_timing=True)
+    counted = P.lbm_get_launches(lat.ctx)
     t_start.record(stream)
     for i, (a, b) in enumerate(evs):
         one_step(a, b, devs[2 * i * windows: 2 * (i + 1) * windows])
@@ -448,10 +446,9 @@ def time_variant(args, dtype, gx_d, gy_d, torch, P, nsteps, nwarm, events=True, 
     dom_launches = nev * (block // big)
     lat.close()
     del out5
-    per_iter = launches_per_iterate(iters, args.check_every, spl, wave_on, most)
     checks = iters // args.check_every      # each adds one residual-finish launch
     return {"total_ms": total_ms, "iter_ms": iter_ms, "steps": nsteps, "spl": spl, "iters": iters,
-            "step_launches": nsteps * per_iter, "launches": nsteps * (per_iter + checks + 1),
+            "step_launches": step_launches, "launches": step_launches + nsteps * (checks + 1),
             "dom_ms": dom_ms, "dom_launches": dom_launches, "big": big, "wave": wave_on}
 
 
@@ -465,12 +462,12 @@ def fp64_peak(P):
         return FP64_PEAK_GINST, "nominal GB300 FP64 rate (1.25 TFLOP/s with FMA = 2 flops); measurement failed: %s" % e
 
 
-def dominant_block(check_every, spl, wave=False, most=0):
+def dominant_block(check_every, spl, wave=False):
     """(steps, k): the first steps of a residual window, which the library
     runs as whole plain launches of k steps each, k the longest launch of the
     window (lbm_iterate_checked plans the window's check_every - 1 plain steps
     so; see plan_plain)."""
-    sizes = plan_plain(check_every - check_launch_steps(check_every, spl, wave), spl, wave, most)
+    sizes = plan_plain(check_every - check_launch_steps(check_every, spl, wave), spl, wave)
     if not sizes:
         return 0, spl
     big = sizes[0]

@@ -150,7 +150,7 @@ int lbm_get_host_transfer(lbm_ctx *ctx, int *mode);
  * so results differ from one step per launch by less than that format's
  * rounding (and lie closer to the FP64 result).  Since the grouping cannot
  * change an LBM_F32 state, k = 4 on the wavefront schedule lets LBM_F32
- * launches take as many steps as suit the lattice, up to seven
+ * launches take as many steps as suit the lattice, up to six
  * (lbm_get_launch_steps); LBM_F16S keeps groups of four.  Available for LBM_F32 and
  * LBM_F16S storage on any lattice.  Until this function or lbm_set_wavefront is
  * called, LBM_F32 lattices take whichever schedule their size suits (strips of
@@ -169,6 +169,10 @@ int lbm_get_steps_per_launch(lbm_ctx *ctx, int *k);
 /* The most pseudo-time steps a plain (unchecked) launch of this context
  * advances under its settings.  Errors: LBM_ERR_ARG (null), LBM_ERR_CUDA. */
 int lbm_get_launch_steps(lbm_ctx *ctx, int *k);
+
+/* Kernels launched since the context was created to advance its lattice (each
+ * stream-collide launch counts one, whatever number of steps it takes). */
+int lbm_get_launches(lbm_ctx *ctx, int64_t *n);
 
 /* Wavefront schedule of launches of three or more steps (rows > 0: segments
  * of `rows` rows; rows = -1: segments chosen per launch), or the tile schedule

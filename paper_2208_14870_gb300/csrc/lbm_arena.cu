@@ -65,32 +65,20 @@ __device__ __forceinline__ void add_to_problem(double* dst, const double w[kRes]
 // thread) into the problem's FP64 accumulator.
 template <int S>
 __device__ __forceinline__ void tile_to_problem(const ResAcc<S>& acc, double* dst,
-                                                double (&red)[kRes][kThreads / 32]) {
-    const int tid = threadIdx.y * 32 + threadIdx.x, lane = tid & 31, warp = tid >> 5;
+                                                double (*red)[32]) {
+    const int tid = threadIdx.y * 32 + threadIdx.x;
     double v[kRes];
-    res_to_double<S>(acc, v);
+    acc.to_double(v);
     warp_reduce_res(v);
-    if (lane == 0)
-        for (int k = 0; k < kRes; ++k) red[k][warp] = v[k];
-    __syncthreads();
-    if (tid == 0) {
-        double m[kRes] = {0.0, 0.0, 0.0, 0.0, 0.0};
-        for (int w = 0; w < kThreads / 32; ++w) {
-            m[0] = fmax(m[0], red[0][w]);
-            m[1] = fmax(m[1], red[1][w]);
-            m[2] += red[2][w];
-            m[3] += red[3][w];
-            m[4] = fmax(m[4], red[4][w]);
-        }
-        add_to_problem(dst, m);
-    }
+    block_reduce_res(v, red, tid, kThreads / 32);
+    if (tid == 0) add_to_problem(dst, v);
     __syncthreads();
 }
 
 template <int S, int V>
 __global__ void __launch_bounds__(kThreads, 2) k_arena_chunk(const BatchArgs A) {
     cg::grid_group grid = cg::this_grid();
-    __shared__ double red[kRes][kThreads / 32];
+    __shared__ double red[kRes][32];
     const int ntiles = *A.ntiles;
     for (int s = 0; s < A.nsteps; ++s) {
         const bool last = (s == A.nsteps - 1);
@@ -126,7 +114,7 @@ template <int S>
 __global__ void __launch_bounds__(kT2Threads, 2) k_arena_chunk2(const BatchArgs A) {
     cg::grid_group grid = cg::this_grid();
     extern __shared__ float t2_smem[];
-    __shared__ double red[kRes][kThreads / 32];
+    __shared__ double red[kRes][32];
     const int ntiles = *A.ntiles;
     const int npairs = A.nsteps / 2;
     for (int s = 0; s < npairs; ++s) {
@@ -163,12 +151,12 @@ k_arena_strips(const BatchArgs A, const uint2* items, int count, int group) {
     const PairCoef c = pair_coef(prob_coef(P));
     const int ns = (P.nx + kArenaOX - 1) / kArenaOX;
     const int strip = (int)tl.y % ns, y0 = (int)tl.y / ns * P.seg, rows = min(P.seg, P.ny - y0);
-    const uint32_t sm = (uint32_t)__cvta_generic_to_shared(strip_mem) + warp * st_warp_smem<S, T>();
-    ResAcc<S> acc;
+    const uint32_t sm = (uint32_t)__cvta_generic_to_shared(strip_mem) + warp * st_warp_smem<S, T, CHECK>();
+    ResAcc2 acc;
     if (CHECK && P.check) {
         strip_walk<S, false, T, true, kArenaOX>(a, c, sm, strip, y0, rows, acc);
         double w[kRes];
-        res_to_double<S>(acc, w);
+        acc.to_double(w);
         warp_reduce_res(w);
         if ((threadIdx.x & 31) == 0) add_to_problem(A.acc + (int64_t)tl.x * kRes, w);
     } else {
@@ -181,7 +169,7 @@ template <int S, bool CHECK>
 __global__ void __launch_bounds__(kT2Threads, 2)
 k_arena_pairs(const BatchArgs A, const uint2* items, int group) {
     extern __shared__ float t2_smem[];
-    __shared__ double red[kRes][kThreads / 32];
+    __shared__ double red[kRes][32];
     after_predecessor();
     const uint2 tl = items[blockIdx.x];
     const BatchProb P = A.probs[tl.x];
@@ -245,7 +233,7 @@ cudaError_t launch_arena_force(const ForceIn& f, cudaStream_t st) {
 
 template <int S, int T, bool CHECK>
 static cudaError_t launch_strips_k(const BatchArgs& a, const uint2* items, int count, int group, cudaStream_t st) {
-    constexpr int SM = kArenaNW * st_warp_smem<S, T>();
+    constexpr int SM = kArenaNW * st_warp_smem<S, T, CHECK>();
     const auto kernel = k_arena_strips<S, T, CHECK>;
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SM);
     if (e != cudaSuccess) return e;

@@ -45,6 +45,8 @@ int set_last_error(int code, const std::string& msg) {
 }
 }  // namespace lbm
 
+constexpr int kWavePlan = 128;    // longest run of plain steps wave_plan plans exactly
+
 struct lbm_ctx {
     int device = 0;
     int nx = 0, ny = 0, dtype = 0;
@@ -86,8 +88,11 @@ struct lbm_ctx {
                                    // with the segment chosen per launch (wave_seg)
     int nsm = 0;                   // multiprocessors of the device
     int64_t nblocks2 = 0;          // grid of the two-step check launch
-    StripShape shape[kStTMax + 1]; // strip launches per step count ([0]: checked), cleared by lbm_set_wavefront
-    int wave_T = 0;                // FP32: steps per plain strip launch (0: not chosen yet)
+    StripShape shape[2][kStTMax + 1];   // strip launches per step count, plain and checked, cleared by lbm_set_wavefront
+    int wave_T = 0;                // FP32 strip launches (wave_plan; 0: not planned yet)
+    uint8_t wave_first[kWavePlan + 1] = {};
+    double wave_cost[kWavePlan + 1] = {};
+    int64_t launches = 0;          // kernels launched to advance the lattice
     bool auto_plan = true;         // FP32: strip or tile launches as they suit the lattice, until the
                                    // caller sets a schedule (lbm_set_steps_per_launch, lbm_set_wavefront)
     int plan = 0;                  // 0: not chosen yet, 1: strips, 2: register tiles (tile)
@@ -155,8 +160,9 @@ Coef<T> coef(lbm_rates r) {
 
 // Residual of a check launch whose blocks wrote partials only.
 cudaError_t finish_residual_launch(lbm_ctx* c, int64_t grid) {
-    k_residual_finish<<<1, kFinishThreads, 0, c->stream>>>(c->partials, grid, c->result);
-    return cudaGetLastError();
+    const int threads = grid < kFinishThreads ? (int)((grid + 31) / 32 * 32) : kFinishThreads;
+    return launch_after(k_residual_finish, dim3(1), dim3(threads), 0, c->stream, (const double*)c->partials, grid,
+                        c->result);
 }
 
 int ensure_partials(lbm_ctx* c, int64_t sets);
@@ -169,6 +175,7 @@ cudaError_t launch_tile64(lbm_ctx* c, int T, bool check) {
     if (e == cudaSuccess && check) e = finish_residual_launch(c, std::min(tile64_count(t, c->nx, c->ny), c->nblocks));
     if (e == cudaSuccess) {
         c->cur ^= 1;
+        ++c->launches;
         c->step += T;
         c->staged_fields = false;
     }
@@ -187,6 +194,7 @@ cudaError_t launch_step(lbm_ctx* c, bool check) {
     if (e == cudaSuccess) {
         c->ghosts_ok = false;
         c->cur ^= 1;
+        ++c->launches;
         c->step += 1;
         c->staged_fields = false;
     }
@@ -204,6 +212,7 @@ cudaError_t launch_step2(lbm_ctx* c, bool check) {
     if (e == cudaSuccess) {
         c->ghosts_ok = false;
         c->cur ^= 1;
+        ++c->launches;
         c->step += 2;
         c->staged_fields = false;
     }
@@ -219,6 +228,7 @@ cudaError_t launch_step3(lbm_ctx* c) {
     if (e == cudaSuccess) {
         c->ghosts_ok = false;
         c->cur ^= 1;
+        ++c->launches;
         c->step += 3;
         c->staged_fields = false;
     }
@@ -230,7 +240,7 @@ bool wave_on(const lbm_ctx* c) { return c->wave != 0 && wave_fits(c->nx, c->ny);
 // The shape of a strip launch of T steps (kept per context: it depends on the
 // sizes and the lbm_set_wavefront setting only).
 cudaError_t wave_shape(lbm_ctx* c, int T, bool check, StripShape* out) {
-    StripShape& sh = c->shape[check ? 0 : T];
+    StripShape& sh = c->shape[check][T];
     if (sh.T == 0) {
         int warps = 0;
         const StepParams a = params(c, c->cur);
@@ -238,42 +248,67 @@ cudaError_t wave_shape(lbm_ctx* c, int T, bool check, StripShape* out) {
         const cudaError_t e = c->dtype == LBM_F32 ? strip_f32(a, cf, c->gen, T, check, 1, &warps, c->stream)
                                                   : strip_f16s(a, cf, c->gen, T, check, 1, &warps, c->stream);
         if (e != cudaSuccess) return e;
-        sh = strip_shape(c->dtype, T, c->nx, c->ny, c->nsm > 0 ? c->nsm : 1, warps, c->wave);
+        sh = strip_shape(c->dtype, T, check, c->nx, c->ny, c->nsm > 0 ? c->nsm : 1, warps, c->wave);
     }
     *out = sh;
     return cudaSuccess;
 }
 
-// Steps per plain strip launch of FP32 storage: the count with the fewest
-// modelled cycles per step, memory traffic included (its states are the same
-// bits whatever the grouping).  Every launch moves 72 bytes per node, 3.0
-// cycles per 768 bytes at 6.2 TB/s, unless the lattice stays in the L2 cache.
-cudaError_t wave_steps(lbm_ctx* c, int* T) {
-    if (c->wave_T == 0) {
-        const double bytes = 72.0 * (double)c->n;
-        const double mem = bytes > 1.2e8 ? bytes / 6.2e12 * 2.0e9 : 0.0;
-        double best = 0.0;
-        int bt = 0;
-        for (int t = 4; t <= kStTMax; ++t) {
-            StripShape sh;
-            const cudaError_t e = wave_shape(c, t, false, &sh);
-            if (e != cudaSuccess) return e;
-            const double per = (sh.cost > mem ? sh.cost : mem) / t;
-            if (bt == 0 || per < best) {
-                best = per;
-                bt = t;
+// Groups of FP32 strip launches: for every n up to kWavePlan the steps of the
+// launch to take first, of those that cover n steps in the fewest modelled
+// cycles (FP32 states are the same bits whatever the grouping); n = 1 runs as a
+// single step.  wave_T: the group with the fewest cycles per step.
+cudaError_t wave_plan(lbm_ctx* c) {
+    if (c->wave_T) return cudaSuccess;
+    double cost[kStTMax + 1] = {0.0, 3000.0 + 72.0 * (double)c->n / 3040.0};
+    int best = 2;
+    for (int t = 2; t <= kStTMax; ++t) {
+        StripShape sh;
+        const cudaError_t e = wave_shape(c, t, false, &sh);
+        if (e != cudaSuccess) return e;
+        cost[t] = sh.cost;
+        if (cost[t] * best < cost[best] * t) best = t;
+    }
+    c->wave_cost[0] = 0.0;
+    for (int n = 1; n <= kWavePlan; ++n) {
+        c->wave_cost[n] = 0.0;
+        for (int t = 1; t <= kStTMax && t <= n; ++t) {
+            const double v = cost[t] + c->wave_cost[n - t];
+            if (t == 1 || v < c->wave_cost[n]) {
+                c->wave_cost[n] = v;
+                c->wave_first[n] = (uint8_t)t;
             }
         }
-        c->wave_T = bt;
     }
-    *T = c->wave_T;
+    c->wave_T = best;
     return cudaSuccess;
 }
 
-// Blocks (partial sets) of the checked launch of four steps.
-int64_t strip_check_blocks(const lbm_ctx* c, int seg) {
-    const int64_t items = strip_count(c->dtype, 4, c->nx) * ((c->ny + seg - 1) / seg);
-    return (items + st_nw<4>() - 1) / st_nw<4>();
+// The first launch of n plain steps, and the modelled cycles of all of them.
+int wave_first(const lbm_ctx* c, int64_t n) { return n > kWavePlan ? c->wave_T : c->wave_first[n]; }
+double wave_cost(const lbm_ctx* c, int64_t n) {
+    const int64_t groups = n > kWavePlan ? (n - kWavePlan + c->wave_T - 1) / c->wave_T : 0;
+    return groups * (c->wave_cost[c->wave_T]) + c->wave_cost[n - groups * c->wave_T];
+}
+
+// Steps of the checked strip launch that ends a window of n >= 4 steps: four,
+// or (FP32, without a set number of steps per launch below four) the cheaper of
+// four and five with the plain launches before it.
+cudaError_t wave_check_steps(lbm_ctx* c, int64_t n, int* T) {
+    *T = 4;
+    if (c->dtype != LBM_F32 || n < 5) return cudaSuccess;
+    StripShape a, b;
+    cudaError_t e = wave_plan(c);
+    if (e == cudaSuccess) e = wave_shape(c, 4, true, &a);
+    if (e == cudaSuccess) e = wave_shape(c, 5, true, &b);
+    if (e == cudaSuccess && b.cost + wave_cost(c, n - 5) < a.cost + wave_cost(c, n - 4)) *T = 5;
+    return e;
+}
+
+// Blocks (partial sets) of a checked strip launch.
+int64_t strip_check_blocks(const lbm_ctx* c, int T, int seg) {
+    const int64_t items = strip_count(c->dtype, T, c->nx) * ((c->ny + seg - 1) / seg);
+    return (items + kStNW - 1) / kStNW;
 }
 
 cudaError_t launch_strip(lbm_ctx* c, int T, bool check) {
@@ -282,7 +317,7 @@ cudaError_t launch_strip(lbm_ctx* c, int T, bool check) {
     if (e != cudaSuccess) return e;
     int64_t blocks = 0;
     if (check) {
-        blocks = strip_check_blocks(c, sh.seg);
+        blocks = strip_check_blocks(c, T, sh.seg);
         if (ensure_partials(c, blocks) != LBM_OK) return cudaErrorMemoryAllocation;
     }
     if (!c->ghosts_ok) {
@@ -299,6 +334,7 @@ cudaError_t launch_strip(lbm_ctx* c, int T, bool check) {
     if (e == cudaSuccess && check) e = finish_residual_launch(c, blocks);
     if (e == cudaSuccess) {
         c->cur ^= 1;
+        ++c->launches;
         c->step += T;
         c->staged_fields = false;
     }
@@ -314,12 +350,9 @@ cudaError_t choose_plan(lbm_ctx* c) {
     c->tile = tile_shape(c->nx, c->ny, c->nsm > 0 ? c->nsm : 1);
     c->plan = 2;
     if (c->ghost) {
-        int T = 0;
-        StripShape sh;
-        cudaError_t e = wave_steps(c, &T);
-        if (e == cudaSuccess) e = wave_shape(c, T, false, &sh);
+        const cudaError_t e = wave_plan(c);
         if (e != cudaSuccess) return e;
-        if (sh.cost * c->tile.T < c->tile.cost * T) c->plan = 1;
+        if (c->wave_cost[c->wave_T] * c->tile.T < c->tile.cost * c->wave_T) c->plan = 1;
     }
     return cudaSuccess;
 }
@@ -336,6 +369,7 @@ cudaError_t launch_tile(lbm_ctx* c, int T, bool check) {
     if (e == cudaSuccess) {
         c->ghosts_ok = false;
         c->cur ^= 1;
+        ++c->launches;
         c->step += T;
         c->staged_fields = false;
     }
@@ -366,17 +400,14 @@ cudaError_t run_tiles(lbm_ctx* c, int64_t n, bool check) {
     return e;
 }
 
-// n plain steps in strip launches of up to T steps: whole groups, then the
-// rest in one launch, or two for T + 1.
+// n plain steps in strip launches (FP32).
 cudaError_t run_strips(lbm_ctx* c, int64_t n) {
-    int T = 0;
-    cudaError_t e = wave_steps(c, &T);
-    while (n >= 2 && e == cudaSuccess) {
-        const int t = n >= T && n != T + 1 ? T : (n == T + 1 ? (T + 1) / 2 : (int)n);
-        e = launch_strip(c, t, false);
+    cudaError_t e = wave_plan(c);
+    while (n > 0 && e == cudaSuccess) {
+        const int t = wave_first(c, n);
+        e = t > 1 ? launch_strip(c, t, false) : launch_step(c, false);
         n -= t;
     }
-    if (n > 0 && e == cudaSuccess) e = launch_step(c, false);
     return e;
 }
 
@@ -441,8 +472,10 @@ cudaError_t run_window(lbm_ctx* c, int64_t to_check) {
         }
     }
     if (to_check >= 4 && (auto_on(c) || (c->spl >= 4 && wave_on(c)))) {
-        e = run_plain(c, to_check - 4);
-        return e == cudaSuccess ? launch_strip(c, 4, true) : e;
+        int T = 0;
+        e = wave_check_steps(c, to_check, &T);
+        if (e == cudaSuccess) e = run_plain(c, to_check - T);
+        return e == cudaSuccess ? launch_strip(c, T, true) : e;
     }
     if (c->spl >= 2 && to_check >= 2) {
         e = run_plain(c, to_check - 2);
@@ -744,9 +777,11 @@ int lbm_create_ex(int nx, int ny, double lambda, double mu, int dtype, const lbm
     if (e == cudaSuccess) e = alloc(&c->snap, snap_bytes);
     c->partials_len = std::max(c->nblocks, c->nblocks2);
     if (e == cudaSuccess && dtype != LBM_F64 && (wave_on(c) || (dtype == LBM_F32 && c->ghost))) {
-        StripShape sh;
-        e = wave_shape(c, 4, true, &sh);
-        c->partials_len = std::max(c->partials_len, strip_check_blocks(c, sh.seg));
+        for (int T = 4; T <= (dtype == LBM_F32 ? 5 : 4) && e == cudaSuccess; ++T) {
+            StripShape sh;
+            e = wave_shape(c, T, true, &sh);
+            c->partials_len = std::max(c->partials_len, strip_check_blocks(c, T, sh.seg));
+        }
     }
     if (e == cudaSuccess && dtype == LBM_F32) {
         e = choose_plan(c);
@@ -816,7 +851,16 @@ int lbm_get_launch_steps(lbm_ctx* c, int* k) {
     *k = c->spl >= 4 && !wave_on(c) ? 3 : c->spl;
     if (auto_on(c)) CK(choose_plan(c));
     if (auto_on(c) && c->plan == 2) *k = c->tile.T;
-    else if (c->dtype == LBM_F32 && (auto_on(c) || (c->spl >= 4 && wave_on(c)))) CK(wave_steps(c, k));
+    else if (c->dtype == LBM_F32 && (auto_on(c) || (c->spl >= 4 && wave_on(c)))) {
+        CK(wave_plan(c));
+        *k = c->wave_T;
+    }
+    return LBM_OK;
+}
+
+int lbm_get_launches(lbm_ctx* c, int64_t* n) {
+    if (!c || !n) return fail(LBM_ERR_ARG, "lbm_get_launches: null pointer");
+    *n = c->launches;
     return LBM_OK;
 }
 
@@ -829,7 +873,8 @@ int lbm_set_wavefront(lbm_ctx* c, int rows) {
         return fail(LBM_ERR_ARG, "lbm_set_wavefront: the wavefront kernel needs FP32 or FP16-shifted storage");
     c->wave = rows;
     c->auto_plan = false;
-    for (auto& sh : c->shape) sh = StripShape();
+    for (auto& kind : c->shape)
+        for (auto& sh : kind) sh = StripShape();
     c->wave_T = 0;
     return LBM_OK;
 }

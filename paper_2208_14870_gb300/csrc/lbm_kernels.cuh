@@ -52,7 +52,6 @@ constexpr int max_vec() {
     return S == S_F64 ? 2 : (S == S_F16S ? LBM_F16S_V : 4);
 }
 constexpr int kThreads = 32 * BY;
-constexpr int kMaxWarps = 16;          // warps of the largest block that reduces residuals
 
 template <int S> struct StoreT;
 // T: collision arithmetic, P: stored population, G: stored force.
@@ -100,11 +99,34 @@ __device__ __forceinline__ T ldg(const T* p) { return __ldg(p); }
 template <int S> struct ResSnap { float2 u, v; };          // (hi, lo) per component
 template <> struct ResSnap<S_F64> { double u, v; };
 
+// A thread's partial as FP64 (a NaN among the maxima -- an infinite difference --
+// is left to the flag).
+__device__ __forceinline__ double pair_to_double(float h, float l) { return (double)h + (double)l; }
+__device__ __forceinline__ double max_to_double(float h, float l) {
+    const double v = pair_to_double(h, l);
+    return v >= 0.0 ? v : 0.0;
+}
+
 template <int S> struct ResAcc {
     float dh = 0.f, dl = 0.f, uh = 0.f, ul = 0.f, d2h = 0.f, d2l = 0.f, u2h = 0.f, u2l = 0.f, bad = 0.f;
+    // [max|du|, max|u|, sum du^2, sum u^2, flag]
+    __device__ __forceinline__ void to_double(double w[kRes]) const {
+        w[0] = max_to_double(dh, dl);
+        w[1] = max_to_double(uh, ul);
+        w[2] = pair_to_double(d2h, d2l);
+        w[3] = pair_to_double(u2h, u2l);
+        w[4] = bad;
+    }
 };
 template <> struct ResAcc<S_F64> {
     double d = 0.0, u = 0.0, d2 = 0.0, u2 = 0.0, bad = 0.0;
+    __device__ __forceinline__ void to_double(double w[kRes]) const {
+        w[0] = d >= 0.0 ? d : 0.0;
+        w[1] = u >= 0.0 ? u : 0.0;
+        w[2] = d2;
+        w[3] = u2;
+        w[4] = bad;
+    }
 };
 
 // max(m, |h + l|) on normalised pairs (|l| <= ulp(h) / 2), lexicographically.
@@ -196,33 +218,145 @@ __device__ __forceinline__ void check_node(const StepParams& a, int64_t n, int64
     }
 }
 
-// The thread's partials in FP64: [max|du|, max|u|, sum du^2, sum u^2, flag].
-template <int S>
-__device__ __forceinline__ void res_to_double(const ResAcc<S>& acc, double w[kRes]) {
-    if constexpr (S == S_F64) {
-        w[0] = acc.d;
-        w[1] = acc.u;
-        w[2] = acc.d2;
-        w[3] = acc.u2;
-        w[4] = acc.bad;
-    } else {
-        w[0] = (double)acc.dh + (double)acc.dl;
-        w[1] = (double)acc.uh + (double)acc.ul;
-        w[2] = (double)acc.d2h + (double)acc.d2l;
-        w[3] = (double)acc.u2h + (double)acc.u2l;
-        w[4] = acc.bad;
-    }
+// Combination of kRes partials across a warp's lanes (result in every lane).
+// The maxima and the flag are non-negative doubles, which order like their bit
+// patterns: they are combined as integers (an FP64 instruction takes 64 cycles
+// of a scheduler), the sums in FP64.
+__device__ __forceinline__ double max_bits(double a, double b) {
+    const unsigned long long x = (unsigned long long)__double_as_longlong(a), y = (unsigned long long)__double_as_longlong(b);
+    return __longlong_as_double((long long)(x > y ? x : y));
 }
-
-// Warp-level FP64 combination of kRes partials (result in every lane).
+__device__ __forceinline__ void combine_res(double w[kRes], const double v[kRes]) {
+    w[0] = max_bits(w[0], v[0]);
+    w[1] = max_bits(w[1], v[1]);
+    w[2] += v[2];
+    w[3] += v[3];
+    w[4] = max_bits(w[4], v[4]);
+}
 __device__ __forceinline__ void warp_reduce_res(double w[kRes]) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-        w[0] = fmax(w[0], __shfl_xor_sync(0xffffffffu, w[0], o));
-        w[1] = fmax(w[1], __shfl_xor_sync(0xffffffffu, w[1], o));
-        w[2] += __shfl_xor_sync(0xffffffffu, w[2], o);
-        w[3] += __shfl_xor_sync(0xffffffffu, w[3], o);
-        w[4] = fmax(w[4], __shfl_xor_sync(0xffffffffu, w[4], o));
+        double v[kRes];
+#pragma unroll
+        for (int k = 0; k < kRes; ++k) v[k] = __shfl_xor_sync(0xffffffffu, w[k], o);
+        combine_res(w, v);
+    }
+}
+// The same across the block's warps (at most 32): every lane of every warp
+// brings its warp's partials, thread 0's w receives the block's.
+__device__ __forceinline__ void block_reduce_res(double w[kRes], double (*sh)[32], int tid, int nwarps) {
+    const int lane = tid & 31, warp = tid >> 5;
+    if (lane == 0)
+        for (int k = 0; k < kRes; ++k) sh[k][warp] = w[k];
+    __syncthreads();
+    if (warp == 0) {
+        for (int k = 0; k < kRes; ++k) w[k] = lane < nwarps ? sh[k][lane] : 0.0;
+        warp_reduce_res(w);
+    }
+}
+
+// The residual check of two nodes at a time, in packed instructions: the
+// partials of the low and the high node of a lane's pairs are kept apart until
+// the end, where the halves a lane owns count (own0, own1).
+struct ResAcc2 {
+    float dh[2] = {0.f, 0.f}, dl[2] = {0.f, 0.f}, uh[2] = {0.f, 0.f}, ul[2] = {0.f, 0.f};
+    pair_t d2h = 0, d2l = 0, u2h = 0, u2l = 0, fin = 0;   // fin: 0 until a displacement is not finite
+    bool own0 = false, own1 = false;
+    __device__ __forceinline__ void to_double(double w[kRes]) const {
+        const bool own[2] = {own0, own1};
+        float a[2], b[2], c[2], d[2], f[2];
+        unpk(fin, f[0], f[1]);
+        unpk(d2h, a[0], a[1]);
+        unpk(d2l, b[0], b[1]);
+        unpk(u2h, c[0], c[1]);
+        unpk(u2l, d[0], d[1]);
+        for (int k = 0; k < kRes; ++k) w[k] = 0.0;
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            if (own[h]) {
+                const double v[kRes] = {max_to_double(dh[h], dl[h]), max_to_double(uh[h], ul[h]),
+                                        pair_to_double(a[h], b[h]), pair_to_double(c[h], d[h]), f[h] == 0.0f ? 0.0 : 1.0};
+                combine_res(w, v);
+            }
+    }
+};
+
+// two_sum (lbm_core.cuh) on pairs.
+__device__ __forceinline__ pair_t two_sum2(pair_t a, pair_t b, pair_t& e) {
+    const pair_t s = add2(a, b), bb = sub2(s, a);
+    e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
+    return s;
+}
+__device__ __forceinline__ pair_t two_diff2(pair_t a, pair_t b, pair_t& e) {      // a - b
+    const pair_t s = sub2(a, b), bb = sub2(s, a);
+    e = sub2(sub2(a, sub2(s, bb)), add2(b, bb));
+    return s;
+}
+// s += a^2 + b^2, a and b in two parts each (pair_add_square's terms of both
+// squares, joined before they meet the sum).
+__device__ __forceinline__ void pair_add_squares2(pair_t& sh, pair_t& sl, pair_t ah, pair_t al, pair_t bh, pair_t bl) {
+    float a0, a1, b0, b1;
+    unpk(ah, a0, a1);
+    unpk(bh, b0, b1);
+    const pair_t p = pk(__fmul_rn(a0, a0), __fmul_rn(a1, a1)), q = pk(__fmul_rn(b0, b0), __fmul_rn(b1, b1));
+    const pair_t np = pk(__fmul_rn(-a0, a0), __fmul_rn(-a1, a1)), nq = pk(__fmul_rn(-b0, b0), __fmul_rn(-b1, b1));
+    const pair_t ea = fma2(add2(ah, ah), al, fma2(ah, ah, np)), eb = fma2(add2(bh, bh), bl, fma2(bh, bh, nq));
+    pair_t t, t2;
+    const pair_t w = two_sum2(p, q, t), s = two_sum2(sh, w, t2);
+    const pair_t x = add2(add2(sl, t2), add2(t, add2(ea, eb))), r = add2(s, x);
+    sl = sub2(x, sub2(r, s));
+    sh = r;
+}
+// max over both of |h + l| into (mh, ml): one test for two candidates, which
+// few nodes pass once a thread's maximum is established.
+__device__ __forceinline__ void pair_max_abs2(float& mh, float& ml, float h, float l, float g, float m) {
+    if (fmaxf(fabsf(h), fabsf(g)) >= mh) {
+        pair_max_abs(mh, ml, h, l);
+        pair_max_abs(mh, ml, g, m);
+    }
+}
+
+// Residual check of a lane's two nodes (pulled populations f, force gx, gy):
+// check_node's arithmetic for FP32 and FP16-shifted storage.  o0, o1: their
+// snapshot entries; store(u0, v0, u1, v1) writes the new ones.
+template <int S, typename STORE>
+__device__ __forceinline__ void check_pair(ResAcc2& acc, const ResSnap<S>& o0, const ResSnap<S>& o1, const pair_t f[8],
+                                           pair_t gx, pair_t gy, STORE&& store) {
+    const pair_t half = splat(0.5f);
+    pair_t er, es, e12, e21, ea, eb, e10, e01, eu, ev;
+    const pair_t r = two_diff2(f[4], f[6], er), s = two_diff2(f[5], f[7], es);
+    const pair_t m12 = two_diff2(r, s, e12), m21 = two_sum2(r, s, e21);
+    const pair_t a = two_diff2(f[0], f[2], ea), b = two_diff2(f[1], f[3], eb);
+    const pair_t m10 = two_sum2(a, m12, e10), m01 = two_sum2(b, m21, e01);
+    const pair_t u = two_sum2(m10, fma2(half, gx, 0), eu), v = two_sum2(m01, fma2(half, gy, 0), ev);
+    const pair_t ulo = add2(add2(add2(eu, e10), add2(ea, e12)), sub2(er, es));
+    const pair_t vlo = add2(add2(add2(ev, e01), add2(eb, e21)), add2(er, es));
+    pair_t ul, vl;
+    const pair_t uh = two_sum2(u, ulo, ul), vh = two_sum2(v, vlo, vl);
+    float4 n0, n1;                                // (u hi, u lo, v hi, v lo) of either node
+    unpk(uh, n0.x, n1.x);
+    unpk(ul, n0.y, n1.y);
+    unpk(vh, n0.z, n1.z);
+    unpk(vl, n0.w, n1.w);
+    store(make_float2(n0.x, n0.y), make_float2(n0.z, n0.w), make_float2(n1.x, n1.y), make_float2(n1.z, n1.w));
+    pair_t e, ul2, vl2;
+    pair_t du = two_diff2(uh, pk(o0.u.x, o1.u.x), e);
+    du = two_sum2(du, add2(e, sub2(ul, pk(o0.u.y, o1.u.y))), ul2);
+    pair_t dv = two_diff2(vh, pk(o0.v.x, o1.v.x), e);
+    dv = two_sum2(dv, add2(e, sub2(vl, pk(o0.v.y, o1.v.y))), vl2);
+    pair_add_squares2(acc.d2h, acc.d2l, du, ul2, dv, vl2);
+    pair_add_squares2(acc.u2h, acc.u2l, uh, ul, vh, vl);
+    acc.fin = fma2(uh, 0, fma2(vh, 0, acc.fin));
+    float x[2], y[2], p[2], q[2];
+    unpk(du, x[0], x[1]);
+    unpk(ul2, y[0], y[1]);
+    unpk(dv, p[0], p[1]);
+    unpk(vl2, q[0], q[1]);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const float4 n = h ? n1 : n0;
+        pair_max_abs2(acc.dh[h], acc.dl[h], x[h], y[h], p[h], q[h]);
+        pair_max_abs2(acc.uh[h], acc.ul[h], n.x, n.y, n.z, n.w);
     }
 }
 
@@ -387,31 +521,20 @@ __device__ __forceinline__ void scatter_local(const StepParams& a, int64_t idx,
 // check; without one (the library's own check launches) the blocks stop after
 // writing their partials and k_residual_finish combines them in a separate
 // launch.
-template <int S>
-__device__ __forceinline__ void residual_reduce(const StepParams& a, const ResAcc<S>& acc) {
-    __shared__ double sh[kRes][kMaxWarps];
+template <typename ACC>
+__device__ __forceinline__ void residual_reduce(const StepParams& a, const ACC& acc) {
+    __shared__ double sh[kRes][32];
     __shared__ bool is_last;
     const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-    const int lane = tid & 31, warp = tid >> 5;
-    const int nwarps = (blockDim.x * blockDim.y) >> 5;
+    const int nthr = blockDim.x * blockDim.y, nwarps = nthr >> 5;
     double v[kRes];
-    res_to_double<S>(acc, v);
+    acc.to_double(v);
     warp_reduce_res(v);
-    if (lane == 0)
-        for (int k = 0; k < kRes; ++k) sh[k][warp] = v[k];
-    __syncthreads();
+    block_reduce_res(v, sh, tid, nwarps);
     const unsigned int nblocks = gridDim.x * gridDim.y;
     const unsigned int bid = blockIdx.y * gridDim.x + blockIdx.x;
     if (tid == 0) {
-        double w[kRes] = {0.0, 0.0, 0.0, 0.0, 0.0};
-        for (int i = 0; i < nwarps; ++i) {
-            w[0] = fmax(w[0], sh[0][i]);
-            w[1] = fmax(w[1], sh[1][i]);
-            w[2] += sh[2][i];
-            w[3] += sh[3][i];
-            w[4] = fmax(w[4], sh[4][i]);
-        }
-        for (int k = 0; k < kRes; ++k) a.partials[(int64_t)bid * kRes + k] = w[k];
+        for (int k = 0; k < kRes; ++k) a.partials[(int64_t)bid * kRes + k] = v[k];
         if (a.counter != nullptr) {
             __threadfence();
             const unsigned int done = atomicAdd(a.counter, 1u);
@@ -424,48 +547,17 @@ __device__ __forceinline__ void residual_reduce(const StepParams& a, const ResAc
     __syncthreads();
     if (!is_last) return;
     __threadfence();
-    // (four blocks' partials in flight per thread: the grid may have 10^5 blocks)
     double w[kRes] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    const unsigned int nthr = blockDim.x * blockDim.y;
-    unsigned int b = tid;
-    for (; b + 3 * nthr < nblocks; b += 4 * nthr) {
-        double q[4][kRes];
+    for (unsigned int b = tid; b < nblocks; b += nthr) {
+        double q[kRes];
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int k = 0; k < kRes; ++k) q[u][k] = __ldcg(a.partials + (int64_t)(b + u * nthr) * kRes + k);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            w[0] = fmax(w[0], q[u][0]);
-            w[1] = fmax(w[1], q[u][1]);
-            w[2] += q[u][2];
-            w[3] += q[u][3];
-            w[4] = fmax(w[4], q[u][4]);
-        }
-    }
-    for (; b < nblocks; b += nthr) {
-        const double* p = a.partials + (int64_t)b * kRes;
-        w[0] = fmax(w[0], __ldcg(p + 0));
-        w[1] = fmax(w[1], __ldcg(p + 1));
-        w[2] += __ldcg(p + 2);
-        w[3] += __ldcg(p + 3);
-        w[4] = fmax(w[4], __ldcg(p + 4));
+        for (int k = 0; k < kRes; ++k) q[k] = __ldcg(a.partials + (int64_t)b * kRes + k);
+        combine_res(w, q);
     }
     warp_reduce_res(w);
-    __syncthreads();
-    if (lane == 0)
-        for (int k = 0; k < kRes; ++k) sh[k][warp] = w[k];
-    __syncthreads();
+    block_reduce_res(w, sh, tid, nwarps);
     if (tid == 0) {
-        double r[kRes] = {0.0, 0.0, 0.0, 0.0, 0.0};
-        for (int i = 0; i < nwarps; ++i) {
-            r[0] = fmax(r[0], sh[0][i]);
-            r[1] = fmax(r[1], sh[1][i]);
-            r[2] += sh[2][i];
-            r[3] += sh[3][i];
-            r[4] = fmax(r[4], sh[4][i]);
-        }
-        for (int k = 0; k < kRes; ++k) a.result[k] = r[k];
+        for (int k = 0; k < kRes; ++k) a.result[k] = w[k];
         *a.counter = 0u;
         __threadfence();
     }
@@ -547,7 +639,7 @@ k_step(const StepParams a, const Coef<typename StoreT<S>::T> c) {
         const int ty = (int)(t / ntx), tx = (int)(t - (int64_t)ty * ntx);
         step_tile<S, V, GEN, CHECK>(a, c, tx, ty, acc);
     }
-    if (CHECK) residual_reduce<S>(a, acc);
+    if (CHECK) residual_reduce(a, acc);
 }
 
 // Periodic image in [0, n) of a slot coordinate v >= -1.  ANY = false
@@ -636,7 +728,7 @@ k_tile64(const StepParams a, const Coef<double> c, int T, int bx, int by, int nt
             if (T > 1) __syncthreads();
         }
     }
-    if (CHECK) residual_reduce<S_F64>(a, acc);
+    if (CHECK) residual_reduce(a, acc);
 }
 
 // ---------------------------------------------------------------------------
@@ -802,7 +894,7 @@ k_step2(const StepParams a, const Coef<float> c) {
         step2_tile<S, GEN, CHECK, ANY>(a, c, t2_smem, tx, ty, acc);
         if (t + gridDim.x < ntiles) __syncthreads();   // slots are reused by the next tile
     }
-    if (CHECK) residual_reduce<S>(a, acc);
+    if (CHECK) residual_reduce(a, acc);
 }
 
 // ---------------------------------------------------------------------------
@@ -964,7 +1056,7 @@ k_step3(const StepParams a, const Coef<float> c) {
         step3_tile<S, GEN, CHECK, ANY>(a, c, t3_smem, tx, ty, acc);
         if (t + gridDim.x < ntiles) __syncthreads();   // slots are reused by the next tile
     }
-    if (CHECK) residual_reduce<S>(a, acc);
+    if (CHECK) residual_reduce(a, acc);
 }
 
 // ---------------------------------------------------------------------------
@@ -1004,7 +1096,7 @@ k_step3(const StepParams a, const Coef<float> c) {
 // instruction cache and the compiler took 202 registers instead of 150.
 constexpr int kGhost = 8;                        // ghost columns per row end (at least kStTMax + 1)
 constexpr int kStSlots = 64;                     // slot columns of a strip (two per lane)
-constexpr int kStTMax = 7;                       // most steps per launch
+constexpr int kStTMax = 6;                       // most steps per launch (seven: 0.627 ms per step at 16384^2, six 0.611)
 
 template <int S> __host__ __device__ constexpr int st_lag() { return S == S_F16S ? 1 : 0; }
 // halo rows per end, and halo columns: at least as many per side, even on the
@@ -1014,12 +1106,10 @@ template <int S, int T> __host__ __device__ constexpr int st_left() { return (st
 template <int S, int T> __host__ __device__ constexpr int st_ox() {
     return (kStSlots - st_left<S, T>() - st_halo<S, T>()) & ~1;
 }
-// warps per block and resident blocks the kernel is compiled for: twelve warps
-// per SM (168 registers a thread; at 16384^2 with registers for eight warps
-// 87.6 ms per 100 steps against 79.8; T = 7 as 64-thread blocks 447 GLUPS, as
-// 128-thread blocks 411)
-template <int T> __host__ __device__ constexpr int st_nw() { return T >= 7 ? 2 : 4; }
-template <int T> __host__ __device__ constexpr int st_minb() { return T >= 7 ? 6 : 3; }
+// warps per block; the kernel is compiled for three resident blocks, twelve
+// warps per SM (168 registers a thread; at 16384^2 with registers for eight warps
+// 87.6 ms per 100 steps against 79.8)
+constexpr int kStNW = 4;
 // rows copied ahead of the rows in use, and population rows held: FP32 has the
 // rows above, at and below level 1 in use, FP16S the decoded row
 template <int S> __host__ __device__ constexpr int st_la() { return S == S_F16S ? 3 : 1; }
@@ -1035,10 +1125,12 @@ template <int S, int T> __host__ __device__ constexpr int st_ring() {
 constexpr int kStCols = 72;
 template <int S> __host__ __device__ constexpr int st_row() { return S == S_F16S ? kStCols * (8 * 2 + 8) : kStCols * 8 * 4; }
 constexpr int kStFRow = 2 * kStCols * 4;
-template <int S, int T> __host__ __device__ constexpr int st_warp_smem() {
-    return kWvD * st_row<S>() + st_ring<S, T>() * kStFRow;
+template <int S, int T, bool CHECK> __host__ __device__ constexpr int st_warp_smem() {
+    return kWvD * st_row<S>() + st_ring<S, T>() * kStFRow + (CHECK ? 2048 : 0);
 }
-template <int S, int T> __host__ __device__ constexpr int st_smem() { return st_nw<T>() * st_warp_smem<S, T>(); }
+template <int S, int T, bool CHECK> __host__ __device__ constexpr int st_smem() {
+    return kStNW * st_warp_smem<S, T, CHECK>();
+}
 
 template <int B>
 __device__ __forceinline__ void copy_async(uint32_t dst, const void* src) {
@@ -1080,7 +1172,7 @@ __device__ __forceinline__ pair_t opaque(pair_t p, uint32_t a) {
 // OX: output columns of a strip (at most st_ox).
 template <int S, bool GEN, int T, bool CHECK, int OX = st_ox<S, T>()>
 __device__ __forceinline__ void strip_walk(const StepParams& a, const PairCoef& ca, uint32_t sm, int strip, int y0,
-                                           int rows, ResAcc<S>& acc) {
+                                           int rows, ResAcc2& acc) {
     static_assert(OX % 2 == 0 && OX <= st_ox<S, T>(), "pairs, within the slots");
     constexpr int LAG = st_lag<S>(), H = st_halo<S, T>(), HL = st_left<S, T>(),
                   LA = st_la<S>(), R = st_ring<S, T>(), ROW = st_row<S>();
@@ -1104,6 +1196,7 @@ __device__ __forceinline__ void strip_walk(const StepParams& a, const PairCoef& 
     const int64_t n = a.plane;
     const int nit = rows + 2 * H;
     const uint32_t frc = sm + kWvD * ROW;                   // force ring
+    const uint32_t snp = frc + R * kStFRow + lane * 32;      // snapshot entries of two rows (CHECK)
     const uint32_t own = (uint32_t)(xs - xa0);               // the lane's first column within a row
     // Copies of a row: 16-byte chunks, chunk q = lane + 32 m (FP32: 18 per
     // plane, eight populations, then the force; FP16S: 9 per plane, eight
@@ -1157,6 +1250,10 @@ __device__ __forceinline__ void strip_walk(const StepParams& a, const PairCoef& 
     // image, 0 without one); one(dx, k) stores column k of the pair at the
     // pair's place + dx.
     auto image = [&](bool own, int x) { return !own ? 0 : (x < kGhost ? nx : (x >= nx - kGhost ? -nx : 0)); };
+    if (CHECK) {
+        acc.own0 = ok;
+        acc.own1 = two;
+    }
     const int off0 = image(ok, xs), off1 = image(two, xs + 1);
     const bool edge = __any_sync(0xffffffffu, off0 != 0 || off1 != 0 || ok != two);
     auto images = [&](auto&& one) {
@@ -1169,12 +1266,17 @@ __device__ __forceinline__ void strip_walk(const StepParams& a, const PairCoef& 
     auto iter = [&](int i, auto k_c) {
         constexpr int K = decltype(k_c)::value;
         pair_t f[8];
-        ResSnap<S> sn0{}, sn1{};
-        if (CHECK && i >= 2 * H && ok) {
-            sn0 = snap_load<S>(a, n, (int64_t)so);
-            sn1 = snap_load<S>(a, n, (int64_t)so + 1);
-        }
         __syncwarp();                             // every lane is done with the rows this copy replaces
+        if (CHECK && ok && i + 1 >= 2 * H && i + 1 < nit) {
+            // snapshot entries of the next output row, in this row's group of
+            // copies (the entry after an odd lattice's last column is in the plane,
+            // too): as loads into registers the assembler moved them down to
+            // their use
+            const float2* sp = static_cast<const float2*>(a.snap) + (i >= 2 * H ? so + pitch : so);
+            const uint32_t d = snp + ((i + 1) & 1) * 1024;
+            copy_async<16>(d, sp);
+            copy_async<16>(d + 16, sp + n);
+        }
         copy_row(i + AHEAD);                      // (rows past the last are copied too: any row is in range)
         asm volatile("cp.async.wait_group %0;" ::"n"(LA) : "memory");
         __syncwarp();                             // the rows of this iteration have arrived for every lane
@@ -1273,14 +1375,25 @@ __device__ __forceinline__ void strip_walk(const StepParams& a, const PairCoef& 
             }
             // level T: the output row
             pair_t fs[8];
-            if (CHECK && ok) {
-                float fl[8], fh[8], gxl, gxh, gyl, gyh;
-#pragma unroll
-                for (int p = 0; p < 8; ++p) unpk(f[p], fl[p], fh[p]);
-                unpk(gx, gxl, gxh);
-                unpk(gy, gyl, gyh);
-                check_node<S>(a, n, (int64_t)so, acc, sn0, fl, gxl, gyl, 0.0f, 0.0f);
-                if (xs + 1 < nx) check_node<S>(a, n, (int64_t)so + 1, acc, sn1, fh, gxh, gyh, 0.0f, 0.0f);
+            if (CHECK) {
+                ResSnap<S> sn0, sn1;
+                pair_t e0, e1;
+                lds_pairs(snp + (i & 1) * 1024, e0, e1);
+                unpk(e0, sn0.u.x, sn0.u.y);
+                unpk(e1, sn1.u.x, sn1.u.y);
+                lds_pairs(snp + (i & 1) * 1024 + 16, e0, e1);
+                unpk(e0, sn0.v.x, sn0.v.y);
+                unpk(e1, sn1.v.x, sn1.v.y);
+                check_pair<S>(acc, sn0, sn1, f, gx, gy, [&](float2 u0, float2 v0, float2 u1, float2 v1) {
+                    float2* sp = static_cast<float2*>(a.snap) + so;
+                    if (two) {
+                        *reinterpret_cast<float4*>(sp) = make_float4(u0.x, u0.y, u1.x, u1.y);
+                        *reinterpret_cast<float4*>(sp + n) = make_float4(v0.x, v0.y, v1.x, v1.y);
+                    } else if (ok) {
+                        sp[0] = u0;
+                        sp[n] = v0;
+                    }
+                });
             }
             if constexpr (S == S_F32) {
                 Pop2<!GEN>(m, c).all(c, fs);
@@ -1352,19 +1465,19 @@ __device__ __forceinline__ void strip_walk(const StepParams& a, const PairCoef& 
 }
 
 template <int S, bool GEN, int T, bool CHECK>
-__global__ void __launch_bounds__(32 * st_nw<T>(), st_minb<T>())
+__global__ void __launch_bounds__(32 * kStNW, 3)
 k_strip(const StepParams a, const PairCoef c, int seg, int nstrips, int items) {
     extern __shared__ float4 st_mem[];
     const int warp = threadIdx.x >> 5;
-    const int item = (int)blockIdx.x * st_nw<T>() + warp;
+    const int item = (int)blockIdx.x * kStNW + warp;
     after_predecessor();
-    ResAcc<S> acc;
+    ResAcc2 acc;
     if (item < items) {
         const int strip = item % nstrips, y0 = (item / nstrips) * seg;
-        const uint32_t sm = (uint32_t)__cvta_generic_to_shared(st_mem) + warp * st_warp_smem<S, T>();
+        const uint32_t sm = (uint32_t)__cvta_generic_to_shared(st_mem) + warp * st_warp_smem<S, T, CHECK>();
         strip_walk<S, GEN, T, CHECK>(a, c, sm, strip, y0, min(seg, a.ny - y0), acc);
     }
-    if (CHECK) residual_reduce<S>(a, acc);
+    if (CHECK) residual_reduce(a, acc);
 }
 
 // ---------------------------------------------------------------------------
@@ -1462,9 +1575,24 @@ k_tile(const StepParams a, const PairCoef ca, int T, int ntx) {
     __syncthreads();
     const int s0 = 2 * lane;
     const bool ok0 = s0 >= H && s0 < kStSlots - H && xs < nx, ok1 = s0 + 1 >= H && s0 + 1 < kStSlots - H && xs + 1 < nx;
-    ResAcc<S_F32> acc;
+    ResAcc2 acc;
+    acc.own0 = ok0;
+    acc.own1 = ok1;
+    // the check's snapshot entries of the coming row, loaded one row ahead
+    ResSnap<S_F32> sn[2];
+    auto owned_row = [&](int r) {
+        const int q = warp * RR + r;
+        return q >= H && q < nw * RR - H && ys + r < ny;
+    };
+    auto snap_row = [&](int r) {
+        if (!owned_row(r)) return;
+        const int64_t idx = (int64_t)(ys + r) * a.pitch + xs;
+        if (ok0) sn[0] = snap_load<S_F32>(a, pl, idx);
+        if (ok1) sn[1] = snap_load<S_F32>(a, pl, idx + 1);
+    };
     for (int t = 0; t < T; ++t) {
         const bool last = t == T - 1;
+        if (CHECK && last) snap_row(0);
         const uint32_t par = (t & 1) ? par_bytes : 0;
         const uint32_t above = slot(warp - 1) + par, below = slot(warp + 1) + par + 768;
         pair_t u2 = lds_pair(above), u5 = lds_pair(above + 256), nu6 = lds_pair(above + 512);
@@ -1484,8 +1612,14 @@ k_tile(const StepParams a, const PairCoef ca, int T, int ntx) {
             const Post2 m = collide2<GEN>(moments2(o, c), gx[r], gy[r], c);
             const Pop2<!GEN> w(m, c);
             if (last) {
-                const int y = ys + r, q = warp * RR + r;
-                if (q >= H && q < nw * RR - H && y < ny) {
+                ResSnap<S_F32> now[2];
+                if (CHECK) {
+                    now[0] = sn[0];
+                    now[1] = sn[1];
+                    if (r + 1 < RR) snap_row(r + 1);
+                }
+                if (owned_row(r)) {
+                    const int y = ys + r;
                     pair_t fs[8];
                     w.all(c, fs);
                     const int64_t idx = (int64_t)y * a.pitch + xs;
@@ -1499,16 +1633,18 @@ k_tile(const StepParams a, const PairCoef ca, int T, int ntx) {
                     }
                     if (CHECK) {
                         const pair_t f[8] = {s[r].m1, u2, s[r].m3, d4, u5, neg2(nu6), d7, neg2(nd8)};
-                        float fl[8], fh[8], gxl, gxh, gyl, gyh;
-#pragma unroll
-                        for (int p = 0; p < 8; ++p) unpk(f[p], fl[p], fh[p]);
-                        unpk(gx[r], gxl, gxh);
-                        unpk(gy[r], gyl, gyh);
-                        if (ok0)
-                            check_node<S_F32>(a, pl, idx, acc, snap_load<S_F32>(a, pl, idx), fl, gxl, gyl, 0.0f, 0.0f);
-                        if (ok1)
-                            check_node<S_F32>(a, pl, idx + 1, acc, snap_load<S_F32>(a, pl, idx + 1), fh, gxh, gyh,
-                                              0.0f, 0.0f);
+                        check_pair<S_F32>(acc, now[0], now[1], f, gx[r], gy[r],
+                                          [&](float2 u0, float2 v0, float2 u1, float2 v1) {
+                                              float2* sp = static_cast<float2*>(a.snap) + idx;
+                                              if (ok0) {
+                                                  sp[0] = u0;
+                                                  sp[pl] = v0;
+                                              }
+                                              if (ok1) {
+                                                  sp[1] = u1;
+                                                  sp[pl + 1] = v1;
+                                              }
+                                          });
                     }
                 }
             }
@@ -1530,7 +1666,7 @@ k_tile(const StepParams a, const PairCoef ca, int T, int ntx) {
         put(next + 768, s[0].d4, s[0].d7, s[0].nd8);
         __syncthreads();
     }
-    if (CHECK) residual_reduce<S_F32>(a, acc);
+    if (CHECK) residual_reduce(a, acc);
 }
 
 // Destinations of the five solution fields u_x, u_y, sigma_xx, sigma_yy,
@@ -1551,12 +1687,25 @@ inline FieldOut field_planes(double* out, int64_t n) {
     return o;
 }
 
+// x 2^(e - 896) in FP64 (e in [836, 956]) by integer operations: the conversion
+// instructions run on the FP64 pipe.  A subnormal, infinity or NaN sets odd (and
+// gives no meaningful value).
+__device__ __forceinline__ double to_double(float x, int e, bool& odd) {
+    const uint32_t b = __float_as_uint(x), m = b & 0x7fffffffu;
+    odd |= m != 0 && m - 0x00800000u >= 0x7f000000u;
+    const uint32_t hi = (b & 0x80000000u) | (m ? (m >> 3) + ((uint32_t)e << 20) : 0u);
+    return __hiloint2double((int)hi, (int)(m << 29));
+}
+// log2 of a power of two.
+__device__ __forceinline__ int ilogb2(float p) { return (int)(__float_as_uint(p) >> 23) - 127; }
+
 // Solution fields of the current state (Table 2, Eq. compute_bared), FP64.
 template <int S>
 __global__ void __launch_bounds__(kThreads)
 k_fields(const StepParams a, const Coef<double> c, typename StoreT<S>::T theta, const FieldOut out) {
     using T = typename StoreT<S>::T;
     using G = typename StoreT<S>::G;
+    after_predecessor();
     const int nx = a.nx, ny = a.ny;
     const int y = blockIdx.y * BY + threadIdx.y;
     const int x = blockIdx.x * 32 + threadIdx.x;
@@ -1567,6 +1716,10 @@ k_fields(const StepParams a, const Coef<double> c, typename StoreT<S>::T theta, 
     gather<S>(a, r0, rm, rp, x, wrap_dec(x, nx), wrap_inc(x, nx), f, theta);
     const int64_t idx = r0 + x;
     const G gxs = static_cast<const G*>(a.gx)[idx], gys = static_cast<const G*>(a.gy)[idx];
+    // FP64 work is what bounds the recovery on GB300 (64 cycles of a scheduler
+    // per warp instruction): nine FP64 instructions per node.  cs, cd: the
+    // factors of Eq. compute_bared with Table 2's -1/2.
+    const double cs = -0.5 * c.bs, cd = -0.5 * c.bd;
     double u, v, m11, ms, md;
     if constexpr (S == S_F64) {
         const Mom<double> m = moments(f);
@@ -1576,13 +1729,15 @@ k_fields(const StepParams a, const Coef<double> c, typename StoreT<S>::T theta, 
         ms = m.ms;
         md = m.md;
     } else {
-        // FP32 populations: the moments as exact FP32 pairs (TwoSum), each
-        // joined in FP64 once -- GB300 issues FP64 at a small fraction of the
-        // FP32 rate, and this keeps the recovery's FP64 work to the joins and
-        // the products of Eq. compute_bared
+        // FP32 populations: the moments as exact FP32 pairs (TwoSum), converted
+        // by integer operations (out of the state's scaled units on the way,
+        // FP16S) and joined in FP64 once
+        const int e = S == S_F16S ? 896 - ilogb2(a.hscale) : 896;
+        bool odd = false;
+        auto join = [&](float h, float l) { return to_double(h, e, odd) + to_double(l, e, odd); };
         const float4 w = exact_displacement(f, gxs, gys);
-        u = (double)w.x + (double)w.y;
-        v = (double)w.z + (double)w.w;
+        u = join(w.x, w.y);
+        v = join(w.z, w.w);
         float ep, eq, e13, e24, e11, e22, ed, et, es;
         const float p = two_sum(f[4], f[6], ep), q = two_sum(f[5], f[7], eq);
         const float h11 = two_sum(p, -q, e11), h22 = two_sum(p, q, e22);
@@ -1590,18 +1745,27 @@ k_fields(const StepParams a, const Coef<double> c, typename StoreT<S>::T theta, 
         const float hd = two_sum(s13, -s24, ed), ht = two_sum(s13, s24, et);
         const float l22 = __fadd_rn(e22, __fadd_rn(ep, eq));
         const float hs = two_sum(ht, 2.0f * h22, es);   // m_s = (f1+f3) + (f2+f4) + 2 m_22
-        m11 = (double)h11 + (double)__fadd_rn(e11, __fsub_rn(ep, eq));
-        md = (double)hd + (double)__fadd_rn(ed, __fsub_rn(e13, e24));
-        ms = (double)hs + (double)__fadd_rn(__fadd_rn(es, __fadd_rn(et, __fadd_rn(e13, e24))), 2.0f * l22);
+        const float l11 = __fadd_rn(e11, __fsub_rn(ep, eq)), ld = __fadd_rn(ed, __fsub_rn(e13, e24));
+        const float ls = __fadd_rn(__fadd_rn(es, __fadd_rn(et, __fadd_rn(e13, e24))), 2.0f * l22);
+        m11 = join(h11, l11);
+        md = join(hd, ld);
+        ms = join(hs, ls);
+        if (odd) {
+            const double s = S == S_F16S ? (double)a.hinv : 1.0;
+            u = ((double)w.x + (double)w.y) * s;
+            v = ((double)w.z + (double)w.w) * s;
+            m11 = ((double)h11 + (double)l11) * s;
+            md = ((double)hd + (double)ld) * s;
+            ms = ((double)hs + (double)ls) * s;
+        }
     }
-    // (FP16S: back from the state's scaled units, a power of two)
-    const double un = S == S_F16S ? (double)a.hinv : 1.0;
-    const double mb11 = c.b11 * m11, mbs = c.bs * ms, mbd = c.bd * md;
+    // (un: the joins return the fields' own unit)
+    const double t = cd * md, mb11 = c.b11 * m11, un = 1.0;
     const int64_t o = out.tr ? (int64_t)x * ny + y : (int64_t)y * nx + x;
-    if (out.p[0]) out.p[0][o] = u * un;
-    if (out.p[1]) out.p[1][o] = v * un;
-    if (out.p[2]) out.p[2][o] = -0.5 * (mbs + mbd) * un;
-    if (out.p[3]) out.p[3][o] = -0.5 * (mbs - mbd) * un;
+    if (out.p[0]) out.p[0][o] = u;
+    if (out.p[1]) out.p[1][o] = v;
+    if (out.p[2]) out.p[2][o] = fma(cs, ms, t);
+    if (out.p[3]) out.p[3][o] = fma(cs, ms, -t);
     if (out.p[4]) out.p[4][o] = -mb11 * un;
 }
 
@@ -1852,34 +2016,34 @@ struct StripShape {
 };
 
 // Rows per segment of a launch of T steps that takes the fewest cycles on
-// `nsm` multiprocessors of `warps` resident warps each.  A warp's iteration
-// costs about 70 + 115 w cycles per level with w warps on its scheduler, and a
-// segment of seg rows takes seg + 2 (halo rows) iterations, so the best
-// segments are those whose warps just fill a whole number of waves
-// (4096 x 3000, T = 5: 213 to 229 us with 32 to 256 rows chosen by halving,
-// 164 us with the 125 rows that fill one wave).  rows > 0 fixes the segment.
-inline StripShape strip_shape(int dtype, int T, int nx, int ny, int nsm, int warps, int rows) {
+// `nsm` multiprocessors of `warps` resident warps each, and its cost.  Fitted on
+// GB300 (300 x 2000 to 16384^2, T = 2 .. 6; within 10 %): a warp's iteration costs
+// 70 + 115 w cycles per level with w warps on its scheduler, and a segment of seg
+// rows takes seg + 2 (halo rows) iterations, so the best segments are those whose
+// warps just fill a whole number of waves (4096 x 3000, T = 5: 213 to 229 us with
+// 32 to 256 rows chosen by halving, 155 us with the 125 rows that fill one
+// wave); a checked row costs 2300 cycles more; the state moves at 3.0 kB per
+// cycle (6.2 TB/s).  rows > 0 fixes the segment.
+inline StripShape strip_shape(int dtype, int T, bool check, int nx, int ny, int nsm, int warps, int rows) {
     const int64_t ns = strip_count(dtype, T, nx);
     const int halo = T - 1 + (dtype == S_F16S ? 1 : 0);
+    // (short launches wait longer for their rows)
+    const double slow = T == 2 ? 1.6 : (T == 3 ? 1.3 : (T == 4 ? 1.08 : 1.0));
+    const double mem = (double)nx * ny * ((dtype == S_F16S ? 56 : 72) + (check ? 32 : 0)) / 3040.0;
     StripShape best;
     auto consider = [&](int64_t seg) {
         if (seg < 1) seg = 1;
         if (seg > ny) seg = ny;
         const int64_t items = ns * ((ny + seg - 1) / seg), slots = (int64_t)nsm * warps;
-        double cost = 0.0;
-        for (int64_t left = items; left > 0; left -= slots) {
-            const int64_t now = left < slots ? left : slots;
-            const double w = (double)((now + 4 * nsm - 1) / (4 * nsm));
-            const double one = (double)(seg + 2 * halo) * (T * (70.0 + 115.0 * w) + 150.0);
-            if (left > 8 * slots) {                // many waves: they run into one another
-                const double waves = (double)(left - 4 * slots) / (double)slots;
-                cost += waves * one;
-                left = 4 * slots + slots;
-                continue;
-            }
-            cost += one;
-        }
-        cost += 3000.0;                            // the launch itself
+        auto wave = [&](double w) {
+            return slow * (double)(seg + 2 * halo) * (T * (70.0 + 115.0 * w) + 150.0) + (check ? 2300.0 * seg : 0.0);
+        };
+        // full waves (many run into one another), then what is left
+        const int64_t full = (items - 1) / slots, rest = items - full * slots;
+        const double part = full < 8 ? wave((double)((rest + 4 * nsm - 1) / (4 * nsm)))
+                                     : wave(warps / 4.0) * (double)rest / (double)slots;
+        const double busy = full * wave(warps / 4.0) + part;
+        const double cost = 3000.0 + pow(pow(busy, 6.0) + pow(mem, 6.0), 1.0 / 6.0);
         if (best.seg == 0 || cost < best.cost) {
             best.T = T;
             best.seg = (int)seg;
@@ -1984,8 +2148,8 @@ inline TileShape tile_shape(int nx, int ny, int nsm) {
 cudaError_t tile_f32(const StepParams& a, const Coef<float>& c, bool gen, const TileShape& t, bool check,
                      cudaStream_t st);
 
-// T fused steps on the wavefront schedule (k_strip; FP32: T = 2 .. 7, FP16S:
-// T = 3, 4; check: T = 4 with the residual on the last step), segments of seg
+// T fused steps on the wavefront schedule (k_strip; FP32: T = 2 .. 6, FP16S:
+// T = 3, 4; check: T = 4, FP32 also 5, with the residual on the last step), segments of seg
 // rows.  warps non-null: only the resident warps per multiprocessor of that
 // kernel.  Defined with each storage type's kernels.
 cudaError_t strip_f32(const StepParams& a, const Coef<float>& c, bool gen, int T, bool check, int seg, int* warps,

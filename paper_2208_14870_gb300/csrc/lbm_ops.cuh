@@ -86,7 +86,7 @@ static cudaError_t launch_strip_k(const StepParams& a, const Coef<float>& c, int
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     const auto kernel = k_strip<S, GEN, T, CHECK>;
-    constexpr int NW = st_nw<T>(), SM = st_smem<S, T>();
+    constexpr int NW = kStNW, SM = st_smem<S, T, CHECK>();
     {
         std::lock_guard<std::mutex> lock(mu);
         if (!resident[dev]) {
@@ -170,8 +170,7 @@ cudaError_t Ops<S>::step(const StepParams& a, const Coef<T>& c, int V, bool gen,
 template <int S>
 cudaError_t Ops<S>::fields(const StepParams& a, const Coef<double>& c, T theta, const FieldOut& out,
                            cudaStream_t st) {
-    k_fields<S><<<step_grid(a.nx, a.ny, 1), dim3(32, BY), 0, st>>>(a, c, theta, out);
-    return cudaGetLastError();
+    return launch_after(k_fields<S>, step_grid(a.nx, a.ny, 1), dim3(32, BY), 0, st, a, c, theta, out);
 }
 
 template <int S>

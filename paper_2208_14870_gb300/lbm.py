@@ -61,6 +61,7 @@ _SIGS = {
     "lbm_get_host_transfer": (_c.c_int, [_vp, _c.POINTER(_c.c_int)]),
     "lbm_set_steps_per_launch": (_c.c_int, [_vp, _c.c_int]),
     "lbm_get_steps_per_launch": (_c.c_int, [_vp, _c.POINTER(_c.c_int)]),
+    "lbm_get_launches": (_c.c_int, [_vp, _c.POINTER(_i64)]),
     "lbm_get_launch_steps": (_c.c_int, [_vp, _c.POINTER(_c.c_int)]),
     "lbm_set_wavefront": (_c.c_int, [_vp, _c.c_int]),
     "lbm_get_wavefront": (_c.c_int, [_vp, _c.POINTER(_c.c_int)]),
@@ -174,6 +175,12 @@ def lbm_get_steps_per_launch(ctx: int) -> int:
     k = _c.c_int()
     _check(_lib.lbm_get_steps_per_launch(ctx, _c.byref(k)), "lbm_get_steps_per_launch")
     return k.value
+
+
+def lbm_get_launches(ctx: int) -> int:
+    n = _i64()
+    _check(_lib.lbm_get_launches(ctx, _c.byref(n)), "lbm_get_launches")
+    return n.value
 
 
 def lbm_get_launch_steps(ctx: int) -> int:

@@ -1,4 +1,4 @@
-"""Strip kernel (two to seven steps per launch, one warp per strip of 64 slot
+"""Strip kernel (two to six steps per launch, one warp per strip of 64 slot
 columns) against one step per launch, at the sizes where its copies, halos
 and pairs can go wrong: widths that are no multiple of a 16-byte chunk (every
 remainder of eight), odd widths, whole numbers of strips and one column more,
@@ -55,6 +55,44 @@ def test_f32_general_rates_and_checks(nx, ny):
         assert np.array_equal(_state(nx, ny, "f32", 4, -1, steps, **kw), ref), steps
     ref = _state(nx, ny, "f32", 1, 0, 37, **kw)
     assert np.array_equal(_state(nx, ny, "f32", 4, -1, 37, check_every=9, **kw), ref)
+
+
+# Checked launches of four and of five steps (windows of five steps end in one
+# launch), with the residual of the last check.
+@pytest.mark.parametrize("nx,ny", [(256, 8), (257, 9), (364, 40), (261, 8)])
+@pytest.mark.parametrize("every", [4, 5, 9, 10])
+def test_f32_checked_launches(nx, ny, every):
+    lam, mu = W.lame_2d(1.0, 0.3)
+    gx, gy = np.random.RandomState(nx + ny).standard_normal((2, ny, nx)) / max(nx, ny) ** 2
+    res = []
+    for spl, wave in ((1, 0), (4, -1), (4, 3)):
+        with Lattice(nx, ny, lam, mu, "f32") as lat:
+            lat.steps_per_launch, lat.wavefront = spl, wave
+            lat.set_force(gx, gy)
+            r = lat.iterate_checked(4 * every, every)
+            res.append((lat.populations(), r))
+    for pops, r in res[1:]:
+        assert np.array_equal(pops, res[0][0])
+        assert np.allclose(r, res[0][1], rtol=1e-12, atol=0.0)
+
+
+# Recovery of the fields from FP32 states: subnormal populations convert like
+# their multiples by a power of two, and an overflow stays in its own node.
+@pytest.mark.parametrize("nx,ny", [(5, 3), (33, 9), (256, 8)])
+def test_f32_fields_of_subnormal_and_overflowing_states(nx, ny):
+    lam, mu = W.lame_2d(1.0, 0.3)
+    k = np.random.RandomState(nx).randint(-5, 6, (8, ny, nx)).astype(np.float64)
+    got = []
+    with Lattice(nx, ny, lam, mu, "f32") as lat:
+        for e in (-149, -100):
+            lat.set_populations(k * 2.0 ** e)
+            got.append(lat.fields())
+        k[1, 1, 2] = k[3, 1, 2] = 3e38
+        lat.set_populations(k)
+        bad = lat.fields()
+    assert np.array_equal(got[0] * 2.0 ** 49, got[1])
+    at = ~np.isfinite(bad).all(axis=0)
+    assert at[1, 2] and at.sum() == 1
 
 
 @pytest.mark.parametrize("nx,ny", SIZES)
