@@ -46,14 +46,6 @@ FALLBACK_HBM_GBS = 6800.0
 WAVE_MIN_NX = 256
 BYTES_PER_LAUNCH_NODE = {"f64": 8 * 8 * 2 + 2 * 8, "f32": 8 * 4 * 2 + 2 * 4, "f16s": (8 * 2 + 2 * 4) * 2 + 2 * 4}
 FORCE_SEED = 0x2208_14870
-# FP64 storage runs its collision on the FP64 pipe: 34 FP64 instructions per
-# lattice update (collide_f64: 15 additions, 3 products, 16 fused
-# multiply-adds per node), i.e. 50 flops.
-# Every FP64 instruction takes one slot of the pipe, whose nominal rate on
-# GB300 is 1.25 TFLOP/s counting an FMA as 2 flops, i.e. 625 G instructions/s.
-FP64_INSTR_PER_LUP = 34
-FP64_FLOPS_PER_LUP = 50
-FP64_PEAK_GINST = 625.0
 # DRAM traffic per stream-collide launch from one ncu capture, keyed by dtype,
 # steps per launch and schedule, with the hash of the kernel code it was taken
 # on (null in the bench line once the code changes; comments do not count).
@@ -452,16 +444,6 @@ def time_variant(args, dtype, gx_d, gy_d, torch, P, nsteps, nwarm, events=True, 
             "dom_ms": dom_ms, "dom_launches": dom_launches, "big": big, "wave": wave_on}
 
 
-def fp64_peak(P):
-    """The FP64 roofline denominator: the device's measured FP64 FMA rate
-    (lbm_fp64_fma_rate), else the nominal rate."""
-    try:
-        return float(P.lbm_fp64_fma_rate()), ("measured: lbm_fp64_fma_rate (8 independent dependent-DFMA "
-                                              "chains per thread, every SM full, CUDA events)")
-    except Exception as e:  # noqa: BLE001
-        return FP64_PEAK_GINST, "nominal GB300 FP64 rate (1.25 TFLOP/s with FMA = 2 flops); measurement failed: %s" % e
-
-
 def dominant_block(check_every, spl, wave=False):
     """(steps, k): the first steps of a residual window, which the library
     runs as whole plain launches of k steps each, k the longest launch of the
@@ -543,15 +525,9 @@ def run_ours(args, ws, rank, local):
                 "achieved_gbs": b / pl / 1e9, "frac_of_measured_hbm": b / pl / 1e9 / peak,
                 "bytes_per_lup": BYTES_PER_LAUNCH_NODE[dt] / r["big"]}
             if dt == "f64":
-                # FP64 is bound by the FP64 pipe, not by HBM: FP64 instructions
-                # per second over the device's measured FP64 FMA rate
-                gi = FP64_INSTR_PER_LUP * n * n / pl / 1e9
-                fpk, fkind = fp64_peak(P)
+                # (the collision runs in integers, so HBM bounds FP64 as well)
                 variants[name]["roofline"] = {
-                    "bound": "alu", "achieved": gi, "peak": fpk, "unit": "G FP64 instr/s",
-                    "frac": gi / fpk, "peak_kind": fkind,
-                    "fp64_instructions_per_lup": FP64_INSTR_PER_LUP, "flops_per_lup": FP64_FLOPS_PER_LUP,
-                    "achieved_tflops": FP64_FLOPS_PER_LUP * n * n / pl / 1e12}
+                    "bound": "hbm", "achieved": b / pl / 1e9, "peak": peak, "unit": "GB/s", "frac": b / pl / 1e9 / peak}
 
     e2e = None
     if not args.no_e2e:

@@ -135,8 +135,6 @@ StepParams params(const lbm_ctx* c, int src) {
 template <typename T>
 Coef<T> coef(lbm_rates r) {
     Coef<T> c;
-    // (a multiple of 2^-53, see collide_f64; no change to a theta rounded to FP32)
-    if (sizeof(T) == 8 && r.theta >= kThetaExact) r.theta = theta_f64(r.theta);
     // quarter form (exact scaling by 1/4 before the rounding to T)
     c.q11 = T(0.25 * (1.0 - r.w11));
     c.qs = T(0.25 * (1.0 - r.ws));
@@ -151,10 +149,7 @@ Coef<T> coef(lbm_rates r) {
     c.b11 = T(1.0 - 0.5 * r.w11);
     c.bs = T(1.0 - 0.5 * r.ws);
     c.bd = T(1.0 - 0.5 * r.wd);
-    c.qsd = T(0.25 * (1.0 - r.ws) + 0.25 * (1.0 - r.wd));
-    c.qds = T(0.25 * (1.0 - r.ws) - 0.25 * (1.0 - r.wd));
-    c.qs2 = T(0.5 * (1.0 - r.ws));
-    c.twoctheta = T(2.0 * (1.0 - r.theta));
+    set_factors(c);
     return c;
 }
 
@@ -169,10 +164,10 @@ int ensure_partials(lbm_ctx* c, int64_t sets);
 
 // T steps of FP64 storage (check: the last one is the residual-check step).
 cudaError_t launch_tile64(lbm_ctx* c, int T, bool check) {
-    Tile64Shape t = c->tile64;
-    t.T = T;
-    cudaError_t e = tile_f64(params(c, c->cur), coef<double>(c->rates), c->gen, t, check, c->nblocks, c->stream);
-    if (e == cudaSuccess && check) e = finish_residual_launch(c, std::min(tile64_count(t, c->nx, c->ny), c->nblocks));
+    const Tile64Shape t = tile64(T, c->tile64.bx, c->tile64.by);
+    int64_t blocks = 0;
+    cudaError_t e = tile_f64(params(c, c->cur), coef<double>(c->rates), c->gen, t, check, &blocks, c->stream);
+    if (e == cudaSuccess && check) e = finish_residual_launch(c, blocks);
     if (e == cudaSuccess) {
         c->cur ^= 1;
         ++c->launches;
@@ -737,7 +732,6 @@ int lbm_create_ex(int nx, int ny, double lambda, double mu, int dtype, const lbm
     c->rates.w22 = 1.0 / (tau22 + 0.5);
     c->rates.theta = theta;
     c->gen = !(c->rates.w12 == 1.0 && c->rates.w22 == 1.0);
-    if (dtype == LBM_F64 && theta < kThetaExact) c->gen = true;   // collide_f64 needs 1 - theta exact
     if (dtype == LBM_F64) {
         c->V = 1;
         c->tile64 = tile64_shape(nx, ny, c->nsm > 0 ? c->nsm : 1);
@@ -746,7 +740,12 @@ int lbm_create_ex(int nx, int ny, double lambda, double mu, int dtype, const lbm
         c->V = nx >= 32 * vmax ? vmax : 1;
     }
     // residual-check grids: one block per tile up to kMaxCheckBlocks
-    c->nblocks = std::min(dtype == LBM_F64 ? tile64_count(c->tile64, nx, ny) : step_tiles(nx, ny, c->V), kMaxCheckBlocks);
+    c->nblocks = std::min(step_tiles(nx, ny, c->V), kMaxCheckBlocks);
+    if (dtype == LBM_F64)   // the most of the checked launches of 1 .. T steps
+        for (int T = 1; T <= c->tile64.T; ++T) {
+            const dim3 g = tile64_grid(tile64(T, c->tile64.bx, c->tile64.by), nx, ny, kMaxCheckBlocks);
+            c->nblocks = std::max<int64_t>(c->nblocks, (int64_t)g.x * g.y);
+        }
     if (dtype != LBM_F64) {
         c->nblocks2 = std::min(step2_tiles(nx, ny), kMaxCheckBlocks);
         // four steps per launch on the wavefront schedule where it fits, else

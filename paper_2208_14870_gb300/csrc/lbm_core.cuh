@@ -32,6 +32,24 @@ struct Mom {
     T m10, m01, m11, ms, md, m12, m21, m22;
 };
 
+// A factor in [-1/2, 1/2) as a multiple of 2^-64: its upper and lower halves, the
+// lower one without its last bit (step_fixed).
+struct Factor {
+    int hi, lo;
+};
+inline Factor factor(double v) {
+    const int64_t b = llrint(ldexp(v, 64));
+    return {(int)(b >> 32), (int)((uint32_t)b >> 1)};
+}
+// The same constants as factors (FP64 storage); fixed: all of them are in range.
+template <typename T>
+struct CoefFixed {};
+template <>
+struct CoefFixed<double> {
+    Factor k11, ks, kd, kw12t, k12, kw21t, k21, k22;
+    int fixed;
+};
+
 // Per-lattice constants of the collision in compute precision, in the
 // quarter form collide returns (every factor of a second-order moment
 // divided by 4; see collide):
@@ -39,19 +57,22 @@ struct Mom {
 //   qw12t = w12 theta / 4, q12 = (1 - w12)/4, ...          (m^eq_12 = theta mbar_10)
 //   qtheta = theta / 4; theta itself for the FP16-shifted store
 template <typename T>
-struct Coef {
+struct Coef : CoefFixed<T> {
     T q11, qs, qd;
     T qw12t, q12, qw21t, q21, q22;
     T qtheta, theta;
     T b11, bs, bd;   // 1 - w/2 (bared moments, Eq. compute_bared)
-    // collide_f64: q_s + q_d, q_s - q_d, 2 q_s, 2 (1 - theta)
-    T qsd, qds, qs2, twoctheta;
 };
-
-// theta of FP64 storage as a multiple of 2^-53 (within 2^-54 of theta), for
-// theta >= kThetaExact; below that collide_f64 is not used.
-constexpr double kThetaExact = 0.125;
-inline double theta_f64(double theta) { return nearbyint(theta * 9007199254740992.0) / 9007199254740992.0; }
+inline void set_factors(Coef<float>&) {}
+inline void set_factors(Coef<double>& c) {
+    const double q[8] = {c.q11, c.qs, c.qd, c.qw12t, c.q12, c.qw21t, c.q21, c.q22};
+    Factor* k[8] = {&c.k11, &c.ks, &c.kd, &c.kw12t, &c.k12, &c.kw21t, &c.k21, &c.k22};
+    c.fixed = 1;
+    for (int i = 0; i < 8; ++i) {
+        if (fabs(q[i]) < 0.499) *k[i] = factor(q[i]);
+        else c.fixed = 0;
+    }
+}
 
 // Raw moments of eight populations, Eq. moments and Eq. replace_raw, written
 // as a butterfly: with p = f5 + f7, q = f6 + f8, r = f5 - f7, s = f6 - f8,
@@ -181,35 +202,121 @@ __device__ __forceinline__ void collide_populations(const Mom<T>& m, T gx, T gy,
     populations<!GEN>(collide<T, GEN>(m, gx, gy, c, u, v), f);
 }
 
-// The same step of FP64 storage at the standard rates, from the pulled
-// populations.  GB300's FP64 pipe issues two lanes per cycle and SM and is what
-// bounds FP64 storage, so the collision is merged with the back-transformation
-// to 34 FP64 instructions instead of 42:
-//   P, Q = q_s m_s +- q_d m_d = (q_s +- q_d) s13 + (q_s -+ q_d) s24 + 2 q_s m_22,
-//   A = m*_10 - theta u = (1 - theta) u + g_x / 2   (m*_10 = u + g_x / 2),
-//   f5, f7 = X +- theta/4 (u + v), f6, f8 = -X +- theta/4 (v - u), X = q_11 m_11,
-// with s13 = f1 + f3, s24 = f2 + f4.  The first moments of the result are m*_10,
-// m*_01 up to rounding only if the theta of A and the theta / 4 of f5 .. f8 are
-// the same number: theta is a multiple of 2^-53, so that 1 - theta is exact
-// (coef<double>).  Measured at 1500 x 1100: 137 -> 114 us per step.
-__device__ __forceinline__ void collide_f64(const double f[8], double gx, double gy, const Coef<double>& c,
-                                            double& u, double& v, double o[8]) {
-    const double p = f[4] + f[6], q = f[5] + f[7], r = f[4] - f[6], s = f[5] - f[7];
-    const double s13 = f[0] + f[2], s24 = f[1] + f[3];
-    u = fma(0.5, gx, (f[0] - f[2]) + (r - s));
-    v = fma(0.5, gy, (f[1] - f[3]) + (r + s));
-    const double w = c.qs2 * (p + q), X = c.q11 * (p - q);
-    const double P = fma(c.qsd, s13, fma(c.qds, s24, w)), Q = fma(c.qds, s13, fma(c.qsd, s24, w));
-    const double A = fma(c.twoctheta, u, gx), B = fma(c.twoctheta, v, gy);   // 2 (m*_10 - theta u)
-    const double su = u + v, sv = v - u;
-    o[0] = fma(0.25, A, P);
-    o[2] = fma(-0.25, A, P);
-    o[1] = fma(0.25, B, Q);
-    o[3] = fma(-0.25, B, Q);
-    o[4] = fma(c.qtheta, su, X);
-    o[6] = fma(-c.qtheta, su, X);
-    o[5] = fma(c.qtheta, sv, -X);
-    o[7] = fma(-c.qtheta, sv, -X);
+// The same step of FP64 storage.  GB300's FP64 pipe takes 64 cycles of a
+// scheduler per warp instruction, an integer instruction one or two, so the step
+// runs in integers: the node's populations and half forces become multiples of
+// one unit, 2^-58 of the power of two above the largest of them (at least five
+// bits more than FP64 holds of that one), their sums are exact, its five
+// products (eight at general rates) are good to about a unit, and the results
+// are rounded to FP64 once.  No result is off by more than FP64 arithmetic's
+// own rounding of the sums, and the first moments of the result are mbar + g / 2 up
+// to that last rounding.  About 600 integer instructions, two cycles of the ALU
+// for 360 of them, against 34 FP64 ones (2176 cycles): 1500 x 1100 116 -> 44 us
+// per step, 64 x 64 2.05 -> 1.45 us, before the FP64 pipe took some results:
+// three of them with few warps per scheduler (64 x 64: none 1.41 us, two 1.40,
+// three 1.39, five 1.52), four with many (WIDE; 1500 x 1100: none 42.6 us, two
+// 40.8, three 39.6, four and five 38.7, six 44.0), where the signs go to the FMA
+// pipe as well (38.7 against 40.5; with few warps 1.41 against 1.34).
+// Nodes of infinities, NaN or values near the ends of the exponent range, and
+// rates with a factor of 1/2 or more, take FP64 arithmetic.
+// m (below 2^63) with the sign of the word w.  FMA: most of the work on the FMA pipe (a multiplication by the sign) instead
+// of the ALU, which bounds the step where many warps share a scheduler; slower
+// where one warp runs alone.
+template <bool FMA>
+__device__ __forceinline__ int64_t signed_as(uint64_t m, int w) {
+    const int t = w >> 31;
+    if (!FMA) return ((int64_t)m ^ (int64_t)t) - (int64_t)t;
+    const uint32_t s = (uint32_t)(t | 1), ml = (uint32_t)m, mh = (uint32_t)(m >> 32);
+    uint32_t lo, hi;
+    // (-m = m (2^32 - 1) - m 2^32 in 64 bits)
+    asm("{\n\t.reg .b64 r;\n\tmul.wide.u32 r, %2, %4;\n\tmov.b64 {%0, %1}, r;\n\tmad.lo.s32 %1, %3, %4, %1;\n\t"
+        "mad.lo.s32 %1, %2, %5, %1;\n\t}" : "=&r"(lo), "=&r"(hi) : "r"(ml), "r"(mh), "r"(s), "r"(t));
+    return (int64_t)((uint64_t)hi << 32 | lo);
+}
+// x as a multiple of the unit; h: one more halving.
+template <bool FMA>
+__device__ __forceinline__ int64_t to_fixed(double x, uint32_t e, int h) {
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const uint32_t d = (e - (hi & 0x7ff00000u)) >> 20;
+    uint64_t m = ((uint64_t)((hi & 0x000fffffu) | 0x00100000u) << 32 | lo) << (5 - h);
+    asm("shr.u64 %0, %0, %1;" : "+l"(m) : "r"(d));                 // (64 and more: zero)
+    return signed_as<FMA>(m, (int)hi);
+}
+// v units (|v| < 2^63), rounded to FP64 (ties to even).
+template <bool FMA>
+__device__ __forceinline__ double from_fixed(int64_t v, uint32_t e) {
+    const int vh = (int)(v >> 32);
+    const uint64_t a = (uint64_t)signed_as<FMA>((uint64_t)v, vh);
+    const uint32_t ah = (uint32_t)(a >> 32), x = ah ? ah : (uint32_t)a;
+    int t;                                                         // the highest set bit, 0 .. 62 (-1: none)
+    asm("bfind.u32 %0, %1;" : "=r"(t) : "r"(x));
+    if (ah) t += 32;
+    const uint64_t b = a << (62 - t), m = (b + 511 + (((uint32_t)b >> 10) & 1)) >> 10;   // [2^52, 2^53], or 0
+    uint32_t hi = (uint32_t)(m >> 32);
+    if (x) hi += ((uint32_t)t << 20) + (e - (58u << 20));
+    return __hiloint2double((int)(hi | (vh & 0x80000000)), (int)(uint32_t)m);
+}
+// The same by two FP64 additions: v's upper word above 2^84 + 2^63
+// units, its lower word above 2^52; the first difference is exact.
+__device__ __forceinline__ double from_fixed_fp64(int64_t v, uint32_t e) {
+    const int k = (int)(e + (27u << 20));
+    const double d1 = __hiloint2double(k, (int)((uint32_t)(v >> 32) ^ 0x80000000u));
+    const double d2 = __hiloint2double((int)(e - (5u << 20)), (int)(uint32_t)v);
+    return (d1 - __hiloint2double(k, (int)0x80100000u)) + d2;      // 2^84 + 2^63 + 2^52
+}
+// a times a factor, within about a unit (|a| < 2^62).
+__device__ __forceinline__ int64_t mul_fixed(Factor k, int64_t a) {
+    const int ah = (int)(a >> 32), al = (int)((uint32_t)a >> 1);
+    const int64_t t = (int64_t)ah * k.lo + (int64_t)al * k.hi;
+    return (int64_t)ah * k.hi + (t >> 31);
+}
+
+// The N-th of a node's results: the first three (WIDE: four) on the FP64 pipe.
+template <bool WIDE, int N>
+__device__ __forceinline__ double result(int64_t v, uint32_t e) {
+    return N < (WIDE ? 4 : 3) ? from_fixed_fp64(v, e) : from_fixed<WIDE>(v, e);
+}
+
+template <bool GEN, bool WIDE>
+__device__ __forceinline__ void step_f64(const double f[8], double gx, double gy, const Coef<double>& c, double& u,
+                                         double& v, double o[8]) {
+    uint32_t e = 0;
+#pragma unroll
+    for (int p = 0; p < 8; ++p) e = max(e, (uint32_t)__double2hiint(f[p]) & 0x7ff00000u);
+    e = max(e, (uint32_t)__double2hiint(gx) & 0x7ff00000u);
+    e = max(e, (uint32_t)__double2hiint(gy) & 0x7ff00000u);
+    if (!c.fixed || e - (100u << 20) > (1900u << 20)) {
+        collide_populations<GEN>(moments(f), gx, gy, c, u, v, o);
+        return;
+    }
+    int64_t F[8];
+#pragma unroll
+    for (int p = 0; p < 8; ++p) F[p] = to_fixed<WIDE>(f[p], e, 0);
+    const int64_t hx = to_fixed<WIDE>(gx, e, 1), hy = to_fixed<WIDE>(gy, e, 1);
+    const int64_t p = F[4] + F[6], q = F[5] + F[7], r = F[4] - F[6], s = F[5] - F[7];
+    const int64_t m11 = p - q, m22 = p + q, m12 = r - s, m21 = r + s;
+    const int64_t U = (F[0] - F[2]) + m12 + hx, V = (F[1] - F[3]) + m21 + hy;
+    const int64_t s13 = F[0] + F[2], s24 = F[1] + F[3];
+    const int64_t X = mul_fixed(c.k11, m11), S = mul_fixed(c.ks, s13 + s24 + 2 * m22), D = mul_fixed(c.kd, s13 - s24);
+    int64_t Tu = mul_fixed(c.kw12t, U), Tv = mul_fixed(c.kw21t, V), W = 0;
+    if (GEN) {
+        Tu += mul_fixed(c.k12, m12);
+        Tv += mul_fixed(c.k21, m21);
+        W = mul_fixed(c.k22, m22);
+    }
+    // m*_10 - m*_12 and m*_01 - m*_21, halved without a loss
+    const int64_t A = U + hx - 4 * Tu, B = V + hy - 4 * Tv, Ah = A >> 1, Bh = B >> 1;
+    const int64_t P = S + D - 2 * W, Q = S - D - 2 * W;
+    o[0] = result<WIDE, 0>(P + Ah, e);
+    o[2] = result<WIDE, 1>(P - (A - Ah), e);
+    o[1] = result<WIDE, 2>(Q + Bh, e);
+    o[3] = result<WIDE, 3>(Q - (B - Bh), e);
+    o[4] = result<WIDE, 4>(W + X + (Tu + Tv), e);
+    o[6] = result<WIDE, 5>(W + X - (Tu + Tv), e);
+    o[5] = result<WIDE, 6>(W - X + (Tv - Tu), e);
+    o[7] = result<WIDE, 7>(W - X - (Tv - Tu), e);
+    u = from_fixed<false>(U, e);
+    v = from_fixed<false>(V, e);
 }
 
 // Shifted FP16 storage.  The equilibrium-type part of a post-collision state

@@ -611,9 +611,9 @@ __device__ __forceinline__ void step_tile(const StepParams& a,
         const int x = xb + 32 * j;
         if (x < nx) {
             const int64_t idx = r0 + x;
-            if constexpr (S == S_F64 && !GEN) {
+            if constexpr (S == S_F64) {
                 T u, v, fs[8];
-                collide_f64(f[j], gx[j], gy[j], c, u, v, fs);
+                step_f64<GEN, true>(f[j], gx[j], gy[j], c, u, v, fs);
                 store_state<S>(a, idx, fs, 0.0f, 0.0f);
                 if (CHECK) check_node<S>(a, n, idx, acc, so[j], f[j], gx[j], gy[j], u, v);
             } else {
@@ -655,51 +655,73 @@ __device__ __forceinline__ int wrap_slot(int v, int n) {
     return v;
 }
 
+// Pulled populations and stored ones of FP64 storage, by node indices of 31 bits
+// (a state of 2^31 nodes is larger than the device's memory).
+__device__ __forceinline__ void pull64(const StepParams& a, int r0, int rm, int rp, int x, int xm, int xp, double f[8]) {
+    const double* s = static_cast<const double*>(a.src);
+    const int64_t pl = a.plane;
+    f[0] = ldg(s + 0 * pl + (r0 + xm));                       // f_p(x) = f*_p(x - c_p)
+    f[1] = ldg(s + 1 * pl + (rm + x));
+    f[2] = ldg(s + 2 * pl + (r0 + xp));
+    f[3] = ldg(s + 3 * pl + (rp + x));
+    f[4] = ldg(s + 4 * pl + (rm + xm));
+    f[5] = ldg(s + 5 * pl + (rm + xp));
+    f[6] = ldg(s + 6 * pl + (rp + xp));
+    f[7] = ldg(s + 7 * pl + (rp + xm));
+}
+__device__ __forceinline__ void push64(const StepParams& a, int idx, const double f[8]) {
+    double* d = static_cast<double*>(a.dst);
+#pragma unroll
+    for (int p = 0; p < 8; ++p) (d + p * a.plane)[idx] = f[p];
+}
+
+// A launch of FP64 storage: T steps; T > 1: blocks of bx x by nodes (k_tile64),
+// T = 1: k_one64.
+constexpr int kT64Max = 4;        // most steps per launch
+struct Tile64Shape {
+    int T = 0, bx = 0, by = 0;
+    int inv[kT64Max] = {};        // step t: 2^16 / (width of its slots), rounded up
+    double cost = 0.0;            // modelled cycles of one launch
+};
+
 // ---------------------------------------------------------------------------
 // T pseudo-time steps per launch of FP64 storage (T >= 1, a run-time count).
 //
-// FP64 storage is bound by the FP64 pipe (a warp instruction takes 64 cycles of
-// one of an SM's four schedulers, whatever its active lanes), so a small lattice has to be spread
-// over all SMs, in whole warps: a block owns bx x by nodes, holds the states
-// between its steps in shared memory over a halo that shrinks by one node per
-// step, and its threads take the slots of a step in linear order.  Several
-// steps per launch recompute the halos but save launches; tile64_shape weighs
-// the two.  Large lattices take T = 1 (no halo).  Measured: 1500 x 1100 116 us per
-// step (tiles of 64 x 8 with two nodes per thread 121 with the same arithmetic,
-// 137 before it), 0.77 of the FP64 pipe's measured rate in 34 instructions per
-// update; 64 x 64 2.05 us (8.3).
+// A step of a node is some 600 instructions in a row (step_f64), so a small
+// lattice has to be spread over all SMs, in whole warps: a block owns bx x by
+// nodes, holds the states between its steps in shared memory over a halo that
+// shrinks by one node per step, and its threads take the slots of a step in
+// linear order.  Several steps per launch recompute the halos but save launches;
+// tile64_shape weighs the two.  64 x 64: 1.39 us per step (8.3 with one step of
+// 64 x 8 tiles per launch, 2.05 with these tiles on the FP64 pipe).
 template <bool GEN, bool CHECK>
-__global__ void __launch_bounds__(128)
-k_tile64(const StepParams a, const Coef<double> c, int T, int bx, int by, int ntx, int64_t ntiles) {
+__global__ void __launch_bounds__(256)
+k_tile64(const StepParams a, const Coef<double> c, const __grid_constant__ Tile64Shape sh, int nty) {
     extern __shared__ double tile64_mem[];
-    const int nx = a.nx, ny = a.ny, H = T - 1, sw = bx + 2 * H, sh = by + 2 * H, area = sw * sh;
-    const int64_t pl = a.plane;
-    const double* gxp = static_cast<const double*>(a.gx);
-    const double* gyp = static_cast<const double*>(a.gy);
-    double* dst = static_cast<double*>(a.dst);
+    const int nx = a.nx, ny = a.ny, H = sh.T - 1, sw = sh.bx + 2 * H, area = sw * (sh.by + 2 * H);
+    const int pitch = (int)a.pitch;
     ResAcc<S_F64> acc;
     after_predecessor();
-    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const int ty = (int)(tile / ntx), tx = (int)(tile - (int64_t)ty * ntx);
-        const int x0 = tx * bx - H, y0 = ty * by - H;         // node of slot (0, 0)
-        for (int t = 0; t < T; ++t) {
-            const bool last = t == T - 1;
-            const int aw = sw - 2 * t, count = aw * (sh - 2 * t);
+    const int x0 = (int)blockIdx.x * sh.bx - H;               // node of slot (0, 0)
+    for (int ty = blockIdx.y; ty < nty; ty += gridDim.y) {
+        const int y0 = ty * sh.by - H;
+        for (int t = 0; t <= H; ++t) {
+            const bool last = t == H;
+            const int aw = sw - 2 * t, count = aw * (sh.by + 2 * (H - t)), inv = sh.inv[t];
             const double* from = tile64_mem + (t & 1) * 8 * area;
             double* to = tile64_mem + ((t + 1) & 1) * 8 * area;
             for (int i = threadIdx.x; i < count; i += blockDim.x) {
-                const int q = i / aw, sx = t + i - q * aw, sy = t + q;
+                const int q = (i * inv) >> 16, sx = t + i - q * aw, sy = t + q;   // q = i / aw
                 int x = x0 + sx, y = y0 + sy;
                 if (last && (x >= nx || y >= ny)) continue;
                 if (!last) {
                     x = wrap_slot<true>(x, nx);
                     y = wrap_slot<true>(y, ny);
                 }
-                const int64_t row = (int64_t)y * a.pitch, idx = row + x;
+                const int row = y * pitch, idx = row + x;
                 double f[8];
                 if (t == 0) {
-                    gather<S_F64>(a, row, (int64_t)wrap_dec(y, ny) * a.pitch, (int64_t)wrap_inc(y, ny) * a.pitch, x,
-                                  wrap_dec(x, nx), wrap_inc(x, nx), f, c.theta);
+                    pull64(a, row, wrap_dec(y, ny) * pitch, wrap_inc(y, ny) * pitch, x, wrap_dec(x, nx), wrap_inc(x, nx), f);
                 } else {
                     const double* p = from + sy * sw + sx;
                     f[0] = p[0 * area - 1];                   // f_p(x) = f*_p(x - c_p)
@@ -711,22 +733,47 @@ k_tile64(const StepParams a, const Coef<double> c, int T, int bx, int by, int nt
                     f[6] = p[6 * area + sw + 1];
                     f[7] = p[7 * area + sw - 1];
                 }
-                const double gx = ldg(gxp + idx), gy = ldg(gyp + idx);
+                const double gx = ldg(static_cast<const double*>(a.gx) + idx), gy = ldg(static_cast<const double*>(a.gy) + idx);
                 double u, v, fs[8];
-                if (GEN) collide_populations<true>(moments(f), gx, gy, c, u, v, fs);
-                else collide_f64(f, gx, gy, c, u, v, fs);
+                step_f64<GEN, false>(f, gx, gy, c, u, v, fs);
                 if (last) {
-                    if (CHECK) check_node<S_F64>(a, pl, idx, acc, snap_load<S_F64>(a, pl, idx), f, gx, gy, u, v);
-#pragma unroll
-                    for (int p = 0; p < 8; ++p) dst[p * pl + idx] = fs[p];
+                    if (CHECK) check_node<S_F64>(a, a.plane, idx, acc, snap_load<S_F64>(a, a.plane, idx), f, gx, gy, u, v);
+                    push64(a, idx, fs);
                 } else {
                     double* o = to + sy * sw + sx;
 #pragma unroll
                     for (int p = 0; p < 8; ++p) o[p * area] = fs[p];
                 }
             }
-            if (T > 1) __syncthreads();
+            if (H) __syncthreads();
         }
+    }
+    if (CHECK) residual_reduce(a, acc);
+}
+
+// One step per launch of FP64 storage (lattices of some 200 x 200 nodes and more):
+// blocks of 32 x 4 nodes.  1500 x 1100: 38.7 us per step, 238 MB of populations
+// and force at 6.1 TB/s (k_tile64 at T = 1 47 us, with 64-bit tile divisions and
+// addresses; on the FP64 pipe 116, with tiles of 64 x 8 137).
+constexpr int kOne64Rows = 4;
+template <bool GEN, bool CHECK>
+__global__ void __launch_bounds__(32 * kOne64Rows)
+k_one64(const StepParams a, const Coef<double> c, int nty) {
+    const int nx = a.nx, ny = a.ny, pitch = (int)a.pitch;
+    ResAcc<S_F64> acc;
+    after_predecessor();
+    const int x = (int)blockIdx.x * 32 + threadIdx.x;
+    for (int ty = blockIdx.y; ty < nty; ty += gridDim.y) {
+        const int y = ty * kOne64Rows + threadIdx.y;
+        if (x >= nx || y >= ny) continue;
+        const int row = y * pitch, idx = row + x;
+        double f[8];
+        pull64(a, row, wrap_dec(y, ny) * pitch, wrap_inc(y, ny) * pitch, x, wrap_dec(x, nx), wrap_inc(x, nx), f);
+        const double gx = ldg(static_cast<const double*>(a.gx) + idx), gy = ldg(static_cast<const double*>(a.gy) + idx);
+        double u, v, fs[8];
+        step_f64<GEN, true>(f, gx, gy, c, u, v, fs);
+        if (CHECK) check_node<S_F64>(a, a.plane, idx, acc, snap_load<S_F64>(a, a.plane, idx), f, gx, gy, u, v);
+        push64(a, idx, fs);
     }
     if (CHECK) residual_reduce(a, acc);
 }
@@ -2065,39 +2112,46 @@ inline StripShape strip_shape(int dtype, int T, bool check, int nx, int ny, int 
     return best;
 }
 
-// A tile launch of FP64 storage (k_tile64): T steps, blocks of bx x by nodes.
-struct Tile64Shape {
-    int T = 0, bx = 0, by = 0;
-    double cost = 0.0;            // modelled cycles of one launch
-};
-inline int64_t tile64_count(const Tile64Shape& t, int nx, int ny) {
-    return (int64_t)((nx + t.bx - 1) / t.bx) * ((ny + t.by - 1) / t.by);
-}
 inline int tile64_smem(const Tile64Shape& t) {
     return t.T > 1 ? 2 * 8 * 8 * (t.bx + 2 * (t.T - 1)) * (t.by + 2 * (t.T - 1)) : 0;
 }
+// Blocks of bx x by nodes in two dimensions, at most `most` of them in all if
+// the width allows it (each then takes several, one below the other).
+inline dim3 tile64_grid(const Tile64Shape& t, int nx, int ny, int64_t most) {
+    const int64_t w = (nx + t.bx - 1) / t.bx, h = (ny + t.by - 1) / t.by;
+    const int64_t cap = std::max<int64_t>(1, std::min<int64_t>(65535, most / w));
+    return dim3((unsigned)w, (unsigned)std::min(h, cap));
+}
+inline Tile64Shape tile64(int T, int bx, int by) {
+    Tile64Shape t;
+    t.T = T;
+    t.bx = T > 1 ? bx : 32;
+    t.by = T > 1 ? by : kOne64Rows;
+    for (int s = 0; s < T; ++s) {
+        const int aw = t.bx + 2 * (T - 1 - s);
+        t.inv[s] = (65536 + aw - 1) / aw;
+    }
+    return t;
+}
 
-// The FP64 tile launch with the fewest modelled cycles per step.  Fitted on
-// GB300 (8 x 8 to 1500 x 1100 lattices, T = 1 .. 5): each of an SM's four
-// schedulers issues one FP64 warp instruction in 64 cycles, so a step takes
-// about 1100 + 2250 ceil(W / 4) cycles with W warps of slots on an SM, and a
-// launch 2800 besides.  64 x 64: T = 3 on 8 x 4 nodes, 2.05 us per step (T = 1
-// 2.94, the 64 x 8 tiles before 8.3); 256 x 256: T = 1 on 32 x 2, 6.8 (9.8).
+// The FP64 launch with the fewest modelled cycles per step.  Fitted on GB300 (1 x 1
+// to 1500 x 1100, T = 1 .. 4; within 5 %): W warps of slots on an SM's scheduler
+// take 1060 W cycles (T = 1: 820 W), a step of a tile 1030 and a launch 2330
+// (T = 1: 3350) besides.  64 x 64: T = 4 on 8 x 4 nodes, 1.39 us per step (T = 3
+// 1.45, T = 1 2.09); 256 x 256: T = 1, 3.3 us (T = 2 on 16 x 8 3.5).
 inline Tile64Shape tile64_shape(int nx, int ny, int nsm) {
-    const int tiles[4][2] = {{8, 4}, {16, 4}, {32, 2}, {32, 4}};
+    const int tiles[5][2] = {{8, 4}, {16, 4}, {8, 8}, {16, 8}, {32, 4}};
     Tile64Shape best;
-    for (int T = 1; T <= 3; ++T)
+    for (int T = 1; T <= kT64Max; ++T)
         for (const auto& b : tiles) {
-            Tile64Shape t;
-            t.T = T;
-            t.bx = b[0];
-            t.by = b[1];
-            const int64_t here = (tile64_count(t, nx, ny) + nsm - 1) / nsm;   // tiles per SM
-            t.cost = 2800.0;
+            Tile64Shape t = tile64(T, b[0], b[1]);
+            const dim3 g = tile64_grid(t, nx, ny, (int64_t)1 << 40);
+            const int64_t here = ((int64_t)g.x * ((ny + t.by - 1) / t.by) + nsm - 1) / nsm;   // tiles per SM
+            t.cost = T > 1 ? 2330.0 : 2320.0;
             for (int s = 0; s < T; ++s) {
                 const int slots = (t.bx + 2 * (T - 1 - s)) * (t.by + 2 * (T - 1 - s));
                 const int64_t warps = here * ((slots + 31) / 32);
-                t.cost += 1100.0 + 2250.0 * (double)((warps + 3) / 4);
+                t.cost += 1030.0 + (T > 1 ? 1060.0 : 820.0) * (double)((warps + 3) / 4);
             }
             if (best.T == 0 || t.cost * best.T < 0.999 * best.cost * t.T) best = t;
         }
@@ -2105,7 +2159,7 @@ inline Tile64Shape tile64_shape(int nx, int ny, int nsm) {
 }
 
 cudaError_t tile_f64(const StepParams& a, const Coef<double>& c, bool gen, const Tile64Shape& t, bool check,
-                     int64_t max_blocks, cudaStream_t st);
+                     int64_t* blocks, cudaStream_t st);
 
 // A tile launch: T steps, blocks of NW warps of RR rows.
 struct TileShape {

@@ -70,7 +70,7 @@ int scratch_for_device(int dev, double** out) {
 template <typename T>
 Coef<T> standard_coef(double lambda, double mu) {
     // Table 1 with theta = 1/3 and w_12 = w_21 = w_22 = 1; Eq. relaxation_rate.
-    const double theta = sizeof(T) == 8 ? theta_f64(1.0 / 3.0) : 1.0 / 3.0, K = lambda + mu;
+    const double theta = 1.0 / 3.0, K = lambda + mu;
     const double w11 = 1.0 / (mu / theta + 0.5);
     const double ws = 1.0 / (2.0 * K / (1.0 + theta) + 0.5);
     const double wd = 1.0 / (2.0 * mu / (1.0 - theta) + 0.5);
@@ -88,10 +88,7 @@ Coef<T> standard_coef(double lambda, double mu) {
     c.b11 = T(1.0 - 0.5 * w11);
     c.bs = T(1.0 - 0.5 * ws);
     c.bd = T(1.0 - 0.5 * wd);
-    c.qsd = T(0.25 * (1.0 - ws) + 0.25 * (1.0 - wd));
-    c.qds = T(0.25 * (1.0 - ws) - 0.25 * (1.0 - wd));
-    c.qs2 = T(0.5 * (1.0 - ws));
-    c.twoctheta = T(2.0 * (1.0 - theta));
+    set_factors(c);
     return c;
 }
 

@@ -4,21 +4,29 @@
 namespace lbm {
 template struct Ops<S_F64>;
 
-// check: at most max_blocks blocks (partial sets)
+// blocks: of the launch (partial sets of a checked one)
 cudaError_t tile_f64(const StepParams& a, const Coef<double>& c, bool gen, const Tile64Shape& t, bool check,
-                     int64_t max_blocks, cudaStream_t st) {
-    const int64_t tiles = tile64_count(t, a.nx, a.ny);
-    const int64_t blocks = check && tiles > max_blocks ? max_blocks : tiles;
-    if (t.T < 1 || tile64_smem(t) > 48 * 1024 || blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-    const int ntx = (a.nx + t.bx - 1) / t.bx;
-    // whole warps for the slots of the first step, at most four
+                     int64_t* blocks, cudaStream_t st) {
+    const dim3 grid = tile64_grid(t, a.nx, a.ny, check ? kMaxCheckBlocks : (int64_t)1 << 40);
+    *blocks = (int64_t)grid.x * grid.y;
+    if (t.T < 1 || t.T > kT64Max || tile64_smem(t) > 48 * 1024 || a.plane > 0x7fffffffLL) return cudaErrorInvalidValue;
+    const int nty = (a.ny + t.by - 1) / t.by;
+    if (t.T == 1) {
+        const dim3 block(32, kOne64Rows);
+        if (gen)
+            return check ? launch_after(k_one64<true, true>, grid, block, 0, st, a, c, nty)
+                         : launch_after(k_one64<true, false>, grid, block, 0, st, a, c, nty);
+        return check ? launch_after(k_one64<false, true>, grid, block, 0, st, a, c, nty)
+                     : launch_after(k_one64<false, false>, grid, block, 0, st, a, c, nty);
+    }
+    // whole warps for the slots of the first step, at most eight
     const int slots = (t.bx + 2 * (t.T - 1)) * (t.by + 2 * (t.T - 1)), warps = (slots + 31) / 32;
-    const dim3 grid((unsigned)blocks), block(32 * (warps < 4 ? warps : 4));
+    const dim3 block(32 * (warps < 8 ? warps : 8));
     const size_t sm = tile64_smem(t);
     if (gen)
-        return check ? launch_after(k_tile64<true, true>, grid, block, sm, st, a, c, t.T, t.bx, t.by, ntx, tiles)
-                     : launch_after(k_tile64<true, false>, grid, block, sm, st, a, c, t.T, t.bx, t.by, ntx, tiles);
-    return check ? launch_after(k_tile64<false, true>, grid, block, sm, st, a, c, t.T, t.bx, t.by, ntx, tiles)
-                 : launch_after(k_tile64<false, false>, grid, block, sm, st, a, c, t.T, t.bx, t.by, ntx, tiles);
+        return check ? launch_after(k_tile64<true, true>, grid, block, sm, st, a, c, t, nty)
+                     : launch_after(k_tile64<true, false>, grid, block, sm, st, a, c, t, nty);
+    return check ? launch_after(k_tile64<false, true>, grid, block, sm, st, a, c, t, nty)
+                 : launch_after(k_tile64<false, false>, grid, block, sm, st, a, c, t, nty);
 }
 }  // namespace lbm

@@ -152,6 +152,52 @@ def test_f64_tiles_equal_single_steps(nx, ny, kw):
         assert np.allclose(ra, rb, rtol=1e-13, atol=0.0)
 
 
+# FP64 collision in integers (step_f64) against long double, one step: populations
+# of mixed magnitudes, zeros, and scales on either side of the lines to FP64
+# arithmetic (2^-923 and 2^977).  Integers: the last rounding and eight units of
+# 2^-58 of the largest value's power of two, so 2^-54 of the largest value; FP64:
+# at most 32 roundings of sums of twelve populations.
+@pytest.mark.parametrize("scale,integers", [(0, True), (-880, True), (940, True), (-990, False), (1000, False)])
+@pytest.mark.parametrize("kw", [dict(), dict(tau12=0.9, tau22=0.3)])
+def test_f64_step_against_long_double(scale, integers, kw):
+    nx, ny = 37, 11
+    lam, mu = (np.longdouble(v) for v in W.lame_2d(1.0, 0.3))
+    rng = np.random.RandomState(scale + 2000)
+    f = rng.standard_normal((8, ny, nx)) * 2.0 ** rng.randint(-40, 1, (8, ny, nx))
+    f[rng.random_sample(f.shape) < 0.1] = 0.0
+    f[:, 3, :5] = 0.0
+    g = rng.standard_normal((2, ny, nx)) * 2.0 ** rng.randint(-60, 1, (2, ny, nx))
+    g[:, 3, :3] = 0.0
+    f, g = np.ldexp(f, scale), np.ldexp(g, scale)
+    with Lattice(nx, ny, float(lam), float(mu), "f64", **kw) as lat:
+        lat.set_force(g[0], g[1])
+        lat.set_populations(f)
+        lat.iterate(1)
+        got = lat.populations()
+    one = np.longdouble(1)
+    th, t12, t22 = one / 3, np.longdouble(kw.get("tau12", 0.5)), np.longdouble(kw.get("tau22", 0.5))
+    w11, w12, w22 = one / (mu / th + one / 2), one / (t12 + one / 2), one / (t22 + one / 2)
+    ws, wd = one / (2 * (lam + mu) / (1 + th) + one / 2), one / (2 * mu / (1 - th) + one / 2)
+    f, g = np.ldexp(f, -scale).astype(np.longdouble), np.ldexp(g, -scale).astype(np.longdouble)
+    p, q, r, s = f[4] + f[6], f[5] + f[7], f[4] - f[6], f[5] - f[7]
+    u, v = f[0] - f[2] + (r - s) + g[0] / 2, f[1] - f[3] + (r + s) + g[1] / 2
+    s13, s24 = f[0] + f[2], f[1] + f[3]
+    m11, m22 = (1 - w11) * (p - q) / 4, (1 - w22) * (p + q) / 4
+    ms, md = (1 - ws) * (s13 + s24 + 2 * (p + q)) / 4, (1 - wd) * (s13 - s24) / 4
+    m12, m21 = (w12 * th * u + (1 - w12) * (r - s)) / 4, (w12 * th * v + (1 - w12) * (r + s)) / 4
+    A, B = (u + g[0] / 2 - 4 * m12) / 2, (v + g[1] / 2 - 4 * m21) / 2
+    P_, Q_ = ms + md - 2 * m22, ms - md - 2 * m22
+    o = [P_ + A, Q_ + B, P_ - A, Q_ - B, m22 + m11 + m12 + m21, m22 - m11 + m21 - m12, m22 + m11 - m12 - m21,
+         m22 - m11 - m21 + m12]
+    top = np.maximum(abs(f).max(axis=0), abs(g).max(axis=0))
+    for k, (cx, cy) in enumerate([(1, 0), (0, 1), (-1, 0), (0, -1), (1, 1), (-1, 1), (-1, -1), (1, -1)]):
+        want, big = np.roll(o[k], (cy, cx), (0, 1)), np.roll(top, (cy, cx), (0, 1))
+        err = abs(np.ldexp(got[k].astype(np.longdouble), -scale) - want)
+        # (the rates are FP64 numbers: 2^-53 of sums of up to twelve populations)
+        tol = 2.0 ** -53 * abs(want) + (2.0 ** -54 + 2.0 ** -50) * big if integers else 2.0 ** -44 * big + 2.0 ** -70
+        assert (err <= tol).all(), k
+
+
 def _problems(sizes):
     out = []
     for i, (nx, ny) in enumerate(sizes):
