@@ -93,9 +93,10 @@ struct lbm_ctx {
     uint8_t wave_first[kWavePlan + 1] = {};
     double wave_cost[kWavePlan + 1] = {};
     int64_t launches = 0;          // kernels launched to advance the lattice
-    bool auto_plan = true;         // FP32: strip or tile launches as they suit the lattice, until the
+    bool auto_plan = true;         // FP32, FP16S: strip or tile launches as they suit the lattice, until the
                                    // caller sets a schedule (lbm_set_steps_per_launch, lbm_set_wavefront)
-    int plan = 0;                  // 0: not chosen yet, 1: strips, 2: register tiles (tile)
+    int plan = 0;                  // 0: not chosen yet, 1: strips, 2: register tiles (tile), 3: FP16S single
+                                   // or paired steps
     TileShape tile;
     Tile64Shape tile64;            // FP64
 };
@@ -232,6 +233,9 @@ cudaError_t launch_step3(lbm_ctx* c) {
 
 bool wave_on(const lbm_ctx* c) { return c->wave != 0 && wave_fits(c->nx, c->ny); }
 
+// Steps of a whole group of plain steps (groups_of).
+int group_steps(const lbm_ctx* c) { return c->spl >= 4 && wave_on(c) ? 4 : std::min(c->spl, 3); }
+
 // The shape of a strip launch of T steps (kept per context: it depends on the
 // sizes and the lbm_set_wavefront setting only).
 cudaError_t wave_shape(lbm_ctx* c, int T, bool check, StripShape* out) {
@@ -336,30 +340,49 @@ cudaError_t launch_strip(lbm_ctx* c, int T, bool check) {
     return e;
 }
 
-// FP32 without a schedule set by the caller: strips or register tiles,
+// FP32 and FP16S without a schedule set by the caller: strips or register tiles,
 // whichever the models say takes fewer cycles per step (every plan gives the
 // same states).  Tiles win up to about 10^6 nodes, where a strip launch is bound
-// by the latency of its rows (333 x 517: 1.1 against 2.1 us per step).
+// by the latency of its rows (FP32 333 x 517: 1.1 against 2.1 us per step; FP16S
+// 300 x 300 1.09 against 1.77, 700 x 500 2.1 / 2.9, 1000 x 700 4.03 / 3.89; 90 x
+// 2413 1.67 / 2.86, with three-step tiles 3.07; 255 x 8000 12.7 / 10.05, 15.6).
+// FP16S lattices that one or two steps at a time are rounded on (narrow or flat
+// ones) have no strips: tiles (33 x 64: 0.79 us per step, single steps 4.1;
+// 63 x 8000 5.4 / 8.2), and single or paired steps where those lattices are so
+// long that their traffic is cheaper than the tiles' halos.
 cudaError_t choose_plan(lbm_ctx* c) {
     if (c->plan) return cudaSuccess;
-    c->tile = tile_shape(c->nx, c->ny, c->nsm > 0 ? c->nsm : 1);
+    const int nsm = c->nsm > 0 ? c->nsm : 1, group = c->dtype == LBM_F32 ? 1 : group_steps(c);
+    c->tile = tile_shape(c->dtype, group, c->nx, c->ny, nsm);
     c->plan = 2;
-    if (c->ghost) {
+    if (c->dtype == LBM_F32 && c->ghost) {
         const cudaError_t e = wave_plan(c);
         if (e != cudaSuccess) return e;
         if (c->wave_cost[c->wave_T] * c->tile.T < c->tile.cost * c->wave_T) c->plan = 1;
+    } else if (c->dtype == LBM_F16S && c->ghost && group >= 3) {
+        StripShape sh;
+        const cudaError_t e = wave_shape(c, group, false, &sh);
+        if (e != cudaSuccess) return e;
+        if (sh.cost * c->tile.T < c->tile.cost * group) c->plan = 1;
+    } else if (c->dtype == LBM_F16S) {
+        // (one or two steps per launch: at most the start of a launch and the traffic)
+        if ((6200.0 + 56.0 * (double)c->n / 3040.0) * c->tile.T < c->tile.cost * group) c->plan = 3;
     }
     return cudaSuccess;
 }
 
 bool auto_on(const lbm_ctx* c) { return c->auto_plan && c->dtype == LBM_F32; }
+bool auto16(const lbm_ctx* c) { return c->auto_plan && c->dtype == LBM_F16S; }
 
-cudaError_t launch_tile(lbm_ctx* c, int T, bool check) {
+// rounds: as tile_f16s.
+cudaError_t launch_tile(lbm_ctx* c, int T, bool check, unsigned rounds = 0) {
     TileShape t = c->tile;
     t.T = T;
     const int64_t blocks = tile_count(t, c->nx, c->ny);
     if (check && ensure_partials(c, blocks) != LBM_OK) return cudaErrorMemoryAllocation;
-    cudaError_t e = tile_f32(params(c, c->cur), coef<float>(c->rates), c->gen, t, check, c->stream);
+    cudaError_t e = c->dtype == LBM_F32
+        ? tile_f32(params(c, c->cur), coef<float>(c->rates), c->gen, t, check, c->stream)
+        : tile_f16s(params(c, c->cur), coef<float>(c->rates), c->gen, t, check, rounds, c->stream);
     if (e == cudaSuccess && check) e = finish_residual_launch(c, blocks);
     if (e == cudaSuccess) {
         c->ghosts_ok = false;
@@ -407,45 +430,81 @@ cudaError_t run_strips(lbm_ctx* c, int64_t n) {
 }
 
 // T = 3 or 4 plain steps in one launch: the strip kernel where it is on and
-// fits, else (T = 3) the three-step tile kernel.
+// fits (or was chosen), else (T = 3) the three-step tile kernel.
 cudaError_t launch_multi(lbm_ctx* c, int T) {
-    if (!wave_on(c)) return T == 3 ? launch_step3(c) : cudaErrorInvalidValue;
+    if (!wave_on(c) && !(auto16(c) && c->plan == 1)) return T == 3 ? launch_step3(c) : cudaErrorInvalidValue;
     return launch_strip(c, T, false);
 }
 
-// n plain steps, grouped into launches of c->spl steps (four only on the
-// wavefront schedule, else three); a remainder of one step is avoided where
-// possible (4 = 2 + 2, 5 = 3 + 2), since a pair of steps costs about as much
-// as one step alone.  FP32 on the wavefront schedule takes up to seven steps
-// per launch (wave_steps); FP16-shifted storage rounds to FP16 where a launch
-// ends, so its groups stay the documented ones.
+// The groups of n plain steps that c->spl sets: `whole` of `big` steps (four only on
+// the wavefront schedule, else three), then the rest; a remainder of one step
+// is avoided where possible (4 = 2 + 2, 5 = 3 + 2), since a pair of steps costs
+// about as much as one step alone.  FP16-shifted storage rounds to FP16 where a
+// group ends.
+struct Groups {
+    int64_t whole = 0;
+    int big = 0, nrest = 0, rest[4] = {};
+};
+Groups groups_of(const lbm_ctx* c, int64_t n) {
+    Groups g;
+    g.big = group_steps(c);
+    g.whole = n / g.big;
+    n %= g.big;
+    if (g.big >= 3 && n == 1 && g.whole >= 1) {
+        --g.whole;
+        n += g.big;
+    }
+    if (g.big == 4 && n >= 3) {
+        g.rest[g.nrest++] = 3;
+        n -= 3;
+    }
+    for (; n >= 2; n -= 2) g.rest[g.nrest++] = 2;
+    if (n > 0) g.rest[g.nrest++] = 1;
+    return g;
+}
+
+cudaError_t launch_group(lbm_ctx* c, int T) {
+    return T >= 3 ? launch_multi(c, T) : (T == 2 ? launch_step2(c, false) : launch_step(c, false));
+}
+
+// n plain steps of FP16-shifted storage and a last group of `check` steps that
+// ends in the residual-check step (0: none) on register tiles: as many groups per
+// launch as the tile takes, the state rounded after each.
+cudaError_t run_tiles16(lbm_ctx* c, int64_t n, int check) {
+    const Groups g = groups_of(c, n);
+    cudaError_t e = cudaSuccess;
+    int T = 0;
+    unsigned rounds = 0;
+    auto flush = [&](bool checked) {
+        if (T > 0 && e == cudaSuccess) e = launch_tile(c, T, checked, rounds);
+        T = 0;
+        rounds = 0;
+    };
+    auto add = [&](int t) {
+        if (T + t > c->tile.T) flush(false);
+        if (T > 0) rounds |= 1u << (T - 1);
+        T += t;
+    };
+    for (int64_t i = 0; i < g.whole && e == cudaSuccess; ++i) add(g.big);
+    for (int i = 0; i < g.nrest; ++i) add(g.rest[i]);
+    if (check) add(check);
+    flush(check != 0);
+    return e;
+}
+
+// n plain steps: as the plan has it, or in launches of a group each.
 cudaError_t run_plain(lbm_ctx* c, int64_t n) {
     cudaError_t e = cudaSuccess;
-    const bool wave = wave_on(c);
     if (c->dtype == LBM_F64) return run_tiles64(c, n, false);
-    if (auto_on(c)) {
+    if (c->auto_plan) {
         e = choose_plan(c);
         if (e != cudaSuccess) return e;
-        return c->plan == 2 ? run_tiles(c, n, false) : run_strips(c, n);
+        if (c->plan == 2) return c->dtype == LBM_F32 ? run_tiles(c, n, false) : run_tiles16(c, n, 0);
     }
-    if (c->spl >= 4 && wave && c->dtype == LBM_F32) return run_strips(c, n);
-    const int big = c->spl >= 4 && wave ? 4 : (c->spl >= 3 ? 3 : 0);
-    if (big) {
-        int64_t groups = n / big, r = n % big;
-        if (r == 1 && groups >= 1) {
-            --groups;
-            r += big;
-        }
-        for (int64_t i = 0; i < groups && e == cudaSuccess; ++i) e = launch_multi(c, big);
-        n = r;
-        if (big == 4 && n >= 3 && e == cudaSuccess) {
-            e = launch_multi(c, 3);
-            n -= 3;
-        }
-    }
-    if (c->spl >= 2)
-        for (; n >= 2 && e == cudaSuccess; n -= 2) e = launch_step2(c, false);
-    for (; n > 0 && e == cudaSuccess; --n) e = launch_step(c, false);
+    if (auto_on(c) || (c->spl >= 4 && wave_on(c) && c->dtype == LBM_F32)) return run_strips(c, n);
+    const Groups g = groups_of(c, n);
+    for (int64_t i = 0; i < g.whole && e == cudaSuccess; ++i) e = launch_group(c, g.big);
+    for (int i = 0; i < g.nrest && e == cudaSuccess; ++i) e = launch_group(c, g.rest[i]);
     return e;
 }
 
@@ -464,6 +523,14 @@ cudaError_t run_window(lbm_ctx* c, int64_t to_check) {
         if (to_check < 4) {
             e = run_strips(c, to_check - 1);
             return e == cudaSuccess ? launch_step(c, true) : e;
+        }
+    }
+    if (auto16(c)) {
+        e = choose_plan(c);
+        if (e != cudaSuccess) return e;
+        if (c->plan == 2) {
+            const int last = to_check >= 4 && group_steps(c) == 4 ? 4 : (c->spl >= 2 && to_check >= 2 ? 2 : 1);
+            return run_tiles16(c, to_check - last, last);
         }
     }
     if (to_check >= 4 && (auto_on(c) || (c->spl >= 4 && wave_on(c)))) {
@@ -782,7 +849,7 @@ int lbm_create_ex(int nx, int ny, double lambda, double mu, int dtype, const lbm
             c->partials_len = std::max(c->partials_len, strip_check_blocks(c, T, sh.seg));
         }
     }
-    if (e == cudaSuccess && dtype == LBM_F32) {
+    if (e == cudaSuccess && dtype != LBM_F64) {
         e = choose_plan(c);
         c->partials_len = std::max(c->partials_len, c->plan == 2 ? tile_count(c->tile, nx, ny) : int64_t(0));
     }

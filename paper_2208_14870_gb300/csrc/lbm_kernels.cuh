@@ -632,6 +632,7 @@ __device__ __forceinline__ void step_tile(const StepParams& a,
 template <int S, int V, bool GEN, bool CHECK>
 __global__ void __launch_bounds__(kThreads, CHECK ? 2 : (S == S_F32 ? LBM_MINB_F32 : (S == S_F16S ? LBM_MINB_F16S : LBM_MINB_F64)))
 k_step(const StepParams a, const Coef<typename StoreT<S>::T> c) {
+    after_predecessor();
     const int ntx = (a.nx + 32 * V - 1) / (32 * V);
     const int64_t ntiles = (int64_t)ntx * ((a.ny + BY - 1) / BY);
     ResAcc<S> acc;
@@ -932,6 +933,7 @@ template <int S, bool GEN, bool CHECK, bool ANY>
 __global__ void __launch_bounds__(kT2Threads,
                                   CHECK ? LBM_MINB_T2_CHECK : (S == S_F16S ? LBM_MINB_T2_F16S : LBM_MINB_T2))
 k_step2(const StepParams a, const Coef<float> c) {
+    after_predecessor();
     extern __shared__ float t2_smem[];
     const int ntx = (a.nx + kT2OX - 1) / kT2OX;
     const int64_t ntiles = (int64_t)ntx * ((a.ny + kT2OY - 1) / kT2OY);
@@ -1094,6 +1096,7 @@ __device__ __forceinline__ void step3_tile(const StepParams& a, const Coef<float
 template <int S, bool GEN, bool CHECK, bool ANY>
 __global__ void __launch_bounds__(kT2Threads, LBM_MINB_T3)
 k_step3(const StepParams a, const Coef<float> c) {
+    after_predecessor();
     extern __shared__ float t3_smem[];
     const int ntx = (a.nx + kT3OX - 1) / kT3OX;
     const int64_t ntiles = (int64_t)ntx * ((a.ny + kT3OY - 1) / kT3OY);
@@ -1209,6 +1212,31 @@ __device__ __forceinline__ float lds_float(uint32_t a) {
 __device__ __forceinline__ pair_t opaque(pair_t p, uint32_t a) {
     asm volatile("st.shared.b64 [%0], %1;" ::"r"(a), "l"(p) : "memory");
     return lds_pair(a);
+}
+
+// FP16S: the deviations of the state after a collision, rounded to FP16 (h, and
+// widened again in r), and the carriers that absorb the first moments of the
+// rounding (store_f16s).
+template <bool GEN>
+__device__ __forceinline__ void round_state(const Post2& m, const PairCoef& c, __half2 h[8], pair_t r[8], pair_t& c10,
+                                            pair_t& c01) {
+    Post2 w = m;
+    w.m10 = w.m01 = 0;
+    w.m12 = fma2(splat(-c.qtheta), m.m10, m.m12);
+    w.m21 = fma2(splat(-c.qtheta), m.m01, m.m21);
+    pair_t fs[8];
+    Pop2<!GEN>(w, c).all(c, fs);
+#pragma unroll
+    for (int p = 0; p < 8; ++p) {
+        float lo, hi;
+        unpk(fs[p], lo, hi);
+        h[p] = __floats2half2_rn(lo, hi);
+        const float2 b = __half22float2(h[p]);
+        r[p] = pk(b.x, b.y);
+    }
+    const pair_t r46 = sub2(r[4], r[6]), r57 = sub2(r[5], r[7]);
+    c10 = sub2(m.m10, add2(sub2(r[0], r[2]), sub2(r46, r57)));
+    c01 = sub2(m.m01, add2(sub2(r[1], r[3]), add2(r46, r57)));
 }
 
 // One strip and segment.  sm: the warp's shared memory (shared-space address).
@@ -1458,32 +1486,17 @@ __device__ __forceinline__ void strip_walk(const StepParams& a, const PairCoef& 
                     }
                 }
             } else {
-                // the deviations, rounded to FP16, and the carriers that absorb
-                // the first moments of the rounding (store_f16s)
-                Post2 w = m;
-                w.m10 = w.m01 = 0;
-                w.m12 = fma2(splat(-c.qtheta), m.m10, m.m12);
-                w.m21 = fma2(splat(-c.qtheta), m.m01, m.m21);
-                Pop2<!GEN>(w, c).all(c, fs);
                 __half* d = static_cast<__half*>(a.dst) + so;
                 __half2 hs[8];
-                pair_t r[8];
+                pair_t c10, c01;
+                round_state<GEN>(m, c, hs, fs, c10, c01);
+                if (two) {
 #pragma unroll
-                for (int p = 0; p < 8; ++p) {
-                    float lo, hi;
-                    unpk(fs[p], lo, hi);
-                    const __half2 h = __floats2half2_rn(lo, hi);
-                    if (two) *reinterpret_cast<__half2*>(d + p * a.plane) = h;
-                    hs[p] = h;
-                    const float2 b = __half22float2(h);
-                    r[p] = pk(b.x, b.y);
+                    for (int p = 0; p < 8; ++p) *reinterpret_cast<__half2*>(d + p * a.plane) = hs[p];
                 }
-                const pair_t r46 = sub2(r[4], r[6]), r57 = sub2(r[5], r[7]);
-                const pair_t e10 = add2(sub2(r[0], r[2]), sub2(r46, r57));
-                const pair_t e01 = add2(sub2(r[1], r[3]), add2(r46, r57));
                 float4 v;
-                unpk(sub2(m.m10, e10), v.x, v.z);
-                unpk(sub2(m.m01, e01), v.y, v.w);
+                unpk(c10, v.x, v.z);
+                unpk(c01, v.y, v.w);
                 float2* cd = reinterpret_cast<float2*>(a.cdst) + so;
                 if (two) *reinterpret_cast<float4*>(cd) = v;
                 if (edge) {
@@ -1553,9 +1566,9 @@ k_strip(const StepParams a, const PairCoef c, int seg, int nstrips, int items) {
 // (wavefront 4.0).  A launch of T steps takes 2.8 us (start, loads, stores) and
 // 0.24 us per step (8 warps of two rows) to 0.67 us (12 warps of four): FMA-pipe
 // and latency bound, 2 to 3 warps per scheduler.
-template <int RR, bool GEN, bool CHECK>
+template <int S, int RR, bool GEN, bool CHECK>
 __global__ void __launch_bounds__(512, 1)
-k_tile(const StepParams a, const PairCoef ca, int T, int ntx) {
+k_tile(const StepParams a, const PairCoef ca, int T, int ntx, unsigned rounds) {
     extern __shared__ float4 tile_mem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int nx = a.nx, ny = a.ny, H = T - 1;
@@ -1576,27 +1589,65 @@ k_tile(const StepParams a, const PairCoef ca, int T, int ntx) {
         return v < 0 ? v + n : v;
     };
     const int xa = wrapped(xs - 1, nx), xb = wrapped(xs, nx), xc = wrapped(xs + 1, nx), xd = wrapped(xs + 2, nx);
-    const float* src = static_cast<const float*>(a.src);
+    using P = typename StoreT<S>::P;
+    const P* src = static_cast<const P*>(a.src);
     const int64_t pl = a.plane;
+    const float k1 = 0.5f * (1.0f - c.theta), k5 = 0.25f * c.theta;   // (FP16S: pull_decode)
     struct Row {
         pair_t m1, m3, u2, u5, nu6, d4, d7, nd8;
     } s[RR];
     pair_t gx[RR], gy[RR];
     auto ld2 = [&](const float* p, int x0, int x1) { return pk(ldg(p + x0), ldg(p + x1)); };
+    // The populations pulled from memory row y; parts: 1 those with c_y = +1, 2
+    // those with c_y = 0, 4 those with c_y = -1 (6 and 8 negated).
+    auto pull = [&](int64_t y, int parts, Row& q) {
+        const int64_t row = y * a.pitch;
+        const P* p = src + row;
+        if constexpr (S == S_F32) {
+            if (parts & 2) {
+                q.m1 = ld2(p, xa, xb);
+                q.m3 = ld2(p + 2 * pl, xc, xd);
+            }
+            if (parts & 1) {
+                q.u2 = ld2(p + pl, xb, xc);
+                q.u5 = ld2(p + 4 * pl, xa, xb);
+                q.nu6 = ld2(p + 5 * pl, xc, xd);
+            }
+            if (parts & 4) {
+                q.d4 = ld2(p + 3 * pl, xb, xc);
+                q.d7 = ld2(p + 6 * pl, xc, xd);
+                q.nd8 = ld2(p + 7 * pl, xa, xb);
+            }
+        } else {
+            auto h2 = [&](int k, int x0, int x1) {
+                return pk(__half2float(ldg(p + k * pl + x0)), __half2float(ldg(p + k * pl + x1)));
+            };
+            const float2* cr = reinterpret_cast<const float2*>(a.csrc) + row;
+            const float2 ca_ = ldg(cr + xa), cb = ldg(cr + xb), cc = ldg(cr + xc), cd = ldg(cr + xd);
+            const pair_t l0 = pk(ca_.x, cb.x), l1 = pk(ca_.y, cb.y), r0 = pk(cc.x, cd.x), r1 = pk(cc.y, cd.y);
+            const pair_t m1 = pk(cb.y, cc.y);
+            if (parts & 2) {
+                q.m1 = fma2(splat(k1), l0, h2(0, xa, xb));
+                q.m3 = fma2(splat(-k1), r0, h2(2, xc, xd));
+            }
+            if (parts & 1) {
+                q.u2 = fma2(splat(k1), m1, h2(1, xb, xc));
+                q.u5 = fma2(splat(k5), add2(l0, l1), h2(4, xa, xb));
+                q.nu6 = fma2(splat(-k5), sub2(r0, r1), h2(5, xc, xd));
+            }
+            if (parts & 4) {
+                q.d4 = fma2(splat(-k1), m1, h2(3, xb, xc));
+                q.d7 = fma2(splat(-k5), add2(r0, r1), h2(6, xc, xd));
+                q.nd8 = fma2(splat(k5), sub2(l0, l1), h2(7, xa, xb));
+            }
+        }
+    };
 #pragma unroll
     for (int r = 0; r < RR; ++r) {
-        const int64_t row = (int64_t)wrapped(ys + r, ny) * a.pitch;
-        const float* p = src + row;
-        s[r].m1 = ld2(p, xa, xb);
-        s[r].u2 = ld2(p + pl, xb, xc);
-        s[r].m3 = ld2(p + 2 * pl, xc, xd);
-        s[r].d4 = ld2(p + 3 * pl, xb, xc);
-        s[r].u5 = ld2(p + 4 * pl, xa, xb);
-        s[r].nu6 = ld2(p + 5 * pl, xc, xd);
-        s[r].d7 = ld2(p + 6 * pl, xc, xd);
-        s[r].nd8 = ld2(p + 7 * pl, xa, xb);
-        gx[r] = ld2(static_cast<const float*>(a.gx) + row, xb, xc);
-        gy[r] = ld2(static_cast<const float*>(a.gy) + row, xb, xc);
+        const int y = wrapped(ys + r, ny);
+        pull(y, 7, s[r]);
+        gx[r] = ld2(static_cast<const float*>(a.gx) + (int64_t)y * a.pitch, xb, xc);
+        gy[r] = ld2(static_cast<const float*>(a.gy) + (int64_t)y * a.pitch, xb, xc);
     }
 #pragma unroll
     for (int r = 0; r < RR; ++r) {
@@ -1612,12 +1663,14 @@ k_tile(const StepParams a, const PairCoef ca, int T, int ntx) {
     put(slot(warp), s[RR - 1].u2, s[RR - 1].u5, s[RR - 1].nu6);
     put(slot(warp) + 768, s[0].d4, s[0].d7, s[0].nd8);
     if (warp == 0) {               // the row before the tile, whose upward movers step 1 pulls
-        const float* p = src + (int64_t)wrapped(ys - 1, ny) * a.pitch;
-        put(slot(-1), ld2(p + pl, xb, xc), ld2(p + 4 * pl, xa, xb), neg2(ld2(p + 5 * pl, xc, xd)));
+        Row q;
+        pull(wrapped(ys - 1, ny), 1, q);
+        put(slot(-1), q.u2, q.u5, neg2(q.nu6));
     }
     if (warp == nw - 1) {          // the row after it
-        const float* p = src + (int64_t)wrapped(ys + RR, ny) * a.pitch;
-        put(slot(nw) + 768, ld2(p + 3 * pl, xb, xc), ld2(p + 6 * pl, xc, xd), neg2(ld2(p + 7 * pl, xa, xb)));
+        Row q;
+        pull(wrapped(ys + RR, ny), 4, q);
+        put(slot(nw) + 768, q.d4, q.d7, neg2(q.nd8));
     }
     __syncthreads();
     const int s0 = 2 * lane;
@@ -1626,7 +1679,7 @@ k_tile(const StepParams a, const PairCoef ca, int T, int ntx) {
     acc.own0 = ok0;
     acc.own1 = ok1;
     // the check's snapshot entries of the coming row, loaded one row ahead
-    ResSnap<S_F32> sn[2];
+    ResSnap<S> sn[2];
     auto owned_row = [&](int r) {
         const int q = warp * RR + r;
         return q >= H && q < nw * RR - H && ys + r < ny;
@@ -1634,8 +1687,8 @@ k_tile(const StepParams a, const PairCoef ca, int T, int ntx) {
     auto snap_row = [&](int r) {
         if (!owned_row(r)) return;
         const int64_t idx = (int64_t)(ys + r) * a.pitch + xs;
-        if (ok0) sn[0] = snap_load<S_F32>(a, pl, idx);
-        if (ok1) sn[1] = snap_load<S_F32>(a, pl, idx + 1);
+        if (ok0) sn[0] = snap_load<S>(a, pl, idx);
+        if (ok1) sn[1] = snap_load<S>(a, pl, idx + 1);
     };
     for (int t = 0; t < T; ++t) {
         const bool last = t == T - 1;
@@ -1657,9 +1710,38 @@ k_tile(const StepParams a, const PairCoef ca, int T, int ntx) {
             }
             const Opp2 o = opposites2(s[r].m1, u2, s[r].m3, d4, u5, nu6, d7, nd8);
             const Post2 m = collide2<GEN>(moments2(o, c), gx[r], gy[r], c);
-            const Pop2<!GEN> w(m, c);
+            // the populations after the collision, or (FP16S, where the state is
+            // rounded: after the steps of `rounds`, and the last) the rounded
+            // deviations and the carriers
+            pair_t w[8], c10 = 0, c01 = 0;
+            const bool round = S == S_F16S && (last || (rounds >> t & 1));
+            if (!round) {
+                const Pop2<!GEN> q(m, c);
+                w[0] = q.f1(c);
+                w[1] = q.f2(c);
+                w[2] = q.f3(c);
+                w[3] = q.f4(c);
+                w[4] = q.f5();
+                w[5] = q.nf6();
+                w[6] = q.f7();
+                w[7] = q.nf8();
+            } else {
+                __half2 h[8];
+                round_state<GEN>(m, c, h, w, c10, c01);
+                if (!last) {
+                    const pair_t sum = add2(c10, c01), dif = sub2(c10, c01);
+                    w[0] = fma2(splat(k1), c10, w[0]);
+                    w[1] = fma2(splat(k1), c01, w[1]);
+                    w[2] = fma2(splat(-k1), c10, w[2]);
+                    w[3] = fma2(splat(-k1), c01, w[3]);
+                    w[4] = fma2(splat(k5), sum, w[4]);
+                    w[5] = fma2(splat(k5), dif, neg2(w[5]));
+                    w[6] = fma2(splat(-k5), sum, w[6]);
+                    w[7] = fma2(splat(-k5), dif, neg2(w[7]));
+                }
+            }
             if (last) {
-                ResSnap<S_F32> now[2];
+                ResSnap<S> now[2];
                 if (CHECK) {
                     now[0] = sn[0];
                     now[1] = sn[1];
@@ -1667,20 +1749,26 @@ k_tile(const StepParams a, const PairCoef ca, int T, int ntx) {
                 }
                 if (owned_row(r)) {
                     const int y = ys + r;
-                    pair_t fs[8];
-                    w.all(c, fs);
                     const int64_t idx = (int64_t)y * a.pitch + xs;
-                    float* d = static_cast<float*>(a.dst) + idx;
+                    P* d = static_cast<P*>(a.dst) + idx;
 #pragma unroll
                     for (int p = 0; p < 8; ++p) {
                         float lo, hi;
-                        unpk(fs[p], lo, hi);
-                        if (ok0) d[p * pl] = lo;
-                        if (ok1) d[p * pl + 1] = hi;
+                        unpk(S == S_F32 && (p == 5 || p == 7) ? neg2(w[p]) : w[p], lo, hi);
+                        if (ok0) d[p * pl] = P(lo);            // (FP16S: exact)
+                        if (ok1) d[p * pl + 1] = P(hi);
+                    }
+                    if constexpr (S == S_F16S) {
+                        float4 v;
+                        unpk(c10, v.x, v.z);
+                        unpk(c01, v.y, v.w);
+                        float2* cd = reinterpret_cast<float2*>(a.cdst) + idx;
+                        if (ok0) cd[0] = make_float2(v.x, v.y);
+                        if (ok1) cd[1] = make_float2(v.z, v.w);
                     }
                     if (CHECK) {
                         const pair_t f[8] = {s[r].m1, u2, s[r].m3, d4, u5, neg2(nu6), d7, neg2(nd8)};
-                        check_pair<S_F32>(acc, now[0], now[1], f, gx[r], gy[r],
+                        check_pair<S>(acc, now[0], now[1], f, gx[r], gy[r],
                                           [&](float2 u0, float2 v0, float2 u1, float2 v1) {
                                               float2* sp = static_cast<float2*>(a.snap) + idx;
                                               if (ok0) {
@@ -1698,14 +1786,14 @@ k_tile(const StepParams a, const PairCoef ca, int T, int ntx) {
             u2 = s[r].u2;
             u5 = s[r].u5;
             nu6 = s[r].nu6;
-            s[r].u2 = w.f2(c);
-            s[r].d4 = w.f4(c);
-            s[r].m1 = from_left(w.f1(c));
-            s[r].m3 = from_right(w.f3(c));
-            s[r].u5 = from_left(w.f5());
-            s[r].nu6 = from_right(w.nf6());
-            s[r].d7 = from_right(w.f7());
-            s[r].nd8 = from_left(w.nf8());
+            s[r].u2 = w[1];
+            s[r].d4 = w[3];
+            s[r].m1 = from_left(w[0]);
+            s[r].m3 = from_right(w[2]);
+            s[r].u5 = from_left(w[4]);
+            s[r].nu6 = from_right(w[5]);
+            s[r].d7 = from_right(w[6]);
+            s[r].nd8 = from_left(w[7]);
         }
         if (last) break;
         const uint32_t next = slot(warp) + (par_bytes - par);
@@ -2174,13 +2262,16 @@ inline int tile_smem(int NW) { return 2 * (NW + 2) * 6 * 256; }
 
 // The tile launch with the fewest modelled cycles per step.  Fitted to
 // launches back to back on GB300 (2 .. 12 steps, 4 .. 16 warps, one block per
-// multiprocessor): a step costs a warp about 50 + 97 w cycles per row with w
+// multiprocessor): an FP32 step costs a warp about 50 + 97 w cycles per row with w
 // warps on its scheduler; start, loads and stores together 3500 cycles and 145
-// per slot row of a multiprocessor.  16 warps are resident.
-inline TileShape tile_shape(int nx, int ny, int nsm) {
+// per slot row of a multiprocessor.  16 warps are resident.  FP16S (1 x 1 to
+// 1400 x 1400, 95 % of the launches within 20 %, the choice within 4 % of the best): 303 + 61 w cycles
+// per row and step, 49 w more where the state is rounded, which is every `group`
+// steps; a launch takes whole groups.
+inline TileShape tile_shape(int dtype, int group, int nx, int ny, int nsm) {
     TileShape best;
     for (int T = 2; T <= 12; ++T)
-        for (int RR = 2; RR <= 4; RR += 2)
+        for (int RR = 2; RR <= 4 && T % group == 0; RR += 2)
             for (int NW = 2; NW <= 16; ++NW) {
                 TileShape t;
                 t.T = T;
@@ -2191,7 +2282,10 @@ inline TileShape tile_shape(int nx, int ny, int nsm) {
                 const int64_t waves = (blocks + slots - 1) / slots;
                 const int64_t here = ((blocks < slots ? blocks : slots) + nsm - 1) / nsm * NW;   // warps
                 const double w = (double)((here + 3) / 4);
-                t.cost = 3500.0 + (double)waves * (145.0 * RR * here + T * RR * (50.0 + 97.0 * w));
+                if (dtype == S_F32)
+                    t.cost = 3500.0 + (double)waves * (145.0 * RR * here + T * RR * (50.0 + 97.0 * w));
+                else
+                    t.cost = 2000.0 + (double)waves * RR * (177.0 * here + T * (303.0 + 61.0 * w) + T / group * 49.0 * w);
                 if (best.T == 0 || t.cost * best.T < best.cost * t.T) best = t;
             }
     return best;
@@ -2201,6 +2295,10 @@ inline TileShape tile_shape(int nx, int ny, int nsm) {
 // step is the residual-check step (one partial set per block).
 cudaError_t tile_f32(const StepParams& a, const Coef<float>& c, bool gen, const TileShape& t, bool check,
                      cudaStream_t st);
+// The same of FP16-shifted storage; bit t of rounds: the state is rounded after
+// step t (as by a launch that ends there).
+cudaError_t tile_f16s(const StepParams& a, const Coef<float>& c, bool gen, const TileShape& t, bool check,
+                      unsigned rounds, cudaStream_t st);
 
 // T fused steps on the wavefront schedule (k_strip; FP32: T = 2 .. 6, FP16S:
 // T = 3, 4; check: T = 4, FP32 also 5, with the residual on the last step), segments of seg

@@ -1,5 +1,5 @@
-// Strip kernels (k_strip, three or four steps per launch) for the LBM_F16S
-// population storage.
+// Strip kernels (k_strip, three or four steps per launch) and register tiles for
+// the LBM_F16S population storage.
 #include "lbm_ops.cuh"
 
 namespace lbm {
@@ -11,5 +11,10 @@ cudaError_t strip_f16s(const StepParams& a, const Coef<float>& c, bool gen, int 
         case 4: return launch_strip_t<S_F16S, 4, false>(a, c, gen, seg, warps, st);
         default: return cudaErrorInvalidValue;
     }
+}
+
+cudaError_t tile_f16s(const StepParams& a, const Coef<float>& c, bool gen, const TileShape& t, bool check,
+                      unsigned rounds, cudaStream_t st) {
+    return launch_tile<S_F16S>(a, c, gen, t, check, rounds, st);
 }
 }  // namespace lbm

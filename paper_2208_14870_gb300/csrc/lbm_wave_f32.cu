@@ -19,40 +19,8 @@ cudaError_t strip_f32(const StepParams& a, const Coef<float>& c, bool gen, int T
     }
 }
 
-template <int RR, bool GEN, bool CHECK>
-static cudaError_t launch_tile_k(const StepParams& a, const Coef<float>& c, const TileShape& t, cudaStream_t st) {
-    static std::mutex mu;
-    static bool done[64] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    const auto kernel = k_tile<RR, GEN, CHECK>;
-    {
-        std::lock_guard<std::mutex> lock(mu);
-        if (!done[dev]) {
-            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, tile_smem(16));
-            if (e != cudaSuccess) return e;
-            done[dev] = true;
-        }
-    }
-    const int ox = kStSlots - 2 * (t.T - 1);
-    const int64_t blocks = tile_count(t, a.nx, a.ny);
-    if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-    return launch_after(kernel, dim3((unsigned)blocks), dim3(32 * t.NW), tile_smem(t.NW), st, a, pair_coef(c), t.T,
-                        (a.nx + ox - 1) / ox);
-}
-
-template <int RR>
-static cudaError_t launch_tile(const StepParams& a, const Coef<float>& c, bool gen, const TileShape& t, bool check,
-                               cudaStream_t st) {
-    if (gen) return check ? launch_tile_k<RR, true, true>(a, c, t, st) : launch_tile_k<RR, true, false>(a, c, t, st);
-    return check ? launch_tile_k<RR, false, true>(a, c, t, st) : launch_tile_k<RR, false, false>(a, c, t, st);
-}
-
 cudaError_t tile_f32(const StepParams& a, const Coef<float>& c, bool gen, const TileShape& t, bool check,
                      cudaStream_t st) {
-    if (t.T < 1 || t.NW < 1 || t.NW > 16 || t.NW * t.RR - 2 * (t.T - 1) < 1 || t.T > 16) return cudaErrorInvalidValue;
-    return t.RR == 2 ? launch_tile<2>(a, c, gen, t, check, st) : launch_tile<4>(a, c, gen, t, check, st);
+    return launch_tile<S_F32>(a, c, gen, t, check, 0, st);
 }
 }  // namespace lbm

@@ -128,6 +128,31 @@ def test_default_plan_equals_single_steps(nx, ny, kw):
             assert np.allclose(res[0][1], res[1][1], rtol=1e-12, atol=0.0), (steps, check)
 
 
+# FP16S: the default plan (tiles that round where a group of steps ends, strips)
+# against the same groups, one launch each: every group length (one, two, three
+# and four steps), lattices smaller than a tile, ragged ones, windows whose
+# groups do not divide them.
+@pytest.mark.parametrize("nx,ny", [(1, 1), (5, 3), (33, 64), (63, 30), (64, 23), (70, 24), (100, 15), (100, 75), (200, 300),
+                                   (255, 40), (256, 8), (300, 300), (90, 2413)])
+@pytest.mark.parametrize("kw", [dict(), dict(tau12=0.9, tau22=0.3)])
+def test_f16s_default_plan_equals_groups(nx, ny, kw):
+    lam, mu = W.lame_2d(1.0, 0.3)
+    rng = np.random.RandomState(nx * 1000 + ny)
+    gx, gy = rng.standard_normal((2, ny, nx)) / max(nx, ny) ** 2
+    for steps, check in ((1, 0), (2, 0), (7, 0), (29, 0), (29, 1), (40, 7), (41, 20)):
+        res = []
+        for groups in (True, False):
+            with Lattice(nx, ny, lam, mu, "f16s", **kw) as lat:
+                if groups:
+                    lat.steps_per_launch = lat.steps_per_launch
+                lat.set_force(gx, gy)
+                r = lat.iterate_checked(steps, check) if check else lat.iterate(steps)
+                res.append((lat.populations(), r))
+        assert np.array_equal(res[0][0], res[1][0]), (steps, check)
+        if check:
+            assert np.allclose(res[0][1], res[1][1], rtol=1e-12, atol=0.0), (steps, check)
+
+
 # FP64 tiles (k_tile64): several steps per launch against one step per launch
 # (an iterate call of one step is one), on lattices smaller than a tile, ragged
 # ones and large ones.
