@@ -212,11 +212,8 @@ __device__ __forceinline__ void collide_populations(const Mom<T>& m, T gx, T gy,
 // own rounding of the sums, and the first moments of the result are mbar + g / 2 up
 // to that last rounding.  About 600 integer instructions, two cycles of the ALU
 // for 360 of them, against 34 FP64 ones (2176 cycles): 1500 x 1100 116 -> 44 us
-// per step, 64 x 64 2.05 -> 1.45 us, before the FP64 pipe took some results:
-// three of them with few warps per scheduler (64 x 64: none 1.41 us, two 1.40,
-// three 1.39, five 1.52), four with many (WIDE; 1500 x 1100: none 42.6 us, two
-// 40.8, three 39.6, four and five 38.7, six 44.0), where the signs go to the FMA
-// pipe as well (38.7 against 40.5; with few warps 1.41 against 1.34).
+// per step; with the signs on the FMA pipe 42.6, and with two, three, four, five,
+// six of the results on the FP64 pipe 40.8, 39.6, 38.7, 38.7, 44.0 us.
 // Nodes of infinities, NaN or values near the ends of the exponent range, and
 // rates with a factor of 1/2 or more, take FP64 arithmetic.
 // m (below 2^63) with the sign of the word w.  FMA: most of the work on the FMA pipe (a multiplication by the sign) instead
@@ -271,13 +268,7 @@ __device__ __forceinline__ int64_t mul_fixed(Factor k, int64_t a) {
     return (int64_t)ah * k.hi + (t >> 31);
 }
 
-// The N-th of a node's results: the first three (WIDE: four) on the FP64 pipe.
-template <bool WIDE, int N>
-__device__ __forceinline__ double result(int64_t v, uint32_t e) {
-    return N < (WIDE ? 4 : 3) ? from_fixed_fp64(v, e) : from_fixed<WIDE>(v, e);
-}
-
-template <bool GEN, bool WIDE>
+template <bool GEN>
 __device__ __forceinline__ void step_f64(const double f[8], double gx, double gy, const Coef<double>& c, double& u,
                                          double& v, double o[8]) {
     uint32_t e = 0;
@@ -291,8 +282,8 @@ __device__ __forceinline__ void step_f64(const double f[8], double gx, double gy
     }
     int64_t F[8];
 #pragma unroll
-    for (int p = 0; p < 8; ++p) F[p] = to_fixed<WIDE>(f[p], e, 0);
-    const int64_t hx = to_fixed<WIDE>(gx, e, 1), hy = to_fixed<WIDE>(gy, e, 1);
+    for (int p = 0; p < 8; ++p) F[p] = to_fixed<true>(f[p], e, 0);
+    const int64_t hx = to_fixed<true>(gx, e, 1), hy = to_fixed<true>(gy, e, 1);
     const int64_t p = F[4] + F[6], q = F[5] + F[7], r = F[4] - F[6], s = F[5] - F[7];
     const int64_t m11 = p - q, m22 = p + q, m12 = r - s, m21 = r + s;
     const int64_t U = (F[0] - F[2]) + m12 + hx, V = (F[1] - F[3]) + m21 + hy;
@@ -307,16 +298,76 @@ __device__ __forceinline__ void step_f64(const double f[8], double gx, double gy
     // m*_10 - m*_12 and m*_01 - m*_21, halved without a loss
     const int64_t A = U + hx - 4 * Tu, B = V + hy - 4 * Tv, Ah = A >> 1, Bh = B >> 1;
     const int64_t P = S + D - 2 * W, Q = S - D - 2 * W;
-    o[0] = result<WIDE, 0>(P + Ah, e);
-    o[2] = result<WIDE, 1>(P - (A - Ah), e);
-    o[1] = result<WIDE, 2>(Q + Bh, e);
-    o[3] = result<WIDE, 3>(Q - (B - Bh), e);
-    o[4] = result<WIDE, 4>(W + X + (Tu + Tv), e);
-    o[6] = result<WIDE, 5>(W + X - (Tu + Tv), e);
-    o[5] = result<WIDE, 6>(W - X + (Tv - Tu), e);
-    o[7] = result<WIDE, 7>(W - X - (Tv - Tu), e);
+    o[0] = from_fixed_fp64(P + Ah, e);
+    o[2] = from_fixed_fp64(P - (A - Ah), e);
+    o[1] = from_fixed_fp64(Q + Bh, e);
+    o[3] = from_fixed_fp64(Q - (B - Bh), e);
+    o[4] = from_fixed<true>(W + X + (Tu + Tv), e);
+    o[6] = from_fixed<true>(W + X - (Tu + Tv), e);
+    o[5] = from_fixed<true>(W - X + (Tv - Tu), e);
+    o[7] = from_fixed<true>(W - X - (Tv - Tu), e);
     u = from_fixed<false>(U, e);
     v = from_fixed<false>(V, e);
+}
+
+// step_f64 of one node on two lanes, 2k (h = 0) and 2k + 1 (h = 1), for launches
+// of few warps: half the conversions each, 500 instructions in a row (with those of
+// k_tile64 around it) instead of 800.  Lane h holds populations h, h + 2, h + 4 and h + 6 in f[0 .. 3] and the
+// force's component h, and receives the same populations of the result and the
+// component w of the displacement.  The bits are step_f64's.  Every lane of the
+// warp calls it.  (No signs on the FMA pipe and no results on the FP64 pipe: with
+// one or two warps per scheduler both only lengthen the chain, 64 x 64 1.34
+// against 1.41 us per step.)
+template <bool GEN>
+__device__ __forceinline__ void step_f64_half(const double f[4], double g, int h, const Coef<double>& c, double& w,
+                                              double o[4]) {
+    constexpr unsigned ALL = 0xffffffffu;
+    uint32_t e = 0;
+#pragma unroll
+    for (int p = 0; p < 4; ++p) e = max(e, (uint32_t)__double2hiint(f[p]) & 0x7ff00000u);
+    e = max(e, (uint32_t)__double2hiint(g) & 0x7ff00000u);
+    e = max(e, __shfl_xor_sync(ALL, e, 1));
+    const bool slow = !c.fixed || e - (100u << 20) > (1900u << 20);
+    auto other = [&](int64_t v) { return __shfl_xor_sync(ALL, v, 1); };
+    const int64_t t = -h;                                    // (v ^ t) - t: v on lane 0, -v on lane 1
+    const int64_t A0 = to_fixed<false>(f[0], e, 0), A2 = to_fixed<false>(f[1], e, 0), B0 = to_fixed<false>(f[2], e, 0),
+                  B1 = to_fixed<false>(f[3], e, 0), H = to_fixed<false>(g, e, 1);
+    const int64_t sB = B0 + B1, dB = B0 - B1, sA = A0 + A2, dA = A0 - A2;
+    const int64_t sBo = other(sB), dBo = other(dB), sAo = other(sA);
+    const int64_t m = dB - ((dBo ^ t) - t);                  // m_12 = r - s, m_21 = s + r
+    const int64_t U = dA + m + H;
+    const int64_t X = mul_fixed(c.k11, ((sB - sBo) ^ t) - t);
+    const int64_t S = mul_fixed(c.ks, sA + sAo + 2 * (sB + sBo)), D = mul_fixed(c.kd, ((sA - sAo) ^ t) - t);
+    int64_t T = mul_fixed(c.kw12t, U), W = 0;                // (w_21 = w_12)
+    if (GEN) {
+        T += mul_fixed(c.k12, m);
+        W = mul_fixed(c.k22, sB + sBo);
+    }
+    const int64_t To = other(T);
+    const int64_t A = U + H - 4 * T, Ah = A >> 1, P = S + ((D ^ t) - t) - 2 * W;
+    const int64_t Xs = W + ((X ^ t) - t), Z = T + ((To ^ t) - t);
+    o[0] = from_fixed<false>(P + Ah, e);
+    o[1] = from_fixed<false>(P - (A - Ah), e);
+    o[2] = from_fixed<false>(Xs + Z, e);
+    o[3] = from_fixed<false>(Xs - Z, e);
+    w = from_fixed<false>(U, e);
+    if (__any_sync(ALL, slow)) {
+        double a[8], gx = __shfl_xor_sync(ALL, g, 1), gy = gx, u, v, r[8];
+        if (h) gy = g;
+        else gx = g;
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+            const double q = __shfl_xor_sync(ALL, f[p], 1);
+            a[2 * p] = h ? q : f[p];
+            a[2 * p + 1] = h ? f[p] : q;
+        }
+        if (slow) {
+            collide_populations<GEN>(moments(a), gx, gy, c, u, v, r);
+#pragma unroll
+            for (int p = 0; p < 4; ++p) o[p] = h ? r[2 * p + 1] : r[2 * p];
+            w = h ? v : u;
+        }
+    }
 }
 
 // Shifted FP16 storage.  The equilibrium-type part of a post-collision state

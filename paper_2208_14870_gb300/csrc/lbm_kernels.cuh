@@ -613,7 +613,7 @@ __device__ __forceinline__ void step_tile(const StepParams& a,
             const int64_t idx = r0 + x;
             if constexpr (S == S_F64) {
                 T u, v, fs[8];
-                step_f64<GEN, true>(f[j], gx[j], gy[j], c, u, v, fs);
+                step_f64<GEN>(f[j], gx[j], gy[j], c, u, v, fs);
                 store_state<S>(a, idx, fs, 0.0f, 0.0f);
                 if (CHECK) check_node<S>(a, n, idx, acc, so[j], f[j], gx[j], gy[j], u, v);
             } else {
@@ -679,6 +679,7 @@ __device__ __forceinline__ void push64(const StepParams& a, int idx, const doubl
 // A launch of FP64 storage: T steps; T > 1: blocks of bx x by nodes (k_tile64),
 // T = 1: k_one64.
 constexpr int kT64Max = 4;        // most steps per launch
+constexpr int kT64Smem = 48 * 1024;
 struct Tile64Shape {
     int T = 0, bx = 0, by = 0;
     int inv[kT64Max] = {};        // step t: 2^16 / (width of its slots), rounded up
@@ -689,61 +690,85 @@ struct Tile64Shape {
 // T pseudo-time steps per launch of FP64 storage (T >= 1, a run-time count).
 //
 // A step of a node is some 600 instructions in a row (step_f64), so a small
-// lattice has to be spread over all SMs, in whole warps: a block owns bx x by
-// nodes, holds the states between its steps in shared memory over a halo that
-// shrinks by one node per step, and its threads take the slots of a step in
-// linear order.  Several steps per launch recompute the halos but save launches;
-// tile64_shape weighs the two.  64 x 64: 1.39 us per step (8.3 with one step of
-// 64 x 8 tiles per launch, 2.05 with these tiles on the FP64 pipe).
+// lattice is spread over all SMs, and every node over two lanes (step_f64_half): a
+// block owns bx x by nodes, holds the states between its steps in shared memory
+// over a halo that shrinks by one node per step, and its threads take the slots
+// of a step in linear order.  The periodic images of the slots' columns and rows
+// come from a table that is made before the wait for the predecessor.  Several
+// steps per launch recompute the halos but save launches; tile64_shape weighs
+// the two.  64 x 64: 1.11 us per step (one lane per node 1.39, two without the
+// table 1.21; on the FP64 pipe 2.05, one step of 64 x 8 tiles per launch 8.3).
+// What is left is latency: of a launch's 2 us, and of about 0.5 us per step.
 template <bool GEN, bool CHECK>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(512)
 k_tile64(const StepParams a, const Coef<double> c, const __grid_constant__ Tile64Shape sh, int nty) {
     extern __shared__ double tile64_mem[];
-    const int nx = a.nx, ny = a.ny, H = sh.T - 1, sw = sh.bx + 2 * H, area = sw * (sh.by + 2 * H);
-    const int pitch = (int)a.pitch;
+    const int nx = a.nx, ny = a.ny, H = sh.T - 1, sw = sh.bx + 2 * H, sr = sh.by + 2 * H, area = sw * sr;
     ResAcc<S_F64> acc;
-    after_predecessor();
     const int x0 = (int)blockIdx.x * sh.bx - H;               // node of slot (0, 0)
+    // the lane's half of a node: populations h, h + 2, h + 4, h + 6 and the force's
+    // component h; f_p(x) = f*_p(x - c_p)
+    const int h = threadIdx.x & 1, d1 = h ? 1 : -1;
+    const int64_t pl = a.plane;
+    const double *src = static_cast<const double*>(a.src) + h * pl, *force = static_cast<const double*>(h ? a.gy : a.gx);
+    double* dst = static_cast<double*>(a.dst) + h * pl;
+    const int off0 = h * area + (h ? -sw : -1), off1 = (2 + h) * area + (h ? sw : 1), off2 = (4 + h) * area - sw + d1,
+              off3 = (6 + h) * area + sw - d1;
+    // lattice column, and first node of the lattice row, of the slots -1 .. sw, -1 .. sr
+    int* col = reinterpret_cast<int*>(tile64_mem + 16 * area) + 1;
+    int* row = col + sw + 2;
     for (int ty = blockIdx.y; ty < nty; ty += gridDim.y) {
         const int y0 = ty * sh.by - H;
+        for (int i = threadIdx.x; i < sw + sr + 4; i += blockDim.x) {
+            const bool c = i < sw + 2;
+            const int n = c ? nx : ny, v = (c ? x0 + i : y0 + i - (sw + 2)) - 1, m = v % n;
+            col[i - 1] = (m < 0 ? m + n : m) * (c ? 1 : (int)a.pitch);
+        }
+        __syncthreads();
+        after_predecessor();
         for (int t = 0; t <= H; ++t) {
             const bool last = t == H;
             const int aw = sw - 2 * t, count = aw * (sh.by + 2 * (H - t)), inv = sh.inv[t];
             const double* from = tile64_mem + (t & 1) * 8 * area;
             double* to = tile64_mem + ((t + 1) & 1) * 8 * area;
-            for (int i = threadIdx.x; i < count; i += blockDim.x) {
-                const int q = (i * inv) >> 16, sx = t + i - q * aw, sy = t + q;   // q = i / aw
-                int x = x0 + sx, y = y0 + sy;
-                if (last && (x >= nx || y >= ny)) continue;
-                if (!last) {
-                    x = wrap_slot<true>(x, nx);
-                    y = wrap_slot<true>(y, ny);
-                }
-                const int row = y * pitch, idx = row + x;
-                double f[8];
+            // two lanes per slot; whole warps go round, past the last slot too
+            for (int i = threadIdx.x; (i & ~31) < 2 * count; i += blockDim.x) {
+                const int slot = min(i >> 1, count - 1);
+                const int q = (slot * inv) >> 16, sx = t + slot - q * aw, sy = t + q;   // q = slot / aw
+                const bool own = (i >> 1) < count && (!last || (x0 + sx < nx && y0 + sy < ny));
+                const int x = col[sx], y = row[sy], idx = y + x, at = sy * sw + sx;
+                double f[4];
                 if (t == 0) {
-                    pull64(a, row, wrap_dec(y, ny) * pitch, wrap_inc(y, ny) * pitch, x, wrap_dec(x, nx), wrap_inc(x, nx), f);
+                    const int rm = row[sy - 1], rp = row[sy + 1], xl = col[sx + d1], xr = col[sx - d1];
+                    f[0] = ldg(src + (h ? rm + x : y + xl));
+                    f[1] = ldg(src + 2 * pl + (h ? rp + x : y + xr));
+                    f[2] = ldg(src + 4 * pl + (rm + xl));
+                    f[3] = ldg(src + 6 * pl + (rp + xr));
                 } else {
-                    const double* p = from + sy * sw + sx;
-                    f[0] = p[0 * area - 1];                   // f_p(x) = f*_p(x - c_p)
-                    f[1] = p[1 * area - sw];
-                    f[2] = p[2 * area + 1];
-                    f[3] = p[3 * area + sw];
-                    f[4] = p[4 * area - sw - 1];
-                    f[5] = p[5 * area - sw + 1];
-                    f[6] = p[6 * area + sw + 1];
-                    f[7] = p[7 * area + sw - 1];
+                    f[0] = from[at + off0];
+                    f[1] = from[at + off1];
+                    f[2] = from[at + off2];
+                    f[3] = from[at + off3];
                 }
-                const double gx = ldg(static_cast<const double*>(a.gx) + idx), gy = ldg(static_cast<const double*>(a.gy) + idx);
-                double u, v, fs[8];
-                step_f64<GEN, false>(f, gx, gy, c, u, v, fs);
-                if (last) {
-                    if (CHECK) check_node<S_F64>(a, a.plane, idx, acc, snap_load<S_F64>(a, a.plane, idx), f, gx, gy, u, v);
-                    push64(a, idx, fs);
-                } else {
-                    double* o = to + sy * sw + sx;
+                const double g = ldg(force + idx);
+                double w, fs[4];
+                step_f64_half<GEN>(f, g, h, c, w, fs);
+                if (!last) {
+                    if (own) {
 #pragma unroll
-                    for (int p = 0; p < 8; ++p) o[p * area] = fs[p];
+                        for (int p = 0; p < 4; ++p) to[at + (2 * p + h) * area] = fs[p];
+                    }
+                    continue;
+                }
+                if (CHECK) {
+                    const double v = __shfl_xor_sync(0xffffffffu, w, 1);
+                    const double zero[8] = {};
+                    if (own && h == 0)
+                        check_node<S_F64>(a, pl, idx, acc, snap_load<S_F64>(a, pl, idx), zero, 0.0, 0.0, w, v);
+                }
+                if (own) {
+#pragma unroll
+                    for (int p = 0; p < 4; ++p) (dst + 2 * p * pl)[idx] = fs[p];
                 }
             }
             if (H) __syncthreads();
@@ -754,8 +779,8 @@ k_tile64(const StepParams a, const Coef<double> c, const __grid_constant__ Tile6
 
 // One step per launch of FP64 storage (lattices of some 200 x 200 nodes and more):
 // blocks of 32 x 4 nodes.  1500 x 1100: 38.7 us per step, 238 MB of populations
-// and force at 6.1 TB/s (k_tile64 at T = 1 47 us, with 64-bit tile divisions and
-// addresses; on the FP64 pipe 116, with tiles of 64 x 8 137).
+// and force at 6.1 TB/s (with 64-bit tile divisions and
+// addresses 47; on the FP64 pipe 116, with tiles of 64 x 8 137).
 constexpr int kOne64Rows = 4;
 template <bool GEN, bool CHECK>
 __global__ void __launch_bounds__(32 * kOne64Rows)
@@ -772,7 +797,7 @@ k_one64(const StepParams a, const Coef<double> c, int nty) {
         pull64(a, row, wrap_dec(y, ny) * pitch, wrap_inc(y, ny) * pitch, x, wrap_dec(x, nx), wrap_inc(x, nx), f);
         const double gx = ldg(static_cast<const double*>(a.gx) + idx), gy = ldg(static_cast<const double*>(a.gy) + idx);
         double u, v, fs[8];
-        step_f64<GEN, true>(f, gx, gy, c, u, v, fs);
+        step_f64<GEN>(f, gx, gy, c, u, v, fs);
         if (CHECK) check_node<S_F64>(a, a.plane, idx, acc, snap_load<S_F64>(a, a.plane, idx), f, gx, gy, u, v);
         push64(a, idx, fs);
     }
@@ -2201,7 +2226,8 @@ inline StripShape strip_shape(int dtype, int T, bool check, int nx, int ny, int 
 }
 
 inline int tile64_smem(const Tile64Shape& t) {
-    return t.T > 1 ? 2 * 8 * 8 * (t.bx + 2 * (t.T - 1)) * (t.by + 2 * (t.T - 1)) : 0;
+    const int w = t.bx + 2 * (t.T - 1), h = t.by + 2 * (t.T - 1);
+    return t.T > 1 ? 2 * 8 * 8 * w * h + 4 * (w + h + 4) : 0;
 }
 // Blocks of bx x by nodes in two dimensions, at most `most` of them in all if
 // the width allows it (each then takes several, one below the other).
@@ -2223,23 +2249,24 @@ inline Tile64Shape tile64(int T, int bx, int by) {
 }
 
 // The FP64 launch with the fewest modelled cycles per step.  Fitted on GB300 (1 x 1
-// to 1500 x 1100, T = 1 .. 4; within 5 %): W warps of slots on an SM's scheduler
-// take 1060 W cycles (T = 1: 820 W), a step of a tile 1030 and a launch 2330
-// (T = 1: 3350) besides.  64 x 64: T = 4 on 8 x 4 nodes, 1.39 us per step (T = 3
-// 1.45, T = 1 2.09); 256 x 256: T = 1, 3.3 us (T = 2 on 16 x 8 3.5).
+// to 1500 x 1100, T = 1 .. 4; within 4 %, the choice within 2 % of the best): W
+// warps on an SM's scheduler take 660 W cycles in a tile (780 W in k_one64), a step
+// of a tile 320 and a launch 2830 (3290) besides.  64 x 64: T = 3 on 8 x 4 nodes,
+// 1.11 us per step (T = 1 2.1); 256 x 256: T = 1, 3.3 us (T = 2 on 16 x 16 3.9).
 inline Tile64Shape tile64_shape(int nx, int ny, int nsm) {
-    const int tiles[5][2] = {{8, 4}, {16, 4}, {8, 8}, {16, 8}, {32, 4}};
+    const int tiles[9][2] = {{4, 4}, {8, 2}, {16, 2}, {8, 4}, {16, 4}, {8, 8}, {16, 8}, {32, 4}, {16, 16}};
     Tile64Shape best;
     for (int T = 1; T <= kT64Max; ++T)
         for (const auto& b : tiles) {
             Tile64Shape t = tile64(T, b[0], b[1]);
+            if (tile64_smem(t) > kT64Smem) continue;
             const dim3 g = tile64_grid(t, nx, ny, (int64_t)1 << 40);
             const int64_t here = ((int64_t)g.x * ((ny + t.by - 1) / t.by) + nsm - 1) / nsm;   // tiles per SM
-            t.cost = T > 1 ? 2330.0 : 2320.0;
+            t.cost = T > 1 ? 2830.0 : 3290.0;
             for (int s = 0; s < T; ++s) {
                 const int slots = (t.bx + 2 * (T - 1 - s)) * (t.by + 2 * (T - 1 - s));
-                const int64_t warps = here * ((slots + 31) / 32);
-                t.cost += 1030.0 + (T > 1 ? 1060.0 : 820.0) * (double)((warps + 3) / 4);
+                const int64_t warps = here * (T > 1 ? (slots + 15) / 16 : (slots + 31) / 32);
+                t.cost += T > 1 ? 320.0 + 660.0 * (double)((warps + 3) / 4) : 780.0 * (double)((warps + 3) / 4);
             }
             if (best.T == 0 || t.cost * best.T < 0.999 * best.cost * t.T) best = t;
         }
