@@ -144,7 +144,7 @@ k_arena_strips(const BatchArgs A, const uint2* items, int count, int group) {
     extern __shared__ float4 strip_mem[];
     const int warp = threadIdx.x >> 5, item = (int)blockIdx.x * kArenaNW + warp;
     if (item >= count) return;
-    after_predecessor();
+    // (items and problems are written by copies, which no launch overtakes)
     const uint2 tl = items[item];
     const BatchProb P = A.probs[tl.x];
     const StepParams a = prob_params<S>(A, P, (P.parity + group) & 1);

@@ -1269,7 +1269,9 @@ __device__ __forceinline__ void round_state(const Post2& m, const PairCoef& c, _
 // beyond either end hold the periodic images, so that a strip's rows are
 // contiguous and its copies aligned wherever it lies; the strips that own the
 // outermost kGhost columns store their images too.
-// OX: output columns of a strip (at most st_ox).
+// OX: output columns of a strip (at most st_ox).  Waits for the previous launch
+// (after_predecessor) just before the first copy: 1024^2 1.684 -> 1.669 ms per 400
+// steps, FP16S 1000 x 700 1.664 -> 1.637.
 template <int S, bool GEN, int T, bool CHECK, int OX = st_ox<S, T>()>
 __device__ __forceinline__ void strip_walk(const StepParams& a, const PairCoef& ca, uint32_t sm, int strip, int y0,
                                            int rows, ResAcc2& acc) {
@@ -1537,6 +1539,7 @@ __device__ __forceinline__ void strip_walk(const StepParams& a, const PairCoef& 
 
     using K0 = std::integral_constant<int, 0>;
     using K1 = std::integral_constant<int, 1>;
+    after_predecessor();
 #pragma unroll
     for (int r = 0; r < AHEAD; ++r) copy_row(r);
     int i = 0;
@@ -1555,7 +1558,6 @@ k_strip(const StepParams a, const PairCoef c, int seg, int nstrips, int items) {
     extern __shared__ float4 st_mem[];
     const int warp = threadIdx.x >> 5;
     const int item = (int)blockIdx.x * kStNW + warp;
-    after_predecessor();
     ResAcc2 acc;
     if (item < items) {
         const int strip = item % nstrips, y0 = (item / nstrips) * seg;
