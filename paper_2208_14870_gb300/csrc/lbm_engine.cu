@@ -488,13 +488,12 @@ int ArenaEngine::launch_strip_chunk(std::string* err) {
     return LBM_OK;
 }
 
-int ArenaEngine::run_chunk(int V, float* device_ms, std::string* err) {
+int ArenaEngine::start_chunk(int V, std::string* err) {
     if (V != 1 && V != 2 && V != 4 && !(V == kTileTwoStep && k_ % 2 == 0) && !(V == kTileWave && k_ % 4 == 0)) {
         if (err) *err = "arena: tile code must be 1, 2 or 4 warps of 32, two-step tiles with an even chunk, "
                         "or the wavefront chunk with a chunk of a multiple of 4 steps";
         return LBM_ERR_ARG;
     }
-    if (device_ms) *device_ms = 0.0f;
     if (nrunning_ == 0) return LBM_OK;
     if (tiles_dirty_ || tiles_V_ != V) {
         int rc = upload_tiles(V, err);
@@ -553,6 +552,12 @@ int ArenaEngine::run_chunk(int V, float* device_ms, std::string* err) {
         ECK(cudaMemcpyAsync(h_acc_, d_acc_, sizeof(double) * kRes * probs_.size(), cudaMemcpyDeviceToHost, st_));
     }
     ECK(cudaEventRecord(ev1_, st_));
+    return LBM_OK;
+}
+
+int ArenaEngine::finish_chunk(int V, float* device_ms, std::string* err) {
+    if (device_ms) *device_ms = 0.0f;
+    if (nrunning_ == 0) return LBM_OK;
     ECK(cudaStreamSynchronize(st_));
     if (device_ms) ECK(cudaEventElapsedTime(device_ms, ev0_, ev1_));
     for (int s = 0; s < (int)probs_.size(); ++s) {

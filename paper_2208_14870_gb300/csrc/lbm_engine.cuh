@@ -72,9 +72,16 @@ public:
     // LBM_ERR_ARG if a problem admitted since init has a non-finite force entry
     // (FP16S problems are refused by admit already).
     int check_forces(std::string* err);
-    // One chunk of check_every steps for every running problem; afterwards
-    // finished problems are in state P_DONE (not yet released).
-    int run_chunk(int V, float* device_ms, std::string* err);
+    // One chunk of check_every steps for every running problem, launched on the
+    // engine's streams, and the wait for it; afterwards finished problems are in
+    // state P_DONE (not yet released).  No other call between the two.
+    int start_chunk(int V, std::string* err);
+    int finish_chunk(int V, float* device_ms, std::string* err);
+    int run_chunk(int V, float* device_ms, std::string* err) {
+        if (device_ms) *device_ms = 0.0f;
+        const int rc = start_chunk(V, err);
+        return rc ? rc : finish_chunk(V, device_ms, err);
+    }
     // Solution fields of count finished (or running) problems into host arrays,
     // FP64, lattice units; outs holds 5 nullable host arrays (ux, uy, sxx, syy,
     // sxy) per problem.

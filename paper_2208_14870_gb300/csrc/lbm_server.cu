@@ -121,8 +121,15 @@ void lbm_server::run() {
         lk.unlock();
         std::string err;
         float ms[2] = {0.0f, 0.0f};
+        // Strip chunks of the two arenas run side by side: neither fills the GPU with
+        // small problems (12 of them, 100 steps: 1.19 -> 1.08 ms).  The other chunk
+        // kernels meet at grid barriers and have the device to themselves.
+        const bool both = tile_v == kTileWave;
         for (int a = 0; a < 2 && rc == LBM_OK; ++a)
-            if (arena[a]->running() > 0) rc = arena[a]->run_chunk(tile_v, &ms[a], &err);
+            if (arena[a]->running() > 0)
+                rc = both ? arena[a]->start_chunk(tile_v, &err) : arena[a]->run_chunk(tile_v, &ms[a], &err);
+        for (int a = 0; a < 2 && rc == LBM_OK && both; ++a)
+            if (arena[a]->running() > 0) rc = arena[a]->finish_chunk(tile_v, &ms[a], &err);
         lk.lock();
         if (rc != LBM_OK) {
             failed = rc;
@@ -130,7 +137,7 @@ void lbm_server::run() {
             break;
         }
         ++chunks;
-        device_ms += ms[0] + ms[1];
+        device_ms += both ? std::max(ms[0], ms[1]) : ms[0] + ms[1];   // (side by side: the longer one)
         for (auto& q : queue) {
             auto it = reqs.find(q);
             if (it != reqs.end()) ++it->second->bypassed;
