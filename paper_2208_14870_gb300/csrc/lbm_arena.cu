@@ -1,6 +1,8 @@
 // lbm_arena.cu -- the kernels of the packed lattice arena (see lbm_arena.cuh):
 // strip items, and the persistent chunk kernels, one instantiation per storage
 // type (FP32, FP16-shifted) and tile width.
+#include <mutex>
+
 #include "lbm_arena.cuh"
 
 namespace lbm {
@@ -154,13 +156,13 @@ k_arena_strips(const BatchArgs A, const uint2* items, int count, int group) {
     const uint32_t sm = (uint32_t)__cvta_generic_to_shared(strip_mem) + warp * st_warp_smem<S, T, CHECK>();
     ResAcc2 acc;
     if (CHECK && P.check) {
-        strip_walk<S, false, T, true, kArenaOX>(a, c, sm, strip, y0, rows, acc);
+        strip_walk<S, false, T, true, kArenaOX>(a, c, sm, strip, y0, rows, acc, P.half != 0);
         double w[kRes];
         acc.to_double(w);
         warp_reduce_res(w);
         if ((threadIdx.x & 31) == 0) add_to_problem(A.acc + (int64_t)tl.x * kRes, w);
     } else {
-        strip_walk<S, false, T, false, kArenaOX>(a, c, sm, strip, y0, rows, acc);
+        strip_walk<S, false, T, false, kArenaOX>(a, c, sm, strip, y0, rows, acc, P.half != 0);
     }
 }
 
@@ -231,11 +233,27 @@ cudaError_t launch_arena_force(const ForceIn& f, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+// A kernel's dynamic shared memory above 48 KB, allowed once per device.
+template <auto* KERNEL>
+static cudaError_t allow_smem_once(int bytes) {
+    static std::mutex mu;
+    static bool done[64] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    std::lock_guard<std::mutex> lock(mu);
+    if (done[dev]) return cudaSuccess;
+    e = cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    done[dev] = e == cudaSuccess;
+    return e;
+}
+
 template <int S, int T, bool CHECK>
 static cudaError_t launch_strips_k(const BatchArgs& a, const uint2* items, int count, int group, cudaStream_t st) {
     constexpr int SM = kArenaNW * st_warp_smem<S, T, CHECK>();
     const auto kernel = k_arena_strips<S, T, CHECK>;
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SM);
+    const cudaError_t e = allow_smem_once<k_arena_strips<S, T, CHECK>>(SM);
     if (e != cudaSuccess) return e;
     return launch_after(kernel, dim3((unsigned)((count + kArenaNW - 1) / kArenaNW)), dim3(32 * kArenaNW), SM, st, a, items,
                         count, group);
@@ -247,9 +265,6 @@ cudaError_t launch_arena_strips(int dtype, int T, bool check, const BatchArgs& a
         if (T == 4)
             return check ? launch_strips_k<S_F16S, 4, true>(a, items, count, group, st)
                          : launch_strips_k<S_F16S, 4, false>(a, items, count, group, st);
-        if (T == 2)
-            return check ? launch_strips_k<S_F16S, 2, true>(a, items, count, group, st)
-                         : launch_strips_k<S_F16S, 2, false>(a, items, count, group, st);
         return cudaErrorInvalidValue;
     }
     if (check) {
@@ -266,7 +281,7 @@ cudaError_t launch_arena_strips(int dtype, int T, bool check, const BatchArgs& a
 
 template <int S, bool CHECK>
 static cudaError_t launch_pairs_k(const BatchArgs& a, const uint2* items, int count, int group, cudaStream_t st) {
-    const cudaError_t e = cudaFuncSetAttribute(k_arena_pairs<S, CHECK>, cudaFuncAttributeMaxDynamicSharedMemorySize, kT2Smem);
+    const cudaError_t e = allow_smem_once<k_arena_pairs<S, CHECK>>(kT2Smem);
     if (e != cudaSuccess) return e;
     return launch_after(k_arena_pairs<S, CHECK>, dim3((unsigned)count), dim3(kT2Threads), kT2Smem, st, a, items, group);
 }

@@ -41,6 +41,7 @@ struct BatchProb {
     int64_t plane;     // elements between planes
     int nx, ny, pitch, check, dtype, parity;   // check: this chunk's last step checks
     int seg;                            // strip chunk: rows per item
+    int half;                           // ... FP16S: the state is rounded after every second step
     float q11, qs, qd, qtheta, theta, hscale, hinv;   // rates in the quarter form of collide
 };
 
@@ -113,8 +114,9 @@ private:
 constexpr int kTileTwoStep = 3;
 
 // Tile code of the strip chunk: every launch advances the listed items by a
-// group of steps (FP32 five; FP16S four for lattices from 256 x 8 on and two for
-// smaller ones, as its states round to FP16 where a launch ends).  Strips have
+// group of steps (FP32 five; FP16S four, of which lattices below 256 x 8 round
+// their state after the second one too: in launches of their own, two steps each,
+// 12 small problems of a server took 1.08 ms per 100 steps instead of 0.94).  Strips have
 // kArenaOX output columns whatever the group, so that one item list serves a
 // chunk; problems without ghost columns take pairs of steps on two-step tiles.
 // Chunk lengths: multiples of 4.

@@ -238,7 +238,7 @@ int ArenaEngine::admit(int nx, int ny, double lambda, double mu, const double* g
     ECK(cudaMemsetAsync(pop_[0] + p.pop_off, 0, p.pop_bytes, st_));
     if (dtype_ == S_F16S) ECK(cudaMemsetAsync(car_[0] + p.car_off, 0, p.car_bytes, st_));
     p.parity = 0;
-    p.cls = !p.ghost ? C_PAIRS : (dtype_ == S_F16S && !arena_wide(p.nx, p.ny) ? C_SHORT : C_LONG);
+    p.cls = p.ghost ? C_STRIPS : C_PAIRS;
     p.lambda = lambda;
     p.mu = mu;
     // Table 1 / Eq. relaxation_rate with theta = 1/3, w_12 = w_21 = w_22 = 1
@@ -447,7 +447,7 @@ int ArenaEngine::ensure_graph(int V, std::string* err) {
 // Steps of the launches that advance a class of problems by a chunk of k steps
 // (k a multiple of 4); the last one carries the check.
 static std::vector<int> chunk_groups(int dtype, int cls, int k) {
-    if (cls == C_PAIRS || cls == C_SHORT) return std::vector<int>(k / 2, 2);
+    if (cls == C_PAIRS) return std::vector<int>(k / 2, 2);
     if (dtype == S_F16S || k < 5) return std::vector<int>(k / 4, 4);
     // fives after the rest (two threes where it would be one step)
     std::vector<int> g;
@@ -525,6 +525,7 @@ int ArenaEngine::start_chunk(int V, std::string* err) {
             b.dtype = dtype_;
             b.parity = p.parity;
             b.seg = wave_seg_;
+            b.half = dtype_ == S_F16S && !arena_wide(p.nx, p.ny) ? 1 : 0;
             b.q11 = p.q11;
             b.qs = p.qs;
             b.qd = p.qd;

@@ -15,10 +15,9 @@ namespace lbm {
 
 enum ProbState { P_FREE = 0, P_RUNNING = 1, P_DONE = 2 };
 
-// Strip chunk: strips of the storage type's long groups (FP32 five steps, FP16S
-// four), strips of pairs of steps (FP16S below 256 x 8), two-step tiles
+// Strip chunk: strips (FP32 five steps per launch, FP16S four), or two-step tiles
 // (problems without ghost columns).
-enum ProbClass { C_LONG = 0, C_SHORT = 1, C_PAIRS = 2, kClasses = 3 };
+enum ProbClass { C_STRIPS = 0, C_PAIRS = 1, kClasses = 2 };
 
 struct HostProb {
     int state = P_FREE;
@@ -127,11 +126,11 @@ private:
     uint2* d_tiles_ = nullptr;
     int64_t tiles_cap_ = 0;
     int* d_ntiles_ = nullptr;
-    int class_begin_[kClasses + 1] = {0, 0, 0, 0};   // strip chunk: item ranges of the classes
+    int class_begin_[kClasses + 1] = {};   // strip chunk: item ranges of the classes
     int strip_blocks_ = 0;                            // largest launch so far
     int ghosts_begin_ = 0, ghosts_end_ = 0;           // ... and of the problems whose ghost columns are stale
-    cudaStream_t side_[kClasses - 1] = {nullptr, nullptr};   // the classes run side by side
-    cudaEvent_t fork_ = nullptr, join_[kClasses - 1] = {nullptr, nullptr};
+    cudaStream_t side_[kClasses - 1] = {};   // the classes run side by side
+    cudaEvent_t fork_ = nullptr, join_[kClasses - 1] = {};
     uint2* h_tiles_ = nullptr;        // pinned
     int64_t h_tiles_cap_ = 0;
     int tiles_V_ = 0;                 // V the device tile list was built for

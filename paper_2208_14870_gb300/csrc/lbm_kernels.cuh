@@ -1269,12 +1269,13 @@ __device__ __forceinline__ void round_state(const Post2& m, const PairCoef& c, _
 // beyond either end hold the periodic images, so that a strip's rows are
 // contiguous and its copies aligned wherever it lies; the strips that own the
 // outermost kGhost columns store their images too.
+// half (FP16S): the state is rounded after every second step, as by launches of two.
 // OX: output columns of a strip (at most st_ox).  Waits for the previous launch
 // (after_predecessor) just before the first copy: 1024^2 1.684 -> 1.669 ms per 400
 // steps, FP16S 1000 x 700 1.664 -> 1.637.
 template <int S, bool GEN, int T, bool CHECK, int OX = st_ox<S, T>()>
 __device__ __forceinline__ void strip_walk(const StepParams& a, const PairCoef& ca, uint32_t sm, int strip, int y0,
-                                           int rows, ResAcc2& acc) {
+                                           int rows, ResAcc2& acc, bool half = false) {
     static_assert(OX % 2 == 0 && OX <= st_ox<S, T>(), "pairs, within the slots");
     constexpr int LAG = st_lag<S>(), H = st_halo<S, T>(), HL = st_left<S, T>(),
                   LA = st_la<S>(), R = st_ring<S, T>(), ROW = st_row<S>();
@@ -1405,6 +1406,24 @@ __device__ __forceinline__ void strip_walk(const StepParams& a, const PairCoef& 
             mid[b][0] = from_left(g(1));
             mid[b][1] = from_right(g(3));
         };
+        // Over boundary b: the state of rounded deviations (6 and 8 negated) and
+        // carriers, decoded (pull_decode).
+        auto cross_rounded = [&](int b, pair_t c10, pair_t c01, auto&& stored) {
+            const float k1 = 0.5f * (1.0f - c.theta), k5 = 0.25f * c.theta;
+            const pair_t sum = add2(c10, c01), dif = sub2(c10, c01);
+            cross(b, [&](int p) {
+                switch (p) {
+                    case 1: return fma2(splat(k1), c10, stored(0));
+                    case 2: return fma2(splat(k1), c01, stored(1));
+                    case 3: return fma2(splat(-k1), c10, stored(2));
+                    case 4: return fma2(splat(-k1), c01, stored(3));
+                    case 5: return fma2(splat(k5), sum, stored(4));
+                    case 6: return fma2(splat(k5), dif, stored(5));
+                    case 7: return fma2(splat(-k5), sum, stored(6));
+                    default: return fma2(splat(-k5), dif, stored(7));
+                }
+            });
+        };
         if constexpr (S == S_F32) {
             // f_p(x) = f*_p(x - c_p), from rows i - 1, i and i + 1 (local rows
             // of the copies start one above the strip's, hence the + 1)
@@ -1427,30 +1446,15 @@ __device__ __forceinline__ void strip_walk(const StepParams& a, const PairCoef& 
 #pragma unroll
                 for (int p = 0; p < 8; ++p) f[p] = w[p];
         } else {
-            // the populations of the lane's columns in row i (pull_decode)
+            // the populations of the lane's columns in row i
             const uint32_t r = sm + (i & (kWvD - 1)) * ROW;
-            const float k1 = 0.5f * (1.0f - c.theta), k5 = 0.25f * c.theta;
             pair_t e0, e1;                        // (m*_10, m*_01) of either column
             lds_pairs(r + kStCols * 16 + own * 8, e0, e1);
-            const pair_t c10 = pk(pk_lo(e0), pk_lo(e1)), c01 = pk(pk_hi(e0), pk_hi(e1));
-            const pair_t sum = add2(c10, c01), dif = sub2(c10, c01);
-            auto stored = [&](int p) {            // (populations 6 and 8 cross negated)
+            cross_rounded(0, pk(pk_lo(e0), pk_lo(e1)), pk(pk_hi(e0), pk_hi(e1)), [&](int p) {
                 uint32_t h = lds_u32(r + (p * kStCols + own) * 2);
                 if (p == 5 || p == 7) h ^= 0x80008000u;
                 const float2 v = __half22float2(*reinterpret_cast<__half2*>(&h));
                 return pk(v.x, v.y);
-            };
-            cross(0, [&](int p) {
-                switch (p) {
-                    case 1: return fma2(splat(k1), c10, stored(0));
-                    case 2: return fma2(splat(k1), c01, stored(1));
-                    case 3: return fma2(splat(-k1), c10, stored(2));
-                    case 4: return fma2(splat(-k1), c01, stored(3));
-                    case 5: return fma2(splat(k5), sum, stored(4));
-                    case 6: return fma2(splat(k5), dif, stored(5));
-                    case 7: return fma2(splat(-k5), sum, stored(6));
-                    default: return fma2(splat(-k5), dif, stored(7));
-                }
             });
         }
 #pragma unroll
@@ -1459,6 +1463,13 @@ __device__ __forceinline__ void strip_walk(const StepParams& a, const PairCoef& 
             const uint32_t fr = frc + ((i + OFF - LAG - (j - 1)) & (R - 1)) * kStFRow + own * 4;
             const pair_t gx = lds_pair(fr), gy = lds_pair(fr + kStCols * 4);
             const Post2 m = collide2<GEN>(moments2(o, c), gx, gy, c);
+            if (S == S_F16S && j < T && j % 2 == 0 && half) {
+                __half2 h[8];
+                pair_t w[8], c10, c01;
+                round_state<GEN>(m, c, h, w, c10, c01);
+                cross_rounded(j - 1 + LAG, c10, c01, [&](int p) { return p == 5 || p == 7 ? neg2(w[p]) : w[p]; });
+                continue;
+            }
             if (j < T) {
                 const Pop2<!GEN> w(m, c);
                 cross(j - 1 + LAG, [&](int p) {
