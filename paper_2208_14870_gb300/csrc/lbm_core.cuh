@@ -41,13 +41,15 @@ inline Factor factor(double v) {
     const int64_t b = llrint(ldexp(v, 64));
     return {(int)(b >> 32), (int)((uint32_t)b >> 1)};
 }
-// The same constants as factors (FP64 storage); fixed: all of them are in range.
+// The same constants as factors (FP64 storage); fixed, fields_fixed: all of them
+// are in range.
 template <typename T>
 struct CoefFixed {};
 template <>
 struct CoefFixed<double> {
     Factor k11, ks, kd, kw12t, k12, kw21t, k21, k22;
-    int fixed;
+    Factor h11, hs, hd;            // -b / 2 of the bared moments (recovery of the fields)
+    int fixed, fields_fixed;
 };
 
 // Per-lattice constants of the collision in compute precision, in the
@@ -71,6 +73,13 @@ inline void set_factors(Coef<double>& c) {
     for (int i = 0; i < 8; ++i) {
         if (fabs(q[i]) < 0.499) *k[i] = factor(q[i]);
         else c.fixed = 0;
+    }
+    const double b[3] = {-0.5 * c.b11, -0.5 * c.bs, -0.5 * c.bd};
+    Factor* h[3] = {&c.h11, &c.hs, &c.hd};
+    c.fields_fixed = 1;
+    for (int i = 0; i < 3; ++i) {
+        if (fabs(b[i]) < 0.499) *h[i] = factor(b[i]);
+        else c.fields_fixed = 0;
     }
 }
 
@@ -238,6 +247,14 @@ __device__ __forceinline__ int64_t to_fixed(double x, uint32_t e, int h) {
     uint64_t m = ((uint64_t)((hi & 0x000fffffu) | 0x00100000u) << 32 | lo) << (5 - h);
     asm("shr.u64 %0, %0, %1;" : "+l"(m) : "r"(d));                 // (64 and more: zero)
     return signed_as<FMA>(m, (int)hi);
+}
+// An FP32 x as a multiple of 2^-58 of the power of two above the largest value of
+// exponent field e.
+__device__ __forceinline__ int64_t to_fixed(float x, uint32_t e, int h) {
+    const uint32_t b = __float_as_uint(x), d = (e - (b & 0x7f800000u)) >> 23;
+    uint64_t m = (uint64_t)((b & 0x007fffffu) | 0x00800000u) << (34 - h);
+    asm("shr.u64 %0, %0, %1;" : "+l"(m) : "r"(d));
+    return signed_as<true>(m, (int)b);
 }
 // v units (|v| < 2^63), rounded to FP64 (ties to even).
 template <bool FMA>

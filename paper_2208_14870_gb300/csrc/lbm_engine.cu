@@ -644,6 +644,7 @@ cudaError_t ArenaEngine::launch_fields(int slot, double* dst) {
     c.bs = 1.0 - 0.5 * ws;
     c.bd = 1.0 - 0.5 * wd;
     c.theta = theta;
+    set_factors(c);
     FieldOut o = field_planes(dst, p.n);
     if (p.tr) {
         // back to the caller's lattice: u_x <-> u_y, sigma_xx <-> sigma_yy,

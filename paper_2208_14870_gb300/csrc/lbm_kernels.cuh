@@ -1860,15 +1860,6 @@ inline FieldOut field_planes(double* out, int64_t n) {
     return o;
 }
 
-// x 2^(e - 896) in FP64 (e in [836, 956]) by integer operations: the conversion
-// instructions run on the FP64 pipe.  A subnormal, infinity or NaN sets odd (and
-// gives no meaningful value).
-__device__ __forceinline__ double to_double(float x, int e, bool& odd) {
-    const uint32_t b = __float_as_uint(x), m = b & 0x7fffffffu;
-    odd |= m != 0 && m - 0x00800000u >= 0x7f000000u;
-    const uint32_t hi = (b & 0x80000000u) | (m ? (m >> 3) + ((uint32_t)e << 20) : 0u);
-    return __hiloint2double((int)hi, (int)(m << 29));
-}
 // log2 of a power of two.
 __device__ __forceinline__ int ilogb2(float p) { return (int)(__float_as_uint(p) >> 23) - 127; }
 
@@ -1889,56 +1880,62 @@ k_fields(const StepParams a, const Coef<double> c, typename StoreT<S>::T theta, 
     gather<S>(a, r0, rm, rp, x, wrap_dec(x, nx), wrap_inc(x, nx), f, theta);
     const int64_t idx = r0 + x;
     const G gxs = static_cast<const G*>(a.gx)[idx], gys = static_cast<const G*>(a.gy)[idx];
-    // FP64 work is what bounds the recovery on GB300 (64 cycles of a scheduler
-    // per warp instruction): nine FP64 instructions per node.  cs, cd: the
-    // factors of Eq. compute_bared with Table 2's -1/2.
-    const double cs = -0.5 * c.bs, cd = -0.5 * c.bd;
-    double u, v, m11, ms, md;
-    if constexpr (S == S_F64) {
-        const Mom<double> m = moments(f);
-        u = m.m10 + 0.5 * gxs;
-        v = m.m01 + 0.5 * gys;
-        m11 = m.m11;
-        ms = m.ms;
-        md = m.md;
+    // In integers, as the FP64 collision (step_f64): FP64 arithmetic, 64 cycles of a
+    // scheduler per warp instruction, would bound the recovery.  The unit is 2^-58
+    // of the power of two above the node's largest value, so every sum of FP32
+    // values is exact to a unit (pairs of FP32 sums were to 2^-44); sxx, syy, sxy
+    // are Eq. compute_bared with Table 2's factors.  Three of the five results leave
+    // through the FP64 pipe (16384^2 FP32: none 4.63 ms, two 4.48, three 4.26, four
+    // 4.64; five with nine FP64 instructions per node 5.57, all in FP64 10.3).
+    uint32_t e = 0;
+    auto top = [&](auto v) {
+        if constexpr (S == S_F64) e = max(e, (uint32_t)__double2hiint(v) & 0x7ff00000u);
+        else e = max(e, __float_as_uint(v) & 0x7f800000u);
+    };
+#pragma unroll
+    for (int p = 0; p < 8; ++p) top(f[p]);
+    top(gxs);
+    top(gys);
+    double u, v, sxx, syy, mb11;
+    const bool fixed = c.fields_fixed && (S == S_F64 ? e - (100u << 20) <= (1900u << 20) : e - (64u << 23) < (191u << 23));
+    if (fixed) {
+        auto fix = [&](auto w, int h) {
+            if constexpr (S == S_F64) return to_fixed<true>(w, e, h);
+            else return to_fixed(w, e, h);
+        };
+        int64_t F[8];
+#pragma unroll
+        for (int p = 0; p < 8; ++p) F[p] = fix(f[p], 0);
+        const int64_t hx = fix(gxs, 1), hy = fix(gys, 1);
+        const int64_t p = F[4] + F[6], q = F[5] + F[7], r = F[4] - F[6], s = F[5] - F[7];
+        const int64_t U = (F[0] - F[2]) + (r - s) + hx, V = (F[1] - F[3]) + (r + s) + hy;
+        const int64_t s13 = F[0] + F[2], s24 = F[1] + F[3];
+        const int64_t X = mul_fixed(c.h11, p - q), P = mul_fixed(c.hs, s13 + s24 + 2 * (p + q)), D = mul_fixed(c.hd, s13 - s24);
+        // exponent field of the same power of two in FP64 (FP16S: out of the state's scaled units)
+        const uint32_t e64 = S == S_F64 ? e : (e >> 3) + ((uint32_t)(896 - (S == S_F16S ? ilogb2(a.hscale) : 0)) << 20);
+        u = from_fixed_fp64(U, e64);
+        v = from_fixed_fp64(V, e64);
+        sxx = from_fixed_fp64(P + D, e64);
+        syy = from_fixed<true>(P - D, e64);
+        mb11 = from_fixed<true>(-2 * X, e64);
     } else {
-        // FP32 populations: the moments as exact FP32 pairs (TwoSum), converted
-        // by integer operations (out of the state's scaled units on the way,
-        // FP16S) and joined in FP64 once
-        const int e = S == S_F16S ? 896 - ilogb2(a.hscale) : 896;
-        bool odd = false;
-        auto join = [&](float h, float l) { return to_double(h, e, odd) + to_double(l, e, odd); };
-        const float4 w = exact_displacement(f, gxs, gys);
-        u = join(w.x, w.y);
-        v = join(w.z, w.w);
-        float ep, eq, e13, e24, e11, e22, ed, et, es;
-        const float p = two_sum(f[4], f[6], ep), q = two_sum(f[5], f[7], eq);
-        const float h11 = two_sum(p, -q, e11), h22 = two_sum(p, q, e22);
-        const float s13 = two_sum(f[0], f[2], e13), s24 = two_sum(f[1], f[3], e24);
-        const float hd = two_sum(s13, -s24, ed), ht = two_sum(s13, s24, et);
-        const float l22 = __fadd_rn(e22, __fadd_rn(ep, eq));
-        const float hs = two_sum(ht, 2.0f * h22, es);   // m_s = (f1+f3) + (f2+f4) + 2 m_22
-        const float l11 = __fadd_rn(e11, __fsub_rn(ep, eq)), ld = __fadd_rn(ed, __fsub_rn(e13, e24));
-        const float ls = __fadd_rn(__fadd_rn(es, __fadd_rn(et, __fadd_rn(e13, e24))), 2.0f * l22);
-        m11 = join(h11, l11);
-        md = join(hd, ld);
-        ms = join(hs, ls);
-        if (odd) {
-            const double s = S == S_F16S ? (double)a.hinv : 1.0;
-            u = ((double)w.x + (double)w.y) * s;
-            v = ((double)w.z + (double)w.w) * s;
-            m11 = ((double)h11 + (double)l11) * s;
-            md = ((double)hd + (double)ld) * s;
-            ms = ((double)hs + (double)ls) * s;
-        }
+        double w[8];
+        const double scale = S == S_F16S ? (double)a.hinv : 1.0;
+#pragma unroll
+        for (int p = 0; p < 8; ++p) w[p] = (double)f[p] * scale;
+        const Mom<double> m = moments(w);
+        u = m.m10 + 0.5 * ((double)gxs * scale);
+        v = m.m01 + 0.5 * ((double)gys * scale);
+        sxx = -0.5 * (c.bs * m.ms + c.bd * m.md);
+        syy = -0.5 * (c.bs * m.ms - c.bd * m.md);
+        mb11 = c.b11 * m.m11;
     }
-    // (un: the joins return the fields' own unit)
-    const double t = cd * md, mb11 = c.b11 * m11, un = 1.0;
+    const double un = 1.0;         // (the fields' own unit)
     const int64_t o = out.tr ? (int64_t)x * ny + y : (int64_t)y * nx + x;
     if (out.p[0]) out.p[0][o] = u;
     if (out.p[1]) out.p[1][o] = v;
-    if (out.p[2]) out.p[2][o] = fma(cs, ms, t);
-    if (out.p[3]) out.p[3][o] = fma(cs, ms, -t);
+    if (out.p[2]) out.p[2][o] = sxx;
+    if (out.p[3]) out.p[3][o] = syy;
     if (out.p[4]) out.p[4][o] = -mb11 * un;
 }
 
