@@ -62,7 +62,7 @@ struct lbm_ctx {
     void* snap = nullptr;          // residual snapshot: 2 planes of entries of 8 bytes (ResSnap)
     double* partials = nullptr;    // residual partial sets, kRes doubles each
     int64_t partials_len = 0;      // partial sets the buffer holds
-    double* result = nullptr;      // kRes doubles (device)
+    double* result = nullptr;      // kRes doubles, in pinned
     unsigned long long* absmax = nullptr;
     unsigned int* bad = nullptr;
     double* pinned = nullptr;      // kRes + 2 doubles (pinned host)
@@ -622,7 +622,6 @@ void free_all(lbm_ctx* c) {
     if (c->force) cudaFree(c->force);
     if (c->snap) cudaFree(c->snap);
     if (c->partials) cudaFree(c->partials);
-    if (c->result) cudaFree(c->result);
     if (c->absmax) cudaFree(c->absmax);
     if (c->bad) cudaFree(c->bad);
     if (c->staging) cudaFree(c->staging);
@@ -716,10 +715,8 @@ const void* mapped_host(const void* p) {
 
 // Reads the residual of the last check; returns r_inf etc. in out[0..4].
 int read_residual(lbm_ctx* c, double out[kRes]) {
-    CK(cudaMemcpyAsync(c->pinned, c->result, kRes * sizeof(double), cudaMemcpyDeviceToHost,
-                       c->stream));
     CK(cudaStreamSynchronize(c->stream));
-    for (int k = 0; k < kRes; ++k) out[k] = c->pinned[k];
+    for (int k = 0; k < kRes; ++k) out[k] = c->result[k];
     return LBM_OK;
 }
 
@@ -854,17 +851,22 @@ int lbm_create_ex(int nx, int ny, double lambda, double mu, int dtype, const lbm
         c->partials_len = std::max(c->partials_len, c->plan == 2 ? tile_count(c->tile, nx, ny) : int64_t(0));
     }
     if (e == cudaSuccess) e = alloc((void**)&c->partials, sizeof(double) * kRes * c->partials_len);
-    if (e == cudaSuccess) e = alloc((void**)&c->result, sizeof(double) * kRes);
     if (e == cudaSuccess) e = alloc((void**)&c->absmax, sizeof(unsigned long long));
     if (e == cudaSuccess) e = alloc((void**)&c->bad, sizeof(unsigned int));
+    // host words the device writes and copies into: two of the force upload, then
+    // the result of the last check (written in place: a copy after it would
+    // cost every lbm_solve window 3 us more)
     if (e == cudaSuccess) e = cudaMallocHost((void**)&c->pinned, sizeof(double) * (kRes + 2));
+    if (e == cudaSuccess) {
+        c->result = c->pinned + 2;
+        std::fill(c->result, c->result + kRes, 0.0);
+    }
     if (e == cudaSuccess) e = cudaMemset(c->pop[0], 0, pb);
     if (e == cudaSuccess) e = cudaMemset(c->pop[1], 0, pb);
     if (e == cudaSuccess && dtype == LBM_F16S) e = cudaMemset(c->car[0], 0, cb);
     if (e == cudaSuccess && dtype == LBM_F16S) e = cudaMemset(c->car[1], 0, cb);
     if (e == cudaSuccess) e = cudaMemset(c->force, 0, fb);
     if (e == cudaSuccess) e = cudaMemset(c->snap, 0, snap_bytes);
-    if (e == cudaSuccess) e = cudaMemset(c->result, 0, sizeof(double) * kRes);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
         int code = cuda_fail(e, "lbm_create: device allocation");

@@ -118,6 +118,14 @@ template <int S> struct ResAcc {
         w[4] = bad;
     }
 };
+// Combination of kRes partials across a warp's lanes (result in every lane).
+// The maxima and the flag are non-negative doubles, which order like their bit
+// patterns: they are combined as integers (an FP64 instruction takes 64 cycles
+// of a scheduler), the sums in FP64.
+__device__ __forceinline__ double max_bits(double a, double b) {
+    const unsigned long long x = (unsigned long long)__double_as_longlong(a), y = (unsigned long long)__double_as_longlong(b);
+    return __longlong_as_double((long long)(x > y ? x : y));
+}
 template <> struct ResAcc<S_F64> {
     double d = 0.0, u = 0.0, d2 = 0.0, u2 = 0.0, bad = 0.0;
     __device__ __forceinline__ void to_double(double w[kRes]) const {
@@ -187,8 +195,9 @@ __device__ __forceinline__ void check_node(const StepParams& a, int64_t n, int64
         sp[idx] = u;
         sp[n + idx] = v;
         const double du = u - old.u, dv = v - old.v;
-        acc.d = fmax(acc.d, fmax(fabs(du), fabs(dv)));
-        acc.u = fmax(acc.u, fmax(fabs(u), fabs(v)));
+        // (maxima by the ALU; a NaN among them is left to the flag)
+        acc.d = max_bits(acc.d, max_bits(fabs(du), fabs(dv)));
+        acc.u = max_bits(acc.u, max_bits(fabs(u), fabs(v)));
         acc.d2 += du * du + dv * dv;
         acc.u2 += u * u + v * v;
         if (!(isfinite(u) && isfinite(v))) acc.bad = 1.0;
@@ -216,15 +225,6 @@ __device__ __forceinline__ void check_node(const StepParams& a, int64_t n, int64
         pair_add_square(acc.u2h, acc.u2l, w.z, w.w);
         if (!(isfinite(w.x) && isfinite(w.z))) acc.bad = 1.0f;
     }
-}
-
-// Combination of kRes partials across a warp's lanes (result in every lane).
-// The maxima and the flag are non-negative doubles, which order like their bit
-// patterns: they are combined as integers (an FP64 instruction takes 64 cycles
-// of a scheduler), the sums in FP64.
-__device__ __forceinline__ double max_bits(double a, double b) {
-    const unsigned long long x = (unsigned long long)__double_as_longlong(a), y = (unsigned long long)__double_as_longlong(b);
-    return __longlong_as_double((long long)(x > y ? x : y));
 }
 __device__ __forceinline__ void combine_res(double w[kRes], const double v[kRes]) {
     w[0] = max_bits(w[0], v[0]);
