@@ -281,6 +281,57 @@ struct ResAcc2 {
     }
 };
 
+// (h, l) += (g, m), pairs (about 2^-45 relative).
+__device__ __forceinline__ void pair_add(float& h, float& l, float g, float m) {
+    float e;
+    const float s = two_sum(h, g, e), x = __fadd_rn(__fadd_rn(l, m), e), r = __fadd_rn(s, x);
+    l = __fsub_rn(x, __fsub_rn(r, s));
+    h = r;
+}
+
+// The partials of a thread's, warp's or block's nodes as pairs: combined as they
+// are, and converted to FP64 once per block (an FP64 instruction takes 64 cycles
+// of a scheduler: with conversions and sums in every thread they were 5 us of
+// a checked launch of k_tile).
+struct ResPart {
+    float dh, dl, uh, ul, d2h, d2l, u2h, u2l;
+    bool bad;
+    __device__ __forceinline__ void add(const ResPart& o) {
+        pair_max_abs(dh, dl, o.dh, o.dl);
+        pair_max_abs(uh, ul, o.uh, o.ul);
+        pair_add(d2h, d2l, o.d2h, o.d2l);
+        pair_add(u2h, u2l, o.u2h, o.u2l);
+        bad |= o.bad;
+    }
+    __device__ __forceinline__ void add_warp() {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            auto get = [&](float v) { return __shfl_xor_sync(0xffffffffu, v, o); };
+            add(ResPart{get(dh), get(dl), get(uh), get(ul), get(d2h), get(d2l), get(u2h), get(u2l), false});
+        }
+        bad = __any_sync(0xffffffffu, bad);
+    }
+    __device__ __forceinline__ void to_double(double w[kRes]) const {
+        w[0] = max_to_double(dh, dl);
+        w[1] = max_to_double(uh, ul);
+        w[2] = pair_to_double(d2h, d2l);
+        w[3] = pair_to_double(u2h, u2l);
+        w[4] = bad ? 1.0 : 0.0;
+    }
+};
+__device__ __forceinline__ ResPart res_part(const ResAcc2& r) {
+    float a[2], b[2], c[2], d[2], f[2];
+    unpk(r.fin, f[0], f[1]);
+    unpk(r.d2h, a[0], a[1]);
+    unpk(r.d2l, b[0], b[1]);
+    unpk(r.u2h, c[0], c[1]);
+    unpk(r.u2l, d[0], d[1]);
+    const ResPart none{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, false};
+    ResPart p = r.own0 ? ResPart{r.dh[0], r.dl[0], r.uh[0], r.ul[0], a[0], b[0], c[0], d[0], f[0] != 0.0f} : none;
+    p.add(r.own1 ? ResPart{r.dh[1], r.dl[1], r.uh[1], r.ul[1], a[1], b[1], c[1], d[1], f[1] != 0.0f} : none);
+    return p;
+}
+
 // two_sum (lbm_core.cuh) on pairs.
 __device__ __forceinline__ pair_t two_sum2(pair_t a, pair_t b, pair_t& e) {
     const pair_t s = add2(a, b), bb = sub2(s, a);
@@ -521,6 +572,23 @@ __device__ __forceinline__ void scatter_local(const StepParams& a, int64_t idx,
 // check; without one (the library's own check launches) the blocks stop after
 // writing their partials and k_residual_finish combines them in a separate
 // launch.
+// Paired partials combined as pairs (no counter): the block's partial set.
+__device__ __forceinline__ void residual_reduce_pairs(const StepParams& a, const ResAcc2& acc) {
+    __shared__ ResPart sh[32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    ResPart p = res_part(acc);
+    p.add_warp();
+    if (lane == 0) sh[warp] = p;
+    __syncthreads();
+    if (warp != 0) return;
+    if (lane < (int)(blockDim.x >> 5)) p = sh[lane];
+    else p = ResPart{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, false};
+    p.add_warp();
+    if (lane != 0) return;
+    double w[kRes];
+    p.to_double(w);
+    for (int k = 0; k < kRes; ++k) a.partials[(int64_t)blockIdx.x * kRes + k] = w[k];
+}
 template <typename ACC>
 __device__ __forceinline__ void residual_reduce(const StepParams& a, const ACC& acc) {
     __shared__ double sh[kRes][32];
@@ -1839,7 +1907,7 @@ k_tile(const StepParams a, const PairCoef ca, int T, int ntx, unsigned rounds) {
         put(next + 768, s[0].d4, s[0].d7, s[0].nd8);
         __syncthreads();
     }
-    if (CHECK) residual_reduce(a, acc);
+    if (CHECK) residual_reduce_pairs(a, acc);
 }
 
 // Destinations of the five solution fields u_x, u_y, sigma_xx, sigma_yy,
