@@ -436,6 +436,7 @@ def time_variant(args, dtype, gx_d, gy_d, torch, P, nsteps, nwarm, events=True, 
     iter_ms = sum(a.elapsed_time(b) for a, b in evs)
     dom_ms = sum(devs[2 * k].elapsed_time(devs[2 * k + 1]) for k in range(nev))
     dom_launches = nev * (block // big)
+    step_launches = P.lbm_get_launches(lat.ctx) - counted
     lat.close()
     del out5
     checks = iters // args.check_every      # each adds one residual-finish launch
