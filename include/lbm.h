@@ -54,8 +54,10 @@ extern "C" {
 
 typedef struct lbm_ctx lbm_ctx;
 
-/* Population storage type.  Collision arithmetic is FP64 for LBM_F64 and
- * FP32 for the other two.
+/* Population storage type.  Collision arithmetic is FP32 for LBM_F32 and
+ * LBM_F16S; for LBM_F64 it is 64-bit integer (a node's values as multiples of
+ * 2^-58 of the largest of them, the results rounded to FP64 once: no less exact
+ * than FP64 arithmetic), and FP64 at the ends of the exponent range.
  *  LBM_F64  : 8 FP64 planes.
  *  LBM_F32  : 8 FP32 planes.
  *  LBM_F16S : "shifted" FP16 storage: per node the first post-collision
@@ -141,8 +143,8 @@ int lbm_get_host_transfer(lbm_ctx *ctx, int *mode);
  * this runs on tiles (the tile and a halo of one node per extra step in shared
  * memory); four steps need the wavefront schedule (lbm_set_wavefront), and
  * without it k = 4 runs as k = 3.  A residual check (lbm_iterate_checked,
- * lbm_solve) falls on the last step of a launch: of a four-step wavefront
- * launch where that schedule runs, else of a launch of at most two steps;
+ * lbm_solve) falls on the last step of a launch: of four steps (LBM_F32: or
+ * five) on the wavefront schedule, else of at most two steps;
  * steps left over when n is not a multiple of k run in shorter launches.  With LBM_F32 storage the
  * arithmetic per node is unchanged and the state after every launch equals
  * that of the same steps taken one per launch, bit for bit.  With LBM_F16S
@@ -153,13 +155,14 @@ int lbm_get_host_transfer(lbm_ctx *ctx, int *mode);
  * launches take as many steps as suit the lattice, up to six
  * (lbm_get_launch_steps); LBM_F16S keeps groups of four.  Available for LBM_F32 and
  * LBM_F16S storage on any lattice.  Until this function or lbm_set_wavefront is
- * called, LBM_F32 lattices take whichever schedule their size suits (strips of
- * the wavefront schedule, or tiles held in registers, of up to twelve steps per
- * launch), which gives the same states; the default is 4 (wavefront schedule) from
+ * called, LBM_F32 and LBM_F16S lattices take whichever schedule their size suits
+ * (strips of the wavefront schedule, or tiles held in registers, of up to twelve
+ * steps per launch; LBM_F16S states are rounded where the groups below end, also
+ * inside a launch), which gives the same states; the default is 4 (wavefront schedule) from
  * nx >= 256 and ny >= 8 on, else 3 from nx >= 64 and ny >= 16 on (a smaller
  * lattice fills the on-chip tile more than once and is faster one step per
  * launch).  LBM_F64 storage takes k = 1
- * only (the library itself groups up to three steps of a small LBM_F64 lattice
+ * only (the library itself groups up to four steps of a small LBM_F64 lattice
  * into a launch, with the same states).  Paper: the scheme advances one step at a time; grouping steps into
  * launches is a schedule of the same steps, not part of the method.
  * Errors: LBM_ERR_ARG (k outside 1..4, or k > 1 with LBM_F64 storage). */
@@ -339,36 +342,34 @@ const char *lbm_last_error(void);
 /* ---------------------------------------------------------------------------
  * Batched solves.  Many independent periodic problems (each the setting of
  * Sec. 2 with its own size, Lame parameters and body force) are solved in one
- * packed device arena by a persistent cooperative kernel: every step walks the
- * tiles of all running problems, a grid-wide barrier separates steps, and the
- * residual check of Sec. 2.1 (reading of lbm_solve) is fused into the last step
- * of each chunk of check_every steps, per problem.  Converged problems drop
- * out of the tile list between chunks.  The chunk (accumulator reset, kernel,
- * read-back) is replayed from a CUDA graph.  The tile shape is chosen by an
+ * packed device arena, in chunks of check_every steps; the residual check of
+ * Sec. 2.1 (reading of lbm_solve) is fused into the last step of each chunk,
+ * per problem, and converged problems drop out of the work list between
+ * chunks.  When check_every is a multiple of 4, the strip chunk LBM_TILE_WAVE
+ * advances every problem by a group of steps per launch (LBM_F32 five, LBM_F16S
+ * four) on the schedule of lbm_set_wavefront, one warp per strip of 56 output
+ * columns and segment of rows; problems narrower than 16 columns take pairs of
+ * steps on two-step tiles.  The other tile codes run a chunk as one cooperative
+ * kernel, replayed from a CUDA graph, that walks the tiles of all running
+ * problems with grid-wide barriers: tiles 32, 64 or 128 columns wide (tile code
+ * 1, 2, 4: warps of 32 columns, one step per barrier) or, when check_every is
+ * even, LBM_TILE_TWO_STEP tiles (62 x 22 nodes, two steps per tile visit with the
+ * intermediate state on chip and one barrier per pair of steps;
+ * lbm_set_steps_per_launch describes the arithmetic).  The code is chosen by an
  * autotuner that times the first chunks and caches the choice per workload
  * signature in $LBM_AUTOTUNE_CACHE (default ~/.cache/lbm_gb300/autotune.txt;
- * LBM_AUTOTUNE=0 ignores the cache): tiles 32, 64 or 128 columns wide (tile
- * code 1, 2, 4: warps of 32 columns, one step per barrier) or, when
- * check_every is even, LBM_TILE_TWO_STEP tiles (62 x 22 nodes, two steps per
- * tile visit with the intermediate state on chip and one grid barrier per
- * pair of steps; lbm_set_steps_per_launch describes the arithmetic) or, when
- * check_every is a multiple of 4, the wavefront chunk LBM_TILE_WAVE: problems
- * at least 256 columns wide and 8 rows high advance four steps per visit of a
- * wavefront item (a 256-column strip by up to 256 rows on the schedule of
- * lbm_set_wavefront; the rows are halved, down to 16, while the work list
- * would hold fewer than four waves of resident blocks), narrower ones two steps per two-step tile, with two grid
- * barriers per four steps and items taken from a work counter, wavefront
- * items first.  Every tile code computes the same per-node arithmetic; FP32
+ * LBM_AUTOTUNE=0 ignores the cache).  Every tile code computes the same per-node
+ * arithmetic; FP32
  * results are the same bits under every code.  A problem that fits these
  * tiles clearly better with x and y exchanged (narrow and tall, or a width just
- * past a multiple of the strip's 250 output columns) is solved on its
+ * past a multiple of 250 columns) is solved on its
  * transpose: the scheme is symmetric under the exchange (u_x <-> u_y, sigma_xx
  * <-> sigma_yy), the outputs are returned in the caller's orientation and
  * lbm_result.transposed reports it; the result then equals the problem solved
  * as given up to rounding.
  * ------------------------------------------------------------------------- */
 /* Tile codes in lbm_batch_report.tile_v and lbm_stats.tile_v besides the
- * widths 1, 2, 4: two-step tiles, and the wavefront chunk. */
+ * widths 1, 2, 4: two-step tiles, and the strip chunk. */
 #define LBM_TILE_TWO_STEP 3
 #define LBM_TILE_WAVE 5
 
@@ -393,7 +394,7 @@ typedef struct lbm_result {
 
 typedef struct lbm_batch_report {
     int tile_v;                 /* tile code used: 1, 2, 4 (warps of 32 columns), LBM_TILE_TWO_STEP or LBM_TILE_WAVE */
-    int blocks;                 /* grid of the persistent chunk kernel */
+    int blocks;                 /* grid of the chunk kernel (strip chunk: of the largest launch) */
     int64_t chunks;             /* chunk launches */
     int64_t lattice_updates;    /* sum over problems of nodes x steps */
     double device_ms;           /* device time of the chunks (CUDA events) */

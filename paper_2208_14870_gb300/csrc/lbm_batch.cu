@@ -1,6 +1,6 @@
 // lbm_batch.cu -- lbm_batch_solve: many independent periodic problems solved
-// together in one packed arena by the persistent chunk kernel, with the tile
-// width chosen by the autotuner.
+// together in one packed arena, chunk by chunk, with the tile code chosen by the
+// autotuner.
 #include <algorithm>
 #include <chrono>
 #include <cstdlib>

@@ -509,8 +509,8 @@ cudaError_t run_plain(lbm_ctx* c, int64_t n) {
 }
 
 // to_check - 1 plain steps followed by the residual-check step (the last
-// step of the last launch).  On the four-step wavefront schedule the check is
-// the last level of a four-step launch; with three steps per launch on tiles
+// step of the last launch).  On strips the check is the last level of a launch
+// of four (FP32: or five) steps, on register tiles the last step of any; with three steps per launch on tiles
 // it rides on a two-step launch (a three-step tile launch with the check
 // costs twice a plain one, a two-step launch with the check 1.3 times).
 cudaError_t run_window(lbm_ctx* c, int64_t to_check) {

@@ -13,7 +13,7 @@
 #include "lbm_engine.cuh"
 
 static_assert(lbm::kTileTwoStep == LBM_TILE_TWO_STEP, "tile code of two-step tiles");
-static_assert(lbm::kTileWave == LBM_TILE_WAVE, "tile code of the wavefront chunk");
+static_assert(lbm::kTileWave == LBM_TILE_WAVE, "tile code of the strip chunk");
 
 namespace lbm {
 

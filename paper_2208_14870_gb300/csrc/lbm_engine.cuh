@@ -1,6 +1,6 @@
 // lbm_engine.cuh -- host side of the packed lattice arena: admission of
-// problems into arena slots, chunk replay (CUDA graph around the persistent
-// cooperative kernel), per-problem residual bookkeeping, retirement and
+// problems into arena slots, chunks (strip launches, or a CUDA graph around the
+// cooperative kernel of the other tile codes), per-problem residual bookkeeping, retirement and
 // solution recovery.  Shared by lbm_batch_solve and the serving loop.
 #pragma once
 

@@ -5,8 +5,7 @@
 // queued; between chunks the worker admits queued requests whose lattice fits
 // the free arena memory (first-fit, oldest first, with a bound on how long a
 // request can be bypassed by later ones), runs one chunk of check_every steps
-// of every resident problem (one persistent cooperative launch per arena,
-// replayed from a CUDA graph), and retires problems whose residual dropped
+// of every resident problem (strip chunks of both arenas side by side), and retires problems whose residual dropped
 // below their tolerance: their displacement and stress are recovered into
 // host memory owned by the request, their arena memory is freed for the next
 // admissions, and their latency (submission to completion) is recorded.
@@ -281,7 +280,7 @@ int lbm_server_create(size_t hbm_budget_bytes, int check_every, lbm_server** out
             return set_last_error(rc, "lbm_server_create: " + err);
         }
     }
-    // the wavefront chunk by default (chunk length a multiple of 4), else
+    // the strip chunk by default (chunk length a multiple of 4), else
     // two-step tiles (even) or 128-column tiles, unless the autotuner cache
     // holds a choice for this chunk length
     const bool even = check_every % 2 == 0, four = check_every % 4 == 0;

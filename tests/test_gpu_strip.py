@@ -19,7 +19,7 @@ if not torch.cuda.is_available():  # pragma: no cover
 import paper_2208_14870_gb300 as P  # noqa: E402
 from paper_2208_14870_gb300 import Lattice  # noqa: E402
 
-# 280 and 364: whole strips of 56 and 52 output columns (five and seven steps)
+# 280 and 364: whole strips of 56 and 52 output columns (five and six steps)
 SIZES = [(256, 8), (257, 9), (258, 31), (259, 40), (260, 13), (261, 8), (262, 21), (263, 17),
          (280, 33), (281, 10), (364, 12), (365, 25), (1000, 61)]
 
