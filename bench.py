@@ -49,17 +49,15 @@ FORCE_SEED = 0x2208_14870
 # DRAM traffic per stream-collide launch from one ncu capture, keyed by dtype,
 # steps per launch and schedule, with the hash of the kernel code it was taken
 # on (null in the bench line once the code changes; comments do not count).
-# Captured at 8192^2 with 256-row segments (profiles/k_wave_8192_dram_traffic.md):
-# 33 strips of 256 slots and 32 segments, the same column-halo share (256/250
-# per output column) and segment length as the 16384^2 launch, so a launch's
-# traffic is 4x the capture's (nodes x4).  Mean of three launches.
+# Captured at 8192 x 4096 (profiles/k_strip_dram_traffic.md) and scaled by the
+# nodes to 16384^2:
 NCU_TRAFFIC = {
-    "f32_x4w": {"bytes_per_launch": 4 * (2.76050e9 + 2.10493e9), "kernel_hash": "fb0329a445f0d126",
-                "ncu": {"case": "8192^2, 256-row segments, x4", "dram_read_per_launch": 4 * 2.76050e9,
-                        "dram_write_per_launch": 4 * 2.10493e9, "algorithmic_per_launch": 72 * 16384 ** 2}},
-    "f16s_x4w": {"bytes_per_launch": 4 * (2.20988e9 + 1.57011e9), "kernel_hash": "fb0329a445f0d126",
-                 "ncu": {"case": "8192^2, 256-row segments, x4", "dram_read_per_launch": 4 * 2.20988e9,
-                         "dram_write_per_launch": 4 * 1.57011e9, "algorithmic_per_launch": 56 * 16384 ** 2}},
+    "f32_x6w": {"bytes_per_launch": 8 * (1.448276e9 + 1.039006e9), "kernel_hash": "93db48a8c288ed51",
+                "ncu": {"case": "8192 x 4096, x8", "dram_read_per_launch": 8 * 1.448276e9,
+                        "dram_write_per_launch": 8 * 1.039006e9, "algorithmic_per_launch": 72 * 16384 ** 2}},
+    "f16s_x4w": {"bytes_per_launch": 8 * (1.137909e9 + 0.772296e9), "kernel_hash": "93db48a8c288ed51",
+                 "ncu": {"case": "8192 x 4096, x8", "dram_read_per_launch": 8 * 1.137909e9,
+                         "dram_write_per_launch": 8 * 0.772296e9, "algorithmic_per_launch": 56 * 16384 ** 2}},
 }
 
 
