@@ -1251,7 +1251,10 @@ template <int S, int T> __host__ __device__ constexpr int st_ox() {
 }
 // warps per block; the kernel is compiled for three resident blocks, twelve
 // warps per SM (168 registers a thread; at 16384^2 with registers for eight warps
-// 87.6 ms per 100 steps against 79.8)
+// 87.6 ms per 100 steps against 79.8).  With the check for two: at 168 registers
+// it spilled, and its partials were combined in FP64 (T = 5 at 16384^2 6.20 ms,
+// at 1024^2 39.8 us; with two blocks 5.72 and 35.6, and pairs combined as pairs
+// 5.45 and 32.3; FP16S 1000 x 700 28.1 -> 25.1 us, 8192^2 1.45 -> 1.48 ms)
 constexpr int kStNW = 4;
 // rows copied ahead of the rows in use, and population rows held: FP32 has the
 // rows above, at and below level 1 in use, FP16S the decoded row
@@ -1632,7 +1635,7 @@ __device__ __forceinline__ void strip_walk(const StepParams& a, const PairCoef& 
 }
 
 template <int S, bool GEN, int T, bool CHECK>
-__global__ void __launch_bounds__(32 * kStNW, 3)
+__global__ void __launch_bounds__(32 * kStNW, CHECK ? 2 : 3)
 k_strip(const StepParams a, const PairCoef c, int seg, int nstrips, int items) {
     extern __shared__ float4 st_mem[];
     const int warp = threadIdx.x >> 5;
@@ -1643,7 +1646,7 @@ k_strip(const StepParams a, const PairCoef c, int seg, int nstrips, int items) {
         const uint32_t sm = (uint32_t)__cvta_generic_to_shared(st_mem) + warp * st_warp_smem<S, T, CHECK>();
         strip_walk<S, GEN, T, CHECK>(a, c, sm, strip, y0, min(seg, a.ny - y0), acc);
     }
-    if (CHECK) residual_reduce(a, acc);
+    if (CHECK) residual_reduce_pairs(a, acc);
 }
 
 // ---------------------------------------------------------------------------
@@ -2260,7 +2263,7 @@ struct StripShape {
 // rows takes seg + 2 (halo rows) iterations, so the best segments are those whose
 // warps just fill a whole number of waves (4096 x 3000, T = 5: 213 to 229 us with
 // 32 to 256 rows chosen by halving, 155 us with the 125 rows that fill one
-// wave); a checked row costs 2300 cycles more; the state moves at 3.0 kB per
+// wave); a checked row costs 1250 cycles (FP16S 1600) more; the state moves at 3.0 kB per
 // cycle (6.2 TB/s).  rows > 0 fixes the segment.
 inline StripShape strip_shape(int dtype, int T, bool check, int nx, int ny, int nsm, int warps, int rows) {
     const int64_t ns = strip_count(dtype, T, nx);
@@ -2274,7 +2277,7 @@ inline StripShape strip_shape(int dtype, int T, bool check, int nx, int ny, int 
         if (seg > ny) seg = ny;
         const int64_t items = ns * ((ny + seg - 1) / seg), slots = (int64_t)nsm * warps;
         auto wave = [&](double w) {
-            return slow * (double)(seg + 2 * halo) * (T * (70.0 + 115.0 * w) + 150.0) + (check ? 2300.0 * seg : 0.0);
+            return slow * (double)(seg + 2 * halo) * (T * (70.0 + 115.0 * w) + 150.0) + (check ? (dtype == S_F32 ? 1250.0 : 1600.0) * seg : 0.0);
         };
         // full waves (many run into one another), then what is left
         const int64_t full = (items - 1) / slots, rest = items - full * slots;
