@@ -52,10 +52,10 @@ FORCE_SEED = 0x2208_14870
 # Captured at 8192 x 4096 (profiles/k_strip_dram_traffic.md) and scaled by the
 # nodes to 16384^2:
 NCU_TRAFFIC = {
-    "f32_x6w": {"bytes_per_launch": 8 * (1.448276e9 + 1.039006e9), "kernel_hash": "93db48a8c288ed51",
+    "f32_x6w": {"bytes_per_launch": 8 * (1.448276e9 + 1.039006e9), "kernel_hash": "8ed196ce088fc94a",
                 "ncu": {"case": "8192 x 4096, x8", "dram_read_per_launch": 8 * 1.448276e9,
                         "dram_write_per_launch": 8 * 1.039006e9, "algorithmic_per_launch": 72 * 16384 ** 2}},
-    "f16s_x4w": {"bytes_per_launch": 8 * (1.137909e9 + 0.772296e9), "kernel_hash": "93db48a8c288ed51",
+    "f16s_x4w": {"bytes_per_launch": 8 * (1.137909e9 + 0.772296e9), "kernel_hash": "8ed196ce088fc94a",
                  "ncu": {"case": "8192 x 4096, x8", "dram_read_per_launch": 8 * 1.137909e9,
                          "dram_write_per_launch": 8 * 0.772296e9, "algorithmic_per_launch": 56 * 16384 ** 2}},
 }

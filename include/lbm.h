@@ -284,7 +284,8 @@ int lbm_iterate(lbm_ctx *ctx, int64_t n);
  * window between two checks is check_every steps.  The last residual is
  * written to
  * out[0..4] if out is non-null: r_inf, r_2, max|u|, ||u||_2, nonfinite flag
- * (see lbm_solve).  Synchronous when out is non-null. */
+ * (see lbm_solve).  Before the context's first check r_inf and r_2 are infinite and
+ * the others 0.  Synchronous when out is non-null. */
 int lbm_iterate_checked(lbm_ctx *ctx, int64_t n, int check_every, double *out);
 
 /* Iterate until the steady-state residual drops below tol (Sec. 2.1:

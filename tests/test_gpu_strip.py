@@ -221,6 +221,21 @@ def test_f64_step_against_long_double(scale, integers, kw):
         assert (err <= tol).all(), k
 
 
+# Steps that hold no check: the residual of a fresh context is infinite and its
+# norms are zero, whatever an earlier context left in the memory.
+@pytest.mark.parametrize("dtype", ["f64", "f32", "f16s"])
+def test_residual_before_the_first_check(dtype):
+    lam, mu = W.lame_2d(1.0, 0.3)
+    g = np.random.RandomState(3).standard_normal((2, 200, 300)) * 1e-5
+    for steps in (300, 86, 0):
+        with Lattice(300, 200, lam, mu, dtype) as lat:
+            lat.set_force(g[0], g[1])
+            r = lat.iterate_checked(steps, 100)
+            lat.fields()
+        if steps < 100:
+            assert np.array_equal(r, [np.inf, np.inf, 0.0, 0.0, 0.0])
+
+
 def _problems(sizes):
     out = []
     for i, (nx, ny) in enumerate(sizes):
