@@ -1229,11 +1229,13 @@ k_step3(const StepParams a, const Coef<float> c) {
 // The per-node operations are lbm_core.cuh's, so FP32 results equal T
 // single-step launches bit for bit.
 //
-// What bounds it: the five-step FP32 launch moves 72 bytes per node at 6.1 TB/s,
-// 0.90 of the measured copy peak (16384^2, 3.16 ms; the block-wide wavefront
-// kernel before it took 3.31 ms for four steps).  An update issues about 50
-// instructions (that kernel: 90), 27 of them arithmetic, two operations each;
-// FP16S four-step launches are issue-bound at 0.74 of the copy peak (0.63).
+// What bounds it: the five-step FP32 launch moves 72 bytes per node at 6.15 TB/s,
+// 0.90 of the measured copy peak (16384^2, 3.14 ms; the block-wide wavefront
+// kernel before it took 3.31 ms for four steps); six steps (3.67 ms, 0.611 per step)
+// are bound by latency and the FMA pipe (issue 60 %, FMA pipe 58 %, DRAM 64 % of
+// the time, three warps per scheduler).  An update issues 56 instructions (that
+// kernel: 90), 27 of them packed arithmetic, two operations each; FP16S four-step
+// launches, 69 instructions, run at 0.79 of the copy peak (0.63), bound alike.
 // One code copy serves the first iterations too (each level's test is one
 // uniform branch): with a copy of its own for them the code left the
 // instruction cache and the compiler took 202 registers instead of 150.
