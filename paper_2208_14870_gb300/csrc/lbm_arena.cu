@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(256) k_arena_force(const ForceIn f) {
         if (!(isfinite(u) && isfinite(v))) bad = 1;
         m = fmax(m, fmax(fabs(u), fabs(v)));
         float* o = f.out + y * f.pitch + f.ghost + x;
-        const float gx = (float)(f.tr ? v : u), gy = (float)(f.tr ? u : v);
+        const float gx = (float)(f.tr ? v : u) * f.scale, gy = (float)(f.tr ? u : v) * f.scale;
         o[0] = gx;
         o[f.plane] = gy;
         if (x < f.ghost) {

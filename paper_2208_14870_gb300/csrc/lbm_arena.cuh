@@ -179,6 +179,7 @@ struct ForceIn {
     float* out;                // row 0, first ghost column
     int nx, ny, pitch, ghost;
     int64_t plane;
+    float scale;               // of the converted force (a power of two)
     unsigned long long* stat;
 };
 cudaError_t launch_arena_force(const ForceIn& f, cudaStream_t st);
