@@ -223,11 +223,8 @@ int ArenaEngine::admit(int nx, int ny, double lambda, double mu, const double* g
     }
     unsigned long long* stat = d_stat_ + 2 * slot;
     float* force = reinterpret_cast<float*>(fs_ + p.fs_off);
-    // (one copy where the components lie one after the other: small problems are
-    // admitted at the rate of these calls)
-    const bool joined = reinterpret_cast<uintptr_t>(gy) == reinterpret_cast<uintptr_t>(gx) + sizeof(double) * n;
-    ECK(cudaMemcpyAsync(d_force_, gx, sizeof(double) * (joined ? 2 * n : n), cudaMemcpyHostToDevice, st_));
-    if (!joined) ECK(cudaMemcpyAsync(d_force_ + n, gy, sizeof(double) * n, cudaMemcpyHostToDevice, st_));
+    ECK(cudaMemcpyAsync(d_force_, gx, sizeof(double) * n, cudaMemcpyHostToDevice, st_));
+    ECK(cudaMemcpyAsync(d_force_ + n, gy, sizeof(double) * n, cudaMemcpyHostToDevice, st_));
     ECK(cudaMemsetAsync(stat, 0, 2 * sizeof(unsigned long long), st_));
     ECK(cudaMemsetAsync(force, 0, p.fs_bytes, st_));
     ForceIn f{};

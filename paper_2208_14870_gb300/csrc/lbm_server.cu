@@ -40,7 +40,7 @@ struct Request {
     int nx = 0, ny = 0, dtype = LBM_F32;
     double lambda = 0.0, mu = 0.0, tol = 0.0;
     int64_t max_iters = 0;
-    std::unique_ptr<double[]> g;            // both components, until admitted
+    std::unique_ptr<double[]> gx, gy;       // until admitted
     std::unique_ptr<double[]> fields;       // 5 * nx * ny once done
     int state = R_QUEUED;
     int status = LBM_OK;
@@ -179,7 +179,7 @@ int lbm_server::admit_locked() {
             continue;
         }
         std::string err;
-        const int s = arena[a]->admit(r.nx, r.ny, r.lambda, r.mu, r.g.get(), r.g.get() + (int64_t)r.nx * r.ny, r.tol,
+        const int s = arena[a]->admit(r.nx, r.ny, r.lambda, r.mu, r.gx.get(), r.gy.get(), r.tol,
                                       r.max_iters, &err);
         if (s >= 0) {
             r.state = R_RUNNING;
@@ -187,7 +187,8 @@ int lbm_server::admit_locked() {
             r.slot = s;
             r.t_admit = clk::now();
             slot_owner[a][s] = r.ticket;
-            r.g.reset();  // the arena holds the force now
+            r.gx.reset();  // the arena holds the force now
+            r.gy.reset();
             it = queue.erase(it);
             continue;
         }
@@ -327,15 +328,15 @@ int lbm_server_submit(lbm_server* s, const lbm_problem* p, int dtype, double tol
     r->mu = p->mu;
     r->tol = tol;
     r->max_iters = max_iters;
-    r->g.reset(new double[2 * n]);
-    double *gx = r->g.get(), *gy = gx + n;
+    r->gx.reset(new double[n]);
+    r->gy.reset(new double[n]);
     std::atomic<bool> bad{false};
     host_parallel((size_t)n, size_t(1) << 17, [&](size_t b, size_t e) {
         bool any = false;
         for (size_t i = b; i < e; ++i) {
-            gx[i] = p->gx[i];
-            gy[i] = p->gy[i];
-            any |= !std::isfinite(gx[i]) || !std::isfinite(gy[i]);
+            r->gx[i] = p->gx[i];
+            r->gy[i] = p->gy[i];
+            any |= !std::isfinite(r->gx[i]) || !std::isfinite(r->gy[i]);
         }
         if (any) bad = true;
     });
