@@ -1217,9 +1217,8 @@ k_step3(const StepParams a, const Coef<float> c) {
 // i.e. eight values per column and level boundary, and the horizontal movers
 // pass between lanes by shuffles.  A warp shares nothing, so there is no
 // barrier: its shared memory holds the rows on their way from global memory
-// (asynchronous copies LA rows ahead, which need no registers; every lane
-// reads back only what it copied itself) and the force of the last rows,
-// which the levels read one after the other.  The halo is T - 1 columns per
+// (asynchronous copies LA rows ahead, which need no registers) and the force of
+// the last rows, which the levels read one after the other.  The halo is T - 1 columns per
 // side and T - 1 rows per end.
 //
 // FP16-shifted storage decodes the stored deviations and carriers of the
@@ -1273,8 +1272,12 @@ template <int S, int T> __host__ __device__ constexpr int st_ring() {
 constexpr int kStCols = 72;
 template <int S> __host__ __device__ constexpr int st_row() { return S == S_F16S ? kStCols * (8 * 2 + 8) : kStCols * 8 * 4; }
 constexpr int kStFRow = 2 * kStCols * 4;
+// Rows of residual snapshot entries held (CHECK, 1024 bytes each): the row being
+// checked and the st_la rows on their way, each in the group of copies that the
+// wait of its own iteration is the first to cover (a power of two).
+template <int S> __host__ __device__ constexpr int st_snaps() { return S == S_F16S ? 4 : 2; }
 template <int S, int T, bool CHECK> __host__ __device__ constexpr int st_warp_smem() {
-    return kWvD * st_row<S>() + st_ring<S, T>() * kStFRow + (CHECK ? 2048 : 0);
+    return kWvD * st_row<S>() + st_ring<S, T>() * kStFRow + (CHECK ? 1024 * st_snaps<S>() : 0);
 }
 template <int S, int T, bool CHECK> __host__ __device__ constexpr int st_smem() {
     return kStNW * st_warp_smem<S, T, CHECK>();
@@ -1351,7 +1354,8 @@ __device__ __forceinline__ void strip_walk(const StepParams& a, const PairCoef& 
                                            int rows, ResAcc2& acc, bool half = false) {
     static_assert(OX % 2 == 0 && OX <= st_ox<S, T>(), "pairs, within the slots");
     constexpr int LAG = st_lag<S>(), H = st_halo<S, T>(), HL = st_left<S, T>(),
-                  LA = st_la<S>(), R = st_ring<S, T>(), ROW = st_row<S>();
+                  LA = st_la<S>(), R = st_ring<S, T>(), ROW = st_row<S>(), SN = st_snaps<S>();
+    static_assert(SN > LA && (!CHECK || LA <= 2 * H), "a snapshot entry has a slot until it is read, and is copied in time");
     constexpr int OFF = 1 - LAG;                             // copied row of local row i: i + OFF
     constexpr int AHEAD = 2 * OFF + LA;                      // rows copied ahead of iteration i
     constexpr int CA = S == S_F16S ? 8 : 4;                  // columns of a chunk of populations
@@ -1372,7 +1376,7 @@ __device__ __forceinline__ void strip_walk(const StepParams& a, const PairCoef& 
     const int64_t n = a.plane;
     const int nit = rows + 2 * H;
     const uint32_t frc = sm + kWvD * ROW;                   // force ring
-    const uint32_t snp = frc + R * kStFRow + lane * 32;      // snapshot entries of two rows (CHECK)
+    const uint32_t snp = frc + R * kStFRow + lane * 32;      // snapshot entries of SN rows (CHECK)
     const uint32_t own = (uint32_t)(xs - xa0);               // the lane's first column within a row
     // Copies of a row: 16-byte chunks, chunk q = lane + 32 m (FP32: 18 per
     // plane, eight populations, then the force; FP16S: 9 per plane, eight
@@ -1443,13 +1447,13 @@ __device__ __forceinline__ void strip_walk(const StepParams& a, const PairCoef& 
         constexpr int K = decltype(k_c)::value;
         pair_t f[8];
         __syncwarp();                             // every lane is done with the rows this copy replaces
-        if (CHECK && ok && i + 1 >= 2 * H && i + 1 < nit) {
-            // snapshot entries of the next output row, in this row's group of
-            // copies (the entry after an odd lattice's last column is in the plane,
-            // too): as loads into registers the assembler moved them down to
-            // their use
-            const float2* sp = static_cast<const float2*>(a.snap) + (i >= 2 * H ? so + pitch : so);
-            const uint32_t d = snp + ((i + 1) & 1) * 1024;
+        if (CHECK && ok && i + LA >= 2 * H && i + LA < nit) {
+            // snapshot entries of the output row of iteration i + LA, in this row's
+            // group of copies, which is complete then (the entry after an odd
+            // lattice's last column is in the plane, too): as loads into registers
+            // the assembler moved them down to their use
+            const float2* sp = static_cast<const float2*>(a.snap) + (so + (int64_t)min(LA, i + LA - 2 * H) * pitch);
+            const uint32_t d = snp + ((i + LA) & (SN - 1)) * 1024;
             copy_async<16>(d, sp);
             copy_async<16>(d + 16, sp + n);
         }
@@ -1564,10 +1568,10 @@ __device__ __forceinline__ void strip_walk(const StepParams& a, const PairCoef& 
             if (CHECK) {
                 ResSnap<S> sn0, sn1;
                 pair_t e0, e1;
-                lds_pairs(snp + (i & 1) * 1024, e0, e1);
+                lds_pairs(snp + (i & (SN - 1)) * 1024, e0, e1);
                 unpk(e0, sn0.u.x, sn0.u.y);
                 unpk(e1, sn1.u.x, sn1.u.y);
-                lds_pairs(snp + (i & 1) * 1024 + 16, e0, e1);
+                lds_pairs(snp + (i & (SN - 1)) * 1024 + 16, e0, e1);
                 unpk(e0, sn0.v.x, sn0.v.y);
                 unpk(e1, sn1.v.x, sn1.v.y);
                 check_pair<S>(acc, sn0, sn1, f, gx, gy, [&](float2 u0, float2 v0, float2 u1, float2 v1) {
