@@ -40,7 +40,7 @@ struct Request {
     int nx = 0, ny = 0, dtype = LBM_F32;
     double lambda = 0.0, mu = 0.0, tol = 0.0;
     int64_t max_iters = 0;
-    std::unique_ptr<double[]> gx, gy;       // until admitted
+    std::unique_ptr<double[]> gx, gy;       // until the arena's copies of them are done
     std::unique_ptr<double[]> fields;       // 5 * nx * ny once done
     int state = R_QUEUED;
     int status = LBM_OK;
@@ -85,6 +85,7 @@ struct lbm_server {
     uint64_t next_ticket = 1;
     std::map<uint64_t, std::unique_ptr<Request>> reqs;
     std::deque<uint64_t> queue;                 // admission order
+    std::vector<uint64_t> uploading;            // admitted since the stream was last waited for
     std::map<int, uint64_t> slot_owner[2];      // arena slot -> ticket
     // statistics
     int64_t submitted = 0, completed = 0, chunks = 0, lups = 0;
@@ -135,6 +136,12 @@ void lbm_server::run() {
             fail_msg = err;
             break;
         }
+        // the chunk's end was waited for: the arenas hold the forces admitted before it
+        for (uint64_t t : uploading) {
+            reqs[t]->gx.reset();
+            reqs[t]->gy.reset();
+        }
+        uploading.clear();
         ++chunks;
         device_ms += both ? std::max(ms[0], ms[1]) : ms[0] + ms[1];   // (side by side: the longer one)
         for (auto& q : queue) {
@@ -156,6 +163,8 @@ void lbm_server::run() {
         }
     }
     if (failed != LBM_OK) {
+        // (a request that is taken back frees its force: no copy may still read it)
+        cudaStreamSynchronize(stream);
         // fail every outstanding request so that pollers see the error
         for (auto& kv : reqs)
             if (kv.second->state != R_DONE) {
@@ -187,8 +196,7 @@ int lbm_server::admit_locked() {
             r.slot = s;
             r.t_admit = clk::now();
             slot_owner[a][s] = r.ticket;
-            r.gx.reset();  // the arena holds the force now
-            r.gy.reset();
+            uploading.push_back(r.ticket);  // (the copies of its force may still run)
             it = queue.erase(it);
             continue;
         }

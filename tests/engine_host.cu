@@ -1,0 +1,294 @@
+// The host code of the arena and the server (lbm_engine.cu, lbm_server.cu) on a
+// stand-in for the CUDA runtime, without a GPU: device memory is host memory,
+// kernels do nothing but advance the clock of their stream by a millisecond, and
+// copies and fills run, in order, when the stream is waited for -- as late as the
+// runtime allows.  Freeing the source of a copy that has not run is recorded.
+// usage: engine_host SCENARIO; prints "ok" or what is wrong.
+#include <atomic>
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include <functional>
+#include <map>
+#include <mutex>
+#include <new>
+#include <set>
+#include <string>
+#include <vector>
+
+#include "lbm_engine.cu"
+#include "lbm_server.cu"
+
+namespace fake {
+
+// Sources of copies that have not run (no allocation: read from operator delete).
+constexpr int kMost = 1 << 12;
+struct Source {
+    const char* p;
+    size_t n;
+};
+Source sources[kMost];
+int nsources = 0;
+std::atomic_flag lock = ATOMIC_FLAG_INIT;
+std::atomic<int> freed_in_flight{0};
+
+struct Hold {
+    Hold() {
+        while (lock.test_and_set()) {}
+    }
+    ~Hold() { lock.clear(); }
+};
+
+void check_free(const void* p) {
+    if (!p) return;
+    Hold h;
+    for (int i = 0; i < nsources; ++i)
+        if (sources[i].p == p) ++freed_in_flight;
+}
+
+std::mutex mu;
+std::vector<std::function<void()>> work;      // of all streams (each wait runs all of it)
+std::map<char*, size_t> device, pinned;       // allocations
+std::map<void*, double> clocks;               // of the streams, ms
+std::map<void*, double> events;
+size_t device_bytes = 0, device_peak = 0;
+int launches = 0, fail_launch = -1;           // the launch of this number fails
+
+bool within(const std::map<char*, size_t>& m, const void* p, size_t n) {
+    auto it = m.upper_bound((char*)p);
+    if (it == m.begin()) return false;
+    --it;
+    return (char*)p >= it->first && (char*)p + n <= it->first + it->second;
+}
+
+void run_all() {
+    std::vector<std::function<void()>> now;
+    {
+        std::lock_guard<std::mutex> l(mu);
+        now.swap(work);
+    }
+    for (auto& f : now) f();
+    Hold h;
+    nsources = 0;
+}
+
+cudaError_t launch(void* stream) {
+    std::lock_guard<std::mutex> l(mu);
+    if (launches++ == fail_launch) return cudaErrorLaunchFailure;
+    clocks[stream] += 1.0;
+    return cudaSuccess;
+}
+
+}  // namespace fake
+
+#ifndef __CUDA_ARCH__      // (host only)
+void* operator new(size_t n) {
+    if (void* p = std::malloc(n ? n : 1)) return p;
+    throw std::bad_alloc();
+}
+void* operator new[](size_t n) { return operator new(n); }
+void operator delete(void* p) noexcept {
+    fake::check_free(p);
+    std::free(p);
+}
+void operator delete[](void* p) noexcept { operator delete(p); }
+void operator delete(void* p, size_t) noexcept { operator delete(p); }
+void operator delete[](void* p, size_t) noexcept { operator delete(p); }
+
+extern "C" {
+cudaError_t cudaMalloc(void** p, size_t n) {
+    std::lock_guard<std::mutex> l(fake::mu);
+    *p = std::calloc(1, n);
+    fake::device[(char*)*p] = n;
+    fake::device_bytes += n;
+    fake::device_peak = std::max(fake::device_peak, fake::device_bytes);
+    return cudaSuccess;
+}
+cudaError_t cudaFree(void* p) {
+    fake::run_all();
+    std::lock_guard<std::mutex> l(fake::mu);
+    fake::device_bytes -= fake::device[(char*)p];
+    fake::device.erase((char*)p);
+    std::free(p);
+    return cudaSuccess;
+}
+cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) {
+    std::lock_guard<std::mutex> l(fake::mu);
+    *p = std::calloc(1, n);
+    fake::pinned[(char*)*p] = n;
+    return cudaSuccess;
+}
+cudaError_t cudaMallocHost(void** p, size_t n) { return cudaHostAlloc(p, n, 0); }
+cudaError_t cudaFreeHost(void* p) {
+    fake::run_all();
+    std::lock_guard<std::mutex> l(fake::mu);
+    fake::pinned.erase((char*)p);
+    std::free(p);
+    return cudaSuccess;
+}
+cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, enum cudaMemcpyKind, cudaStream_t) {
+    std::lock_guard<std::mutex> l(fake::mu);
+    fake::work.push_back([=] { std::memcpy(d, s, n); });
+    fake::Hold h;
+    if (fake::nsources < fake::kMost) fake::sources[fake::nsources++] = {(const char*)s, n};
+    return cudaSuccess;
+}
+cudaError_t cudaMemsetAsync(void* d, int v, size_t n, cudaStream_t) {
+    std::lock_guard<std::mutex> l(fake::mu);
+    fake::work.push_back([=] { std::memset(d, v, n); });
+    return cudaSuccess;
+}
+cudaError_t cudaPointerGetAttributes(struct cudaPointerAttributes* a, const void* p) {
+    std::lock_guard<std::mutex> l(fake::mu);
+    std::memset(a, 0, sizeof(*a));
+    a->type = fake::within(fake::pinned, p, 1) ? cudaMemoryTypeHost : cudaMemoryTypeUnregistered;
+    return cudaSuccess;
+}
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) {
+    *s = (cudaStream_t)std::malloc(1);
+    return cudaSuccess;
+}
+cudaError_t cudaStreamDestroy(cudaStream_t s) {
+    std::free(s);
+    return cudaSuccess;
+}
+cudaError_t cudaStreamSynchronize(cudaStream_t) {
+    fake::run_all();
+    return cudaSuccess;
+}
+cudaError_t cudaStreamWaitEvent(cudaStream_t s, cudaEvent_t e, unsigned) {
+    std::lock_guard<std::mutex> l(fake::mu);
+    fake::clocks[s] = std::max(fake::clocks[s], fake::events[e]);
+    return cudaSuccess;
+}
+cudaError_t cudaEventCreate(cudaEvent_t* e) {
+    *e = (cudaEvent_t)std::malloc(1);
+    return cudaSuccess;
+}
+cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) { return cudaEventCreate(e); }
+cudaError_t cudaEventDestroy(cudaEvent_t e) {
+    std::free(e);
+    return cudaSuccess;
+}
+cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s) {
+    std::lock_guard<std::mutex> l(fake::mu);
+    fake::events[e] = fake::clocks[s];
+    return cudaSuccess;
+}
+cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t a, cudaEvent_t b) {
+    std::lock_guard<std::mutex> l(fake::mu);
+    *ms = (float)(fake::events[b] - fake::events[a]);
+    return cudaSuccess;
+}
+cudaError_t cudaGetDevice(int* d) {
+    *d = 0;
+    return cudaSuccess;
+}
+cudaError_t cudaSetDevice(int) { return cudaSuccess; }
+cudaError_t cudaDeviceGetAttribute(int* v, enum cudaDeviceAttr, int) {
+    *v = 152;
+    return cudaSuccess;
+}
+const char* cudaGetErrorString(cudaError_t) { return "stand-in"; }
+cudaError_t cudaGetLastError() { return cudaSuccess; }
+cudaError_t cudaStreamBeginCapture(cudaStream_t, enum cudaStreamCaptureMode) { return cudaErrorNotSupported; }
+cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t*) { return cudaErrorNotSupported; }
+cudaError_t cudaGraphInstantiate(cudaGraphExec_t*, cudaGraph_t, unsigned long long) { return cudaErrorNotSupported; }
+cudaError_t cudaGraphDestroy(cudaGraph_t) { return cudaSuccess; }
+cudaError_t cudaGraphExecDestroy(cudaGraphExec_t) { return cudaSuccess; }
+cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) { return cudaErrorNotSupported; }
+cudaError_t cudaLaunchKernel(const void*, dim3, dim3, void**, size_t, cudaStream_t s) { return fake::launch(s); }
+unsigned __cudaPushCallConfiguration(dim3, dim3, size_t, cudaStream_t) { return 0; }
+cudaError_t __cudaPopCallConfiguration(dim3*, dim3*, size_t*, void*) { return cudaSuccess; }
+void** __cudaRegisterFatBinary(void*) {
+    static void* handle;
+    return &handle;
+}
+void __cudaRegisterFatBinaryEnd(void**) {}
+void __cudaUnregisterFatBinary(void**) {}
+void __cudaRegisterFunction(void**, const char*, char*, const char*, int, uint3*, uint3*, dim3*, dim3*, int*) {}
+char __cudaInitModule(void**) { return 0; }
+cudaError_t __cudaGetKernel(cudaKernel_t*, const void*) { return cudaSuccess; }
+cudaError_t __cudaLaunchKernel(cudaKernel_t, dim3, dim3, void**, size_t, cudaStream_t s) { return fake::launch(s); }
+}
+
+#endif
+
+// What the engine launches (lbm_arena.cu, lbm_step_f32.cu, lbm_step_f16s.cu).
+namespace lbm {
+int set_last_error(int code, const std::string&) { return code; }
+cudaError_t launch_arena_chunk(int, int, const BatchArgs&, int, cudaStream_t st) { return fake::launch(st); }
+int arena_occupancy(int, int) { return 1; }
+cudaError_t launch_arena_strips(int, int, bool, const BatchArgs&, const uint2*, int, int, cudaStream_t st) {
+    return fake::launch(st);
+}
+cudaError_t launch_arena_pairs(int, bool, const BatchArgs&, const uint2*, int, int, cudaStream_t st) {
+    return fake::launch(st);
+}
+cudaError_t launch_arena_ghosts(int, const BatchArgs&, const uint2*, int, cudaStream_t st) { return fake::launch(st); }
+cudaError_t launch_arena_force(const ForceIn&, cudaStream_t st) { return fake::launch(st); }
+template <int S>
+cudaError_t Ops<S>::fields(const StepParams&, const Coef<double>&, T, const FieldOut&, cudaStream_t st) {
+    return fake::launch(st);
+}
+__global__ void k_scale_float(float*, int64_t, float) {}
+}  // namespace lbm
+
+namespace {
+
+#define EXPECT(x)                                                          \
+    do {                                                                   \
+        if (!(x)) {                                                        \
+            std::printf("line %d: not so: %s\n", __LINE__, #x);            \
+            std::exit(1);                                                  \
+        }                                                                  \
+    } while (0)
+
+struct Problem {
+    int nx, ny;
+    std::vector<double> gx, gy, out[5];
+    lbm_result r{};
+    Problem(int nx, int ny) : nx(nx), ny(ny), gx((size_t)nx * ny, 1.0), gy(gx) {
+        double** o[5] = {&r.ux, &r.uy, &r.sxx, &r.syy, &r.sxy};
+        for (int k = 0; k < 5; ++k) {
+            out[k].assign(gx.size(), -7.0);
+            *o[k] = out[k].data();
+        }
+    }
+    lbm_problem in() { return {nx, ny, 0.3, 0.4, gx.data(), gy.data()}; }
+};
+
+// The force of an admitted request outlives its copy to the device, also when the
+// chunk after the admission fails and the request is taken back at once.
+void server_force(bool fail) {
+    lbm_server* s = nullptr;
+    EXPECT(lbm_server_create(size_t(64) << 20, 100, &s) == LBM_OK);
+    if (fail) fake::fail_launch = 12;
+    std::vector<Problem> p;
+    for (int i = 0; i < 6; ++i) p.emplace_back(40 + i, 30);
+    std::vector<uint64_t> t;
+    for (int i = 0; i < 6; ++i) {
+        const lbm_problem in = p[i].in();
+        uint64_t ticket = 0;
+        if (lbm_server_submit(s, &in, i % 2 ? LBM_F16S : LBM_F32, 0.0, 300, &ticket) == LBM_OK) t.push_back(ticket);
+        else EXPECT(fail);
+    }
+    for (size_t i = 0; i < t.size(); ++i) {
+        EXPECT(lbm_server_wait(s, t[i], 60.0, &p[i].r) == LBM_OK);
+        EXPECT(fail || p[i].r.iters == 300);
+    }
+    lbm_server_destroy(s);
+    EXPECT(fake::freed_in_flight == 0);
+}
+
+}  // namespace
+
+int main(int argc, char** argv) {
+    const std::string what = argc > 1 ? argv[1] : "";
+    if (what == "server_force") server_force(false);
+    else if (what == "server_force_failing") server_force(true);
+    else return 2;
+    std::printf("ok\n");
+    std::fflush(stdout);
+    std::_Exit(0);      // (the stand-in's maps go last)
+}
