@@ -87,8 +87,9 @@ int ArenaEngine::init(int dtype, int64_t node_capacity, int max_probs, int check
     int dev = 0;
     ECK(cudaGetDevice(&dev));
     ECK(cudaDeviceGetAttribute(&sms_, cudaDevAttrMultiProcessorCount, dev));
-    // (kRowSlack: a strip of the last problem reads past its last row)
-    const int64_t slack = (int64_t)max_probs * kArenaAlign + kRowSlack * 8;
+    // a strip of the last problem reads past its last row: that much of every
+    // buffer is not given out
+    const int64_t over = kRowSlack * 8, slack = (int64_t)max_probs * kArenaAlign + over;
     const int64_t pb = pop_bytes_per_node(dtype) * node_capacity + slack;
     const int64_t cb = car_bytes_per_node(dtype) * node_capacity + slack;
     const int64_t fb = kFsBytesPerNode * node_capacity + slack;
@@ -102,9 +103,9 @@ int ArenaEngine::init(int dtype, int64_t node_capacity, int max_probs, int check
     }
     ECK(cudaMalloc(&fs_, fb));
     dev_bytes_ += fb;
-    apop_.reset(pb);
-    acar_.reset(dtype == S_F16S ? cb : 0);
-    afs_.reset(fb);
+    apop_.reset(pb - over);
+    acar_.reset(dtype == S_F16S ? cb - over : 0);
+    afs_.reset(fb - over);
     probs_.assign(max_probs, HostProb());
     ECK(cudaMalloc(&d_probs_, sizeof(BatchProb) * max_probs));
     ECK(cudaMalloc(&d_acc_, sizeof(double) * kRes * max_probs));

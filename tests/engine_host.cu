@@ -51,6 +51,7 @@ std::vector<std::function<void()>> work;      // of all streams (each wait runs 
 std::map<char*, size_t> device, pinned;       // allocations
 std::map<void*, double> clocks;               // of the streams, ms
 std::map<void*, double> events;
+std::vector<size_t> sizes;                    // of the device allocations, in turn
 size_t device_bytes = 0, device_peak = 0;
 int launches = 0, fail_launch = -1;           // the launch of this number fails
 
@@ -100,6 +101,7 @@ cudaError_t cudaMalloc(void** p, size_t n) {
     std::lock_guard<std::mutex> l(fake::mu);
     *p = std::calloc(1, n);
     fake::device[(char*)*p] = n;
+    fake::sizes.push_back(n);
     fake::device_bytes += n;
     fake::device_peak = std::max(fake::device_peak, fake::device_bytes);
     return cudaSuccess;
@@ -281,12 +283,51 @@ void server_force(bool fail) {
     EXPECT(fake::freed_in_flight == 0);
 }
 
+// A full arena: what a strip reads beyond the rows of the last problem (at most 72
+// columns from eight before its first one) lies within the arena's buffers.
+void full_arena(int dtype) {
+    for (int nx : {16, 57, 64, 113, 200}) {
+        ArenaEngine e;
+        std::string err;
+        const int most = 256;
+        fake::sizes.clear();
+        EXPECT(e.init(dtype, 20000, most, 100, (cudaStream_t)&e, &err) == LBM_OK);
+        int64_t over = 0, pops = 0, cars = 0, fs = 0;
+        std::vector<double> g;
+        for (int ny = 64; ny >= 1;) {
+            g.assign((size_t)nx * ny, 1.0);
+            const int s = e.admit(nx, ny, 0.3, 0.4, g.data(), g.data(), 0.0, 100, &err);
+            if (s < 0) {
+                EXPECT(s == -1);
+                --ny;
+                continue;
+            }
+            const HostProb& p = e.prob(s);
+            if (!p.ghost) continue;
+            // from the first column of a problem to the last column its last strip's copies take
+            const int64_t last = (arena_strips(p.nx) - 1) * kArenaOX - st_left<S_F32, 5>() + kStCols;
+            const int64_t extent = (int64_t)p.pitch * (p.ny - 1) + p.ghost + last;
+            const int64_t b = dtype == S_F16S ? 2 : 4;
+            over = std::max(over, extent - p.plane);
+            pops = std::max(pops, p.pop_off + b * (7 * p.plane + extent));
+            if (dtype == S_F16S) cars = std::max(cars, p.car_off + 8 * extent);
+            fs = std::max(fs, p.fs_off + 4 * (p.plane + extent));
+        }
+        EXPECT(over > 0 && over <= kRowSlack);
+        const bool car = dtype == S_F16S;      // (allocated in turn: populations, carriers, both again, forces)
+        EXPECT(pops <= (int64_t)fake::sizes[0] && fs <= (int64_t)fake::sizes[car ? 4 : 2]);
+        EXPECT(!car || cars <= (int64_t)fake::sizes[1]);
+    }
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
     const std::string what = argc > 1 ? argv[1] : "";
     if (what == "server_force") server_force(false);
     else if (what == "server_force_failing") server_force(true);
+    else if (what == "full_arena_f32") full_arena(S_F32);
+    else if (what == "full_arena_f16s") full_arena(S_F16S);
     else return 2;
     std::printf("ok\n");
     std::fflush(stdout);
