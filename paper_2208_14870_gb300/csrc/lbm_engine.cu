@@ -5,7 +5,9 @@
 #include <cstdlib>
 #include <cstring>
 #include <fstream>
+#include <memory>
 #include <mutex>
+#include <new>
 #include <sstream>
 #include <sys/stat.h>
 
@@ -32,6 +34,40 @@ int cuerr(cudaError_t e, const char* what, std::string* err) {
 
 int64_t pop_bytes_per_node(int dtype) { return dtype == S_F16S ? 8 * 2 : 8 * 4; }
 int64_t car_bytes_per_node(int dtype) { return dtype == S_F16S ? 2 * 4 : 0; }
+// Copies between the caller's arrays and the device.  The runtime refuses host
+// ranges that are pinned in part, or in several parts (arrays that follow one
+// another, pinned each by itself): these go through memory of our own.
+constexpr size_t kBounce = size_t(16) << 20;
+cudaError_t copy_in(void* dst, const void* src, size_t bytes, cudaStream_t st) {
+    cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st);
+    if (e != cudaErrorInvalidValue) return e;
+    cudaGetLastError();
+    const std::unique_ptr<char[]> own(new (std::nothrow) char[std::min(bytes, kBounce)]);
+    if (!own) return cudaErrorMemoryAllocation;
+    e = cudaSuccess;
+    for (size_t at = 0; at < bytes && e == cudaSuccess; at += kBounce) {
+        const size_t len = std::min(bytes - at, kBounce);
+        std::memcpy(own.get(), static_cast<const char*>(src) + at, len);
+        e = cudaMemcpyAsync(static_cast<char*>(dst) + at, own.get(), len, cudaMemcpyHostToDevice, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    }
+    return e;
+}
+cudaError_t copy_out(void* dst, const void* src, size_t bytes, cudaStream_t st) {
+    cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, st);
+    if (e != cudaErrorInvalidValue) return e;
+    cudaGetLastError();
+    const std::unique_ptr<char[]> own(new (std::nothrow) char[std::min(bytes, kBounce)]);
+    if (!own) return cudaErrorMemoryAllocation;
+    e = cudaSuccess;
+    for (size_t at = 0; at < bytes && e == cudaSuccess; at += kBounce) {
+        const size_t len = std::min(bytes - at, kBounce);
+        e = cudaMemcpyAsync(own.get(), static_cast<const char*>(src) + at, len, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e == cudaSuccess) std::memcpy(static_cast<char*>(dst) + at, own.get(), len);
+    }
+    return e;
+}
 // force (2 FP32 planes) + residual snapshot (2 planes of (hi, lo) FP32 pairs)
 constexpr int64_t kFsBytesPerNode = 2 * 4 + 2 * 8;
 
@@ -224,8 +260,8 @@ int ArenaEngine::admit(int nx, int ny, double lambda, double mu, const double* g
     }
     unsigned long long* stat = d_stat_ + 2 * slot;
     float* force = reinterpret_cast<float*>(fs_ + p.fs_off);
-    ECK(cudaMemcpyAsync(d_force_, gx, sizeof(double) * n, cudaMemcpyHostToDevice, st_));
-    ECK(cudaMemcpyAsync(d_force_ + n, gy, sizeof(double) * n, cudaMemcpyHostToDevice, st_));
+    ECK(copy_in(d_force_, gx, sizeof(double) * n, st_));
+    ECK(copy_in(d_force_ + n, gy, sizeof(double) * n, st_));
     ECK(cudaMemsetAsync(stat, 0, 2 * sizeof(unsigned long long), st_));
     ECK(cudaMemsetAsync(force, 0, p.fs_bytes, st_));
     ForceIn f{};
@@ -728,8 +764,7 @@ int ArenaEngine::recover_many(int count, const int* slots, double* const* outs, 
                 int g = f + 1;
                 while (o[f] && g < 5 && o[g] == o[f] + (g - f) * n) ++g;
                 if (o[f])
-                    ECK(cudaMemcpyAsync(o[f], d_fields_ + off + f * n, sizeof(double) * n * (g - f),
-                                        cudaMemcpyDeviceToHost, st_));
+                    ECK(copy_out(o[f], d_fields_ + off + f * n, sizeof(double) * n * (g - f), st_));
                 f = g;
             }
             off += 5 * n;

@@ -128,8 +128,12 @@ cudaError_t cudaFreeHost(void* p) {
     std::free(p);
     return cudaSuccess;
 }
-cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, enum cudaMemcpyKind, cudaStream_t) {
+cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, enum cudaMemcpyKind kind, cudaStream_t) {
     std::lock_guard<std::mutex> l(fake::mu);
+    // (as the runtime does: host ranges that are pinned in part, or in two parts, are refused)
+    const char* h0 = kind == cudaMemcpyDeviceToHost ? (const char*)d : (const char*)s;
+    for (auto& r : fake::pinned)
+        if (h0 < r.first + r.second && h0 + n > r.first && !fake::within(fake::pinned, h0, n)) return cudaErrorInvalidValue;
     fake::work.push_back([=] { std::memcpy(d, s, n); });
     fake::Hold h;
     if (fake::nsources < fake::kMost) fake::sources[fake::nsources++] = {(const char*)s, n};
@@ -320,6 +324,34 @@ void full_arena(int dtype) {
     }
 }
 
+// Forces and results in host memory that is pinned in parts: arrays that follow
+// one another, pinned each by itself, and arrays across the end of a pinned range.
+void pinned_parts(int dtype) {
+    const int nx = 40, ny = 30, n = nx * ny;
+    std::vector<double> mem(7 * n, -7.0);
+    for (int k = 2; k < 7; ++k) fake::pinned[(char*)&mem[k * n]] = n * sizeof(double);
+    fake::pinned[(char*)mem.data()] = n / 2 * sizeof(double);          // half of g_x
+    for (int i = 0; i < 2 * n; ++i) mem[i] = 1.0;
+    ArenaEngine e;
+    std::string err;
+    EXPECT(e.init(dtype, 20000, 4, 100, (cudaStream_t)&e, &err) == LBM_OK);
+    const int s = e.admit(nx, ny, 0.3, 0.4, &mem[0], &mem[n], 0.0, 100, &err);
+    EXPECT(s >= 0);
+    EXPECT(e.run_chunk(kTileWave, nullptr, &err) == LBM_OK && e.prob(s).state == P_DONE);
+    double* outs[5];
+    for (int k = 0; k < 5; ++k) outs[k] = &mem[(2 + k) * n];
+    EXPECT(e.recover_many(1, &s, outs, &err) == LBM_OK);
+    for (int i = 2 * n; i < 7 * n; ++i) EXPECT(mem[i] == 0.0);
+    // pinned in part only
+    fake::pinned.erase((char*)&mem[4 * n]);
+    fake::pinned[(char*)&mem[4 * n]] = 100;
+    std::fill(mem.begin() + 2 * n, mem.end(), -7.0);
+    EXPECT(e.recover_many(1, &s, outs, &err) == LBM_OK);
+    for (int i = 2 * n; i < 7 * n; ++i) EXPECT(mem[i] == 0.0);
+    for (int k = 2; k < 7; ++k) fake::pinned.erase((char*)&mem[k * n]);
+    fake::pinned.erase((char*)mem.data());
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
@@ -328,6 +360,8 @@ int main(int argc, char** argv) {
     else if (what == "server_force_failing") server_force(true);
     else if (what == "full_arena_f32") full_arena(S_F32);
     else if (what == "full_arena_f16s") full_arena(S_F16S);
+    else if (what == "pinned_parts_f32") pinned_parts(S_F32);
+    else if (what == "pinned_parts_f16s") pinned_parts(S_F16S);
     else return 2;
     std::printf("ok\n");
     std::fflush(stdout);
