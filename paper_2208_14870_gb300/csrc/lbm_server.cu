@@ -5,8 +5,8 @@
 // queued; between chunks the worker admits queued requests whose lattice fits
 // the free arena memory (first-fit, oldest first, with a bound on how long a
 // request can be bypassed by later ones), runs one chunk of check_every steps
-// of every resident problem (strip chunks of both arenas side by side), and retires problems whose residual dropped
-// below their tolerance: their displacement and stress are recovered into
+// of every resident problem (both arenas on one stream), and retires problems
+// whose residual dropped below their tolerance: their displacement and stress are recovered into
 // host memory owned by the request, their arena memory is freed for the next
 // admissions, and their latency (submission to completion) is recorded.
 #include <algorithm>
@@ -121,9 +121,10 @@ void lbm_server::run() {
         lk.unlock();
         std::string err;
         float ms[2] = {0.0f, 0.0f};
-        // Strip chunks of the two arenas run side by side: neither fills the GPU with
-        // small problems (12 of them, 100 steps: 1.19 -> 1.08 ms).  The other chunk
-        // kernels meet at grid barriers and have the device to themselves.
+        // Strip chunks: both arenas' launches go out before the first wait, one chunk
+        // after the other on the device, so that launching the second one's 20 to 25
+        // kernels overlaps the first one's work (unless its tables change, which
+        // waits; 12 problems, 100 steps: 1.19 -> 1.08 ms).
         const bool both = tile_v == kTileWave;
         for (int a = 0; a < 2 && rc == LBM_OK; ++a)
             if (arena[a]->running() > 0)
@@ -143,7 +144,7 @@ void lbm_server::run() {
         }
         uploading.clear();
         ++chunks;
-        device_ms += both ? std::max(ms[0], ms[1]) : ms[0] + ms[1];   // (side by side: the longer one)
+        device_ms += ms[0] + ms[1];
         for (auto& q : queue) {
             auto it = reqs.find(q);
             if (it != reqs.end()) ++it->second->bypassed;

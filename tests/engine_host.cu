@@ -287,6 +287,25 @@ void server_force(bool fail) {
     EXPECT(fake::freed_in_flight == 0);
 }
 
+// The device time a server reports is the time its kernels took: one millisecond
+// each here, all of a chunk's on one stream.
+void server_device_ms() {
+    lbm_server* s = nullptr;
+    EXPECT(lbm_server_create(size_t(64) << 20, 100, &s) == LBM_OK);
+    const int before = fake::launches;
+    Problem a(300, 40), b(310, 50);
+    lbm_problem in[2] = {a.in(), b.in()};
+    uint64_t t[2];
+    EXPECT(lbm_server_submit(s, &in[0], LBM_F32, 0.0, 200, &t[0]) == LBM_OK);
+    EXPECT(lbm_server_submit(s, &in[1], LBM_F16S, 0.0, 200, &t[1]) == LBM_OK);
+    EXPECT(lbm_server_wait(s, t[0], 60.0, &a.r) == LBM_OK && lbm_server_wait(s, t[1], 60.0, &b.r) == LBM_OK);
+    lbm_stats st{};
+    EXPECT(lbm_server_stats(s, &st) == LBM_OK);
+    // (two forces and two recoveries are no part of a chunk)
+    EXPECT(st.device_ms == fake::launches - before - 4);
+    lbm_server_destroy(s);
+}
+
 // A full arena: what a strip reads beyond the rows of the last problem (at most 72
 // columns from eight before its first one) lies within the arena's buffers.
 void full_arena(int dtype) {
@@ -358,6 +377,7 @@ int main(int argc, char** argv) {
     const std::string what = argc > 1 ? argv[1] : "";
     if (what == "server_force") server_force(false);
     else if (what == "server_force_failing") server_force(true);
+    else if (what == "server_device_ms") server_device_ms();
     else if (what == "full_arena_f32") full_arena(S_F32);
     else if (what == "full_arena_f16s") full_arena(S_F16S);
     else if (what == "pinned_parts_f32") pinned_parts(S_F32);
