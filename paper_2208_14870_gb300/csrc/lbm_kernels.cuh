@@ -94,8 +94,9 @@ __device__ __forceinline__ T ldg(const T* p) { return __ldg(p); }
 //   FP64 storage: u from the FP64 collision, FP64 snapshot and partials;
 //   FP32 / FP16S: u as an exact FP32 pair from exact_displacement, the
 //   snapshot as (hi, lo) pairs (16 bytes per node, like two FP64 planes), and
-//   pair partials (about 2^-44 relative), converted to FP64 per thread.
-// Warps, blocks and the grid combine the partials in FP64.
+//   pair partials (about 2^-44 relative); the sums are converted to FP64 per thread.
+// Warps, blocks and the grid combine the sums in FP64 (ResPart: the maxima as pairs
+// within a block).
 template <int S> struct ResSnap { float2 u, v; };          // (hi, lo) per component
 template <> struct ResSnap<S_F64> { double u, v; };
 
@@ -289,33 +290,41 @@ __device__ __forceinline__ void pair_add(float& h, float& l, float g, float m) {
     h = r;
 }
 
-// The partials of a thread's, warp's or block's nodes as pairs: combined as they
-// are, and converted to FP64 once per block (an FP64 instruction takes 64 cycles
-// of a scheduler: with conversions and sums in every thread they were 5 us of
-// a checked launch of k_tile).
+// The partials of a thread's, warp's or block's nodes: the maxima as pairs, which
+// lose nothing when they are combined, the sums in FP64 from the thread on (their
+// pairs have FP32's range, which a block's sum may leave).  An FP64 instruction
+// takes 64 cycles of a scheduler: maxima converted in every thread and two
+// sums that cross the warp side by side were 38 of them, 5 us of a checked launch of
+// k_tile.
 struct ResPart {
-    float dh, dl, uh, ul, d2h, d2l, u2h, u2l;
+    float dh, dl, uh, ul;
+    double d2, u2;
     bool bad;
-    __device__ __forceinline__ void add(const ResPart& o) {
-        pair_max_abs(dh, dl, o.dh, o.dl);
-        pair_max_abs(uh, ul, o.uh, o.ul);
-        pair_add(d2h, d2l, o.d2h, o.d2l);
-        pair_add(u2h, u2l, o.u2h, o.u2l);
-        bad |= o.bad;
+    __device__ __forceinline__ void add_maxima(float odh, float odl, float ouh, float oul) {
+        pair_max_abs(dh, dl, odh, odl);
+        pair_max_abs(uh, ul, ouh, oul);
     }
+    // over the warp (in every lane); the sums share their four last steps, d2 in the lower half-warp and u2 in the upper
     __device__ __forceinline__ void add_warp() {
+        constexpr unsigned ALL = 0xffffffffu;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
-            auto get = [&](float v) { return __shfl_xor_sync(0xffffffffu, v, o); };
-            add(ResPart{get(dh), get(dl), get(uh), get(ul), get(d2h), get(d2l), get(u2h), get(u2l), false});
+            auto get = [&](float v) { return __shfl_xor_sync(ALL, v, o); };
+            add_maxima(get(dh), get(dl), get(uh), get(ul));
         }
-        bad = __any_sync(0xffffffffu, bad);
+        const bool upper = threadIdx.x & 16;
+        double s = (upper ? u2 : d2) + __shfl_xor_sync(ALL, upper ? d2 : u2, 16);
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(ALL, s, o);
+        d2 = __shfl_sync(ALL, s, 0);
+        u2 = __shfl_sync(ALL, s, 16);
+        bad = __any_sync(ALL, bad);
     }
     __device__ __forceinline__ void to_double(double w[kRes]) const {
         w[0] = max_to_double(dh, dl);
         w[1] = max_to_double(uh, ul);
-        w[2] = pair_to_double(d2h, d2l);
-        w[3] = pair_to_double(u2h, u2l);
+        w[2] = d2;
+        w[3] = u2;
         w[4] = bad ? 1.0 : 0.0;
     }
 };
@@ -326,9 +335,18 @@ __device__ __forceinline__ ResPart res_part(const ResAcc2& r) {
     unpk(r.d2l, b[0], b[1]);
     unpk(r.u2h, c[0], c[1]);
     unpk(r.u2l, d[0], d[1]);
-    const ResPart none{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, false};
-    ResPart p = r.own0 ? ResPart{r.dh[0], r.dl[0], r.uh[0], r.ul[0], a[0], b[0], c[0], d[0], f[0] != 0.0f} : none;
-    p.add(r.own1 ? ResPart{r.dh[1], r.dl[1], r.uh[1], r.ul[1], a[1], b[1], c[1], d[1], f[1] != 0.0f} : none);
+    ResPart p{0.f, 0.f, 0.f, 0.f, 0.0, 0.0, false};
+    float ah = 0.f, al = 0.f, ch = 0.f, cl = 0.f;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        if (h ? r.own1 : r.own0) {
+            p.add_maxima(r.dh[h], r.dl[h], r.uh[h], r.ul[h]);
+            pair_add(ah, al, a[h], b[h]);
+            pair_add(ch, cl, c[h], d[h]);
+            p.bad |= f[h] != 0.0f;
+        }
+    p.d2 = pair_to_double(ah, al);
+    p.u2 = pair_to_double(ch, cl);
     return p;
 }
 
@@ -572,7 +590,7 @@ __device__ __forceinline__ void scatter_local(const StepParams& a, int64_t idx,
 // check; without one (the library's own check launches) the blocks stop after
 // writing their partials and k_residual_finish combines them in a separate
 // launch.
-// Paired partials combined as pairs (no counter): the block's partial set.
+// Paired partials (no counter): the block's partial set.
 __device__ __forceinline__ void residual_reduce_pairs(const StepParams& a, const ResAcc2& acc) {
     __shared__ ResPart sh[32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -582,7 +600,7 @@ __device__ __forceinline__ void residual_reduce_pairs(const StepParams& a, const
     __syncthreads();
     if (warp != 0) return;
     if (lane < (int)(blockDim.x >> 5)) p = sh[lane];
-    else p = ResPart{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, false};
+    else p = ResPart{0.f, 0.f, 0.f, 0.f, 0.0, 0.0, false};
     p.add_warp();
     if (lane != 0) return;
     double w[kRes];

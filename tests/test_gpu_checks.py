@@ -40,3 +40,27 @@ def test_f16s_strip_residual_beyond_l2(nx, ny):
     want = [np.abs(d).max() / (4 * np.abs(u[1]).max()), np.sqrt((d ** 2).sum() / (u[1] ** 2).sum()) / 4,
             np.abs(u[1]).max(), np.sqrt((u[1] ** 2).sum())]
     assert np.allclose(got[:4], want, rtol=1e-12, atol=0.0) and got[4] == 0.0
+
+
+# Norms whose squares sum to more than FP32 holds over a block, but not over a
+# thread's nodes: a lattice scaled by a power of two has the same residuals and
+# scaled norms.  A uniform force (u = 7.5 at the last check) and a little noise;
+# 2^122 per node, at most 16 nodes a thread.
+@pytest.mark.parametrize("nx,ny,plan", [(100, 75, None), (333, 100, None), (300, 40, (4, 8)), (257, 64, (4, 8))])
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+def test_norms_beyond_fp32_squares(nx, ny, plan, dtype):
+    if dtype == "f64" and plan:
+        pytest.skip("no schedules for FP64 storage")
+    lam, mu = W.lame_2d(1.0, 0.3)
+    g = np.random.RandomState(nx).standard_normal((2, ny, nx)) * 2.0 ** -10
+    g[0] += 1.0
+    got = []
+    for e in (0, 58):
+        with Lattice(nx, ny, lam, mu, dtype) as lat:
+            if plan:
+                lat.steps_per_launch, lat.wavefront = plan
+            lat.set_force(*(g * 2.0 ** e))
+            r = lat.iterate_checked(8, 4)
+            got.append(np.concatenate([r[:2], r[2:4] * 2.0 ** -e, r[4:]]))
+    assert np.isfinite(got[0]).all() and got[0][2] > 7.0
+    assert np.allclose(got[1], got[0], rtol=1e-14, atol=0.0)
