@@ -916,12 +916,16 @@ int lbm_get_launch_steps(lbm_ctx* c, int* k) {
     int rc = check_ctx(c);
     if (rc) return rc;
     if (!k) return fail(LBM_ERR_ARG, "lbm_get_launch_steps: null pointer");
-    *k = c->spl >= 4 && !wave_on(c) ? 3 : c->spl;
-    if (auto_on(c)) CK(choose_plan(c));
-    if (auto_on(c) && c->plan == 2) *k = c->tile.T;
-    else if (c->dtype == LBM_F32 && (auto_on(c) || (c->spl >= 4 && wave_on(c)))) {
+    if (c->dtype == LBM_F64) {
+        *k = c->tile64.T;
+        return LBM_OK;
+    }
+    *k = group_steps(c);
+    if (c->auto_plan) CK(choose_plan(c));
+    if (c->auto_plan && c->plan == 2) *k = c->tile.T;
+    else if (c->dtype == LBM_F32 && (c->auto_plan || (c->spl >= 4 && wave_on(c)))) {
         CK(wave_plan(c));
-        *k = c->wave_T;
+        *k = *std::max_element(c->wave_first, c->wave_first + kWavePlan + 1);   // (wave_T among them)
     }
     return LBM_OK;
 }
