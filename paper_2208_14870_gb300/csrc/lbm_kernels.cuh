@@ -2014,16 +2014,22 @@ k_fields(const StepParams a, const Coef<double> c, typename StoreT<S>::T theta, 
         syy = from_fixed<true>(P - D, e64);
         mb11 = from_fixed<true>(-2 * X, e64);
     } else {
-        double w[8];
-        const double scale = S == S_F16S ? (double)a.hinv : 1.0;
+        uint32_t any = nonzero(gxs) | nonzero(gys);
 #pragma unroll
-        for (int p = 0; p < 8; ++p) w[p] = (double)f[p] * scale;
-        const Mom<double> m = moments(w);
-        u = m.m10 + 0.5 * ((double)gxs * scale);
-        v = m.m01 + 0.5 * ((double)gys * scale);
-        sxx = -0.5 * (c.bs * m.ms + c.bd * m.md);
-        syy = -0.5 * (c.bs * m.ms - c.bd * m.md);
-        mb11 = c.b11 * m.m11;
+        for (int p = 0; p < 8; ++p) any |= nonzero(f[p]);
+        u = v = sxx = syy = mb11 = 0.0;                  // a node of zeros (as in step_f64)
+        if (any) {
+            double w[8];
+            const double scale = S == S_F16S ? (double)a.hinv : 1.0;
+#pragma unroll
+            for (int p = 0; p < 8; ++p) w[p] = (double)f[p] * scale;
+            const Mom<double> m = moments(w);
+            u = m.m10 + 0.5 * ((double)gxs * scale);
+            v = m.m01 + 0.5 * ((double)gys * scale);
+            sxx = -0.5 * (c.bs * m.ms + c.bd * m.md);
+            syy = -0.5 * (c.bs * m.ms - c.bd * m.md);
+            mb11 = c.b11 * m.m11;
+        }
     }
     const double un = 1.0;         // (the fields' own unit)
     const int64_t o = out.tr ? (int64_t)x * ny + y : (int64_t)y * nx + x;
