@@ -56,8 +56,11 @@ typedef struct lbm_ctx lbm_ctx;
 
 /* Population storage type.  Collision arithmetic is FP32 for LBM_F32 and
  * LBM_F16S; for LBM_F64 it is 64-bit integer (a node's values as multiples of
- * 2^-58 of the largest of them, the results rounded to FP64 once: no less exact
- * than FP64 arithmetic), and FP64 at the ends of the exponent range.
+ * 2^-58 of the power of two above the largest of them, the results rounded to FP64
+ * once), and FP64 at the ends of the exponent range.  The integer collision's
+ * error is relative to the node's largest value, below 2^-52.9 of that power of
+ * two before the last rounding; a value more than 2^58 times smaller than the node's
+ * largest one is taken for zero.
  *  LBM_F64  : 8 FP64 planes.
  *  LBM_F32  : 8 FP32 planes.
  *  LBM_F16S : "shifted" FP16 storage: per node the first post-collision

@@ -216,10 +216,14 @@ __device__ __forceinline__ void collide_populations(const Mom<T>& m, T gx, T gy,
 // runs in integers: the node's populations and half forces become multiples of
 // one unit, 2^-58 of the power of two above the largest of them (at least five
 // bits more than FP64 holds of that one), their sums are exact, its five
-// products (eight at general rates) are good to about a unit, and the results
-// are rounded to FP64 once.  No result is off by more than FP64 arithmetic's
-// own rounding of the sums, and the first moments of the result are mbar + g / 2 up
-// to that last rounding.  About 600 integer instructions, two cycles of the ALU
+// products (eight at general rates) are good to two and a half units, and the results
+// are rounded to FP64 once.  So the error is bounded relative to the node's largest
+// value: before the last rounding a population is within 20 units of the exact
+// result (34 at general rates; each input loses less than a unit), 2^-53.7 (2^-52.9) of
+// that power of two, where FP64 arithmetic rounds at 2^-53 of each of its partial
+// sums.  A value far below the node's largest one has fewer bits than
+// FP64 would keep of it until it meets the others in a sum, and none from 2^-58
+// on.  The first moments of the result are mbar + g / 2 up to the last rounding.  About 600 integer instructions, two cycles of the ALU
 // for 360 of them, against 34 FP64 ones (2176 cycles): 1500 x 1100 116 -> 44 us
 // per step; with the signs on the FMA pipe 42.6, and with two, three, four, five,
 // six of the results on the FP64 pipe 40.8, 39.6, 38.7, 38.7, 44.0 us.
