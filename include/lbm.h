@@ -449,7 +449,8 @@ typedef struct lbm_stats {
     int64_t lattice_updates;   /* sum of nodes x steps of completed problems */
     double device_ms;          /* device time of all chunks */
     int64_t chunks;
-    size_t hbm_bytes;          /* device memory held by the arenas */
+    size_t hbm_bytes;          /* device memory held by the arenas, with the staging of forces and fields, which
+                                  is outside the budget (16 and 40 bytes per node of the largest problem) */
     int peak_running;          /* most problems resident at once */
     int tile_v;                /* tile code: 1, 2, 4 (warps of 32 columns), LBM_TILE_TWO_STEP or LBM_TILE_WAVE */
     int failed;                /* LBM_OK, or the error that stopped the worker */

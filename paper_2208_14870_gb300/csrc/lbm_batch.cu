@@ -114,6 +114,14 @@ extern "C" int lbm_batch_solve(int count, const lbm_problem* probs, int dtype, d
             } catch (...) {   // (no thread to be had: the copies take the faults)
             }
         }
+        int64_t most = 0, fields = 0;
+        for (int i = 0; i < count; ++i) {
+            const lbm_result& r = results[i];
+            const int64_t n = (int64_t)probs[i].nx * probs[i].ny;
+            most = std::max(most, n);
+            if (r.ux || r.uy || r.sxx || r.syy || r.sxy) fields += 5 * n;
+        }
+        rc = eng.reserve_staging(most, fields, &err);
         std::vector<int> slot(count);
         for (int i = 0; i < count && rc == LBM_OK; ++i) {
             const lbm_problem& p = probs[i];

@@ -87,7 +87,6 @@ ArenaEngine::~ArenaEngine() {
     if (d_tiles_) cudaFree(d_tiles_);
     if (d_ntiles_) cudaFree(d_ntiles_);
     if (d_fields_) cudaFree(d_fields_);
-    if (d_force_) cudaFree(d_force_);
     if (d_stat_) cudaFree(d_stat_);
     if (h_acc_) cudaFreeHost(h_acc_);
     if (h_tiles_) cudaFreeHost(h_tiles_);
@@ -130,25 +129,20 @@ int ArenaEngine::init(int dtype, int64_t node_capacity, int max_probs, int check
     const int64_t cb = car_bytes_per_node(dtype) * node_capacity + slack;
     const int64_t fb = kFsBytesPerNode * node_capacity + slack;
     for (int i = 0; i < 2; ++i) {
-        ECK(cudaMalloc(&pop_[i], pb));
-        dev_bytes_ += pb;
-        if (dtype == S_F16S) {
-            ECK(cudaMalloc(&car_[i], cb));
-            dev_bytes_ += cb;
-        }
+        ECK(device_alloc(&pop_[i], pb));
+        if (dtype == S_F16S) ECK(device_alloc(&car_[i], cb));
     }
-    ECK(cudaMalloc(&fs_, fb));
-    dev_bytes_ += fb;
+    ECK(device_alloc(&fs_, fb));
     apop_.reset(pb - over);
     acar_.reset(dtype == S_F16S ? cb - over : 0);
     afs_.reset(fb - over);
     probs_.assign(max_probs, HostProb());
-    ECK(cudaMalloc(&d_probs_, sizeof(BatchProb) * max_probs));
-    ECK(cudaMalloc(&d_acc_, sizeof(double) * kRes * max_probs));
+    ECK(device_alloc(&d_probs_, sizeof(BatchProb) * max_probs));
+    ECK(device_alloc(&d_acc_, sizeof(double) * kRes * max_probs));
     ECK(cudaMallocHost(&h_acc_, sizeof(double) * kRes * max_probs));
-    ECK(cudaMalloc(&d_stat_, 2 * sizeof(unsigned long long) * max_probs));
+    ECK(device_alloc(&d_stat_, 2 * sizeof(unsigned long long) * max_probs));
     ECK(cudaMemsetAsync(d_stat_, 0, 2 * sizeof(unsigned long long) * max_probs, st_));
-    ECK(cudaMalloc(&d_ntiles_, sizeof(int)));
+    ECK(device_alloc(&d_ntiles_, sizeof(int)));
     ECK(cudaMemsetAsync(d_ntiles_, 0, sizeof(int), st_));
     for (int i = 0; i < kClasses - 1; ++i) {
         ECK(cudaStreamCreateWithFlags(&side_[i], cudaStreamNonBlocking));
@@ -157,7 +151,6 @@ int ArenaEngine::init(int dtype, int64_t node_capacity, int max_probs, int check
     ECK(cudaEventCreateWithFlags(&fork_, cudaEventDisableTiming));
     ECK(cudaEventCreate(&ev0_));
     ECK(cudaEventCreate(&ev1_));
-    dev_bytes_ += sizeof(BatchProb) * max_probs + sizeof(double) * kRes * max_probs;
     return LBM_OK;
 }
 
@@ -247,26 +240,21 @@ int ArenaEngine::admit(int nx, int ny, double lambda, double mu, const double* g
     if (!place(p)) return -1;
     // the force: copied as given, converted, transposed and checked on the device
     const int64_t len = 2 * p.plane;
-    if (d_force_cap_ < 2 * n) {
-        if (d_force_) {
-            ECK(cudaStreamSynchronize(st_));
-            cudaFree(d_force_);
-            d_force_ = nullptr;
-            d_force_cap_ = 0;
-        }
-        const int64_t cap = std::max<int64_t>(2 * n, int64_t(1) << 20);
-        ECK(cudaMalloc(&d_force_, sizeof(double) * cap));
-        d_force_cap_ = cap;
+    // (staged where the fields are)
+    const int rc = ensure_fields_buffer(std::max<int64_t>(2 * n, int64_t(1) << 20), err);
+    if (rc) {
+        unplace(p);
+        return rc;
     }
     unsigned long long* stat = d_stat_ + 2 * slot;
     float* force = reinterpret_cast<float*>(fs_ + p.fs_off);
-    ECK(copy_in(d_force_, gx, sizeof(double) * n, st_));
-    ECK(copy_in(d_force_ + n, gy, sizeof(double) * n, st_));
+    ECK(copy_in(d_fields_, gx, sizeof(double) * n, st_));
+    ECK(copy_in(d_fields_ + n, gy, sizeof(double) * n, st_));
     ECK(cudaMemsetAsync(stat, 0, 2 * sizeof(unsigned long long), st_));
     ECK(cudaMemsetAsync(force, 0, p.fs_bytes, st_));
     ForceIn f{};
-    f.gx = d_force_;
-    f.gy = d_force_ + n;
+    f.gx = d_fields_;
+    f.gy = d_fields_ + n;
     f.hx = nx;
     f.tr = tr ? 1 : 0;
     f.out = force;
@@ -409,17 +397,22 @@ int ArenaEngine::upload_tiles(int V, std::string* err) {
         if (h_tiles_) {
             ECK(cudaStreamSynchronize(st_));
             cudaFreeHost(h_tiles_);
+            h_tiles_ = nullptr;
+            h_tiles_cap_ = 0;
         }
-        h_tiles_cap_ = nt + nt / 4 + 1024;
-        ECK(cudaMallocHost(&h_tiles_, sizeof(uint2) * h_tiles_cap_));
+        const int64_t cap = nt + nt / 4 + 1024;
+        ECK(cudaMallocHost(&h_tiles_, sizeof(uint2) * cap));
+        h_tiles_cap_ = cap;
     }
     if (tiles_cap_ < nt) {
         if (d_tiles_) {
             ECK(cudaStreamSynchronize(st_));
-            cudaFree(d_tiles_);
+            device_free(&d_tiles_, sizeof(uint2) * tiles_cap_);
+            tiles_cap_ = 0;
         }
-        tiles_cap_ = nt + nt / 4 + 1024;
-        ECK(cudaMalloc(&d_tiles_, sizeof(uint2) * tiles_cap_));
+        const int64_t cap = nt + nt / 4 + 1024;
+        ECK(device_alloc(&d_tiles_, sizeof(uint2) * cap));
+        tiles_cap_ = cap;
         for (auto& g : graph_)  // the graphs hold the old tile pointer
             if (g) {
                 cudaGraphExecDestroy(g);
@@ -721,21 +714,18 @@ int ArenaEngine::ensure_fields_buffer(int64_t len, std::string* err) {
     if (d_fields_cap_ >= len) return LBM_OK;
     if (d_fields_) {
         ECK(cudaStreamSynchronize(st_));
-        cudaFree(d_fields_);
-        d_fields_ = nullptr;
+        device_free(&d_fields_, sizeof(double) * d_fields_cap_);
         d_fields_cap_ = 0;
     }
-    ECK(cudaMalloc(&d_fields_, sizeof(double) * len));
+    ECK(device_alloc(&d_fields_, sizeof(double) * len));
     d_fields_cap_ = len;
     return LBM_OK;
 }
 
 int ArenaEngine::recover_many(int count, const int* slots, double* const* outs, std::string* err) {
-    // Problems are packed into blocks of kRecoverBlock doubles (a larger problem
-    // is a block of its own): one field launch per problem into a device block,
-    // then copies straight into the callers' arrays, one per problem where its
-    // five arrays lie one after the other.
-    constexpr int64_t kRecoverBlock = int64_t(4) << 20;   // 32 MB of FP64
+    // Problems are packed into blocks of kRecoverBlock doubles: one field launch per
+    // problem into a device block, then copies straight into the callers' arrays,
+    // one per problem where its five arrays lie one after the other.
     int64_t need = 0, all = 0;
     for (int i = 0; i < count; ++i) {
         const HostProb& p = probs_[slots[i]];

@@ -6,6 +6,8 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <atomic>
 #include <string>
 #include <vector>
 
@@ -86,6 +88,11 @@ public:
     // sxy) per problem.
     int recover_many(int count, const int* slots, double* const* outs, std::string* err);
     void release(int slot);
+    // Staging (doubles) that admissions of `most` nodes and a recovery of `fields` field
+    // values in all (0: none), at most 5 * most of one problem, will not have to grow.
+    int reserve_staging(int64_t most, int64_t fields, std::string* err) {
+        return ensure_fields_buffer(std::max(2 * most, fields ? std::max(5 * most, std::min(fields, kRecoverBlock)) : 0), err);
+    }
     const HostProb& prob(int slot) const { return probs_[slot]; }
     int running() const { return nrunning_; }
     int64_t running_tiles(int V) const;
@@ -100,6 +107,22 @@ public:
     cudaStream_t stream() const { return st_; }
 
 private:
+    template <typename T>
+    cudaError_t device_alloc(T** p, int64_t bytes) {
+        const cudaError_t e = cudaMalloc(p, bytes);
+        if (e == cudaSuccess) dev_bytes_ += bytes;
+        else *p = nullptr;
+        return e;
+    }
+    template <typename T>
+    void device_free(T** p, int64_t bytes) {
+        cudaFree(*p);
+        dev_bytes_ -= bytes;
+        *p = nullptr;
+    }
+    // Problems are recovered in blocks of so many doubles (32 MB; a larger problem is a
+    // block of its own).
+    static constexpr int64_t kRecoverBlock = int64_t(4) << 20;
     int upload_tiles(int V, std::string* err);
     int choose_seg() const;
     int launch_strip_chunk(std::string* err);
@@ -137,16 +160,14 @@ private:
     int wave_seg_ = 0;                // rows per strip item of the current list
     bool tiles_dirty_ = true;
     bool desc_dirty_ = true;
-    double* d_force_ = nullptr;       // FP64 staging of the caller's force
-    int64_t d_force_cap_ = 0;
     unsigned long long* d_stat_ = nullptr;   // per problem: max |g|, non-finite flag (ForceIn)
-    double* d_fields_ = nullptr;      // FP64 staging for recovery
+    double* d_fields_ = nullptr;      // FP64 staging: the caller's force, recovered fields
     int64_t d_fields_cap_ = 0;
     cudaGraphExec_t graph_[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
     bool graph_failed_[6] = {false, false, false, false, false, false};
     cudaEvent_t ev0_ = nullptr, ev1_ = nullptr;
     int nrunning_ = 0;
-    int64_t dev_bytes_ = 0;
+    std::atomic<int64_t> dev_bytes_{0};   // (a server's statistics read it while the worker runs)
 };
 
 // Message for lbm_last_error() on this host thread; returns code.

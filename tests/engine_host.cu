@@ -1,6 +1,7 @@
 // The host code of the arena and the server (lbm_engine.cu, lbm_server.cu) on a
 // stand-in for the CUDA runtime, without a GPU: device memory is host memory,
-// kernels do nothing but advance the clock of their stream by a millisecond, and
+// kernels advance the clock of their stream by a millisecond (the recovery fills
+// field k with k + 1, the others do nothing else), and
 // copies and fills run, in order, when the stream is waited for -- as late as the
 // runtime allows.  Freeing the source of a copy that has not run is recorded.
 // usage: engine_host SCENARIO; prints "ok" or what is wrong.
@@ -234,7 +235,14 @@ cudaError_t launch_arena_pairs(int, bool, const BatchArgs&, const uint2*, int, i
 cudaError_t launch_arena_ghosts(int, const BatchArgs&, const uint2*, int, cudaStream_t st) { return fake::launch(st); }
 cudaError_t launch_arena_force(const ForceIn&, cudaStream_t st) { return fake::launch(st); }
 template <int S>
-cudaError_t Ops<S>::fields(const StepParams&, const Coef<double>&, T, const FieldOut&, cudaStream_t st) {
+cudaError_t Ops<S>::fields(const StepParams& a, const Coef<double>&, T, const FieldOut& o, cudaStream_t st) {
+    const int64_t n = (int64_t)a.nx * a.ny;
+    {
+        std::lock_guard<std::mutex> l(fake::mu);
+        fake::work.push_back([=] {
+            for (int k = 0; k < 5; ++k) std::fill(o.p[k], o.p[k] + n, 1.0 + k);
+        });
+    }
     return fake::launch(st);
 }
 __global__ void k_scale_float(float*, int64_t, float) {}
@@ -306,6 +314,29 @@ void server_device_ms() {
     lbm_server_destroy(s);
 }
 
+// The arena says what it holds on the device, and its forces and fields are staged in
+// one buffer.
+void staging(int dtype) {
+    const int nx = 600, ny = 500, n = nx * ny;
+    std::vector<double> g(n, 1.0), out(5 * n);
+    std::string err;
+    const size_t none = fake::device_bytes;
+    ArenaEngine e;
+    EXPECT(e.init(dtype, 620 * 500, 4, 100, (cudaStream_t)&e, &err) == LBM_OK);
+    const size_t empty = fake::device_bytes;
+    EXPECT(e.device_bytes() == (int64_t)(empty - none));
+    const int s = e.admit(nx, ny, 0.3, 0.4, g.data(), g.data(), 0.0, 100, &err);
+    EXPECT(s >= 0 && e.device_bytes() == (int64_t)(fake::device_bytes - none));
+    EXPECT(e.run_chunk(kTileWave, nullptr, &err) == LBM_OK && e.prob(s).state == P_DONE);
+    const size_t ran = e.device_bytes();
+    EXPECT(ran == fake::device_bytes - none);
+    double* outs[5];
+    for (int k = 0; k < 5; ++k) outs[k] = &out[k * n];
+    EXPECT(e.recover_many(1, &s, outs, &err) == LBM_OK);
+    EXPECT(e.device_bytes() == (int64_t)(fake::device_bytes - none));
+    EXPECT(fake::device_peak <= empty + 5 * n * sizeof(double) + (size_t(1) << 20));   // (a megabyte for tables)
+}
+
 // A full arena: what a strip reads beyond the rows of the last problem (at most 72
 // columns from eight before its first one) lies within the arena's buffers.
 void full_arena(int dtype) {
@@ -360,13 +391,13 @@ void pinned_parts(int dtype) {
     double* outs[5];
     for (int k = 0; k < 5; ++k) outs[k] = &mem[(2 + k) * n];
     EXPECT(e.recover_many(1, &s, outs, &err) == LBM_OK);
-    for (int i = 2 * n; i < 7 * n; ++i) EXPECT(mem[i] == 0.0);
+    for (int i = 2 * n; i < 7 * n; ++i) EXPECT(mem[i] == i / n - 1);
     // pinned in part only
     fake::pinned.erase((char*)&mem[4 * n]);
     fake::pinned[(char*)&mem[4 * n]] = 100;
     std::fill(mem.begin() + 2 * n, mem.end(), -7.0);
     EXPECT(e.recover_many(1, &s, outs, &err) == LBM_OK);
-    for (int i = 2 * n; i < 7 * n; ++i) EXPECT(mem[i] == 0.0);
+    for (int i = 2 * n; i < 7 * n; ++i) EXPECT(mem[i] == i / n - 1);
     for (int k = 2; k < 7; ++k) fake::pinned.erase((char*)&mem[k * n]);
     fake::pinned.erase((char*)mem.data());
 }
@@ -378,6 +409,8 @@ int main(int argc, char** argv) {
     if (what == "server_force") server_force(false);
     else if (what == "server_force_failing") server_force(true);
     else if (what == "server_device_ms") server_device_ms();
+    else if (what == "staging_f32") staging(S_F32);
+    else if (what == "staging_f16s") staging(S_F16S);
     else if (what == "full_arena_f32") full_arena(S_F32);
     else if (what == "full_arena_f16s") full_arena(S_F16S);
     else if (what == "pinned_parts_f32") pinned_parts(S_F32);
