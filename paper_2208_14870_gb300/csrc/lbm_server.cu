@@ -238,6 +238,7 @@ void lbm_server::retire(int a, const std::vector<int>& slots, std::unique_lock<s
         Request& r = *reqs[t];
         const HostProb& p = arena[a]->prob(slot);
         r.status = rc != LBM_OK ? rc : p.status;
+        if (rc != LBM_OK) r.fields.reset();     // (not written)
         r.iters = p.steps;
         r.residual = p.residual;
         r.transposed = p.tr ? 1 : 0;

@@ -314,6 +314,22 @@ void server_device_ms() {
     lbm_server_destroy(s);
 }
 
+// A request whose fields could not be recovered says so, and leaves the caller's
+// arrays alone.
+void server_recovery_fails() {
+    lbm_server* s = nullptr;
+    EXPECT(lbm_server_create(size_t(64) << 20, 100, &s) == LBM_OK);
+    Problem p(300, 40);
+    const lbm_problem in = p.in();
+    fake::fail_launch = fake::launches + 1 + 20;       // the force, twenty launches of five steps
+    uint64_t t;
+    EXPECT(lbm_server_submit(s, &in, LBM_F32, 0.0, 100, &t) == LBM_OK);
+    EXPECT(lbm_server_wait(s, t, 60.0, &p.r) == LBM_OK && p.r.status == LBM_ERR_CUDA && p.r.iters == 100);
+    for (auto& o : p.out)
+        for (double v : o) EXPECT(v == -7.0);
+    lbm_server_destroy(s);
+}
+
 // The arena says what it holds on the device, and its forces and fields are staged in
 // one buffer.
 void staging(int dtype) {
@@ -409,6 +425,7 @@ int main(int argc, char** argv) {
     if (what == "server_force") server_force(false);
     else if (what == "server_force_failing") server_force(true);
     else if (what == "server_device_ms") server_device_ms();
+    else if (what == "server_recovery_fails") server_recovery_fails();
     else if (what == "staging_f32") staging(S_F32);
     else if (what == "staging_f16s") staging(S_F16S);
     else if (what == "full_arena_f32") full_arena(S_F32);
