@@ -166,24 +166,6 @@ k_arena_strips(const BatchArgs A, const uint2* items, int count, int group) {
     }
 }
 
-// Two steps of the listed two-step tiles, one block each.
-template <int S, bool CHECK>
-__global__ void __launch_bounds__(kT2Threads, 2)
-k_arena_pairs(const BatchArgs A, const uint2* items, int group) {
-    extern __shared__ float t2_smem[];
-    __shared__ double red[kRes][32];
-    after_predecessor();
-    const uint2 tl = items[blockIdx.x];
-    const BatchProb P = A.probs[tl.x];
-    ResAcc<S> acc;
-    if (CHECK && P.check) {
-        arena_tile2<S, true>(A, P, (int)tl.y, group, t2_smem, acc);
-        tile_to_problem<S>(acc, A.acc + (int64_t)tl.x * kRes, red);
-    } else {
-        arena_tile2<S, false>(A, P, (int)tl.y, group, t2_smem, acc);
-    }
-}
-
 // Ghost columns of the listed problems' current states, one block each.
 template <int S>
 __global__ void __launch_bounds__(256) k_arena_ghosts(const BatchArgs A, const uint2* items) {
@@ -277,22 +259,6 @@ cudaError_t launch_arena_strips(int dtype, int T, bool check, const BatchArgs& a
         case 5: return launch_strips_k<S_F32, 5, false>(a, items, count, group, st);
         default: return cudaErrorInvalidValue;
     }
-}
-
-template <int S, bool CHECK>
-static cudaError_t launch_pairs_k(const BatchArgs& a, const uint2* items, int count, int group, cudaStream_t st) {
-    const cudaError_t e = allow_smem_once<k_arena_pairs<S, CHECK>>(kT2Smem);
-    if (e != cudaSuccess) return e;
-    return launch_after(k_arena_pairs<S, CHECK>, dim3((unsigned)count), dim3(kT2Threads), kT2Smem, st, a, items, group);
-}
-
-cudaError_t launch_arena_pairs(int dtype, bool check, const BatchArgs& a, const uint2* items, int count, int group,
-                               cudaStream_t st) {
-    if (dtype == S_F16S)
-        return check ? launch_pairs_k<S_F16S, true>(a, items, count, group, st)
-                     : launch_pairs_k<S_F16S, false>(a, items, count, group, st);
-    return check ? launch_pairs_k<S_F32, true>(a, items, count, group, st)
-                 : launch_pairs_k<S_F32, false>(a, items, count, group, st);
 }
 
 cudaError_t launch_arena_ghosts(int dtype, const BatchArgs& a, const uint2* items, int count, cudaStream_t st) {

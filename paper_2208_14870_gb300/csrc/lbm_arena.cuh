@@ -13,7 +13,7 @@
 //
 // The strip chunk (kTileWave) launches one kernel per group of steps over the
 // (problem, strip, segment) items of all running problems, one warp per item;
-// the other tile codes run a chunk in one persistent cooperative kernel that
+// the other tile codes, and the problems too narrow for strips, run a chunk in one persistent cooperative kernel that
 // walks the (problem, tile) list grid-stride and synchronises the grid between
 // steps.  The last step of a chunk carries the residual check for the problems
 // flagged in their descriptor (a problem checks every `check_period` chunks of
@@ -118,7 +118,10 @@ constexpr int kTileTwoStep = 3;
 // their state after the second one too: in launches of their own, two steps each,
 // 12 small problems of a server took 1.08 ms per 100 steps instead of 0.94).  Strips have
 // kArenaOX output columns whatever the group, so that one item list serves a
-// chunk; problems without ghost columns take pairs of steps on two-step tiles.
+// chunk; problems without ghost columns take pairs of steps on two-step tiles, all of a
+// chunk's in one cooperative launch beside the strips (a launch per pair: 100
+// problems of sides 8 to 64 1.13 against 0.89 ms per 400 steps, FP16S 1.51 against 1.21; 50 of
+// sides 4 to 15 alone 0.73 against 0.78).
 // Chunk lengths: multiples of 4.
 constexpr int kTileWave = 5;
 constexpr int kArenaOX = 56;
@@ -161,13 +164,11 @@ cudaError_t launch_arena_chunk(int dtype, int V, const BatchArgs& a, int grid, c
 int arena_occupancy(int dtype, int V);
 
 // The strip chunk's launches.  T steps of `count` strip items (check: the last
-// step checks the flagged problems); two steps of `count` two-step tiles; the
-// ghost columns of `count` problems (items: problem numbers).  group: how many
-// groups of steps of its problems ran before in this chunk (buffer parity).
+// step checks the flagged problems); the ghost columns of `count` problems (items:
+// problem numbers).  group: how many groups of steps of its problems ran before in
+// this chunk (buffer parity).
 cudaError_t launch_arena_strips(int dtype, int T, bool check, const BatchArgs& a, const uint2* items, int count,
                                 int group, cudaStream_t st);
-cudaError_t launch_arena_pairs(int dtype, bool check, const BatchArgs& a, const uint2* items, int count, int group,
-                               cudaStream_t st);
 // A problem's force from the caller's FP64 arrays (device memory, hx columns per
 // row) into its FP32 planes of `plane` elements: rows of nx columns with their
 // ghost columns, transposed with the components exchanged for a problem solved

@@ -142,8 +142,8 @@ int ArenaEngine::init(int dtype, int64_t node_capacity, int max_probs, int check
     ECK(cudaMallocHost(&h_acc_, sizeof(double) * kRes * max_probs));
     ECK(device_alloc(&d_stat_, 2 * sizeof(unsigned long long) * max_probs));
     ECK(cudaMemsetAsync(d_stat_, 0, 2 * sizeof(unsigned long long) * max_probs, st_));
-    ECK(device_alloc(&d_ntiles_, sizeof(int)));
-    ECK(cudaMemsetAsync(d_ntiles_, 0, sizeof(int), st_));
+    ECK(device_alloc(&d_ntiles_, 2 * sizeof(int)));
+    ECK(cudaMemsetAsync(d_ntiles_, 0, 2 * sizeof(int), st_));
     for (int i = 0; i < kClasses - 1; ++i) {
         ECK(cudaStreamCreateWithFlags(&side_[i], cudaStreamNonBlocking));
         ECK(cudaEventCreateWithFlags(&join_[i], cudaEventDisableTiming));
@@ -446,10 +446,11 @@ int ArenaEngine::upload_tiles(int V, std::string* err) {
             for (int64_t i = 0; i < m; ++i) h_tiles_[t++] = make_uint2((unsigned)s, (unsigned)i);
         }
     }
-    static thread_local int nt_host;
-    nt_host = (int)t;
+    static thread_local int nt_host[2];
+    nt_host[0] = (int)t;
+    nt_host[1] = V == kTileWave ? class_begin_[C_PAIRS + 1] - class_begin_[C_PAIRS] : 0;
     if (t > 0) ECK(cudaMemcpyAsync(d_tiles_, h_tiles_, sizeof(uint2) * t, cudaMemcpyHostToDevice, st_));
-    ECK(cudaMemcpyAsync(d_ntiles_, &nt_host, sizeof(int), cudaMemcpyHostToDevice, st_));
+    ECK(cudaMemcpyAsync(d_ntiles_, nt_host, sizeof(nt_host), cudaMemcpyHostToDevice, st_));
     ECK(cudaStreamSynchronize(st_));
     tiles_V_ = V;
     tiles_dirty_ = false;
@@ -497,10 +498,9 @@ int ArenaEngine::ensure_graph(int V, std::string* err) {
     return LBM_OK;
 }
 
-// Steps of the launches that advance a class of problems by a chunk of k steps
-// (k a multiple of 4); the last one carries the check.
-static std::vector<int> chunk_groups(int dtype, int cls, int k) {
-    if (cls == C_PAIRS) return std::vector<int>(k / 2, 2);
+// Steps of the launches that advance strip items by a chunk of k steps (k a multiple
+// of 4); the last one carries the check.
+static std::vector<int> chunk_groups(int dtype, int k) {
     if (dtype == S_F16S || k < 5) return std::vector<int>(k / 4, 4);
     // fives after the rest (two threes where it would be one step)
     std::vector<int> g;
@@ -512,7 +512,8 @@ static std::vector<int> chunk_groups(int dtype, int cls, int k) {
     return g;
 }
 
-// One chunk on strips: the classes side by side, each a sequence of launches.
+// One chunk: strips in a sequence of launches, and beside them the problems too narrow
+// for strips in one.
 int ArenaEngine::launch_strip_chunk(std::string* err) {
     const BatchArgs a = chunk_args();
     ECK(cudaMemsetAsync(d_acc_, 0, sizeof(double) * kRes * probs_.size(), st_));
@@ -527,12 +528,18 @@ int ArenaEngine::launch_strip_chunk(std::string* err) {
         const cudaStream_t st = b == 0 ? st_ : side_[b - 1];
         if (b > 0) ECK(cudaStreamWaitEvent(st, fork_, 0));
         const uint2* items = d_tiles_ + class_begin_[c];
-        strip_blocks_ = std::max(strip_blocks_, c == C_PAIRS ? count : (count + 3) / 4);
-        const std::vector<int> groups = chunk_groups(dtype_, c, k_);
-        for (int g = 0; g < (int)groups.size(); ++g) {
-            const bool check = g + 1 == (int)groups.size();
-            if (c == C_PAIRS) ECK(launch_arena_pairs(dtype_, check, a, items, count, g, st));
-            else ECK(launch_arena_strips(dtype_, groups[g], check, a, items, count, g, st));
+        if (c == C_PAIRS && pairs_grid_ == 0) pairs_grid_ = std::max(1, arena_occupancy(dtype_, kTileTwoStep) * sms_);
+        const int blocks = c == C_PAIRS ? std::min(count, pairs_grid_) : (count + 3) / 4;
+        strip_blocks_ = std::max(strip_blocks_, blocks);
+        if (c == C_PAIRS) {
+            BatchArgs p = a;
+            p.tiles = items;
+            p.ntiles = d_ntiles_ + 1;
+            ECK(launch_arena_chunk(dtype_, kTileTwoStep, p, blocks, st));
+        } else {
+            const std::vector<int> groups = chunk_groups(dtype_, k_);
+            for (int g = 0; g < (int)groups.size(); ++g)
+                ECK(launch_arena_strips(dtype_, groups[g], g + 1 == (int)groups.size(), a, items, count, g, st));
         }
         if (b > 0) ECK(cudaEventRecord(join_[b - 1], st));
     }
@@ -619,10 +626,10 @@ int ArenaEngine::finish_chunk(int V, float* device_ms, std::string* err) {
         if (p.state != P_RUNNING) continue;
         p.steps += k_;
         p.lups += p.n * k_;
-        // the buffers swap once per group of steps: k steps, k/2 pairs, or (strip
-        // chunk) the groups of the problem's class
-        const int64_t swaps = V == kTileWave ? (int64_t)chunk_groups(dtype_, p.cls, k_).size()
-                                             : (V == kTileTwoStep ? k_ / 2 : k_);
+        // the buffers swap once per group of steps: k steps, k/2 pairs, or a strip
+        // chunk's groups
+        const int64_t swaps = V == kTileWave && p.cls == C_STRIPS ? (int64_t)chunk_groups(dtype_, k_).size()
+                                                                  : (V == kTileWave || V == kTileTwoStep ? k_ / 2 : k_);
         if (V != kTileWave) p.ghosts_ok = false;
         else if (!p.ghosts_ok) {
             p.ghosts_ok = true;

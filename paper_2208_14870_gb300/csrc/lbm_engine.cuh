@@ -150,6 +150,7 @@ private:
     int64_t tiles_cap_ = 0;
     int* d_ntiles_ = nullptr;
     int class_begin_[kClasses + 1] = {};   // strip chunk: item ranges of the classes
+    int pairs_grid_ = 0;                              // most blocks of the pairs' launch
     int strip_blocks_ = 0;                            // largest launch so far
     int ghosts_begin_ = 0, ghosts_end_ = 0;           // ... and of the problems whose ghost columns are stale
     cudaStream_t side_[kClasses - 1] = {};   // the classes run side by side

@@ -229,9 +229,6 @@ int arena_occupancy(int, int) { return 1; }
 cudaError_t launch_arena_strips(int, int, bool, const BatchArgs&, const uint2*, int, int, cudaStream_t st) {
     return fake::launch(st);
 }
-cudaError_t launch_arena_pairs(int, bool, const BatchArgs&, const uint2*, int, int, cudaStream_t st) {
-    return fake::launch(st);
-}
 cudaError_t launch_arena_ghosts(int, const BatchArgs&, const uint2*, int, cudaStream_t st) { return fake::launch(st); }
 cudaError_t launch_arena_force(const ForceIn&, cudaStream_t st) { return fake::launch(st); }
 template <int S>
@@ -330,6 +327,22 @@ void server_recovery_fails() {
     lbm_server_destroy(s);
 }
 
+// Problems too narrow for strips take one launch per chunk, however many steps.
+void narrow_launches(int dtype) {
+    ArenaEngine e;
+    std::string err;
+    EXPECT(e.init(dtype, 20000, 4, 100, (cudaStream_t)&e, &err) == LBM_OK);
+    std::vector<double> g(100, 1.0);
+    const int s = e.admit(10, 10, 0.3, 0.4, g.data(), g.data(), 0.0, 300, &err);
+    EXPECT(s >= 0 && !e.prob(s).ghost);
+    for (int chunk = 0; chunk < 3; ++chunk) {
+        const int before = fake::launches, parity = e.prob(s).parity;
+        EXPECT(e.run_chunk(kTileWave, nullptr, &err) == LBM_OK);
+        EXPECT(fake::launches == before + 1 && e.prob(s).parity == parity);      // (fifty pairs of steps)
+    }
+    EXPECT(e.prob(s).state == P_DONE && e.prob(s).steps == 300);
+}
+
 // The arena says what it holds on the device, and its forces and fields are staged in
 // one buffer.
 void staging(int dtype) {
@@ -426,6 +439,8 @@ int main(int argc, char** argv) {
     else if (what == "server_force_failing") server_force(true);
     else if (what == "server_device_ms") server_device_ms();
     else if (what == "server_recovery_fails") server_recovery_fails();
+    else if (what == "narrow_launches_f32") narrow_launches(S_F32);
+    else if (what == "narrow_launches_f16s") narrow_launches(S_F16S);
     else if (what == "staging_f32") staging(S_F32);
     else if (what == "staging_f16s") staging(S_F16S);
     else if (what == "full_arena_f32") full_arena(S_F32);
