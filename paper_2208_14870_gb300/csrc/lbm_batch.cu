@@ -126,7 +126,7 @@ extern "C" int lbm_batch_solve(int count, const lbm_problem* probs, int dtype, d
         for (int i = 0; i < count && rc == LBM_OK; ++i) {
             const lbm_problem& p = probs[i];
             int s = eng.admit(p.nx, p.ny, p.lambda, p.mu, p.gx, p.gy, tol, max_iters, &err);
-            if (s == -1) rc = LBM_ERR_OOM, err = "arena full";
+            if (s == ArenaEngine::kNoRoom) rc = LBM_ERR_OOM, err = "arena full";
             else if (s < 0) rc = s;
             slot[i] = s;
         }

@@ -90,6 +90,7 @@ ArenaEngine::~ArenaEngine() {
     if (d_stat_) cudaFree(d_stat_);
     if (h_acc_) cudaFreeHost(h_acc_);
     if (h_tiles_) cudaFreeHost(h_tiles_);
+    if (h_force_) cudaFreeHost(h_force_);
     for (int i = 0; i < kClasses - 1; ++i) {
         if (side_[i]) cudaStreamDestroy(side_[i]);
         if (join_[i]) cudaEventDestroy(join_[i]);
@@ -190,9 +191,107 @@ void ArenaEngine::unplace(const HostProb& p) {
     afs_.release(p.fs_off, p.fs_bytes);
 }
 
-// Problems of at most so many nodes take max |g| on the host: 16 bytes per node to
-// read, against some 15 us for the device's answer.
+// The force of a problem of at most so many nodes is converted on the host, into
+// pinned memory: three calls of the runtime per admission (FP16S four) instead of
+// six.  200 problems of sides 4 to 31 on a server, 400 steps: 10.9 -> 10.0 ms; 100 of
+// sides 16 to 64 7.50 -> 7.11 (up to 1024 nodes 7.35, up to 16384 7.02).
+constexpr int64_t kSmallForce = 4096;
+constexpr int64_t kForceStage = int64_t(1) << 18;      // floats (a problem of 4096 nodes takes at most 2 * 2 * 4096)
+// Up to so many nodes the host looks for max |g| (FP16S): 16 bytes per node to read,
+// against some 15 us for the device's answer.
 constexpr int64_t kHostMax = 16384;
+
+// Max |g| of both components, infinite or NaN if an entry is not finite (of the bit
+// patterns of |g|, which order like the values).
+static double force_max(const double* gx, const double* gy, int64_t n) {
+    uint64_t m = 0;
+    for (const double* g : {gx, gy})
+        for (int64_t i = 0; i < n; ++i) {
+            uint64_t b;
+            std::memcpy(&b, g + i, sizeof b);
+            m = std::max<uint64_t>(m, b & 0x7fffffffffffffffULL);
+        }
+    double gmax;
+    std::memcpy(&gmax, &m, sizeof gmax);
+    return gmax;
+}
+
+// The force planes of a placed problem, whose snapshot is cleared; converted on the
+// host (finite, hexp set).  hx: columns of the caller's arrays.
+int ArenaEngine::admit_small(HostProb& p, int hx, const double* gx, const double* gy, std::string* err) {
+    const int64_t len = 2 * p.plane;
+    if (!h_force_) ECK(cudaMallocHost(&h_force_, sizeof(float) * kForceStage));
+    if (h_force_used_ + len > kForceStage) {
+        ECK(cudaStreamSynchronize(st_));
+        h_force_used_ = 0;
+    }
+    float* h = h_force_ + h_force_used_;
+    h_force_used_ += len;
+    std::memset(h, 0, sizeof(float) * len);
+    const float scale = std::ldexp(1.0f, p.hexp);
+    for (int c = 0; c < 2; ++c) {
+        const double* g = (c == 0) == p.tr ? gy : gx;      // (transposed: components exchanged)
+        for (int y = 0; y < p.ny; ++y) {
+            float* row = h + c * p.plane + (int64_t)y * p.pitch + p.ghost;
+            if (p.tr)
+                for (int x = 0; x < p.nx; ++x) row[x] = (float)g[(int64_t)x * hx + y] * scale;
+            else
+                for (int x = 0; x < p.nx; ++x) row[x] = (float)g[(int64_t)y * hx + x] * scale;
+            for (int x = 0; x < p.ghost; ++x) {
+                row[p.nx + x] = row[x];
+                row[x - p.ghost] = row[p.nx + x - p.ghost];
+            }
+        }
+    }
+    ECK(cudaMemcpyAsync(fs_ + p.fs_off, h, sizeof(float) * len, cudaMemcpyHostToDevice, st_));
+    ECK(cudaMemsetAsync(fs_ + p.fs_off + sizeof(float) * len, 0, p.fs_bytes - sizeof(float) * len, st_));
+    return LBM_OK;
+}
+
+// The same on the device, from a copy of the caller's arrays (in the caller's units
+// and unchecked, but for FP16S up to kHostMax nodes).
+int ArenaEngine::admit_large(HostProb& p, int hx, const double* gx, const double* gy, int slot, std::string* err) {
+    const int64_t n = p.n, len = 2 * p.plane;
+    // (staged where the fields are)
+    const int rc = ensure_fields_buffer(std::max<int64_t>(2 * n, int64_t(1) << 20), err);
+    if (rc) return rc;
+    unsigned long long* stat = d_stat_ + 2 * slot;
+    float* force = reinterpret_cast<float*>(fs_ + p.fs_off);
+    ECK(copy_in(d_fields_, gx, sizeof(double) * n, st_));
+    ECK(copy_in(d_fields_ + n, gy, sizeof(double) * n, st_));
+    ECK(cudaMemsetAsync(stat, 0, 2 * sizeof(unsigned long long), st_));
+    ECK(cudaMemsetAsync(force, 0, p.fs_bytes, st_));
+    ForceIn f{};
+    f.gx = d_fields_;
+    f.gy = d_fields_ + n;
+    f.hx = hx;
+    f.tr = p.tr ? 1 : 0;
+    f.out = force;
+    f.nx = p.nx;
+    f.ny = p.ny;
+    f.pitch = p.pitch;
+    f.ghost = p.ghost;
+    f.plane = p.plane;
+    f.stat = stat;
+    f.scale = std::ldexp(1.0f, p.hexp);
+    ECK(launch_arena_force(f, st_));
+    if (dtype_ != S_F16S || n <= kHostMax) return LBM_OK;
+    unsigned long long got[2];
+    ECK(cudaMemcpyAsync(got, stat, sizeof(got), cudaMemcpyDeviceToHost, st_));
+    ECK(cudaStreamSynchronize(st_));
+    double gmax;
+    std::memcpy(&gmax, &got[0], sizeof(double));
+    if (got[1]) {
+        if (err) *err = "admit: non-finite force";
+        return LBM_ERR_ARG;
+    }
+    p.hexp = f16s_exponent(gmax, p.nx, p.ny);
+    if (p.hexp != 0) {
+        k_scale_float<<<256, 256, 0, st_>>>(force, len, std::ldexp(1.0f, p.hexp));
+        ECK(cudaGetLastError());
+    }
+    return LBM_OK;
+}
 
 int ArenaEngine::admit(int nx, int ny, double lambda, double mu, const double* gx, const double* gy,
                        double tol, int64_t max_iters, std::string* err) {
@@ -207,7 +306,7 @@ int ArenaEngine::admit(int nx, int ny, double lambda, double mu, const double* g
             slot = i;
             break;
         }
-    if (slot < 0) return -1;
+    if (slot < 0) return kNoRoom;
     const int64_t n = (int64_t)nx * ny;
     // a problem that is cheaper on its transpose is solved there: lattice
     // ny x nx, force components exchanged, node (x, y) at x * ny + y
@@ -217,71 +316,22 @@ int ArenaEngine::admit(int nx, int ny, double lambda, double mu, const double* g
     p.ny = tr ? nx : ny;
     p.tr = tr;
     p.n = n;
+    if (!place(p)) return kNoRoom;
     // FP16S keeps its state, the force included, in units scaled by 2^hexp from
-    // max |g| (store_f16s).  Small problems take the maximum here: from the device
-    // it costs a copy and a wait (200 problems of sides 4 to 31: 13.2 against 9.6 ms)
-    const bool small = n <= kHostMax;
-    if (dtype_ == S_F16S && small) {
-        uint64_t m = 0;                           // of the bit patterns of |g|, which order like the values
-        for (const double* g : {gx, gy})
-            for (int64_t i = 0; i < n; ++i) {
-                uint64_t b;
-                std::memcpy(&b, g + i, sizeof b);
-                m = std::max<uint64_t>(m, b & 0x7fffffffffffffffULL);
-            }
-        double gmax;
-        std::memcpy(&gmax, &m, sizeof gmax);
+    // max |g| (store_f16s)
+    if (n <= (dtype_ == S_F16S ? kHostMax : kSmallForce)) {
+        const double gmax = force_max(gx, gy, n);
         if (!std::isfinite(gmax)) {
-            if (err) *err = "admit: non-finite force";
-            return LBM_ERR_ARG;
-        }
-        p.hexp = f16s_exponent(gmax, p.nx, p.ny);
-    }
-    if (!place(p)) return -1;
-    // the force: copied as given, converted, transposed and checked on the device
-    const int64_t len = 2 * p.plane;
-    // (staged where the fields are)
-    const int rc = ensure_fields_buffer(std::max<int64_t>(2 * n, int64_t(1) << 20), err);
-    if (rc) {
-        unplace(p);
-        return rc;
-    }
-    unsigned long long* stat = d_stat_ + 2 * slot;
-    float* force = reinterpret_cast<float*>(fs_ + p.fs_off);
-    ECK(copy_in(d_fields_, gx, sizeof(double) * n, st_));
-    ECK(copy_in(d_fields_ + n, gy, sizeof(double) * n, st_));
-    ECK(cudaMemsetAsync(stat, 0, 2 * sizeof(unsigned long long), st_));
-    ECK(cudaMemsetAsync(force, 0, p.fs_bytes, st_));
-    ForceIn f{};
-    f.gx = d_fields_;
-    f.gy = d_fields_ + n;
-    f.hx = nx;
-    f.tr = tr ? 1 : 0;
-    f.out = force;
-    f.nx = p.nx;
-    f.ny = p.ny;
-    f.pitch = p.pitch;
-    f.ghost = p.ghost;
-    f.plane = p.plane;
-    f.stat = stat;
-    f.scale = std::ldexp(1.0f, p.hexp);
-    ECK(launch_arena_force(f, st_));
-    if (dtype_ == S_F16S && !small) {
-        unsigned long long got[2];
-        ECK(cudaMemcpyAsync(got, stat, sizeof(got), cudaMemcpyDeviceToHost, st_));
-        ECK(cudaStreamSynchronize(st_));
-        double gmax;
-        std::memcpy(&gmax, &got[0], sizeof(double));
-        if (got[1]) {
             unplace(p);
             if (err) *err = "admit: non-finite force";
             return LBM_ERR_ARG;
         }
-        p.hexp = f16s_exponent(gmax, p.nx, p.ny);
-        if (p.hexp != 0) {
-            k_scale_float<<<256, 256, 0, st_>>>(force, len, std::ldexp(1.0f, p.hexp));
-            ECK(cudaGetLastError());
-        }
+        if (dtype_ == S_F16S) p.hexp = f16s_exponent(gmax, p.nx, p.ny);
+    }
+    const int rc = n <= kSmallForce ? admit_small(p, nx, gx, gy, err) : admit_large(p, nx, gx, gy, slot, err);
+    if (rc) {
+        unplace(p);
+        return rc;
     }
     ECK(cudaMemsetAsync(pop_[0] + p.pop_off, 0, p.pop_bytes, st_));
     if (dtype_ == S_F16S) ECK(cudaMemsetAsync(car_[0] + p.car_off, 0, p.car_bytes, st_));
@@ -620,6 +670,7 @@ int ArenaEngine::finish_chunk(int V, float* device_ms, std::string* err) {
     if (device_ms) *device_ms = 0.0f;
     if (nrunning_ == 0) return LBM_OK;
     ECK(cudaStreamSynchronize(st_));
+    h_force_used_ = 0;
     if (device_ms) ECK(cudaEventElapsedTime(device_ms, ev0_, ev1_));
     for (int s = 0; s < (int)probs_.size(); ++s) {
         HostProb& p = probs_[s];

@@ -8,6 +8,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <climits>
 #include <string>
 #include <vector>
 
@@ -65,13 +66,15 @@ public:
     int64_t bytes_for(int64_t n) const;
     // Nodes a problem takes with ghost columns (in the orientation it is solved in).
     static int64_t slots_for(int nx, int ny);
-    // Admit a problem; returns slot >= 0, -1 if it does not fit now, or a
-    // negative lbm status (< -1) on error.  gx, gy: host FP64, nx*ny each.
-    // FP32: the force is checked later, by check_forces.
+    // Admit a problem; returns slot >= 0, kNoRoom if it does not fit now, or a
+    // negative lbm status on error.  gx, gy: host FP64, nx*ny each, read until
+    // the stream has been waited for.  FP32: the force of a large problem is checked
+    // later, by check_forces.
+    static constexpr int kNoRoom = INT_MIN;
     int admit(int nx, int ny, double lambda, double mu, const double* gx, const double* gy,
               double tol, int64_t max_iters, std::string* err);
     // LBM_ERR_ARG if a problem admitted since init has a non-finite force entry
-    // (FP16S problems are refused by admit already).
+    // (small and FP16S problems are refused by admit already).
     int check_forces(std::string* err);
     // One chunk of check_every steps for every running problem, launched on the
     // engine's streams, and the wait for it; afterwards finished problems are in
@@ -128,6 +131,8 @@ private:
     int launch_strip_chunk(std::string* err);
     bool place(HostProb& p);
     void unplace(const HostProb& p);
+    int admit_small(HostProb& p, int hx, const double* gx, const double* gy, std::string* err);
+    int admit_large(HostProb& p, int hx, const double* gx, const double* gy, int slot, std::string* err);
     BatchArgs chunk_args() const;
     cudaError_t launch_fields(int slot, double* dst);
     int ensure_fields_buffer(int64_t len, std::string* err);
@@ -161,6 +166,8 @@ private:
     int wave_seg_ = 0;                // rows per strip item of the current list
     bool tiles_dirty_ = true;
     bool desc_dirty_ = true;
+    float* h_force_ = nullptr;        // pinned: converted forces of small problems
+    int64_t h_force_used_ = 0;        // ... since the stream was last waited for (floats)
     unsigned long long* d_stat_ = nullptr;   // per problem: max |g|, non-finite flag (ForceIn)
     double* d_fields_ = nullptr;      // FP64 staging: the caller's force, recovered fields
     int64_t d_fields_cap_ = 0;

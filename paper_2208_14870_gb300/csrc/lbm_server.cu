@@ -201,7 +201,7 @@ int lbm_server::admit_locked() {
             it = queue.erase(it);
             continue;
         }
-        if (s < -1) return s;  // a real error
+        if (s != ArenaEngine::kNoRoom) return s;  // a real error
         ++memory_waits;
         if (r.bypassed > max_bypass_chunks) blocked[a] = true;
         ++it;

@@ -53,6 +53,8 @@ std::map<char*, size_t> device, pinned;       // allocations
 std::map<void*, double> clocks;               // of the streams, ms
 std::map<void*, double> events;
 std::vector<size_t> sizes;                    // of the device allocations, in turn
+std::vector<char*> bases;
+int calls = 0;                                // copies, fills, launches and waits
 size_t device_bytes = 0, device_peak = 0;
 int launches = 0, fail_launch = -1;           // the launch of this number fails
 
@@ -76,6 +78,7 @@ void run_all() {
 
 cudaError_t launch(void* stream) {
     std::lock_guard<std::mutex> l(mu);
+    ++calls;
     if (launches++ == fail_launch) return cudaErrorLaunchFailure;
     clocks[stream] += 1.0;
     return cudaSuccess;
@@ -103,6 +106,7 @@ cudaError_t cudaMalloc(void** p, size_t n) {
     *p = std::calloc(1, n);
     fake::device[(char*)*p] = n;
     fake::sizes.push_back(n);
+    fake::bases.push_back((char*)*p);
     fake::device_bytes += n;
     fake::device_peak = std::max(fake::device_peak, fake::device_bytes);
     return cudaSuccess;
@@ -135,6 +139,7 @@ cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, enum cudaMemcpyKin
     const char* h0 = kind == cudaMemcpyDeviceToHost ? (const char*)d : (const char*)s;
     for (auto& r : fake::pinned)
         if (h0 < r.first + r.second && h0 + n > r.first && !fake::within(fake::pinned, h0, n)) return cudaErrorInvalidValue;
+    ++fake::calls;
     fake::work.push_back([=] { std::memcpy(d, s, n); });
     fake::Hold h;
     if (fake::nsources < fake::kMost) fake::sources[fake::nsources++] = {(const char*)s, n};
@@ -142,6 +147,7 @@ cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, enum cudaMemcpyKin
 }
 cudaError_t cudaMemsetAsync(void* d, int v, size_t n, cudaStream_t) {
     std::lock_guard<std::mutex> l(fake::mu);
+    ++fake::calls;
     fake::work.push_back([=] { std::memset(d, v, n); });
     return cudaSuccess;
 }
@@ -160,6 +166,7 @@ cudaError_t cudaStreamDestroy(cudaStream_t s) {
     return cudaSuccess;
 }
 cudaError_t cudaStreamSynchronize(cudaStream_t) {
+    ++fake::calls;
     fake::run_all();
     return cudaSuccess;
 }
@@ -276,7 +283,7 @@ void server_force(bool fail) {
     EXPECT(lbm_server_create(size_t(64) << 20, 100, &s) == LBM_OK);
     if (fail) fake::fail_launch = 12;
     std::vector<Problem> p;
-    for (int i = 0; i < 6; ++i) p.emplace_back(40 + i, 30);
+    for (int i = 0; i < 6; ++i) p.emplace_back(40 + i, i < 2 ? 30 : 120);      // (small and large)
     std::vector<uint64_t> t;
     for (int i = 0; i < 6; ++i) {
         const lbm_problem in = p[i].in();
@@ -343,6 +350,45 @@ void narrow_launches(int dtype) {
     EXPECT(e.prob(s).state == P_DONE && e.prob(s).steps == 300);
 }
 
+// Small problems: at most four calls of the runtime per admission, whose force planes
+// hold the caller's values (scaled), transposed where the problem is, with their
+// periodic images and zeros around them; an entry that is not finite is refused as a
+// bad argument.
+void small_forces(int dtype) {
+    ArenaEngine e;
+    std::string err;
+    EXPECT(e.init(dtype, 300000, 128, 100, (cudaStream_t)&e, &err) == LBM_OK);
+    const size_t fs = dtype == S_F16S ? 4 : 2;         // (the force buffer: full_arena)
+    for (auto wh : {std::pair<int, int>{1, 1}, {5, 9}, {16, 16}, {17, 40}, {57, 3}, {16, 250}, {250, 16}, {64, 64}}) {
+        const int nx = wh.first, ny = wh.second;
+        std::vector<double> g[2];
+        for (int c = 0; c < 2; ++c)
+            for (int i = 0; i < nx * ny; ++i) g[c].push_back((c ? -0.375 : 0.25) + i * 0.125);
+        fake::run_all();
+        fake::calls = 0;
+        const int s = e.admit(nx, ny, 0.3, 0.4, g[0].data(), g[1].data(), 0.0, 100, &err);
+        EXPECT(s >= 0 && fake::calls <= (dtype == S_F16S ? 4 : 3) + 1);      // (a reset of the staging at most)
+        fake::run_all();
+        const HostProb& p = e.prob(s);
+        const float* f = (const float*)(fake::bases[fs] + p.fs_off);
+        for (int c = 0; c < 2; ++c)
+            for (int y = 0; y < p.ny; ++y)
+                for (int x = -p.ghost; x < p.pitch - p.ghost; ++x) {
+                    const int xw = (x + p.nx) % p.nx;
+                    const double v = p.tr ? g[1 - c][xw * nx + y] : g[c][y * nx + xw];
+                    const bool in = x < p.nx + p.ghost;
+                    EXPECT(f[c * p.plane + y * p.pitch + p.ghost + x] == (in ? std::ldexp(v, p.hexp) : 0.0));
+                }
+        const float* snap = f + 2 * p.plane;
+        for (int64_t i = 0; i < 4 * p.plane; ++i) EXPECT(snap[i] == 0.0f);
+        g[1].back() = -INFINITY;
+        EXPECT(e.admit(nx, ny, 0.3, 0.4, g[0].data(), g[1].data(), 0.0, 100, &err) == LBM_ERR_ARG);
+        g[1].back() = NAN;
+        EXPECT(e.admit(nx, ny, 0.3, 0.4, g[0].data(), g[1].data(), 0.0, 100, &err) == LBM_ERR_ARG);
+        EXPECT(e.running() == s + 1);
+    }
+}
+
 // The arena says what it holds on the device, and its forces and fields are staged in
 // one buffer.
 void staging(int dtype) {
@@ -381,7 +427,7 @@ void full_arena(int dtype) {
             g.assign((size_t)nx * ny, 1.0);
             const int s = e.admit(nx, ny, 0.3, 0.4, g.data(), g.data(), 0.0, 100, &err);
             if (s < 0) {
-                EXPECT(s == -1);
+                EXPECT(s == ArenaEngine::kNoRoom);
                 --ny;
                 continue;
             }
@@ -406,7 +452,7 @@ void full_arena(int dtype) {
 // Forces and results in host memory that is pinned in parts: arrays that follow
 // one another, pinned each by itself, and arrays across the end of a pinned range.
 void pinned_parts(int dtype) {
-    const int nx = 40, ny = 30, n = nx * ny;
+    const int nx = 80, ny = 80, n = nx * ny;
     std::vector<double> mem(7 * n, -7.0);
     for (int k = 2; k < 7; ++k) fake::pinned[(char*)&mem[k * n]] = n * sizeof(double);
     fake::pinned[(char*)mem.data()] = n / 2 * sizeof(double);          // half of g_x
@@ -441,6 +487,8 @@ int main(int argc, char** argv) {
     else if (what == "server_recovery_fails") server_recovery_fails();
     else if (what == "narrow_launches_f32") narrow_launches(S_F32);
     else if (what == "narrow_launches_f16s") narrow_launches(S_F16S);
+    else if (what == "small_forces_f32") small_forces(S_F32);
+    else if (what == "small_forces_f16s") small_forces(S_F16S);
     else if (what == "staging_f32") staging(S_F32);
     else if (what == "staging_f16s") staging(S_F16S);
     else if (what == "full_arena_f32") full_arena(S_F32);
