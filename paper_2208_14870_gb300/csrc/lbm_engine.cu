@@ -91,6 +91,7 @@ ArenaEngine::~ArenaEngine() {
     if (h_acc_) cudaFreeHost(h_acc_);
     if (h_tiles_) cudaFreeHost(h_tiles_);
     if (h_force_) cudaFreeHost(h_force_);
+    if (h_fields_) cudaFreeHost(h_fields_);
     for (int i = 0; i < kClasses - 1; ++i) {
         if (side_[i]) cudaStreamDestroy(side_[i]);
         if (join_[i]) cudaEventDestroy(join_[i]);
@@ -191,12 +192,15 @@ void ArenaEngine::unplace(const HostProb& p) {
     afs_.release(p.fs_off, p.fs_bytes);
 }
 
-// The force of a problem of at most so many nodes is converted on the host, into
+// A small problem, of at most so many nodes: its force is converted on the host, into
 // pinned memory: three calls of the runtime per admission (FP16S four) instead of
 // six.  200 problems of sides 4 to 31 on a server, 400 steps: 10.9 -> 10.0 ms; 100 of
 // sides 16 to 64 7.50 -> 7.11 (up to 1024 nodes 7.35, up to 16384 7.02).
-constexpr int64_t kSmallForce = 4096;
+constexpr int64_t kSmall = 4096;
 constexpr int64_t kForceStage = int64_t(1) << 18;      // floats (a problem of 4096 nodes takes at most 2 * 2 * 4096)
+// Problems of at most so many nodes are recovered many to a copy (recover_many).
+constexpr int64_t kSmallFields = 2048;
+constexpr int64_t kFieldStage = int64_t(1) << 18;      // doubles
 // Up to so many nodes the host looks for max |g| (FP16S): 16 bytes per node to read,
 // against some 15 us for the device's answer.
 constexpr int64_t kHostMax = 16384;
@@ -319,7 +323,7 @@ int ArenaEngine::admit(int nx, int ny, double lambda, double mu, const double* g
     if (!place(p)) return kNoRoom;
     // FP16S keeps its state, the force included, in units scaled by 2^hexp from
     // max |g| (store_f16s)
-    if (n <= (dtype_ == S_F16S ? kHostMax : kSmallForce)) {
+    if (n <= (dtype_ == S_F16S ? kHostMax : kSmall)) {
         const double gmax = force_max(gx, gy, n);
         if (!std::isfinite(gmax)) {
             unplace(p);
@@ -328,7 +332,7 @@ int ArenaEngine::admit(int nx, int ny, double lambda, double mu, const double* g
         }
         if (dtype_ == S_F16S) p.hexp = f16s_exponent(gmax, p.nx, p.ny);
     }
-    const int rc = n <= kSmallForce ? admit_small(p, nx, gx, gy, err) : admit_large(p, nx, gx, gy, slot, err);
+    const int rc = n <= kSmall ? admit_small(p, nx, gx, gy, err) : admit_large(p, nx, gx, gy, slot, err);
     if (rc) {
         unplace(p);
         return rc;
@@ -783,7 +787,11 @@ int ArenaEngine::ensure_fields_buffer(int64_t len, std::string* err) {
 int ArenaEngine::recover_many(int count, const int* slots, double* const* outs, std::string* err) {
     // Problems are packed into blocks of kRecoverBlock doubles: one field launch per
     // problem into a device block, then copies straight into the callers' arrays,
-    // one per problem where its five arrays lie one after the other.
+    // one per problem where its five arrays lie one after the other.  Small problems
+    // come in one copy per block and are handed out by the host: a copy each into pageable
+    // arrays costs a wait of some 8 us (200 problems of sides 4 to 31 on a server, 400
+    // steps: 10.0 -> 7.7 ms; eight of 64 x 64, which are not small, 1.49 ms a batch, as
+    // small ones 1.64).
     int64_t need = 0, all = 0;
     for (int i = 0; i < count; ++i) {
         const HostProb& p = probs_[slots[i]];
@@ -797,17 +805,44 @@ int ArenaEngine::recover_many(int count, const int* slots, double* const* outs, 
     if (count == 0) return LBM_OK;
     int rc = ensure_fields_buffer(std::max(need, std::min(all, kRecoverBlock)), err);
     if (rc) return rc;
-    for (int i = 0; i < count;) {
-        int j = i;
+    // small problems first, many to a copy
+    std::vector<int> small, large;
+    for (int i = 0; i < count; ++i) (probs_[slots[i]].n <= kSmallFields ? small : large).push_back(i);
+    for (size_t i = 0; i < small.size();) {
+        size_t j = i;
         int64_t used = 0;
-        for (; j < count && (j == i || used + 5 * probs_[slots[j]].n <= d_fields_cap_); ++j) {
-            ECK(launch_fields(slots[j], d_fields_ + used));
-            used += 5 * probs_[slots[j]].n;
+        for (; j < small.size() && used + 5 * probs_[slots[small[j]]].n <= std::min(kFieldStage, d_fields_cap_); ++j) {
+            ECK(launch_fields(slots[small[j]], d_fields_ + used));
+            used += 5 * probs_[slots[small[j]]].n;
+        }
+        if (h_fields_cap_ < used) {
+            if (h_fields_) cudaFreeHost(h_fields_);
+            h_fields_ = nullptr;
+            h_fields_cap_ = 0;
+            const int64_t cap = small.size() == j ? used : kFieldStage;
+            ECK(cudaMallocHost(&h_fields_, sizeof(double) * cap));
+            h_fields_cap_ = cap;
+        }
+        ECK(cudaMemcpyAsync(h_fields_, d_fields_, sizeof(double) * used, cudaMemcpyDeviceToHost, st_));
+        ECK(cudaStreamSynchronize(st_));
+        const double* from = h_fields_;
+        for (; i < j; ++i) {
+            const int64_t n = probs_[slots[small[i]]].n;
+            for (int f = 0; f < 5; ++f, from += n)
+                if (double* to = outs[5 * (int64_t)small[i] + f]) std::memcpy(to, from, sizeof(double) * n);
+        }
+    }
+    for (size_t i = 0; i < large.size();) {
+        size_t j = i;
+        int64_t used = 0;
+        for (; j < large.size() && (j == i || used + 5 * probs_[slots[large[j]]].n <= d_fields_cap_); ++j) {
+            ECK(launch_fields(slots[large[j]], d_fields_ + used));
+            used += 5 * probs_[slots[large[j]]].n;
         }
         int64_t off = 0;
-        for (int q = i; q < j; ++q) {
-            const int64_t n = probs_[slots[q]].n;
-            double* const* o = outs + 5 * (int64_t)q;
+        for (size_t q = i; q < j; ++q) {
+            const int64_t n = probs_[slots[large[q]]].n;
+            double* const* o = outs + 5 * (int64_t)large[q];
             for (int f = 0; f < 5;) {
                 int g = f + 1;
                 while (o[f] && g < 5 && o[g] == o[f] + (g - f) * n) ++g;

@@ -171,6 +171,8 @@ private:
     unsigned long long* d_stat_ = nullptr;   // per problem: max |g|, non-finite flag (ForceIn)
     double* d_fields_ = nullptr;      // FP64 staging: the caller's force, recovered fields
     int64_t d_fields_cap_ = 0;
+    double* h_fields_ = nullptr;      // pinned: recovered fields of small problems
+    int64_t h_fields_cap_ = 0;
     cudaGraphExec_t graph_[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
     bool graph_failed_[6] = {false, false, false, false, false, false};
     cudaEvent_t ev0_ = nullptr, ev1_ = nullptr;

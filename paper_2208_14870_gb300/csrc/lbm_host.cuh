@@ -24,6 +24,10 @@ namespace lbm {
 template <typename F>
 inline void host_parallel(size_t n, size_t grain, F f) {
     const size_t pieces = (n + grain - 1) / grain;
+    if (pieces <= 1) {
+        if (n) f(size_t(0), n);
+        return;
+    }
     std::atomic<size_t> next{0};
     auto work = [&] {
         for (size_t p; (p = next.fetch_add(1)) < pieces;) f(p * grain, std::min(n, (p + 1) * grain));

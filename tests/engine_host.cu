@@ -283,7 +283,7 @@ void server_force(bool fail) {
     EXPECT(lbm_server_create(size_t(64) << 20, 100, &s) == LBM_OK);
     if (fail) fake::fail_launch = 12;
     std::vector<Problem> p;
-    for (int i = 0; i < 6; ++i) p.emplace_back(40 + i, i < 2 ? 30 : 120);      // (small and large)
+    for (int i = 0; i < 6; ++i) p.emplace_back(40 + i, i < 4 ? 120 : 30);      // (large and small)
     std::vector<uint64_t> t;
     for (int i = 0; i < 6; ++i) {
         const lbm_problem in = p[i].in();
@@ -389,6 +389,36 @@ void small_forces(int dtype) {
     }
 }
 
+// Fields of many small problems come in few copies; each goes where its caller wants
+// it, and fields that nobody wants nowhere.
+void small_fields(int dtype) {
+    ArenaEngine e;
+    std::string err;
+    EXPECT(e.init(dtype, 400000, 128, 100, (cudaStream_t)&e, &err) == LBM_OK);
+    std::vector<int> slots;
+    std::vector<std::vector<double>> mem;
+    std::vector<double*> outs;
+    for (int i = 0; i < 100; ++i) {
+        const int nx = i == 50 ? 90 : 8 + i % 38, ny = i == 50 ? 80 : 45 - i % 37;
+        const std::vector<double> g((size_t)nx * ny, 1.0);
+        slots.push_back(e.admit(nx, ny, 0.3, 0.4, g.data(), g.data(), 0.0, 100, &err));
+        EXPECT(slots.back() >= 0);
+        mem.emplace_back(5 * g.size(), -7.0);
+        for (int f = 0; f < 5; ++f) outs.push_back((i + f) % 7 ? &mem.back()[f * g.size()] : nullptr);
+    }
+    EXPECT(e.run_chunk(kTileWave, nullptr, &err) == LBM_OK);
+    fake::calls = 0;
+    EXPECT(e.recover_many(100, slots.data(), outs.data(), &err) == LBM_OK);
+    EXPECT(fake::calls <= 100 + 2 * 2 + 6);        // (two blocks of small ones, the large one's fields)
+    for (int i = 0; i < 100; ++i) {
+        const int64_t n = e.prob(slots[i]).n;
+        for (int f = 0; f < 5; ++f) {
+            const int from = !e.prob(slots[i]).tr || f == 4 ? f : f ^ 1;      // (the transpose's field)
+            for (int64_t k = 0; k < n; ++k) EXPECT(mem[i][f * n + k] == (outs[5 * i + f] ? 1.0 + from : -7.0));
+        }
+    }
+}
+
 // The arena says what it holds on the device, and its forces and fields are staged in
 // one buffer.
 void staging(int dtype) {
@@ -489,6 +519,8 @@ int main(int argc, char** argv) {
     else if (what == "narrow_launches_f16s") narrow_launches(S_F16S);
     else if (what == "small_forces_f32") small_forces(S_F32);
     else if (what == "small_forces_f16s") small_forces(S_F16S);
+    else if (what == "small_fields_f32") small_fields(S_F32);
+    else if (what == "small_fields_f16s") small_fields(S_F16S);
     else if (what == "staging_f32") staging(S_F32);
     else if (what == "staging_f16s") staging(S_F16S);
     else if (what == "full_arena_f32") full_arena(S_F32);

@@ -24,7 +24,7 @@ def program(tmp_path_factory):
 @pytest.mark.parametrize("scenario", ["server_force", "server_force_failing", "server_device_ms", "server_recovery_fails",
                                       "staging_f32", "staging_f16s", "full_arena_f32", "full_arena_f16s", "pinned_parts_f32",
                                       "pinned_parts_f16s", "narrow_launches_f32", "narrow_launches_f16s",
-                                      "small_forces_f32", "small_forces_f16s"])
+                                      "small_forces_f32", "small_forces_f16s", "small_fields_f32", "small_fields_f16s"])
 def test_scenario(program, scenario, tmp_path):
     env = dict(os.environ, LBM_AUTOTUNE_CACHE=str(tmp_path / "autotune.txt"))
     r = subprocess.run([program, scenario], capture_output=True, text=True, timeout=120, env=env)
