@@ -107,6 +107,9 @@ typedef struct lbm_rates {
  * force, the displacement snapshot of the residual check and the reduction
  * scratch on the current device, and sets the state to the equilibrium of
  * u_0 = 0, i.e. all populations zero (Eq. init_cond), with zero force.
+ * LBM_F32 and LBM_F16S rows of 64 columns and more carry up to 23 further columns
+ * (the periodic images the strips read), unless the lattice fits the device only
+ * without them: it then advances on tiles, with the same states.
  * nx, ny >= 1; mu > 0; lambda + mu > 0; dtype one of lbm_dtype.
  * Errors: LBM_ERR_ARG, LBM_ERR_OOM, LBM_ERR_CUDA. */
 int lbm_create(int nx, int ny, double lambda, double mu, int dtype, lbm_ctx **out);

@@ -233,6 +233,10 @@ cudaError_t launch_step3(lbm_ctx* c) {
 
 bool wave_on(const lbm_ctx* c) { return c->wave != 0 && wave_fits(c->nx, c->ny); }
 
+// The wavefront schedule on register tiles: a lattice that fits the device only
+// without ghost columns (lbm_create_ex) has no strips.
+bool wave_tiles(const lbm_ctx* c) { return wave_on(c) && c->spl >= 3 && !c->ghost; }
+
 // Steps of a whole group of plain steps (groups_of).
 int group_steps(const lbm_ctx* c) { return c->spl >= 4 && wave_on(c) ? 4 : std::min(c->spl, 3); }
 
@@ -364,7 +368,7 @@ cudaError_t choose_plan(lbm_ctx* c) {
         const cudaError_t e = wave_shape(c, group, false, &sh);
         if (e != cudaSuccess) return e;
         if (sh.cost * c->tile.T < c->tile.cost * group) c->plan = 1;
-    } else if (c->dtype == LBM_F16S) {
+    } else if (c->dtype == LBM_F16S && group < 3) {
         // (one or two steps per launch: at most the start of a launch and the traffic)
         if ((6200.0 + 56.0 * (double)c->n / 3040.0) * c->tile.T < c->tile.cost * group) c->plan = 3;
     }
@@ -499,8 +503,9 @@ cudaError_t run_plain(lbm_ctx* c, int64_t n) {
     if (c->auto_plan) {
         e = choose_plan(c);
         if (e != cudaSuccess) return e;
-        if (c->plan == 2) return c->dtype == LBM_F32 ? run_tiles(c, n, false) : run_tiles16(c, n, 0);
     }
+    if ((c->auto_plan && c->plan == 2) || wave_tiles(c))
+        return c->dtype == LBM_F32 ? run_tiles(c, n, false) : run_tiles16(c, n, 0);
     if (auto_on(c) || (c->spl >= 4 && wave_on(c) && c->dtype == LBM_F32)) return run_strips(c, n);
     const Groups g = groups_of(c, n);
     for (int64_t i = 0; i < g.whole && e == cudaSuccess; ++i) e = launch_group(c, g.big);
@@ -516,22 +521,18 @@ cudaError_t run_plain(lbm_ctx* c, int64_t n) {
 cudaError_t run_window(lbm_ctx* c, int64_t to_check) {
     cudaError_t e;
     if (c->dtype == LBM_F64) return run_tiles64(c, to_check, true);
-    if (auto_on(c)) {
+    if (c->auto_plan) {
         e = choose_plan(c);
         if (e != cudaSuccess) return e;
-        if (c->plan == 2) return run_tiles(c, to_check, true);
-        if (to_check < 4) {
-            e = run_strips(c, to_check - 1);
-            return e == cudaSuccess ? launch_step(c, true) : e;
-        }
     }
-    if (auto16(c)) {
-        e = choose_plan(c);
-        if (e != cudaSuccess) return e;
-        if (c->plan == 2) {
-            const int last = to_check >= 4 && group_steps(c) == 4 ? 4 : (c->spl >= 2 && to_check >= 2 ? 2 : 1);
-            return run_tiles16(c, to_check - last, last);
-        }
+    if ((c->auto_plan && c->plan == 2) || wave_tiles(c)) {
+        if (c->dtype == LBM_F32) return run_tiles(c, to_check, true);
+        const int last = to_check >= 4 && group_steps(c) == 4 ? 4 : (c->spl >= 2 && to_check >= 2 ? 2 : 1);
+        return run_tiles16(c, to_check - last, last);
+    }
+    if (auto_on(c) && to_check < 4) {
+        e = run_strips(c, to_check - 1);
+        return e == cudaSuccess ? launch_step(c, true) : e;
     }
     if (to_check >= 4 && (auto_on(c) || (c->spl >= 4 && wave_on(c)))) {
         int T = 0;
@@ -615,17 +616,78 @@ int check_ctx(lbm_ctx* c) {
 }
 
 void free_all(lbm_ctx* c) {
+    auto drop = [](auto*& p) {
+        if (p) cudaFree(p);
+        p = nullptr;
+    };
     for (int i = 0; i < 2; ++i) {
-        if (c->pop[i]) cudaFree(c->pop[i]);
-        if (c->car[i]) cudaFree(c->car[i]);
+        drop(c->pop[i]);
+        drop(c->car[i]);
     }
-    if (c->force) cudaFree(c->force);
-    if (c->snap) cudaFree(c->snap);
-    if (c->partials) cudaFree(c->partials);
-    if (c->absmax) cudaFree(c->absmax);
-    if (c->bad) cudaFree(c->bad);
-    if (c->staging) cudaFree(c->staging);
+    drop(c->force);
+    drop(c->snap);
+    drop(c->partials);
+    drop(c->absmax);
+    drop(c->bad);
+    drop(c->staging);
     if (c->pinned) cudaFreeHost(c->pinned);
+    c->pinned = nullptr;
+    c->bytes = 0;
+}
+
+// The buffers of a context whose rows are laid out, cleared, and its plan.
+cudaError_t alloc_ctx(lbm_ctx* c) {
+    const int nx = c->nx, ny = c->ny, dtype = c->dtype;
+    c->plane = round_up((int64_t)c->pitch * ny, 128);
+    const int slack = c->ghost ? kRowSlack : 0;
+    const size_t pb = pop_elem_bytes(dtype) * (8 * c->plane + slack);
+    const size_t fb = force_elem_bytes(dtype) * (2 * c->plane + slack);
+    const size_t cb = sizeof(float) * 2 * (c->plane + slack);
+    auto alloc = [&](void** p, size_t bytes) -> cudaError_t {
+        cudaError_t r = cudaMalloc(p, bytes);
+        if (r == cudaSuccess) c->bytes += bytes;
+        return r;
+    };
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
+        e = alloc(&c->pop[i], pb);
+        if (e == cudaSuccess && dtype == LBM_F16S) e = alloc((void**)&c->car[i], cb);
+    }
+    if (e == cudaSuccess) e = alloc(&c->force, fb);
+    // FP64: two planes of doubles; FP32 / FP16S: two planes of (hi, lo) FP32 pairs
+    const size_t snap_bytes = 16 * (size_t)c->plane;
+    if (e == cudaSuccess) e = alloc(&c->snap, snap_bytes);
+    c->partials_len = std::max(c->nblocks, c->nblocks2);
+    if (e == cudaSuccess && c->ghost && (wave_on(c) || dtype == LBM_F32)) {
+        for (int T = 4; T <= (dtype == LBM_F32 ? 5 : 4) && e == cudaSuccess; ++T) {
+            StripShape sh;
+            e = wave_shape(c, T, true, &sh);
+            c->partials_len = std::max(c->partials_len, strip_check_blocks(c, T, sh.seg));
+        }
+    }
+    if (e == cudaSuccess && dtype != LBM_F64) {
+        e = choose_plan(c);
+        c->partials_len = std::max(c->partials_len, c->plan == 2 ? tile_count(c->tile, nx, ny) : int64_t(0));
+    }
+    if (e == cudaSuccess) e = alloc((void**)&c->partials, sizeof(double) * kRes * c->partials_len);
+    if (e == cudaSuccess) e = alloc((void**)&c->absmax, sizeof(unsigned long long));
+    if (e == cudaSuccess) e = alloc((void**)&c->bad, sizeof(unsigned int));
+    // host words the device writes and copies into: two of the force upload, then
+    // the result of the last check (written in place: a copy after it would
+    // cost every lbm_solve window 3 us more)
+    if (e == cudaSuccess) e = cudaMallocHost((void**)&c->pinned, sizeof(double) * (kRes + 2));
+    if (e == cudaSuccess) {
+        c->result = c->pinned + 2;
+        std::fill(c->result, c->result + kRes, 0.0);
+    }
+    if (e == cudaSuccess) e = cudaMemset(c->pop[0], 0, pb);
+    if (e == cudaSuccess) e = cudaMemset(c->pop[1], 0, pb);
+    if (e == cudaSuccess && dtype == LBM_F16S) e = cudaMemset(c->car[0], 0, cb);
+    if (e == cudaSuccess && dtype == LBM_F16S) e = cudaMemset(c->car[1], 0, cb);
+    if (e == cudaSuccess) e = cudaMemset(c->force, 0, fb);
+    if (e == cudaSuccess) e = cudaMemset(c->snap, 0, snap_bytes);
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    return e;
 }
 
 // FP16-shifted storage: scale exponent from the force (f16s_exponent).
@@ -781,9 +843,6 @@ int lbm_create_ex(int nx, int ny, double lambda, double mu, int dtype, const lbm
     c->ny = ny;
     c->dtype = dtype;
     c->n = (int64_t)nx * ny;
-    c->ghost = row_ghost(dtype, nx);
-    c->pitch = row_pitch(dtype, nx);
-    c->plane = round_up((int64_t)c->pitch * ny, 128);
     // Table 1 and Eq. relaxation_rate: theta tau_11 = mu, (1-theta)/2 tau_d = mu,
     // (1+theta)/2 tau_s = K = lambda + mu, w = 1/(tau + 1/2).
     const double K = lambda + mu;
@@ -820,54 +879,19 @@ int lbm_create_ex(int nx, int ny, double lambda, double mu, int dtype, const lbm
         else if (step2_fits(nx, ny)) c->spl = 2;
     }
 
-    const int slack = c->ghost ? kRowSlack : 0;
-    const size_t pb = pop_elem_bytes(dtype) * (8 * c->plane + slack);
-    const size_t fb = force_elem_bytes(dtype) * (2 * c->plane + slack);
-    const size_t cb = sizeof(float) * 2 * (c->plane + slack);
-    auto alloc = [&](void** p, size_t bytes) -> cudaError_t {
-        cudaError_t r = cudaMalloc(p, bytes);
-        if (r == cudaSuccess) c->bytes += bytes;
-        return r;
-    };
-    e = cudaSuccess;
-    for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
-        e = alloc(&c->pop[i], pb);
-        if (e == cudaSuccess && dtype == LBM_F16S) e = alloc((void**)&c->car[i], cb);
+    // Rows with ghost columns where strips may run; without them if the lattice fits
+    // the device only so (64 columns take a quarter more with them).
+    c->ghost = row_ghost(dtype, nx);
+    c->pitch = row_pitch(dtype, nx);
+    e = alloc_ctx(c);
+    if (e == cudaErrorMemoryAllocation && c->ghost) {
+        cudaGetLastError();
+        free_all(c);
+        c->ghost = 0;
+        c->pitch = nx;
+        c->plan = 0;
+        e = alloc_ctx(c);
     }
-    if (e == cudaSuccess) e = alloc(&c->force, fb);
-    // FP64: two planes of doubles; FP32 / FP16S: two planes of (hi, lo) FP32 pairs
-    const size_t snap_bytes = 16 * (size_t)c->plane;
-    if (e == cudaSuccess) e = alloc(&c->snap, snap_bytes);
-    c->partials_len = std::max(c->nblocks, c->nblocks2);
-    if (e == cudaSuccess && dtype != LBM_F64 && (wave_on(c) || (dtype == LBM_F32 && c->ghost))) {
-        for (int T = 4; T <= (dtype == LBM_F32 ? 5 : 4) && e == cudaSuccess; ++T) {
-            StripShape sh;
-            e = wave_shape(c, T, true, &sh);
-            c->partials_len = std::max(c->partials_len, strip_check_blocks(c, T, sh.seg));
-        }
-    }
-    if (e == cudaSuccess && dtype != LBM_F64) {
-        e = choose_plan(c);
-        c->partials_len = std::max(c->partials_len, c->plan == 2 ? tile_count(c->tile, nx, ny) : int64_t(0));
-    }
-    if (e == cudaSuccess) e = alloc((void**)&c->partials, sizeof(double) * kRes * c->partials_len);
-    if (e == cudaSuccess) e = alloc((void**)&c->absmax, sizeof(unsigned long long));
-    if (e == cudaSuccess) e = alloc((void**)&c->bad, sizeof(unsigned int));
-    // host words the device writes and copies into: two of the force upload, then
-    // the result of the last check (written in place: a copy after it would
-    // cost every lbm_solve window 3 us more)
-    if (e == cudaSuccess) e = cudaMallocHost((void**)&c->pinned, sizeof(double) * (kRes + 2));
-    if (e == cudaSuccess) {
-        c->result = c->pinned + 2;
-        std::fill(c->result, c->result + kRes, 0.0);
-    }
-    if (e == cudaSuccess) e = cudaMemset(c->pop[0], 0, pb);
-    if (e == cudaSuccess) e = cudaMemset(c->pop[1], 0, pb);
-    if (e == cudaSuccess && dtype == LBM_F16S) e = cudaMemset(c->car[0], 0, cb);
-    if (e == cudaSuccess && dtype == LBM_F16S) e = cudaMemset(c->car[1], 0, cb);
-    if (e == cudaSuccess) e = cudaMemset(c->force, 0, fb);
-    if (e == cudaSuccess) e = cudaMemset(c->snap, 0, snap_bytes);
-    if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
         int code = cuda_fail(e, "lbm_create: device allocation");
         free_all(c);
@@ -922,7 +946,7 @@ int lbm_get_launch_steps(lbm_ctx* c, int* k) {
     }
     *k = group_steps(c);
     if (c->auto_plan) CK(choose_plan(c));
-    if (c->auto_plan && c->plan == 2) *k = c->tile.T;
+    if ((c->auto_plan && c->plan == 2) || wave_tiles(c)) *k = c->tile.T;
     else if (c->dtype == LBM_F32 && (c->auto_plan || (c->spl >= 4 && wave_on(c)))) {
         CK(wave_plan(c));
         *k = *std::max_element(c->wave_first, c->wave_first + kWavePlan + 1);   // (wave_T among them)
