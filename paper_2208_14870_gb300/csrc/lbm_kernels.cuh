@@ -39,9 +39,6 @@ namespace lbm {
 #ifndef LBM_F16S_V
 #define LBM_F16S_V 2
 #endif
-#ifndef LBM_MINB_F64
-#define LBM_MINB_F64 3
-#endif
 constexpr int BY = LBM_BY;         // rows per block (block = 32 x BY threads)
 
 enum Storage { S_F64 = 0, S_F32 = 1, S_F16S = 2 };
@@ -716,7 +713,7 @@ __device__ __forceinline__ void step_tile(const StepParams& a,
 }
 
 template <int S, int V, bool GEN, bool CHECK>
-__global__ void __launch_bounds__(kThreads, CHECK ? 2 : (S == S_F32 ? LBM_MINB_F32 : (S == S_F16S ? LBM_MINB_F16S : LBM_MINB_F64)))
+__global__ void __launch_bounds__(kThreads, CHECK ? 2 : (S == S_F32 ? LBM_MINB_F32 : LBM_MINB_F16S))
 k_step(const StepParams a, const Coef<typename StoreT<S>::T> c) {
     after_predecessor();
     const int ntx = (a.nx + 32 * V - 1) / (32 * V);

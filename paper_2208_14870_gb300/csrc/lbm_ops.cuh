@@ -1,6 +1,6 @@
 // lbm_ops.cuh -- launchers of the per-storage kernels; included by exactly one
 // translation unit per storage type (lbm_step_f64.cu, lbm_step_f32.cu,
-// lbm_step_f16s.cu), which instantiates Ops<S> for its type.
+// lbm_step_f16s.cu), which instantiates Ops<S> for its type (FP64: without step).
 #pragma once
 
 #include <mutex>

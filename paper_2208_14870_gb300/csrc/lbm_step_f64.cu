@@ -2,7 +2,10 @@
 #include "lbm_ops.cuh"
 
 namespace lbm {
-template struct Ops<S_F64>;
+// (steps: tile_f64)
+template cudaError_t Ops<S_F64>::fields(const StepParams&, const Coef<double>&, double, const FieldOut&, cudaStream_t);
+template cudaError_t Ops<S_F64>::export_pop(const StepParams&, double, double*, cudaStream_t);
+template cudaError_t Ops<S_F64>::import_pop(const StepParams&, double, const double*, cudaStream_t);
 
 // blocks: of the launch (partial sets of a checked one)
 cudaError_t tile_f64(const StepParams& a, const Coef<double>& c, bool gen, const Tile64Shape& t, bool check,
