@@ -82,10 +82,9 @@ struct lbm_ctx {
     size_t bytes = 0;
     int64_t nblocks = 0;           // grid of the residual-check launch
     int spl = 1;                   // pseudo-time steps per stream-collide launch (1 to 4)
-    int wave = 0;                  // launches of three or four steps: 0 tile kernel, > 0 wavefront
+    int wave = 0;                  // launches of three or more steps: 0 tiles, > 0 strips in segments of so
+                                   // many rows, -1 strips in segments chosen per launch (strip_shape)
     int host_transfer = LBM_HOST_DIRECT;   // lbm_host_transfer
-                                   // kernel with segments of this many rows per block, -1 wavefront
-                                   // with the segment chosen per launch (wave_seg)
     int nsm = 0;                   // multiprocessors of the device
     int64_t nblocks2 = 0;          // grid of the two-step check launch
     StripShape shape[2][kStTMax + 1];   // strip launches per step count, plain and checked, cleared by lbm_set_wavefront

@@ -223,14 +223,14 @@ __device__ __forceinline__ void collide_populations(const Mom<T>& m, T gx, T gy,
 // that power of two, where FP64 arithmetic rounds at 2^-53 of each of its partial
 // sums.  A value far below the node's largest one has fewer bits than
 // FP64 would keep of it until it meets the others in a sum, and none from 2^-58
-// on.  The first moments of the result are mbar + g / 2 up to the last rounding.  About 600 integer instructions, two cycles of the ALU
-// for 360 of them, against 34 FP64 ones (2176 cycles): 1500 x 1100 116 -> 44 us
-// per step; with the signs on the FMA pipe 42.6, and with two, three, four, five,
-// six of the results on the FP64 pipe 40.8, 39.6, 38.7, 38.7, 44.0 us.
-// Nodes of infinities, NaN or values near the ends of the exponent range, and
+// on.  The first moments of the result are mbar + g / 2 up to the last rounding.
+// About 600 integer instructions, two cycles of the ALU for 360 of them, against 34
+// FP64 ones (2176 cycles): 1500 x 1100 116 -> 44 us per step; with the signs on the FMA
+// pipe 43.0, and with two, three, four, five, six of the results on the FP64 pipe
+// 40.2, 39.9, 37.8, 37.8, 41.6 us.  Nodes of infinities, NaN or values near the ends of the exponent range, and
 // rates with a factor of 1/2 or more, take FP64 arithmetic.
-// m (below 2^63) with the sign of the word w.  FMA: most of the work on the FMA pipe (a multiplication by the sign) instead
-// of the ALU, which bounds the step where many warps share a scheduler; slower
+// m (below 2^63) with the sign of the word w.  FMA: most of the work on the FMA pipe
+// (a multiplication by the sign) instead of the ALU, which bounds the step where many warps share a scheduler; slower
 // where one warp runs alone.
 template <bool FMA>
 __device__ __forceinline__ int64_t signed_as(uint64_t m, int w) {

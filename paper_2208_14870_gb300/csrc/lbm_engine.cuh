@@ -158,7 +158,7 @@ private:
     int pairs_grid_ = 0;                              // most blocks of the pairs' launch
     int strip_blocks_ = 0;                            // largest launch so far
     int ghosts_begin_ = 0, ghosts_end_ = 0;           // ... and of the problems whose ghost columns are stale
-    cudaStream_t side_[kClasses - 1] = {};   // the classes run side by side
+    cudaStream_t side_[kClasses - 1] = {};   // strips and narrow problems run side by side
     cudaEvent_t fork_ = nullptr, join_[kClasses - 1] = {};
     uint2* h_tiles_ = nullptr;        // pinned
     int64_t h_tiles_cap_ = 0;

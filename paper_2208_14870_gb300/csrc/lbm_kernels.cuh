@@ -861,8 +861,8 @@ k_tile64(const StepParams a, const Coef<double> c, const __grid_constant__ Tile6
 }
 
 // One step per launch of FP64 storage (lattices of some 200 x 200 nodes and more):
-// blocks of 32 x 4 nodes.  1500 x 1100: 38.7 us per step, 238 MB of populations
-// and force at 6.1 TB/s (with 64-bit tile divisions and
+// blocks of 32 x 4 nodes.  1500 x 1100: 37.8 us per step, 238 MB of populations
+// and force at 6.3 TB/s (with 64-bit tile divisions and
 // addresses 47; on the FP64 pipe 116, with tiles of 64 x 8 137).
 constexpr int kOne64Rows = 4;
 template <bool GEN, bool CHECK>
@@ -1268,9 +1268,10 @@ template <int S, int T> __host__ __device__ constexpr int st_ox() {
 // warps per block; the kernel is compiled for three resident blocks, twelve
 // warps per SM (168 registers a thread; at 16384^2 with registers for eight warps
 // 87.6 ms per 100 steps against 79.8).  With the check for two: at 168 registers
-// it spilled, and its partials were combined in FP64 (T = 5 at 16384^2 6.20 ms,
-// at 1024^2 39.8 us; with two blocks 5.72 and 35.6, and pairs combined as pairs
-// 5.45 and 32.3; FP16S 1000 x 700 28.1 -> 25.1 us, 8192^2 1.45 -> 1.48 ms)
+// it spilled, and every thread's partials were converted (T = 5 at 16384^2 6.20 ms,
+// at 1024^2 39.8 us; with two blocks 5.72 and 35.6).  As ResPart combines them, and
+// with k_residual_finish: 5.52 ms and 35.9 us (sums as pairs 5.46 and 35.5); FP16S
+// 1000 x 700 28.8 us, 8192^2 1.40 ms
 constexpr int kStNW = 4;
 // rows copied ahead of the rows in use, and population rows held: FP32 has the
 // rows above, at and below level 1 in use, FP16S the decoded row
