@@ -356,7 +356,9 @@ const char *lbm_last_error(void);
  * advances every problem by a group of steps per launch (LBM_F32 five, LBM_F16S
  * four) on the schedule of lbm_set_wavefront, one warp per strip of 56 output
  * columns and segment of rows; problems narrower than 16 columns take pairs of
- * steps on two-step tiles.  The other tile codes run a chunk as one cooperative
+ * steps on two-step tiles, in one launch per chunk.  Rows of 16 columns and more
+ * take up to 23 further columns of arena memory (periodic images) where the arena
+ * can hold the problem so.  The other tile codes run a chunk as one cooperative
  * kernel, replayed from a CUDA graph, that walks the tiles of all running
  * problems with grid-wide barriers: tiles 32, 64 or 128 columns wide (tile code
  * 1, 2, 4: warps of 32 columns, one step per barrier) or, when check_every is
