@@ -52,12 +52,12 @@ FORCE_SEED = 0x2208_14870
 # Captured at 8192 x 4096 (profiles/k_strip_dram_traffic.md) and scaled by the
 # nodes to 16384^2:
 NCU_TRAFFIC = {
-    "f32_x6w": {"bytes_per_launch": 8 * (1.448233e9 + 1.039082e9), "kernel_hash": "3a0b8c7c1b3e86e5",
-                "ncu": {"case": "8192 x 4096, x8", "dram_read_per_launch": 8 * 1.448233e9,
-                        "dram_write_per_launch": 8 * 1.039082e9, "algorithmic_per_launch": 72 * 16384 ** 2}},
-    "f16s_x4w": {"bytes_per_launch": 8 * (1.137914e9 + 0.772039e9), "kernel_hash": "3a0b8c7c1b3e86e5",
-                 "ncu": {"case": "8192 x 4096, x8", "dram_read_per_launch": 8 * 1.137914e9,
-                         "dram_write_per_launch": 8 * 0.772039e9, "algorithmic_per_launch": 56 * 16384 ** 2}},
+    "f32_x6w": {"bytes_per_launch": 8 * (1.447921e9 + 1.038954e9), "kernel_hash": "7ffac5f12813b451",
+                "ncu": {"case": "8192 x 4096, x8", "dram_read_per_launch": 8 * 1.447921e9,
+                        "dram_write_per_launch": 8 * 1.038954e9, "algorithmic_per_launch": 72 * 16384 ** 2}},
+    "f16s_x4w": {"bytes_per_launch": 8 * (1.138100e9 + 0.772273e9), "kernel_hash": "7ffac5f12813b451",
+                 "ncu": {"case": "8192 x 4096, x8", "dram_read_per_launch": 8 * 1.138100e9,
+                         "dram_write_per_launch": 8 * 0.772273e9, "algorithmic_per_launch": 56 * 16384 ** 2}},
 }
 
 

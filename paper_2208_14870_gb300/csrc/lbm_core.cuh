@@ -356,7 +356,9 @@ __device__ __forceinline__ void step_f64(const double f[8], double gx, double gy
 // component w of the displacement.  The bits are step_f64's.  Every lane of the
 // warp calls it.  (No signs on the FMA pipe and no results on the FP64 pipe: with
 // one or two warps per scheduler both only lengthen the chain, 64 x 64 1.34
-// against 1.41 us per step.)
+// against 1.41 us per step.  Nor are nodes of zeros told apart: 64 x 64 with one
+// forced node, twelve steps, 37 -> 17 us, but every other launch lost 0.4 to 1.4 %, and a
+// small lattice is filled within some tens of steps.)
 template <bool GEN>
 __device__ __forceinline__ void step_f64_half(const double f[4], double g, int h, const Coef<double>& c, double& w,
                                               double o[4]) {
@@ -391,16 +393,6 @@ __device__ __forceinline__ void step_f64_half(const double f[4], double g, int h
     o[3] = from_fixed<false>(Xs - Z, e);
     w = from_fixed<false>(U, e);
     if (__any_sync(ALL, slow)) {
-        uint32_t any = nonzero(g);
-#pragma unroll
-        for (int p = 0; p < 4; ++p) any |= nonzero(f[p]);
-        any |= __shfl_xor_sync(ALL, any, 1);
-        if (any == 0) {
-            w = 0.0;
-#pragma unroll
-            for (int p = 0; p < 4; ++p) o[p] = 0.0;
-        }
-        if (!__any_sync(ALL, slow && any)) return;
         double a[8], gx = __shfl_xor_sync(ALL, g, 1), gy = gx, u, v, r[8];
         if (h) gy = g;
         else gx = g;
@@ -410,7 +402,7 @@ __device__ __forceinline__ void step_f64_half(const double f[4], double g, int h
             a[2 * p] = h ? q : f[p];
             a[2 * p + 1] = h ? f[p] : q;
         }
-        if (slow && any) {
+        if (slow) {
             collide_populations<GEN>(moments(a), gx, gy, c, u, v, r);
 #pragma unroll
             for (int p = 0; p < 4; ++p) o[p] = h ? r[2 * p + 1] : r[2 * p];
